@@ -422,9 +422,7 @@ static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_
         if (h->ctomb_bound > h->col_cap / 4) {
             drsf_status st = read_ctl(h, s);
             if (st) return st;
-            // deleted CSR entries = 2 * (deleted edges) - bounded by the
-            // index tombstones (each deleted edge frees two CSR entries)
-            long long ct = 2 * h->ctl_host->htomb + h->ctl_host->ctomb;
+            long long ct = h->ctl_host->ctomb;
             h->ctomb_bound = ct;
             if (ct > h->col_cap / 4) {
                 st = rebuild(h, s, len);

@@ -248,11 +248,11 @@ template <int BT>
 __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long long b0, long long b1) {
     Ctl *ctl = S.ctl;
     BLocal *L = G.L;
-    if (G.tid == 0) L->cnt[0] = L->cnt[1] = L->cnt[2] = 0;
+    if (G.tid == 0) L->cnt[0] = L->cnt[1] = L->cnt[2] = L->cnt[3] = 0;
     gsync();
     // normalisation and index claim: self-loops, repeats and existing edges
     // are dropped; kept keys go to the graph's slice of nkey / nslot
-    int loops = 0, drops = 0;
+    int loops = 0, drops = 0, reuse = 0;
     for (long long i = b0 + G.tid; i < b1; i += G.stride) {
         const int u = d.batch[2 * i], v = d.batch[2 * i + 1];
         if (u == v) {
@@ -260,7 +260,9 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
             continue;
         }
         const u64 key = ekey((uint32_t)u, (uint32_t)v);
-        const long long s = index_claim(S.ix, key);
+        bool reused = false;
+        const long long s = index_claim(S.ix, key, &reused);
+        reuse += reused;
         if (s == LLONG_MIN) atomicOr(&ctl->err, ERR_CAPACITY);
         if (s >= 0) {
             const int p = gappend(&L->cnt[0]);
@@ -272,6 +274,7 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
     }
     gadd(G, 1, loops);
     gadd(G, 2, drops);
+    gadd(G, 3, reuse);
     gsync();
     const int nb = L->cnt[0];
     // CSR append (or overflow) and the cross test rep[u] != rep[v]
@@ -313,6 +316,7 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
         atomicAdd((u64 *)&ctl->edges, (u64)nb);
         atomicAdd((u64 *)&ctl->self_loops, (u64)L->cnt[1]);
         atomicAdd((u64 *)&ctl->dropped, (u64)L->cnt[2]);
+        atomicAdd((u64 *)&ctl->htomb, (u64)(-(long long)L->cnt[3]));
     }
 }
 
@@ -327,7 +331,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
     if (G.tid == 0) L->cnt[0] = L->cnt[1] = L->cnt[2] = L->cnt[3] = L->cnt[4] = L->cnt[5] = 0;
     gsync();
     // normalisation, removal and the cut of deleted tree edges
-    int loops = 0, drops = 0, wins = 0, cuts = 0;
+    int loops = 0, drops = 0, wins = 0, cuts = 0, dead = 0;
     for (long long i = b0 + G.tid; i < b1; i += G.stride) {
         const int u = d.batch[2 * i], v = d.batch[2 * i + 1];
         if (u == v) {
@@ -351,6 +355,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         } else {
             S.g.col[pu] = -1;
             S.g.col[pv] = -1;
+            dead += 2;
         }
         int c = -1, rc = -1;
         if (par_u == v) {
@@ -371,12 +376,14 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
     gadd(G, 2, drops);
     gadd(G, 0, wins);
     gadd(G, 3, cuts);
+    gadd(G, 4, dead);
     gsync();
     const int nwin = L->cnt[0], ncut = L->cnt[3];
     if (G.tid == 0) {
         atomicAdd(&ctl->nb, (u64)nwin);
         atomicAdd((u64 *)&ctl->edges, (u64)(-(long long)nwin));
         atomicAdd((u64 *)&ctl->htomb, (u64)nwin);
+        atomicAdd((u64 *)&ctl->ctomb, (u64)L->cnt[4]);
         atomicAdd(&ctl->ncut, (u64)ncut);
         atomicAdd((u64 *)&ctl->self_loops, (u64)L->cnt[1]);
         atomicAdd((u64 *)&ctl->dropped, (u64)L->cnt[2]);

@@ -67,7 +67,7 @@ struct Ctl {
     u64 ovf_count;          // overflow list length (grows until rebuild)
     long long edges;        // live undirected edges of G
     long long htomb;        // index tombstones
-    long long ctomb;        // CSR tombstones (deleted entries)
+    long long ctomb;        // dead CSR entries (deleted ones, and slots lost to overflow edges)
     long long scanned;      // adjacency entries scanned
     long long self_loops;
     long long dropped;
@@ -121,15 +121,33 @@ __device__ __forceinline__ u64 hslot(u64 k, u64 mask) {
 // Edge index probes (open addressing, linear probing).
 // Insert-if-absent.  Returns the slot when this call claimed it, -1-slot
 // when the key was already present, LLONG_MIN when the table is full.
-__device__ __forceinline__ long long index_claim(Index ix, u64 key) {
+// The claimed slot is the first deleted or empty one of the key's chain, and
+// it is claimed only after the whole chain was seen without the key
+// (*reused tells that it was a deleted one).  While keys are being inserted
+// slots only go from deleted or empty to a key, so two threads with one key
+// meet: a thread whose slot was taken meanwhile looks at the chain again
+// from that slot on, and finds the key the other one wrote there or further
+// along.  Without the reuse an edge that comes back leaves one more deleted
+// slot in its own chain every time: after 1,500 removals of each edge of a
+// 100-edge batch the claim took 1,115 us (R-MAT scale 22) instead of 16.
+__device__ __forceinline__ long long index_claim(Index ix, u64 key, bool *reused) {
     u64 s = hslot(key, ix.mask);
-    for (u64 p = 0; p <= ix.mask; ++p) {
-        u64 cur = __ldcg(&ix.key[s]);
+    long long free_slot = -1;   // first deleted slot of the chain
+    for (u64 p = 0; p <= 2 * ix.mask; ++p) {
+        const u64 cur = __ldcg(&ix.key[s]);
         if (cur == key) return -1 - (long long)s;
+        if (cur == TOMB_KEY && free_slot < 0) free_slot = (long long)s;
         if (cur == EMPTY_KEY) {
-            u64 old = atomicCAS(&ix.key[s], EMPTY_KEY, key);
-            if (old == EMPTY_KEY) return (long long)s;
-            if (old == key) return -1 - (long long)s;
+            const bool dead = free_slot >= 0;
+            const u64 t = dead ? (u64)free_slot : s;
+            const u64 old = atomicCAS(&ix.key[t], dead ? TOMB_KEY : EMPTY_KEY, key);
+            if (old == (dead ? TOMB_KEY : EMPTY_KEY)) {
+                *reused = dead;
+                return (long long)t;
+            }
+            if (old == key) return -1 - (long long)t;
+            s = t;   // another key took the slot
+            free_slot = -1;
         }
         s = (s + 1) & ix.mask;
     }

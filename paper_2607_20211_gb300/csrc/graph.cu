@@ -36,7 +36,8 @@ __global__ void k_create_claim(const int *edges, long long m, Index ix, u64 *dke
         long long s = -1;
         if (u != v) {
             key = ekey((uint32_t)u, (uint32_t)v);
-            s = index_claim(ix, key);
+            bool reused = false;
+            s = index_claim(ix, key, &reused);
             keep = s >= 0;
         }
         agg_count(self_loops, u == v);
@@ -171,7 +172,7 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
     const long long len = ctl->batch_len;
     // block-uniform loop: counters and the list append are aggregated per
     // block (one atomic per block instead of one per warp)
-    long long loops = 0, drops = 0;
+    long long loops = 0, drops = 0, reuse = 0;
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < len; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
         bool keep = false;
@@ -181,9 +182,11 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
             int u = batch[2 * i], v = batch[2 * i + 1];
             if (u != v) {
                 key = ekey((uint32_t)u, (uint32_t)v);
-                s = index_claim(ix, key);
+                bool reused = false;
+                s = index_claim(ix, key, &reused);
                 if (s == LLONG_MIN) atomicOr(&ctl->err, ERR_CAPACITY);
                 keep = s >= 0;
+                reuse += reused;
                 drops += !keep;
             } else {
                 ++loops;
@@ -197,6 +200,7 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
     }
     block_add(&ctl->self_loops, loops);
     block_add(&ctl->dropped, drops);
+    block_add(&ctl->htomb, -reuse);
 }
 
 // Insert, step 2: append each new edge to both CSR rows (warp-aggregated
@@ -285,7 +289,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
     unsigned ep = ctl->epoch;
     // block-uniform loop: counters and the cut list append are aggregated
     // per block (one atomic per block instead of one per warp)
-    long long loops = 0, drops = 0, wins = 0;
+    long long loops = 0, drops = 0, wins = 0, dead = 0;
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < len; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
         int c = -1, rc = -1;
@@ -307,6 +311,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                     } else {
                         g.col[pu] = -1;
                         g.col[pv] = -1;
+                        dead += 2;
                     }
                     if (par_u == v) {
                         c = u;
@@ -344,6 +349,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
     block_add(&ctl->self_loops, loops);
     block_add(&ctl->dropped, drops);
     block_add(&ctl->htomb, wins);
+    block_add(&ctl->ctomb, dead);
     block_add(&ctl->edges, -wins);
     block_add((long long *)&ctl->nb, wins);
 }
