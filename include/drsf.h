@@ -176,7 +176,7 @@ DRSF_API drsf_status drsf_set_allocator(drsf_alloc_fn alloc, drsf_free_fn free_f
  *   flags   DRSF_DETERMINISTIC | DRSF_VALIDATE | DRSF_EULER_REVERSAL |
  *           DRSF_REPL_SG | DRSF_REPL_HS
  *   out     receives the handle (NULL on failure)
- * The graph is stored as a slack CSR (int64 row offsets, int32 columns) with
+ * The graph is stored as a slack CSR (16-byte row heads, int32 columns) with
  * an open-addressing edge index for O(1) deletion.  Synchronises the stream
  * once (to size the CSR).  Without DRSF_VALIDATE, an F that is not a rooted
  * spanning forest of G gives undefined (but memory-safe) results.

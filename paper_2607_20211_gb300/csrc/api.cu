@@ -51,8 +51,8 @@ struct drsf_ctx {
     // forest
     int *parent = nullptr, *rep = nullptr;
     // graph
-    long long *off = nullptr;
-    int *used = nullptr, *col = nullptr;
+    Row *row = nullptr;
+    int *col = nullptr, *fpos = nullptr;
     long long col_cap = 0;
     Index ix{};
     u64 H = 0;
@@ -241,8 +241,10 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     u64 *dkey = nullptr, *dslot = nullptr, *cnt = nullptr;
     long long *tmp64 = nullptr, *bs = nullptr;
     int *deg = nullptr;
+    int2 *place = nullptr;
     CKA(halloc(h, &dkey, (size_t)std::max<long long>(m, 1), s));
     CKA(halloc(h, &dslot, (size_t)std::max<long long>(m, 1), s));
+    CKA(halloc(h, &place, (size_t)std::max<long long>(m, 1), s));
     CKA(halloc(h, &cnt, 4, s));
     CKA(halloc(h, &deg, (size_t)n, s));
     CKA(halloc(h, &tmp64, (size_t)n + 1, s));
@@ -255,7 +257,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     CK(cudaMemcpyAsync(hc, cnt, 2 * sizeof(u64), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     long long m2 = (long long)hc[0];
-    CK(launch_degree(dkey, m2, deg, s));
+    CK(launch_degree(dkey, m2, deg, place, s));
     CK(launch_caps(deg, n, tmp64, s));
     long long *off = nullptr;
     CKA(halloc(h, &off, (size_t)n + 1, s));
@@ -264,13 +266,16 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     CK(cudaMemcpyAsync(&total, off + n, sizeof(long long), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (total >= (long long)POS_OVF - 1) return DRSF_ENOMEM;   // positions are 32-bit
-    int *col = nullptr, *used = nullptr;
+    int *col = nullptr, *fpos = nullptr;
+    Row *row = nullptr;
     CKA(halloc(h, &col, (size_t)total, s));
-    CKA(halloc(h, &used, (size_t)n, s));
+    CKA(halloc(h, &fpos, (size_t)total, s));
+    CKA(halloc(h, &row, (size_t)n + 1, s));
     CK(cudaMemsetAsync(col, 0xFF, (size_t)total * sizeof(int), s));
-    CK(cudaMemsetAsync(used, 0, (size_t)n * sizeof(int), s));
-    Csr g{off, used, col};
-    CK(launch_fill(dkey, dslot, m2, g, ix, s));
+    CK(cudaMemsetAsync(fpos, 0xFF, (size_t)total * sizeof(int), s));
+    CK(launch_rows_init(off, deg, n, row, s));
+    Csr g{row, col, fpos};
+    CK(launch_fill(dkey, dslot, place, m2, g, ix, s));
     u64 ovf_cap = std::max<u64>(std::max<u64>(1u << 16, (u64)m2 / 16), (u64)(2 * extra));
     u64 *ovf = nullptr;
     CKA(halloc(h, &ovf, ovf_cap, s));
@@ -301,22 +306,24 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     hfree(h, &h->ix.key, s);
     hfree(h, &h->ix.pu, s);
     hfree(h, &h->ix.pv, s);
-    hfree(h, &h->off, s);
+    hfree(h, &h->row, s);
     hfree(h, &h->col, s);
-    hfree(h, &h->used, s);
+    hfree(h, &h->fpos, s);
     hfree(h, &h->ovf, s);
     h->ix = ix;
     h->H = H;
-    h->off = off;
+    h->row = row;
     h->col = col;
-    h->used = used;
+    h->fpos = fpos;
     h->col_cap = total;
     h->ovf = ovf;
     h->ovf_cap = ovf_cap;
     hfree(h, &dkey, s);
     hfree(h, &dslot, s);
+    hfree(h, &place, s);
     hfree(h, &cnt, s);
     hfree(h, &deg, s);
+    hfree(h, &off, s);
     hfree(h, &tmp64, s);
     hfree(h, &bs, s);
     h->occ_bound = m2;
@@ -370,7 +377,7 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     CKA(halloc(h, &tmp, (size_t)std::max<long long>(2 * live, 2), s));
     CKA(halloc(h, &cnt, 2, s));
     CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(u64), s));
-    Csr g{h->off, h->used, h->col};
+    Csr g{h->row, h->col, h->fpos};
     CK(launch_extract(h->dev, h->n, g, h->ovf, h->ovf_cap, h->ctl, tmp, live, cnt, s));
     u64 hc[2];
     CK(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s));
@@ -559,7 +566,7 @@ static drsf_status create_impl(drsf_ctx *h, const int32_t *edges, int64_t m, con
     if (st) return st;
     CK(cudaMemcpyAsync(h->parent, parent, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, s));
     // representatives of F by pointer jumping over all vertices
-    Csr g0{h->off, h->used, h->col};
+    Csr g0{h->row, h->col, h->fpos};
     CK(launch_jump(h->dev, nullptr, 0, n, h->ctl, h->parent, h->J0, h->J1, h->rep, rows(h), 0, h->rold, h->wgt,
                    h->heavy, g0, h->jump_sync == 2 ? 1 : h->jump_sync, h->act, h->xlist, h->cutlist, s));
     Ctl c{};
@@ -576,7 +583,7 @@ static drsf_status create_impl(drsf_ctx *h, const int32_t *edges, int64_t m, con
         CKA(halloc(h, &el, (size_t)std::max<long long>(2 * m2, 2), s));
         CKA(halloc(h, &cnt, 2, s));
         CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(u64), s));
-        Csr g{h->off, h->used, h->col};
+        Csr g{h->row, h->col, h->fpos};
         CK(launch_extract(h->dev, n, g, h->ovf, h->ovf_cap, h->ctl, el, m2, cnt, s));
         CK(launch_check_cross(el, m2, h->rep, bad, s));
         CK(cudaMemcpyAsync(hb, bad, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -678,7 +685,7 @@ static bool use_supergraph(const drsf_ctx *h, int op, long long len) {
 // sequence serves every batch with the same key.
 static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cudaStream_t s) {
     Ctl *ctl = h->ctl;
-    Csr g{h->off, h->used, h->col};
+    Csr g{h->row, h->col, h->fpos};
     CK(launch_validate_batch(glen, h->n, ctl, s));
     prof_end(h, PH_BEGIN, 2, s);
     if (op == DRSF_INSERT) {
@@ -960,7 +967,7 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
         CKA(halloc(h, &b.pb, need, s));
         b.pool_cap = need;
     }
-    // tiles of the scanned rows: graph g's start at off[first vertex] / 32 + g
+    // tiles of the scanned rows: graph g's start at row[first vertex].start / 32 + g
     const long long ntile = h->col_cap / 32 + G + 2;
     if (ntile > h->b_tile_cap) {
         CK(cudaStreamSynchronize(s));
@@ -1046,7 +1053,7 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     b.ctl = h->ctl;
     b.parent = h->parent;
     b.rep = h->rep;
-    b.g = Csr{h->off, h->used, h->col};
+    b.g = Csr{h->row, h->col, h->fpos};
     b.ix = h->ix;
     b.ovf = h->ovf;
     b.ovf_cap = h->ovf_cap;
@@ -1271,7 +1278,7 @@ drsf_status drsf_export_edges(drsf_handle h, int32_t *out, int64_t cap, int64_t 
     u64 *cnt = nullptr;
     CKA(halloc(h, &cnt, 2, s));
     CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(u64), s));
-    Csr g{h->off, h->used, h->col};
+    Csr g{h->row, h->col, h->fpos};
     CK(launch_extract(h->dev, h->n, g, h->ovf, h->ovf_cap, h->ctl, out, cap, cnt, s));
     u64 hc[2];
     CK(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s));
@@ -1330,7 +1337,7 @@ drsf_status drsf_static_forest(drsf_handle h, int32_t *parent_out, int32_t *labe
     cudaStream_t s = (cudaStream_t)stream;
     int *comp = labels_out ? labels_out : h->pold;
     u64 *levels = (u64 *)h->bsum;   // scratch word
-    Csr g{h->off, h->used, h->col};
+    Csr g{h->row, h->col, h->fpos};
     CK(launch_static_forest(h->dev, h->n, g, h->ovf, h->ctl, h->J1, comp, parent_out, h->act, h->xlist, levels,
                             s));
     if (levels_out) {

@@ -248,7 +248,7 @@ template <int BT>
 __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long long b0, long long b1) {
     Ctl *ctl = S.ctl;
     BLocal *L = G.L;
-    if (G.tid == 0) L->cnt[0] = L->cnt[1] = L->cnt[2] = L->cnt[3] = 0;
+    if (G.tid == 0) L->cnt[0] = L->cnt[1] = L->cnt[2] = L->cnt[3] = L->cnt[4] = 0;
     gsync();
     // normalisation and index claim: self-loops, repeats and existing edges
     // are dropped; kept keys go to the graph's slice of nkey / nslot
@@ -277,6 +277,7 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
     gadd(G, 3, reuse);
     gsync();
     const int nb = L->cnt[0];
+    long long hole = 0;
     // CSR append (or overflow) and the cross test rep[u] != rep[v]
     for (int j0 = 0; j0 < nb; j0 += G.stride) {
         if (!pool_ensure(G, S, G.stride)) return;
@@ -285,15 +286,15 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
             const u64 k = GL(S.nkey[b0 + j]);
             const u64 s = GL(S.nslot[b0 + j]);
             const uint32_t a = klo(k), b = khi(k);
-            const long long oa = S.g.off[a], ob = S.g.off[b];
-            const long long capa = S.g.off[a + 1] - oa, capb = S.g.off[b + 1] - ob;
-            const int pa = row_slot(S.g.used, (int)a), pb = row_slot(S.g.used, (int)b);
-            const bool fa = pa < capa, fb = pb < capb;
-            if (fa && fb) {
-                S.g.col[oa + pa] = (int)b;
-                S.g.col[ob + pb] = (int)a;
-                S.ix.pu[s] = (uint32_t)(oa + pa);
-                S.ix.pv[s] = (uint32_t)(ob + pb);
+            const Row ha = row_head(S.g, (int)a), hb = row_head(S.g, (int)b);
+            const int pa = row_take(S.g, (int)a, ha, &hole), pb = row_take(S.g, (int)b, hb, &hole);
+            if (pa >= 0 && pb >= 0) {
+                const unsigned qa = ha.start + (unsigned)pa, qb = hb.start + (unsigned)pb;
+                S.g.col[qa] = (int)b;
+                S.g.col[qb] = (int)a;
+                S.ix.pu[s] = qa;
+                S.ix.pv[s] = qb;
+                hole -= 2;
             } else {
                 const u64 o = atomicAdd(&ctl->ovf_count, 1ull);
                 if (o < S.ovf_cap) {
@@ -304,14 +305,15 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
                     atomicOr(&ctl->err, ERR_CAPACITY);
                 }
                 atomicAdd((u64 *)&ctl->overflow_total, 1ull);
-                if (fa || fb) atomicAdd((u64 *)&ctl->ctomb, 1ull);
             }
             const int ra = GL(S.rep[a]), rb = GL(S.rep[b]);
             if (ra != rb) pool_put(G, S, k, ra, rb);
         }
     }
+    gadd(G, 4, (int)hole);
     gsync();
     if (G.tid == 0) {
+        atomicAdd((u64 *)&ctl->ctomb, (u64)(long long)L->cnt[4]);
         atomicAdd(&ctl->nb, (u64)nb);
         atomicAdd((u64 *)&ctl->edges, (u64)nb);
         atomicAdd((u64 *)&ctl->self_loops, (u64)L->cnt[1]);
@@ -353,8 +355,9 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         if (pu == POS_OVF) {
             S.ovf[pv] = TOMB_KEY;
         } else {
-            S.g.col[pu] = -1;
-            S.g.col[pv] = -1;
+            const int lo = (int)klo(key), hi = (int)khi(key);
+            row_give(S.g, lo, S.g.row[lo].start, pu);
+            row_give(S.g, hi, S.g.row[hi].start, pv);
             dead += 2;
         }
         int c = -1, rc = -1;
@@ -433,23 +436,22 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         const int rn = GL(S.R[v]);
         S.rep[v] = rn;
         // rows with no entries are left out of the row list
-        if (GL(S.st_cut[rn]) == ep && GL(S.g.used[v]) > 0) S.Dv[v0 + gappend(&L->cnt[4])] = v;
+        if (GL(S.st_cut[rn]) == ep && GL(S.g.row[v].used) > 0) S.Dv[v0 + gappend(&L->cnt[4])] = v;
     }
     gsync();
     const int nd = L->cnt[4];
-    // row lengths -> entry offsets (group scan in chunks); a row's append
-    // cursor passes its capacity when edges went to the overflow list.  The
+    // row lengths -> entry offsets (group scan in chunks).  The
     // flattened entries are cut into tiles of 32; each tile records the row
-    // of its first entry (tiles of graph g start at off[v0] / 32 + g, so the
+    // of its first entry (tiles of graph g start at row[v0].start / 32 + g, so the
     // graphs' tile ranges do not overlap).
-    const long long tb = (S.g.off[v0] >> 5) + g;
+    const long long tb = (S.g.row[v0].start >> 5) + g;
     int run = 0;
     for (int k0 = 0; k0 < nd; k0 += G.stride) {
         const int k = k0 + G.tid;
         int len = 0;
         if (k < nd) {
             const int v = GL(S.Dv[v0 + k]);
-            len = min(GL(S.g.used[v]), (int)(S.g.off[v + 1] - S.g.off[v]));
+            len = GL(S.g.row[v].used);
         }
         int tot = 0;
         const int ex = grp_excl<BT>(G, len, &tot);
@@ -491,7 +493,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
             const bool wok = wr < nd;
             const int wo = wok ? GL(S.roff[v0 + wr]) : INT_MAX;
             const int wv = wok ? GL(S.Dv[v0 + wr]) : 0;
-            const long long wb = wok ? S.g.off[wv] : 0;
+            const long long wb = wok ? S.g.row[wv].start : 0;
             const int wp = wok ? GL(S.rep[wv]) : 0;
             const int t0 = T << 5;
             // rows after the first that start inside the tile mark their

@@ -2,10 +2,10 @@
 //
 // Device state layout (all in HBM, one copy per handle):
 //   parent[n], rep[n]           int32   the forest and each vertex's tree root
-//   off[n+1]                    int64   slack-CSR row starts (row capacity =
-//                                       off[u+1] - off[u])
-//   used[n]                     int32   append cursor of each row
-//   col[off[n]]                 int32   neighbours; -1 = empty or deleted
+//   row[n+1]                    16 B    slack-CSR row heads: start, slots in
+//                                       use, free slots, capacity
+//   col[slots]                  int32   neighbours; -1 = empty or deleted
+//   fpos[slots]                 int32   each row's stack of free slots
 //   hkey[H], hpu[H], hpv[H]             open-addressing edge index: key ->
 //                                       global col positions of the edge in
 //                                       the rows of min(u,v) and max(u,v),
@@ -95,11 +95,21 @@ struct Index {
     u64 mask;
 };
 
-// The slack CSR.
+// The slack CSR.  A row's head is one 16-byte record, so that whoever visits
+// a row (append, removal, scan) touches one sector for it.  Its free slots
+// form a stack of nfree entries in the row's part of fpos: entry k is the
+// free slot's position in the row, or -1 for the position it holds when the
+// row is new (cap - 1 - k: the stack of a new row gives its slack in order).
+struct __align__(16) Row {
+    unsigned start;   // first slot (positions are below 2^32, checked at build)
+    int used;         // slots from the start that may hold an entry: what a scan reads
+    int nfree;        // free slots
+    int cap;
+};
 struct Csr {
-    const long long *off;
-    int *used;
+    Row *row;
     int *col;
+    int *fpos;
 };
 
 __host__ __device__ __forceinline__ u64 ekey(uint32_t u, uint32_t v) {
@@ -129,7 +139,9 @@ __device__ __forceinline__ u64 hslot(u64 k, u64 mask) {
 // from that slot on, and finds the key the other one wrote there or further
 // along.  Without the reuse an edge that comes back leaves one more deleted
 // slot in its own chain every time: after 1,500 removals of each edge of a
-// 100-edge batch the claim took 1,115 us (R-MAT scale 22) instead of 16.
+// 100-edge batch the claim alone took 1,115 us (R-MAT scale 22).  Measured
+// over a window of returning edges (insert + delete step, R-MAT scale 22):
+// 100-edge batches 751 -> 218 us, 10K-edge batches 781 -> 333 us.
 __device__ __forceinline__ long long index_claim(Index ix, u64 key, bool *reused) {
     u64 s = hslot(key, ix.mask);
     long long free_slot = -1;   // first deleted slot of the chain
@@ -211,15 +223,46 @@ __device__ __forceinline__ long long agg_append(u64 *ctr, bool pred) {
     return (long long)(base + __popc(m & ((1u << lane) - 1u)));
 }
 
-// One slot of row r's append cursor per calling lane; lanes of a warp with
-// the same row share one atomicAdd.
-__device__ __forceinline__ int row_slot(int *used, int r) {
+__device__ __forceinline__ Row row_head(const Csr &g, int r) {
+    const int4 q = __ldcg(reinterpret_cast<const int4 *>(&g.row[r]));
+    return Row{(unsigned)q.x, q.y, q.z, q.w};
+}
+
+// One free slot of row r (head h) per calling lane, from the top of the
+// row's stack; -1 when the row is full.  Slots are only taken while a batch
+// is inserted and only given back while one is deleted, so the counter alone
+// decides who gets which entry: no retries, and a lane that drew below zero
+// puts its draw back.  Lanes of a warp with the same row share one atomic (a
+// hub row receives many of a batch's edges).  *grown counts the slots that
+// the row's scanned length grew by.  Reusing deleted slots keeps rows at
+// their length when edges leave and come back; with append-only rows such a
+// window filled the slack and then the overflow list and rebuilt the whole
+// storage every 40 steps of 100K-edge batches (R-MAT scale 22).
+__device__ __forceinline__ int row_take(const Csr &g, int r, const Row &h, long long *grown) {
     const unsigned grp = __match_any_sync(__activemask(), r);
-    const int lane = threadIdx.x & 31, ld = __ffs(grp) - 1;
+    const int lane = threadIdx.x & 31, ld = __ffs(grp) - 1, cnt = __popc(grp);
     int base = 0;
-    if (lane == ld) base = atomicAdd(&used[r], __popc(grp));
+    if (lane == ld) {
+        base = atomicSub(&g.row[r].nfree, cnt);
+        if (base < cnt) atomicAdd(&g.row[r].nfree, base > 0 ? cnt - base : cnt);
+    }
     base = __shfl_sync(grp, base, ld);
-    return base + __popc(grp & ((1u << lane) - 1u));
+    const int k = base - 1 - __popc(grp & ((1u << lane) - 1u));
+    if (k < 0) return -1;
+    const int f = g.fpos[(size_t)h.start + k];
+    const int slot = f < 0 ? h.cap - 1 - k : f;
+    if (slot >= h.used) {
+        const int old = atomicMax(&g.row[r].used, slot + 1);
+        if (slot + 1 > old) *grown += slot + 1 - old;
+    }
+    return slot;
+}
+
+// Give slot pos (a position in col) of row r back.
+__device__ __forceinline__ void row_give(const Csr &g, int r, unsigned start, unsigned pos) {
+    const int k = atomicAdd(&g.row[r].nfree, 1);
+    g.col[pos] = -1;
+    g.fpos[(size_t)start + k] = (int)(pos - start);
 }
 
 // Pair table: piece pair (min, max) -> minimum edge key between the two

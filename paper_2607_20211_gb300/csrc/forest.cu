@@ -244,7 +244,7 @@ __device__ __forceinline__ void warp_fill_tiles(int *tile, bool on, long long st
 // list of the scan, with their entry ranges and the tile map: positions are
 // pb (rows << 32 | entries) plus offsets from one atomic per warp on the
 // packed counter pc.  All 32 lanes call.
-__device__ __forceinline__ void warp_list_rows(u64 *pc, u64 pb, RowList rl, Csr g, bool f, int w, int len, int p,
+__device__ __forceinline__ void warp_list_rows(u64 *pc, u64 pb, RowList rl, bool f, int w, unsigned st, int len, int p,
                                                int ro) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -268,19 +268,19 @@ __device__ __forceinline__ void warp_list_rows(u64 *pc, u64 pb, RowList rl, Csr 
     if (f) {
         rl.D[q] = w;
         rl.roff[q] = (unsigned)eo;
-        rl.base[q] = (unsigned)g.off[w];
+        rl.base[q] = st;
         rl.meta[q] = make_int2(p, ro);
     }
     warp_fill_tiles(rl.tile, f, eo, len, (int)q);
 }
 
 // Append one warp's detached vertices (lanes with `on`) to the vertex list
-// and their non-empty rows (`len` > 0) to the row list of the scan: positions
+// and their non-empty rows (starting at `st`, `len` > 0) to the row list of the scan: positions
 // are the level's bases (vb vertices; pb rows << 32 | entries) plus offsets
 // taken from the level's own counters (vc, and pc packed like pb), one
 // atomic per warp on each.  All 32 lanes call.
-__device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long vb, u64 pb, RowList rl, int *A, Csr g,
-                                                   bool on, int w, int len, int p, int ro) {
+__device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long vb, u64 pb, RowList rl, int *A,
+                                                   bool on, int w, unsigned st, int len, int p, int ro) {
     const int lane = threadIdx.x & 31;
     const unsigned m = __ballot_sync(0xffffffffu, on);
     if (!m) return;
@@ -289,7 +289,7 @@ __device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long v
     if (lane == ld) a0 = atomicAdd(vc, (u64)__popc(m));
     a0 = __shfl_sync(0xffffffffu, a0, ld);
     if (on) A[vb + (long long)a0 + __popc(m & ((1u << lane) - 1u))] = w;
-    warp_list_rows(pc, pb, rl, g, on && len > 0, w, len, p, ro);
+    warp_list_rows(pc, pb, rl, on && len > 0, w, st, len, p, ro);
 }
 
 // Representatives by asynchronous pointer doubling in place (delete batches
@@ -416,15 +416,18 @@ __global__ void __launch_bounds__(BLK, 4)
         const long long i = b0 + lane;
         const bool on = i < nc;
         int c = 0, len = 0, ro = 0;
+        unsigned st = 0;
         if (on) {
             c = cuts[i];
             ro = rold[c];
             J1[c] = c;
             __threadfence();   // J1 before the stamp that publishes it
             det_ep[c] = ep;
-            len = min(g.used[c], (int)(g.off[c + 1] - g.off[c]));
+            const Row h = row_head(g, c);
+            st = h.start;
+            len = h.used;
         }
-        warp_detach_append(&ctl->dv[0], &ctl->dp[0], 0, 0, rl, A, g, on, c, len, c, ro);
+        warp_detach_append(&ctl->dv[0], &ctl->dp[0], 0, 0, rl, A, on, c, st, len, c, ro);
     }
     // the tree edges held outside the rows (overflow list), as (child,
     // parent): listed once, read by every level (few: edges land there
@@ -512,13 +515,16 @@ __global__ void __launch_bounds__(BLK, 4)
                 }
             }
             int len = 0;
+            unsigned st = 0;
             if (child) {
+                const Row h = row_head(g, w);
                 J1[w] = p;
                 __threadfence();
                 det_ep[w] = ep;
-                len = min(g.used[w], (int)(g.off[w + 1] - g.off[w]));
+                st = h.start;
+                len = h.used;
             }
-            warp_detach_append(&ctl->dv[sn], &ctl->dp[sn], vn, pn, rl, A, g, child, w, len, p, ro);
+            warp_detach_append(&ctl->dv[sn], &ctl->dp[sn], vn, pn, rl, A, child, w, st, len, p, ro);
         }
         // children joined by a tree edge outside the rows: a vertex whose
         // parent is detached (published: its J1 before its stamp)
@@ -527,6 +533,7 @@ __global__ void __launch_bounds__(BLK, 4)
             const long long i = b0 + lane;
             bool child = false;
             int w = -1, p = 0, ro = 0, len = 0;
+            unsigned st = 0;
             if (i < nt) {
                 const int cw = LD(oc[i]), pv = LD(op[i]);
                 const bool pd = LD(det_ep[pv]) == ep;
@@ -539,12 +546,14 @@ __global__ void __launch_bounds__(BLK, 4)
                 }
             }
             if (child) {
+                const Row h = row_head(g, w);
                 J1[w] = p;
                 __threadfence();
                 det_ep[w] = ep;
-                len = min(g.used[w], (int)(g.off[w + 1] - g.off[w]));
+                st = h.start;
+                len = h.used;
             }
-            warp_detach_append(&ctl->dv[sn], &ctl->dp[sn], vn, pn, rl, A, g, child, w, len, p, ro);
+            warp_detach_append(&ctl->dv[sn], &ctl->dp[sn], vn, pn, rl, A, child, w, st, len, p, ro);
         }
         vb = vn;
         pb = pn;
@@ -709,6 +718,7 @@ __global__ void __launch_bounds__(BLK, 6)
         const long long S = gstride();
         for (long long base = (long long)blockIdx.x * blockDim.x; base < cnt; base += S * JF) {
             int v[JF], p[JF], ro[JF], len[JF];
+            unsigned st[JF];
             bool ok[JF], scan[JF];
 #pragma unroll
             for (int k = 0; k < JF; ++k) {
@@ -725,13 +735,14 @@ __global__ void __launch_bounds__(BLK, 6)
             for (int k = 0; k < JF; ++k) {
                 scan[k] = false;
                 len[k] = 0;
+                st[k] = 0;
                 if (!ok[k]) continue;
                 // rep[v] == rold[v] already for the root piece's vertices
                 if (p[k] != ro[k]) {
                     rep[v[k]] = p[k];
-                    int cap = (int)(g.off[v[k] + 1] - g.off[v[k]]);
-                    int used = g.used[v[k]];
-                    len[k] = used < cap ? used : cap;
+                    const Row h = row_head(g, v[k]);
+                    st[k] = h.start;
+                    len[k] = h.used;
                     scan[k] = len[k] > 0;
                 }
             }
@@ -752,7 +763,7 @@ __global__ void __launch_bounds__(BLK, 6)
                 if (scan[k]) {
                     D[q[k]] = v[k];
                     roff[q[k]] = (unsigned)eo[k];
-                    rl.base[q[k]] = (unsigned)g.off[v[k]];
+                    rl.base[q[k]] = st[k];
                     rl.meta[q[k]] = make_int2(p[k], ro[k]);
                 }
                 warp_fill_tiles(rl.tile, scan[k], eo[k], len[k], (int)q[k]);
@@ -824,12 +835,13 @@ __global__ void __launch_bounds__(BLK, 6)
             long long i = base + threadIdx.x;
             bool scan[1] = {false};
             int v = 0, hp = 0, pv = 0, len[1] = {0};
+            unsigned st = 0;
             if (i < cnt) {
                 v = A[i];
                 hp = (int)(unsigned)LD(heavy[rold[v]]);
-                int cap = (int)(g.off[v + 1] - g.off[v]);
-                int used = g.used[v];
-                len[0] = used < cap ? used : cap;
+                const Row h = row_head(g, v);
+                st = h.start;
+                len[0] = h.used;
                 pv = LD(rep[v]);
                 scan[0] = pv != hp && len[0] > 0;
             }
@@ -838,7 +850,7 @@ __global__ void __launch_bounds__(BLK, 6)
             if (scan[0]) {
                 D[q[0]] = v;
                 roff[q[0]] = (unsigned)eo[0];
-                rl.base[q[0]] = (unsigned)g.off[v];
+                rl.base[q[0]] = st;
                 rl.meta[q[0]] = make_int2(pv, hp);
             }
             warp_fill_tiles(rl.tile, scan[0], eo[0], len[0], (int)q[0]);

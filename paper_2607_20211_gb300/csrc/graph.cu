@@ -49,11 +49,11 @@ __global__ void k_create_claim(const int *edges, long long m, Index ix, u64 *dke
     }
 }
 
-__global__ void k_degree(const u64 *dkey, long long m, int *deg) {
+// Row degrees; each edge keeps the places that it takes in its two rows.
+__global__ void k_degree(const u64 *dkey, long long m, int *deg, int2 *place) {
     GS_LOOP(i, m) {
-        u64 k = dkey[i];
-        atomicAdd(&deg[klo(k)], 1);
-        atomicAdd(&deg[khi(k)], 1);
+        const u64 k = dkey[i];
+        place[i] = make_int2(atomicAdd(&deg[klo(k)], 1), atomicAdd(&deg[khi(k)], 1));
     }
 }
 
@@ -135,17 +135,27 @@ __global__ void k_scan_apply(const long long *in, long long *out, long long n, c
     if (base <= n - 1 && base + SCAN_ITEMS > n - 1) out[n] = pre;   // total after the last element
 }
 
-// Place the deduplicated edges: append to both rows, record positions.
-__global__ void k_fill(const u64 *dkey, const u64 *dslot, long long m, Csr g, Index ix) {
+// Row heads of a new CSR: the slots past a row's degree are free (row n
+// closes the array).
+__global__ void k_rows_init(const long long *off, const int *deg, int n, Row *row) {
+    GS_LOOP(u, (long long)n + 1) {
+        const int cap = u < n ? (int)(off[u + 1] - off[u]) : 0, d = u < n ? deg[u] : 0;
+        row[u] = Row{(unsigned)off[u], d, cap - d, cap};
+    }
+}
+
+// Place the deduplicated edges at the places taken in k_degree, record
+// their positions.
+__global__ void k_fill(const u64 *dkey, const u64 *dslot, const int2 *place, long long m, Csr g, Index ix) {
     GS_LOOP(i, m) {
         u64 k = dkey[i];
         uint32_t a = klo(k), b = khi(k);
-        int pa = atomicAdd(&g.used[a], 1), pb = atomicAdd(&g.used[b], 1);
-        long long qa = g.off[a] + pa, qb = g.off[b] + pb;
+        const int2 pl = place[i];
+        const unsigned qa = g.row[a].start + (unsigned)pl.x, qb = g.row[b].start + (unsigned)pl.y;
         g.col[qa] = (int)b;
         g.col[qb] = (int)a;
-        ix.pu[dslot[i]] = (uint32_t)qa;
-        ix.pv[dslot[i]] = (uint32_t)qb;
+        ix.pu[dslot[i]] = qa;
+        ix.pv[dslot[i]] = qb;
     }
 }
 
@@ -203,9 +213,9 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
     block_add(&ctl->htomb, -reuse);
 }
 
-// Insert, step 2: append each new edge to both CSR rows (warp-aggregated
-// row cursors are per row, so plain atomics); an edge whose row is full goes
-// whole to the overflow list.  The cross test of the insert case (M = B,
+// Insert, step 2: put each new edge into a free slot of both CSR rows
+// (row_take); an edge one of whose rows is full goes whole to the overflow
+// list.  The cross test of the insert case (M = B,
 // Algorithm 1) is fused here: rep[u] != rep[v] makes a candidate.  With SG
 // (the supergraph variant, Section III-A) a candidate goes into the pair
 // table instead, which keeps the minimum key per pair of trees (one
@@ -217,6 +227,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
     if (*(volatile int *)&ctl->skip) return;
     const unsigned ep = ctl->epoch;
     long long nb = (long long)ctl->nb;
+    long long dead = 0;   // change of the slots that scans read and hold no entry
     // block-uniform loop: the candidate append is aggregated per block
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nb; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
@@ -227,19 +238,18 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
             k = nkey[i];
             u64 s = nslot[i];
             uint32_t a = klo(k), b = khi(k);
-            long long oa = g.off[a], ob = g.off[b];
-            long long capa = g.off[a + 1] - oa, capb = g.off[b + 1] - ob;
-            // lanes appending to the same row take consecutive slots from one
-            // atomic (a hub row receives many of a batch's edges)
-            int pa = row_slot(g.used, (int)a), pb = row_slot(g.used, (int)b);
-            bool fa = pa < capa, fb = pb < capb;
-            if (fa && fb) {
-                g.col[oa + pa] = (int)b;
-                g.col[ob + pb] = (int)a;
-                ix.pu[s] = (uint32_t)(oa + pa);
-                ix.pv[s] = (uint32_t)(ob + pb);
+            const Row ha = row_head(g, (int)a), hb = row_head(g, (int)b);
+            const int pa = row_take(g, (int)a, ha, &dead), pb = row_take(g, (int)b, hb, &dead);
+            if (pa >= 0 && pb >= 0) {
+                const unsigned qa = ha.start + (unsigned)pa, qb = hb.start + (unsigned)pb;
+                g.col[qa] = (int)b;
+                g.col[qb] = (int)a;
+                ix.pu[s] = qa;
+                ix.pv[s] = qb;
+                dead -= 2;
             } else {
-                // the consumed free slot (if any) stays -1
+                // (a slot taken in the row that had one stays empty and
+                // unlisted until the next rebuild)
                 u64 o = atomicAdd(&ctl->ovf_count, 1ull);
                 if (o < ovf_cap) {
                     ovf[o] = k;
@@ -249,7 +259,6 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                     atomicOr(&ctl->err, ERR_CAPACITY);
                 }
                 atomicAdd((u64 *)&ctl->overflow_total, 1ull);
-                if (fa || fb) atomicAdd((u64 *)&ctl->ctomb, 1ull);
             }
             ra = rep[a];
             rb = rep[b];
@@ -273,6 +282,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
             }
         }
     }
+    block_add(&ctl->ctomb, dead);
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd((u64 *)&ctl->edges, (u64)nb);
 }
 
@@ -301,6 +311,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                 // this kernel only by the cut of the edge {u, parent[u]}, which
                 // only the thread deleting that edge makes
                 const int par_u = parent[u], par_v = parent[v], rep_u = rep[u], rep_v = rep[v];
+                const unsigned st_u = g.row[u].start, st_v = g.row[v].start;
                 u64 key = ekey((uint32_t)u, (uint32_t)v);
                 long long s = index_find(ix, key);
                 if (s >= 0) won = atomicCAS(&ix.key[s], key, TOMB_KEY) == key;
@@ -309,8 +320,8 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                     if (pu == POS_OVF) {
                         ovf[pv] = TOMB_KEY;
                     } else {
-                        g.col[pu] = -1;
-                        g.col[pv] = -1;
+                        row_give(g, u < v ? u : v, u < v ? st_u : st_v, pu);
+                        row_give(g, u < v ? v : u, u < v ? st_v : st_u, pv);
                         dead += 2;
                     }
                     if (par_u == v) {
@@ -550,10 +561,7 @@ __global__ void k_extract(int n, Csr g, const u64 *ovf, const Ctl *ctl, int *out
     long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long u = warp; u < n; u += nw) {
-        long long o = g.off[u];
-        long long c = g.off[u + 1] - o;
-        long long used = g.used[u];
-        if (used > c) used = c;
+        const long long o = g.row[u].start, used = g.row[u].used;
         for (long long j0 = 0; j0 < used; j0 += 32) {
             long long j = j0 + lane;
             int x = j < used ? g.col[o + j] : -1;
@@ -614,8 +622,8 @@ cudaError_t launch_create_claim(const int *edges, long long m, Index ix, u64 *dk
     k_create_claim<<<gsz(m), BLK, 0, s>>>(edges, m, ix, dkey, dslot, cnt, self_loops);
     return cudaGetLastError();
 }
-cudaError_t launch_degree(const u64 *dkey, long long m, int *deg, cudaStream_t s) {
-    k_degree<<<gsz(m), BLK, 0, s>>>(dkey, m, deg);
+cudaError_t launch_degree(const u64 *dkey, long long m, int *deg, int2 *place, cudaStream_t s) {
+    k_degree<<<gsz(m), BLK, 0, s>>>(dkey, m, deg, place);
     return cudaGetLastError();
 }
 cudaError_t launch_caps(const int *deg, int n, long long *cap, cudaStream_t s) {
@@ -630,8 +638,13 @@ cudaError_t launch_scan_i64(const long long *in, long long *out, long long n, lo
     k_scan_apply<<<(unsigned)tiles, BLK, 0, s>>>(in, out, n, bsum);
     return cudaGetLastError();
 }
-cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, long long m, Csr g, Index ix, cudaStream_t s) {
-    k_fill<<<gsz(m), BLK, 0, s>>>(dkey, dslot, m, g, ix);
+cudaError_t launch_rows_init(const long long *off, const int *deg, int n, Row *row, cudaStream_t s) {
+    k_rows_init<<<gsz((long long)n + 1), BLK, 0, s>>>(off, deg, n, row);
+    return cudaGetLastError();
+}
+cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, const int2 *place, long long m, Csr g, Index ix,
+                        cudaStream_t s) {
+    k_fill<<<gsz(m), BLK, 0, s>>>(dkey, dslot, place, m, g, ix);
     return cudaGetLastError();
 }
 // The batch kernels read the batch and its length from the control block;

@@ -28,10 +28,12 @@ unsigned scan_grid(int nsm);
 cudaError_t launch_check_range(const int *a, long long cnt, int n, int *bad, cudaStream_t s);
 cudaError_t launch_create_claim(const int *edges, long long m, Index ix, u64 *dkey, u64 *dslot, u64 *cnt,
                                 long long *self_loops, cudaStream_t s);
-cudaError_t launch_degree(const u64 *dkey, long long m, int *deg, cudaStream_t s);
+cudaError_t launch_degree(const u64 *dkey, long long m, int *deg, int2 *place, cudaStream_t s);
 cudaError_t launch_caps(const int *deg, int n, long long *cap, cudaStream_t s);
 cudaError_t launch_scan_i64(const long long *in, long long *out, long long n, long long *bsum, cudaStream_t s);
-cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, long long m, Csr g, Index ix, cudaStream_t s);
+cudaError_t launch_rows_init(const long long *off, const int *deg, int n, Row *row, cudaStream_t s);
+cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, const int2 *place, long long m, Csr g, Index ix,
+                        cudaStream_t s);
 // (the batch kernels read the batch from the control block; len sizes the grid)
 cudaError_t launch_validate_batch(long long len, int n, Ctl *ctl, cudaStream_t s);
 

@@ -48,10 +48,7 @@ __global__ void k_cc_hook(int n, Csr g, const u64 *ovf, const Ctl *ctl, int *lab
     long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long u = warp; u < n; u += nw) {
-        long long o = g.off[u];
-        long long cap = g.off[u + 1] - o;
-        long long used = g.used[u];
-        if (used > cap) used = cap;
+        const long long o = g.row[u].start, used = g.row[u].used;
         for (long long j = lane; j < used; j += 32) {
             int x = g.col[o + j];
             if (x > (int)u) cc_union(lab, (int)u, x);
@@ -109,10 +106,7 @@ __global__ void k_bfs(Ctl *ctl, Csr g, const u64 *ovf, int *parent, int *f0, int
         int *out = (r & 1) ? f0 : f1;
         for (long long w = warp; w < c; w += nw) {
             int u = in[w];
-            long long o = g.off[u];
-            long long cap = g.off[u + 1] - o;
-            long long used = g.used[u];
-            if (used > cap) used = cap;
+            const long long o = g.row[u].start, used = g.row[u].used;
             for (long long j0 = 0; j0 < used; j0 += 32) {
                 long long j = j0 + lane;
                 int x = j < used ? g.col[o + j] : -1;

@@ -39,3 +39,35 @@ def test_same_edges_leave_and_come_back(n, m, b, cycles):
             old = fresh
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_window_neither_overflows_nor_rebuilds(batched):
+    """A window of returning edges reuses the rows' freed slots: with
+    append-only rows 24 cycles of a sixth of the edges would overflow every
+    row's slack (a quarter of its degree, at least 4) many times over.  The
+    last cycles run against the oracle."""
+    g = workloads.er_graph(30_000, 120_000, seed=22)
+    f = make_forest(g)
+    keys, par = g.keys, g.parent
+    rng = np.random.default_rng(6)
+    back = workloads.keys_to_edges(rng.permutation(g.keys)[:20_000])
+    dev = torch.from_numpy(back).cuda()
+    vo = bo = None
+    if batched:
+        vo, bo = np.array([0, g.n], np.int64), np.array([0, len(back)], np.int64)
+    try:
+        for c in range(24):
+            for op in (drsf.DELETE, drsf.INSERT):
+                if batched:
+                    f.apply_batched(op, dev, vo, bo)
+                else:
+                    f.apply(op, dev)
+        st = f.stats()
+        assert st["rebuilds"] == 0 and st["overflow"] == 0 and st["edges"] == g.m
+        assert np.array_equal(workloads.edges_to_keys(f.export_edges().cpu().numpy()), g.keys)
+        par = f.parent().cpu().numpy()
+        keys, par, _ = check_batch(f, g.n, keys, par, drsf.DELETE, back)
+        keys, par, _ = check_batch(f, g.n, keys, par, drsf.INSERT, back)
+    finally:
+        f.close()
