@@ -232,11 +232,9 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     long long headroom = std::max<long long>(std::max<long long>(m / 2, 1 << 12), 2 * extra);
     u64 H = pow2_at_least((u64)(2 * (m + headroom)));
     Index ix{};
-    CKA(halloc(h, &ix.key, H, s));
-    CKA(halloc(h, &ix.pu, H, s));
-    CKA(halloc(h, &ix.pv, H, s));
+    CKA(halloc(h, &ix.e, H, s));
     ix.mask = H - 1;
-    CK(cudaMemsetAsync(ix.key, 0xFF, H * sizeof(u64), s));
+    CK(cudaMemsetAsync(ix.e, 0xFF, H * sizeof(Entry), s));
 
     u64 *dkey = nullptr, *dslot = nullptr, *cnt = nullptr;
     long long *tmp64 = nullptr, *bs = nullptr;
@@ -303,9 +301,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     }
     CK(cudaStreamSynchronize(s));
     // swap in
-    hfree(h, &h->ix.key, s);
-    hfree(h, &h->ix.pu, s);
-    hfree(h, &h->ix.pv, s);
+    hfree(h, &h->ix.e, s);
     hfree(h, &h->row, s);
     hfree(h, &h->col, s);
     hfree(h, &h->fpos, s);

@@ -292,15 +292,13 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
                 const unsigned qa = ha.start + (unsigned)pa, qb = hb.start + (unsigned)pb;
                 S.g.col[qa] = (int)b;
                 S.g.col[qb] = (int)a;
-                S.ix.pu[s] = qa;
-                S.ix.pv[s] = qb;
+                S.ix.e[s].pos = make_uint2(qa, qb);
                 hole -= 2;
             } else {
                 const u64 o = atomicAdd(&ctl->ovf_count, 1ull);
                 if (o < S.ovf_cap) {
                     S.ovf[o] = k;
-                    S.ix.pu[s] = POS_OVF;
-                    S.ix.pv[s] = (uint32_t)o;
+                    S.ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
                 } else {
                     atomicOr(&ctl->err, ERR_CAPACITY);
                 }
@@ -344,20 +342,20 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         // which only the thread deleting that edge makes
         const int par_u = GL(S.parent[u]), par_v = GL(S.parent[v]), rep_u = GL(S.rep[u]), rep_v = GL(S.rep[v]);
         const u64 key = ekey((uint32_t)u, (uint32_t)v);
-        const long long s = index_find(S.ix, key);
-        const bool won = s >= 0 && atomicCAS(&S.ix.key[s], key, TOMB_KEY) == key;
+        uint2 pos = make_uint2(0, 0);
+        const long long s = index_find(S.ix, key, &pos);
+        const bool won = s >= 0 && atomicCAS(&S.ix.e[s].key, key, TOMB_KEY) == key;
         if (!won) {
             ++drops;
             continue;
         }
         ++wins;
-        const uint32_t pu = S.ix.pu[s], pv = S.ix.pv[s];
-        if (pu == POS_OVF) {
-            S.ovf[pv] = TOMB_KEY;
+        if (pos.x == POS_OVF) {
+            S.ovf[pos.y] = TOMB_KEY;
         } else {
             const int lo = (int)klo(key), hi = (int)khi(key);
-            row_give(S.g, lo, S.g.row[lo].start, pu);
-            row_give(S.g, hi, S.g.row[hi].start, pv);
+            row_give(S.g, lo, S.g.row[lo].start, pos.x);
+            row_give(S.g, hi, S.g.row[hi].start, pos.y);
             dead += 2;
         }
         int c = -1, rc = -1;

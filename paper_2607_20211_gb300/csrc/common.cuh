@@ -6,7 +6,7 @@
 //                                       use, free slots, capacity
 //   col[slots]                  int32   neighbours; -1 = empty or deleted
 //   fpos[slots]                 int32   each row's stack of free slots
-//   hkey[H], hpu[H], hpv[H]             open-addressing edge index: key ->
+//   index[H]                    16 B    open-addressing edge index: key ->
 //                                       global col positions of the edge in
 //                                       the rows of min(u,v) and max(u,v),
 //                                       or (POS_OVF, overflow slot)
@@ -87,11 +87,16 @@ struct Ctl {
     long long det_entries;  // adjacency entries the top-down search read
 };
 
-// The edge index.
+// The edge index.  An entry is one 16-byte record: with keys and positions in
+// arrays of their own a deleted edge touched three sectors of a table far
+// larger than L2 instead of one, an inserted one too.
+struct __align__(16) Entry {
+    u64 key;
+    uint2 pos;      // x: position of the edge in the row of min(u,v), or POS_OVF
+                    // y: position in the row of max(u,v), or overflow slot
+};
 struct Index {
-    u64 *key;
-    uint32_t *pu;   // position of the edge in the row of min(u,v), or POS_OVF
-    uint32_t *pv;   // position in the row of max(u,v), or overflow slot
+    Entry *e;
     u64 mask;
 };
 
@@ -146,13 +151,13 @@ __device__ __forceinline__ long long index_claim(Index ix, u64 key, bool *reused
     u64 s = hslot(key, ix.mask);
     long long free_slot = -1;   // first deleted slot of the chain
     for (u64 p = 0; p <= 2 * ix.mask; ++p) {
-        const u64 cur = __ldcg(&ix.key[s]);
+        const u64 cur = __ldcg(&ix.e[s].key);
         if (cur == key) return -1 - (long long)s;
         if (cur == TOMB_KEY && free_slot < 0) free_slot = (long long)s;
         if (cur == EMPTY_KEY) {
             const bool dead = free_slot >= 0;
             const u64 t = dead ? (u64)free_slot : s;
-            const u64 old = atomicCAS(&ix.key[t], dead ? TOMB_KEY : EMPTY_KEY, key);
+            const u64 old = atomicCAS(&ix.e[t].key, dead ? TOMB_KEY : EMPTY_KEY, key);
             if (old == (dead ? TOMB_KEY : EMPTY_KEY)) {
                 *reused = dead;
                 return (long long)t;
@@ -197,12 +202,17 @@ __device__ __forceinline__ void hook_slot_init(const HookSlots &hs, int a, unsig
     }
 }
 
-// Lookup; -1 when absent.  Deleted entries (TOMB_KEY) are probed past.
-__device__ __forceinline__ long long index_find(Index ix, u64 key) {
+// Lookup; -1 when absent, else the slot and the entry's positions.  Deleted
+// entries (TOMB_KEY) are probed past.
+__device__ __forceinline__ long long index_find(Index ix, u64 key, uint2 *pos) {
     u64 s = hslot(key, ix.mask);
     for (u64 p = 0; p <= ix.mask; ++p) {
-        u64 cur = __ldcg(&ix.key[s]);
-        if (cur == key) return (long long)s;
+        const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(&ix.e[s]));
+        const u64 cur = ((u64)q.y << 32) | q.x;
+        if (cur == key) {
+            *pos = make_uint2(q.z, q.w);
+            return (long long)s;
+        }
         if (cur == EMPTY_KEY) return -1;
         s = (s + 1) & ix.mask;
     }

@@ -154,8 +154,7 @@ __global__ void k_fill(const u64 *dkey, const u64 *dslot, const int2 *place, lon
         const unsigned qa = g.row[a].start + (unsigned)pl.x, qb = g.row[b].start + (unsigned)pl.y;
         g.col[qa] = (int)b;
         g.col[qb] = (int)a;
-        ix.pu[dslot[i]] = qa;
-        ix.pv[dslot[i]] = qb;
+        ix.e[dslot[i]].pos = make_uint2(qa, qb);
     }
 }
 
@@ -244,8 +243,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                 const unsigned qa = ha.start + (unsigned)pa, qb = hb.start + (unsigned)pb;
                 g.col[qa] = (int)b;
                 g.col[qb] = (int)a;
-                ix.pu[s] = qa;
-                ix.pv[s] = qb;
+                ix.e[s].pos = make_uint2(qa, qb);
                 dead -= 2;
             } else {
                 // (a slot taken in the row that had one stays empty and
@@ -253,8 +251,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                 u64 o = atomicAdd(&ctl->ovf_count, 1ull);
                 if (o < ovf_cap) {
                     ovf[o] = k;
-                    ix.pu[s] = POS_OVF;
-                    ix.pv[s] = (uint32_t)o;
+                    ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
                 } else {
                     atomicOr(&ctl->err, ERR_CAPACITY);
                 }
@@ -313,15 +310,15 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                 const int par_u = parent[u], par_v = parent[v], rep_u = rep[u], rep_v = rep[v];
                 const unsigned st_u = g.row[u].start, st_v = g.row[v].start;
                 u64 key = ekey((uint32_t)u, (uint32_t)v);
-                long long s = index_find(ix, key);
-                if (s >= 0) won = atomicCAS(&ix.key[s], key, TOMB_KEY) == key;
+                uint2 pos;
+                long long s = index_find(ix, key, &pos);
+                if (s >= 0) won = atomicCAS(&ix.e[s].key, key, TOMB_KEY) == key;
                 if (won) {
-                    uint32_t pu = ix.pu[s], pv = ix.pv[s];
-                    if (pu == POS_OVF) {
-                        ovf[pv] = TOMB_KEY;
+                    if (pos.x == POS_OVF) {
+                        ovf[pos.y] = TOMB_KEY;
                     } else {
-                        row_give(g, u < v ? u : v, u < v ? st_u : st_v, pu);
-                        row_give(g, u < v ? v : u, u < v ? st_v : st_u, pv);
+                        row_give(g, u < v ? u : v, u < v ? st_u : st_v, pos.x);
+                        row_give(g, u < v ? v : u, u < v ? st_v : st_u, pos.y);
                         dead += 2;
                     }
                     if (par_u == v) {
@@ -597,7 +594,8 @@ __global__ void k_extract(int n, Csr g, const u64 *ovf, const Ctl *ctl, int *out
 __global__ void k_check_tree_edges(int n, const int *parent, Index ix, int *bad) {
     GS_LOOP(v, n) {
         int p = parent[v];
-        if (p != (int)v && index_find(ix, ekey((uint32_t)v, (uint32_t)p)) < 0) atomicOr(bad, 2);
+        uint2 pos;
+        if (p != (int)v && index_find(ix, ekey((uint32_t)v, (uint32_t)p), &pos) < 0) atomicOr(bad, 2);
     }
 }
 
