@@ -137,9 +137,9 @@ enum {
     PH_SCAN,          // delete: cross-edge scan of detached rows + overflow
     PH_HOOK,          // hook-and-compress (replacement edges)
     PH_ORIENT,        // Euler-tour orientation
-    PH_ACTIVE,        // path-reversal set-up + representative refresh
-    PH_MARK,          // pointer-doubling marks
-    PH_REVERSE        // path walks, reversal scatter + attach
+    PH_ACTIVE,        // representative refresh, and the doubling marks and reversal of long paths
+    PH_MARK,          // Euler-tour marks
+    PH_REVERSE        // path walks (Euler: reversal scatter + attach)
 };
 static const char *kPhaseNames[DRSF_NUM_PHASES] = {
     "begin", "ins_claim", "ins_place", "del_claim", "affected", "jump", "scan", "hook", "orient", "active",
@@ -627,11 +627,10 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.coop_hook = coop_blocks_hook(nsm);
     h->dev.coop_hook_small = coop_blocks_hook_small(nsm);
     h->dev.coop_orient = coop_blocks_orient(nsm);
-    h->dev.coop_mark = coop_blocks_mark(nsm);
+    h->dev.coop_finish = coop_blocks_finish(nsm);
     h->dev.coop_bfs = coop_blocks_bfs(nsm);
     h->dev.grid_scan = scan_grid(nsm);
     h->dev.grid_pass = grid_vertex_pass(nsm);
-    h->dev.grid_list = grid_list_pass(nsm);
     h->dev.coop_et = coop_blocks_et(nsm);
     h->dev.coop_detach = coop_blocks_detach(nsm);
     // root search of a delete batch: barrier-free doubling over per-warp
@@ -712,7 +711,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         }
         prof_begin(h, PH_AFF, s);
         CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, h->parent,
-                              h->jump_sync == 2 ? h->J0 : nullptr, 0, s));
+                              h->jump_sync == 2 ? h->J0 : nullptr, s));
         prof_end(h, PH_AFF, 1, s);
         prof_begin(h, PH_JUMP, s);
         if (h->jump_sync == 2) CK(launch_jump_async(h->dev, h->A, ctl, h->J0, h->act, h->xlist, s));
@@ -764,6 +763,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     oa.eroot = h->oeroot;
     oa.cel = h->nx1;   // (the grid ranking's second buffer: unused on the one-block path)
     oa.parent = h->parent;
+    oa.aff_ep = h->aff_ep;
     oa.n = h->n;
     prof_begin(h, PH_ORIENT, s);
     CK(launch_orient(h->dev, ctl, oa, s));
@@ -777,23 +777,28 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         CK(launch_walk(h->dev, ctl, h->chx, h->chy, h->rep, h->parent, h->long_ep, s));
         prof_end(h, PH_REVERSE, 1, s);
     }
-    const unsigned *sel = euler ? h->att_ep : h->long_ep;
+    FinishArgs fa{};
+    fa.A = h->A;
+    fa.n = h->n;
+    fa.rep = h->rep;
+    fa.parent = h->parent;
+    fa.sel_ep = euler ? h->att_ep : h->long_ep;
+    fa.att_x = h->att_x;
+    fa.rep_ep = h->rep_ep;
+    fa.newrep = h->newrep;
+    fa.act = h->act;
+    fa.pold = h->pold;
+    fa.J0 = h->J0;
+    fa.J1 = h->J1;
+    fa.aidx = h->aidx;
+    fa.aroot = h->aroot;
+    fa.mark = h->mark;
+    fa.chx = h->chx;
+    fa.chy = h->chy;
+    fa.euler = euler ? 1 : 0;
     prof_begin(h, PH_ACTIVE, s);
-    if (op == DRSF_DELETE && h->detach_now) {
-        // after a top-down delete the affected list holds the detached
-        // vertices only; a root piece that was re-rooted adds its vertices
-        CK(launch_rootcheck(h->dev, ctl, h->cutlist, h->rold, h->rep_ep, s));
-        CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, h->parent,
-                              nullptr, 1, s));
-    }
-    if (op == DRSF_INSERT)
-        CK(launch_active(h->dev, nullptr, 0, h->n, ctl, h->rep, h->parent, sel, h->att_x, h->rep_ep, h->newrep,
-                         h->act, h->pold, h->J0, h->mark, h->aidx, h->aroot, s));
-    else
-        CK(launch_active(h->dev, h->A, 1, 0, ctl, h->rep, h->parent, sel, h->att_x, h->rep_ep, h->newrep, h->act,
-                         h->pold, h->J0, h->mark, h->aidx, h->aroot, s));
+    CK(launch_finish(h->dev, ctl, fa, s));
     prof_end(h, PH_ACTIVE, 1, s);
-    prof_begin(h, PH_MARK, s);
     if (euler) {
         // Algorithm 3: Euler-tour intervals of the re-rooted pieces
         EtArgs ea{};
@@ -813,14 +818,13 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         ea.nx1 = h->nx1;
         ea.bsum = h->bsum;
         ea.mark = h->mark;
+        prof_begin(h, PH_MARK, s);
         CK(launch_et_marks(h->dev, ctl, ea, s));
-    } else {
-        CK(launch_mark(h->dev, ctl, h->act, h->J0, h->J1, h->mark, h->parent, s));
+        prof_end(h, PH_MARK, 1, s);
+        prof_begin(h, PH_REVERSE, s);
+        CK(launch_reverse(h->dev, ctl, fa, s));
+        prof_end(h, PH_REVERSE, 1, s);
     }
-    prof_end(h, PH_MARK, 1, s);
-    prof_begin(h, PH_REVERSE, s);
-    CK(launch_reverse(h->dev, ctl, h->act, h->pold, h->mark, h->chx, h->chy, h->parent, euler ? 0 : 1, s));
-    prof_end(h, PH_REVERSE, 1, s);
     return DRSF_OK;
 }
 

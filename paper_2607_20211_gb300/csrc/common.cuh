@@ -82,7 +82,8 @@ struct Ctl {
     long long overflow_total;
     const int *batch;       // the current batch (device), set by k_begin
     int td;                 // delete: the detached vertices were found top-down (else: pointer jumping)
-    int need_root;          // delete, top-down: a tree's root piece is re-rooted (list its vertices)
+    int need_root;          // delete: a cut tree's root piece is re-rooted (read after a top-down delete)
+    int nlong;              // some path was too long to be reversed by its walk
     long long det_levels;   // top-down levels of the batch (0: not taken)
     long long det_entries;  // adjacency entries the top-down search read
 };

@@ -103,7 +103,7 @@ __global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
     ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
     ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
     ctl->jump_visits = 0;
-    ctl->td = ctl->need_root = 0;
+    ctl->td = ctl->need_root = ctl->nlong = 0;
     if (ctl->det_skip) {   // the last batch skipped the top-down search
         if (ctl->depth_hint > 0) ctl->depth_hint -= 1;
         ctl->det_skip = 0;
@@ -130,18 +130,13 @@ __global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
 // 32 consecutive vertices), with all IPN loads and gathers in flight before
 // any is used.  A warp's listed vertices take consecutive slots (one block
 // reservation of the warps' totals), in vertex order within the warp.
-// With roots_only (after a top-down search of the detached vertices, when
-// some tree's root piece is re-rooted) only the root pieces' vertices are
-// appended (the detached ones already hold their new representative, which
-// is no stamped old root); otherwise the pass runs only when the top-down
-// search did not (the pointer-jumping path).
+// It runs only when the top-down search of the detached vertices did not (the
+// pointer-jumping path).
 __global__ void __launch_bounds__(BLK) k_aff_collect(int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                                                     unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J,
-                                                     int roots_only) {
+                                                     unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J) {
     static_assert(IPA <= 32, "item masks are 32 bits");
     if (*(volatile int *)&ctl->skip) return;
-    if (roots_only ? !(*(volatile int *)&ctl->td && *(volatile int *)&ctl->need_root) : *(volatile int *)&ctl->td)
-        return;
+    if (*(volatile int *)&ctl->td) return;
     unsigned ep = ctl->epoch;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -170,13 +165,11 @@ __global__ void __launch_bounds__(BLK) k_aff_collect(int n, const int *rep, cons
             if ((in >> k) & 1u) {
                 const int v = (int)(v0 + (long long)k * blockDim.x);
                 A[p + __popc(bk & lt)] = v;
-                if (!roots_only) {
-                    rold[v] = r[k];
-                    if (J) J[v] = par[v];   // seed of the asynchronous doubling
-                    if (r[k] == v) {        // the old root: piece-weight and heaviest-piece slots
-                        w[v] = 0;
-                        heavy[v] = 0;
-                    }
+                rold[v] = r[k];
+                if (J) J[v] = par[v];   // seed of the asynchronous doubling
+                if (r[k] == v) {        // the old root: piece-weight and heaviest-piece slots
+                    w[v] = 0;
+                    heavy[v] = 0;
                 }
             }
             p += __popc(bk);
@@ -581,18 +574,6 @@ __global__ void __launch_bounds__(BLK, 4)
         ctl->depth_hint = (unsigned)lvl;
         ctl->td = 1;
     }
-}
-
-// After the orientation of a top-down delete: does some cut tree's root
-// piece get a new representative (a detached piece with a smaller root id
-// joined its super-tree)?  Then its vertices must be listed for the refresh
-// and the path marks (k_aff_collect with roots_only).
-__global__ void k_rootcheck(Ctl *ctl, const int *cuts, const int *rold, const unsigned *rep_ep) {
-    if (*(volatile int *)&ctl->skip || !*(volatile int *)&ctl->td) return;
-    const unsigned ep = ctl->epoch;
-    const long long nc = (long long)ctl->ncut;
-    for (long long i = gtid(); i < nc; i += gstride())
-        if (rep_ep[rold[cuts[i]]] == ep) ctl->need_root = 1;
 }
 
 // Representatives (Algorithm 1, parallel pointer jumping) of the listed
@@ -1072,8 +1053,11 @@ __global__ void __launch_bounds__(HT, 1024 / HT) k_boruvka(Ctl *ctl, u64 *ck0, i
 // (x in P) gets the oriented edge x -> y, its attach point x and the
 // super-tree's root as its new representative (each non-root piece is the
 // child of exactly one edge: one write per piece; the super-root keeps its
-// representative).
-__device__ __forceinline__ void orient_one(const OrientArgs &a, long long i, bool down, unsigned ep) {
+// representative).  A child that is the root piece of a cut tree (its root
+// was stamped by the cut) is noted: after a top-down delete the affected list
+// holds the detached vertices only, and the refresh then has to pass over
+// all vertices.
+__device__ __forceinline__ void orient_one(Ctl *ctl, const OrientArgs &a, long long i, bool down, unsigned ep) {
     const u64 k = a.er[i];
     const int x0 = (int)klo(k), x1 = (int)khi(k);
     const int p0 = LD(a.ep[2 * i]), p1 = LD(a.ep[2 * i + 1]);
@@ -1085,6 +1069,7 @@ __device__ __forceinline__ void orient_one(const OrientArgs &a, long long i, boo
     a.att_ep[child] = ep;
     a.newrep[child] = LD(a.minp[LD(a.eroot[i])]);
     a.rep_ep[child] = ep;
+    if (a.aff_ep[child] == ep) ctl->need_root = 1;
 }
 
 // Wyllie list ranking of ncore list cells in shared memory by one block:
@@ -1168,7 +1153,7 @@ __device__ void orient_small_core(Ctl *ctl, const OrientArgs &a, const int *cel,
     const int rounds = rank_block(ctl, svc, svn, snc, snn, ncore, &rank);
     for (long long t = threadIdx.x; t < nce; t += blockDim.x) {
         const long long i = LD(cel[t]);
-        orient_one(a, i, rank[a.apos[2 * i]] > rank[a.apos[2 * i + 1]], ep);
+        orient_one(ctl, a, i, rank[a.apos[2 * i]] > rank[a.apos[2 * i + 1]], ep);
     }
     if (threadIdx.x == 0) {
         ctl->ncore = (u64)ncore;
@@ -1328,7 +1313,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs 
         if (nce <= ORIENT_SMALL_EDGES) {
             for (long long i = gtid(); i < ner; i += gstride()) {
                 const unsigned char lf = LD(a.lf[i]);
-                if (lf) orient_one(a, i, lf == 2, ep);
+                if (lf) orient_one(ctl, a, i, lf == 2, ep);
             }
             if (blockIdx.x == 0) orient_small_core(ctl, a, cel, nce, ep);
             return;
@@ -1438,7 +1423,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs 
     for (long long i = gtid(); i < ner; i += gstride()) {
         const unsigned char lf = LD(a.lf[i]);
         const bool down = lf ? lf == 2 : LD(vc[LD(a.apos[2 * i])]) > LD(vc[LD(a.apos[2 * i + 1])]);
-        orient_one(a, i, down, ep);
+        orient_one(ctl, a, i, down, ep);
     }
 }
 
@@ -1481,45 +1466,42 @@ __global__ void k_walk(Ctl *ctl, const int *chx, const int *chy, const int *rep,
                 v = nv;
             }
             long_ep[rep[x]] = ep;
+            ctl->nlong = 1;
         }
     }
     if (rev) atomicAdd((u64 *)&ctl->reversed, (u64)rev);
 }
 
-// Path-reversal set-up fused with the representative refresh: a vertex of a
-// piece that is re-rooted at an attach point x != its root is active (its
-// old parent is saved, J0 seeded, x marked); every vertex of a merged piece
-// takes the super-tree's root as its new rep.
-// IP items per thread and iteration (IPT over a list, IPN over all
-// vertices), k-major as in k_aff_collect, one slot reservation per block.
+// Path-reversal set-up fused with the representative refresh: every vertex
+// of a merged piece takes the super-tree's root as its new rep; with `marks`
+// a vertex of a piece that is reversed through the marks (selected in
+// sel_ep, re-rooted at an attach point x != its root) is active (its old
+// parent is saved, J0 seeded, x marked).
+// IP items per thread and iteration (IPT over a list or few vertices, IPN
+// over many), k-major as in k_aff_collect, one slot reservation per block.
 // Only the pieces stay in registers; the few items whose piece changed are
 // handled from bit masks (the common item costs one stamp gather).
 template <int IP>
-__global__ void __launch_bounds__(BLK)
-    k_active(const int *L, int use_list, long long cnt_static, Ctl *ctl, int *rep, const int *parent,
-             const unsigned *sel_ep, const int *att_x, const unsigned *rep_ep, const int *newrep, int *act, int *pold,
-             int *J0, unsigned char *mark, int *aidx, int *aroot) {
+__device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, const int *L, long long cnt, unsigned ep,
+                                             bool marks) {
     static_assert(IP <= 32, "item masks are 32 bits");
-    if (*(volatile int *)&ctl->skip) return;
-    unsigned ep = ctl->epoch;
-    long long cnt = use_list ? (long long)ctl->naff : cnt_static;
     const long long step = (long long)gridDim.x * blockDim.x * IP;
     for (long long b0 = (long long)blockIdx.x * blockDim.x * IP; b0 < cnt; b0 += step) {
         const long long i0 = b0 + threadIdx.x;
         int p[IP];
-        if (use_list) {
+        if (L) {
 #pragma unroll
             for (int k = 0; k < IP; ++k) {
                 const long long i = i0 + (long long)k * blockDim.x;
                 p[k] = i < cnt ? L[i] : 0;
             }
 #pragma unroll
-            for (int k = 0; k < IP; ++k) p[k] = i0 + (long long)k * blockDim.x < cnt ? rep[p[k]] : 0;
+            for (int k = 0; k < IP; ++k) p[k] = i0 + (long long)k * blockDim.x < cnt ? a.rep[p[k]] : 0;
         } else {
 #pragma unroll
             for (int k = 0; k < IP; ++k) {
                 const long long i = i0 + (long long)k * blockDim.x;
-                p[k] = i < cnt ? rep[i] : 0;
+                p[k] = i < cnt ? a.rep[i] : 0;
             }
         }
         // the pieces selected for the marks are re-rooted child pieces, all
@@ -1527,30 +1509,33 @@ __global__ void __launch_bounds__(BLK)
         unsigned chg = 0;
 #pragma unroll
         for (int k = 0; k < IP; ++k)
-            if (i0 + (long long)k * blockDim.x < cnt && rep_ep[p[k]] == ep) chg |= 1u << k;
+            if (i0 + (long long)k * blockDim.x < cnt && a.rep_ep[p[k]] == ep) chg |= 1u << k;
         unsigned on = 0;
-        for (unsigned m = chg; m; m &= m - 1) {
-            const int k = __ffs(m) - 1;
-            const int pk = p[k];
-            if (sel_ep[pk] == ep && att_x[pk] != pk) on |= 1u << k;
+        long long q = 0;
+        if (marks) {   // (the same value in every thread)
+            for (unsigned m = chg; m; m &= m - 1) {
+                const int k = __ffs(m) - 1;
+                const int pk = p[k];
+                if (a.sel_ep[pk] == ep && a.att_x[pk] != pk) on |= 1u << k;
+            }
+            q = block_reserve(&ctl->nact, __popc(on));
         }
-        long long q = block_reserve(&ctl->nact, __popc(on));
         for (unsigned m = chg; m; m &= m - 1) {
             const int k = __ffs(m) - 1;
             const int pk = p[k];
             const long long i = i0 + (long long)k * blockDim.x;
-            const int v = use_list ? L[i] : (int)i;
+            const int v = L ? L[i] : (int)i;
             if ((on >> k) & 1u) {
-                const int pv = parent[v];
-                act[q] = v;
-                pold[q] = pv;
-                J0[v] = pv;
-                mark[v] = v == att_x[pk];
-                aidx[v] = (int)q;   // dense index (Euler-tour marks)
-                aroot[q] = pk;      // the piece root
+                const int pv = a.parent[v];
+                a.act[q] = v;
+                a.pold[q] = pv;
+                a.J0[v] = pv;
+                a.mark[v] = v == a.att_x[pk];
+                a.aidx[v] = (int)q;   // dense index (Euler-tour marks)
+                a.aroot[q] = pk;      // the piece root
                 ++q;
             }
-            rep[v] = newrep[pk];
+            a.rep[v] = a.newrep[pk];
         }
     }
 }
@@ -1561,19 +1546,14 @@ __global__ void __launch_bounds__(BLK)
 // round j the marks cover distances [0, 2^{j+1}); the loop stops once every
 // J_{j+1} is a root, which bounds the path length.  Marks only ever land on
 // ancestors of x, so reads racing with writes within a round are harmless.
-__global__ void k_mark(Ctl *ctl, const int *act, int *J0, int *J1, unsigned char *mark, const int *parent) {
-    if (*(volatile int *)&ctl->skip) return;
-    long long na = (long long)ctl->nact;
-    if (na == 0) {   // every path was walked (the same value in every block)
-        if (gtid() == 0) ctl->mark_rounds = 0;
-        return;
-    }
-    int *Jc = J0, *Jn = J1;
+// Returns false when a grid barrier gave up or the rounds ran out.
+__device__ bool mark_paths(Ctl *ctl, const FinishArgs &a, long long na) {
+    int *Jc = a.J0, *Jn = a.J1;
     int r = 0;
     for (;; ++r) {
         if (r >= MAX_ROUNDS) {
             if (gtid() == 0) atomicOr(&ctl->err, ERR_ROUNDS);
-            return;
+            return false;
         }
         if (gtid() == 0) ctl->flag[(r + 1) % 3] = 0;
         bool more = false;
@@ -1586,52 +1566,81 @@ __global__ void k_mark(Ctl *ctl, const int *act, int *J0, int *J1, unsigned char
             for (int k = 0; k < JU; ++k) {
                 long long i = base + k * S;
                 ok[k] = i < na;
-                v[k] = ok[k] ? act[i] : 0;
+                v[k] = ok[k] ? LD(a.act[i]) : 0;
             }
 #pragma unroll
             for (int k = 0; k < JU; ++k) {
                 w[k] = ok[k] ? LD(Jc[v[k]]) : 0;
-                mk[k] = ok[k] ? LD(mark[v[k]]) : 0;
+                mk[k] = ok[k] ? LD(a.mark[v[k]]) : 0;
             }
 #pragma unroll
             for (int k = 0; k < JU; ++k) w2[k] = ok[k] ? LD(Jc[w[k]]) : 0;
 #pragma unroll
             for (int k = 0; k < JU; ++k) {
                 if (!ok[k]) continue;
-                if (mk[k]) mark[w[k]] = 1;
+                if (mk[k]) a.mark[w[k]] = 1;
                 Jn[v[k]] = w2[k];
-                more |= parent[w2[k]] != w2[k];
+                more |= a.parent[w2[k]] != w2[k];
             }
         }
         if (__syncthreads_or(more) && threadIdx.x == 0) atomicOr(&ctl->flag[r % 3], 1);
-        if (!grid_barrier(ctl, &ctl->bar[3])) return;
+        if (!grid_barrier(ctl, &ctl->bar[3])) return false;
         int again = *(volatile int *)&ctl->flag[r % 3];
         int *t = Jc; Jc = Jn; Jn = t;
         if (!again) break;
     }
     if (gtid() == 0) ctl->mark_rounds = r + 1;
+    return true;
 }
 
 // ReversePaths + attach (Algorithm 1): for each marked non-root vertex u,
 // parent'[old parent of u] = u (old parents come from the saved snapshot, so
 // no thread reads a pointer another thread rewrites); then parent[x] = y for
 // every oriented replacement edge x -> y.
-__global__ void k_reverse(Ctl *ctl, const int *act, const int *pold, const unsigned char *mark, const int *chx,
-                          const int *chy, int *parent, int walked) {
-    if (*(volatile int *)&ctl->skip) return;
-    long long na = (long long)ctl->nact, ner = (long long)ctl->ner;
-    if (walked && na == 0) return;   // every piece was reversed and attached by its walk
+__device__ __forceinline__ void reverse_marked(Ctl *ctl, const FinishArgs &a, long long na) {
+    const long long ner = (long long)ctl->ner;
     long long c = 0;
     GS_LOOP(i, na) {
-        int v = act[i];
-        int p = pold[i];
-        if (mark[v] && p != v) {
-            parent[p] = v;
+        const int v = LD(a.act[i]);
+        const int p = LD(a.pold[i]);
+        if (LD(a.mark[v]) && p != v) {
+            a.parent[p] = v;
             ++c;
         }
     }
     if (c) atomicAdd((u64 *)&ctl->reversed, (u64)c);
-    GS_LOOP(i, ner) parent[chx[i]] = chy[i];
+    GS_LOOP(i, ner) a.parent[a.chx[i]] = a.chy[i];
+}
+
+// End of a batch: the representative refresh, and, when some walk was too
+// long (ctl->nlong), the doubling marks and the reversal of those pieces, in
+// one cooperative launch: without long walks (the common case) it is one
+// pass and no grid barrier, where two launches that found nothing to do cost
+// 10 us of every batch.  An insert passes over all vertices, a delete over
+// its affected list; after a top-down delete that list holds the detached
+// vertices only, so the rare one that re-rooted a tree's root piece
+// (need_root) passes over all vertices too.  With a.euler the marks are the
+// Euler tour's (a launch of its own) and k_reverse follows it.
+__global__ void __launch_bounds__(BLK, 5) k_finish(Ctl *ctl, FinishArgs a) {
+    if (*(volatile int *)&ctl->skip) return;
+    const unsigned ep = ctl->epoch;
+    const bool marks = a.euler || *(volatile int *)&ctl->nlong;
+    if (ctl->op == DRSF_DELETE && !(ctl->td && *(volatile int *)&ctl->need_root))
+        refresh_pass<IPT>(ctl, a, a.A, (long long)ctl->naff, ep, marks);
+    else if (a.n <= gstride() * IPT)
+        refresh_pass<IPT>(ctl, a, nullptr, a.n, ep, marks);
+    else
+        refresh_pass<IPN>(ctl, a, nullptr, a.n, ep, marks);
+    if (a.euler || !marks) return;
+    if (!grid_barrier(ctl, &ctl->bar[3])) return;
+    const long long na = (long long)*(volatile u64 *)&ctl->nact;
+    if (na == 0) return;
+    if (!mark_paths(ctl, a, na)) return;
+    reverse_marked(ctl, a, na);
+}
+__global__ void k_reverse(Ctl *ctl, FinishArgs a) {
+    if (*(volatile int *)&ctl->skip) return;
+    reverse_marked(ctl, a, (long long)ctl->nact);
 }
 
 // Component labels: smallest vertex id per tree (drsf_labels).
@@ -1667,13 +1676,10 @@ static unsigned coop_blocks(const void *fn, int nsm, int cap_per_sm) {
     if (per > cap_per_sm) per = cap_per_sm;
     return (unsigned)(per * nsm);
 }
-// The vertex passes (k_aff_collect, k_active) loop over their range with
+// The vertex passes (k_aff_collect, k_finish) loop over their range with
 // the blocks that are resident at once: no partial last wave.
-unsigned grid_vertex_pass(int nsm) {
-    unsigned a = coop_blocks((const void *)k_aff_collect, nsm, 8), b = coop_blocks((const void *)k_active<IPN>, nsm, 8);
-    return a < b ? a : b;
-}
-unsigned grid_list_pass(int nsm) { return coop_blocks((const void *)k_active<IPT>, nsm, 8); }
+unsigned grid_vertex_pass(int nsm) { return coop_blocks((const void *)k_aff_collect, nsm, 8); }
+unsigned coop_blocks_finish(int nsm) { return coop_blocks((const void *)k_finish, nsm, 8); }
 unsigned coop_blocks_jump(int nsm) {
     // the three root-search variants share one launch bound; take the least
     unsigned a = coop_blocks((const void *)k_jump<0>, nsm, 8), b = coop_blocks((const void *)k_jump<1>, nsm, 8),
@@ -1698,17 +1704,14 @@ unsigned coop_blocks_orient(int nsm) {
     if (per > 2) per = 2;
     return (unsigned)(per * nsm);
 }
-unsigned coop_blocks_mark(int nsm) { return coop_blocks((const void *)k_mark, nsm, 4); }
 
 cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s) {
     k_begin<<<1, 32, 0, s>>>(ctl, op, len, batch);
     return cudaGetLastError();
 }
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, int roots_only,
-                               cudaStream_t s) {
-    k_aff_collect<<<d.grid_pass, BLK, 0, s>>>(n, rep, aff_ep, A, rold, w, heavy, ctl, par, J, roots_only);
-    (void)d;
+                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, cudaStream_t s) {
+    k_aff_collect<<<d.grid_pass, BLK, 0, s>>>(n, rep, aff_ep, A, rold, w, heavy, ctl, par, J);
     return cudaGetLastError();
 }
 cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf,
@@ -1720,11 +1723,6 @@ cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *pa
                     (void *)&det_ep,  (void *)&det_claim, (void *)&rold,    (void *)&budget_v,   (void *)&budget_e,
                     (void *)&max_levels, (void *)&oc,    (void *)&op};
     return cudaLaunchCooperativeKernel((const void *)k_detach, d.coop_detach, BLK, args, 0, s);
-}
-cudaError_t launch_rootcheck(const Dev &d, Ctl *ctl, const int *cuts, const int *rold, const unsigned *rep_ep,
-                             cudaStream_t s) {
-    k_rootcheck<<<d.nsm, BLK, 0, s>>>(ctl, cuts, rold, rep_ep);
-    return cudaGetLastError();
 }
 unsigned coop_blocks_detach(int nsm) { return coop_blocks((const void *)k_detach, nsm, 4); }
 cudaError_t launch_jump_async(const Dev &d, const int *A, Ctl *ctl, int *J, int *X, int *Y, cudaStream_t s) {
@@ -1760,26 +1758,12 @@ cudaError_t launch_walk(const Dev &d, Ctl *ctl, const int *chx, const int *chy, 
     k_walk<<<d.grid, BLK, 0, s>>>(ctl, chx, chy, rep, parent, long_ep);
     return cudaGetLastError();
 }
-cudaError_t launch_active(const Dev &d, const int *L, int use_list, long long cnt_static, Ctl *ctl, int *rep,
-                          const int *parent, const unsigned *sel_ep, const int *att_x, const unsigned *rep_ep,
-                          const int *newrep, int *act, int *pold, int *J0, unsigned char *mark, int *aidx,
-                          int *aroot, cudaStream_t s) {
-    if (use_list)
-        k_active<IPT><<<d.grid_list, BLK, 0, s>>>(L, use_list, cnt_static, ctl, rep, parent, sel_ep, att_x, rep_ep,
-                                                  newrep, act, pold, J0, mark, aidx, aroot);
-    else
-        k_active<IPN><<<d.grid_pass, BLK, 0, s>>>(L, use_list, cnt_static, ctl, rep, parent, sel_ep, att_x, rep_ep,
-                                                  newrep, act, pold, J0, mark, aidx, aroot);
-    return cudaGetLastError();
+cudaError_t launch_finish(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s) {
+    void *args[] = {(void *)&ctl, (void *)&a};
+    return cudaLaunchCooperativeKernel((const void *)k_finish, d.coop_finish, BLK, args, 0, s);
 }
-cudaError_t launch_mark(const Dev &d, Ctl *ctl, const int *act, int *J0, int *J1, unsigned char *mark,
-                        const int *parent, cudaStream_t s) {
-    void *args[] = {(void *)&ctl, (void *)&act, (void *)&J0, (void *)&J1, (void *)&mark, (void *)&parent};
-    return cudaLaunchCooperativeKernel((const void *)k_mark, d.coop_mark, BLK, args, 0, s);
-}
-cudaError_t launch_reverse(const Dev &d, Ctl *ctl, const int *act, const int *pold, const unsigned char *mark,
-                           const int *chx, const int *chy, int *parent, int walked, cudaStream_t s) {
-    k_reverse<<<d.grid, BLK, 0, s>>>(ctl, act, pold, mark, chx, chy, parent, walked);
+cudaError_t launch_reverse(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s) {
+    k_reverse<<<d.grid, BLK, 0, s>>>(ctl, a);
     return cudaGetLastError();
 }
 cudaError_t launch_labels(int n, const int *rep, int *tmp, int *out, cudaStream_t s) {

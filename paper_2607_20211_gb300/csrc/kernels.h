@@ -14,13 +14,12 @@ struct Dev {
     unsigned coop_hook;        // (1024-thread blocks)
     unsigned coop_hook_small;  // (256-thread blocks, for large batches)
     unsigned coop_orient;
-    unsigned coop_mark;
+    unsigned coop_finish;
     unsigned coop_bfs;
     unsigned coop_et;
     unsigned coop_detach;
     unsigned grid_scan;   // row scan: the co-resident block count
-    unsigned grid_pass;   // passes over all n vertices (affected list, insert refresh): co-resident blocks
-    unsigned grid_list;   // passes over a vertex list (delete refresh): co-resident blocks
+    unsigned grid_pass;   // affected list: co-resident blocks
 };
 
 // graph.cu -------------------------------------------------------------
@@ -78,10 +77,9 @@ cudaError_t launch_check_cross(const int *pairs, long long m, const int *rep, in
 // forest.cu ------------------------------------------------------------
 cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s);
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, int roots_only,
-                               cudaStream_t s);
+                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, cudaStream_t s);
 // delete: detached vertices top-down from the cut vertices (falls back to
-// the pointer jumping above when over budget); root pieces to list after it.
+// the pointer jumping above when over budget).
 // DETACH_LEVELS: its level limit (measured on R-MAT, where it pays, the
 // search takes 2-7 levels; on deep trees each level costs about as much as
 // a whole pointer-jumping round)
@@ -90,8 +88,6 @@ cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *pa
                           u64 ovf_cap, RowList rl, int *A, int *J1, unsigned *det_ep, unsigned *det_claim,
                           const int *rold, long long budget_v, long long budget_e, int max_levels, int *oc, int *op,
                           cudaStream_t s);
-cudaError_t launch_rootcheck(const Dev &d, Ctl *ctl, const int *cuts, const int *rold, const unsigned *rep_ep,
-                             cudaStream_t s);
 unsigned coop_blocks_detach(int nsm);
 cudaError_t launch_jump_async(const Dev &d, const int *A, Ctl *ctl, int *J, int *X, int *Y, cudaStream_t s);
 cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par,
@@ -118,28 +114,35 @@ struct OrientArgs {
     int *eroot;          // per edge: hook-forest root of its super-tree
     int *cel;            // core edges (for the one-block path of small cores)
     const int *parent;   // the forest: pulled into L2 for the walks that follow
+    const unsigned *aff_ep;   // old roots of this batch's cut trees
     long long n;
 };
 cudaError_t launch_orient(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, const int *chx, const int *chy, const int *rep, int *parent,
                         unsigned *long_ep, cudaStream_t s);
-cudaError_t launch_active(const Dev &d, const int *L, int use_list, long long cnt_static, Ctl *ctl, int *rep,
-                          const int *parent, const unsigned *sel_ep, const int *att_x, const unsigned *rep_ep,
-                          const int *newrep, int *act, int *pold, int *J0, unsigned char *mark, int *aidx,
-                          int *aroot, cudaStream_t s);
-cudaError_t launch_mark(const Dev &d, Ctl *ctl, const int *act, int *J0, int *J1, unsigned char *mark,
-                        const int *parent, cudaStream_t s);
-cudaError_t launch_reverse(const Dev &d, Ctl *ctl, const int *act, const int *pold, const unsigned char *mark,
-                           const int *chx, const int *chy, int *parent, int walked, cudaStream_t s);
+struct FinishArgs {
+    const int *A;             // delete: the affected list
+    long long n;
+    int *rep, *parent;
+    const unsigned *sel_ep;   // pieces reversed through the marks
+    const int *att_x;
+    const unsigned *rep_ep;
+    const int *newrep;
+    int *act, *pold, *J0, *J1, *aidx, *aroot;
+    unsigned char *mark;
+    const int *chx, *chy;
+    int euler;
+};
+cudaError_t launch_finish(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s);
+cudaError_t launch_reverse(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s);
 cudaError_t launch_labels(int n, const int *rep, int *tmp, int *out, cudaStream_t s);
 
 unsigned coop_blocks_jump(int nsm);
 unsigned grid_vertex_pass(int nsm);
-unsigned grid_list_pass(int nsm);
+unsigned coop_blocks_finish(int nsm);
 unsigned coop_blocks_hook(int nsm);
 unsigned coop_blocks_hook_small(int nsm);
 unsigned coop_blocks_orient(int nsm);
-unsigned coop_blocks_mark(int nsm);
 cudaError_t launch_barrier_selftest(Ctl *ctl, cudaStream_t s);
 // static.cu ------------------------------------------------------------
 cudaError_t launch_static_forest(const Dev &d, int n, Csr g, const u64 *ovf, Ctl *ctl, int *lab, int *comp,
