@@ -135,11 +135,11 @@ enum {
     PH_AFF,           // delete: affected-vertex list
     PH_JUMP,          // delete: pointer jumping (representatives)
     PH_SCAN,          // delete: cross-edge scan of detached rows + overflow
-    PH_HOOK,          // hook-and-compress (replacement edges)
-    PH_ORIENT,        // Euler-tour orientation
+    PH_HOOK,          // replacement edges: hook-and-compress, orientation, path walks
+    PH_ORIENT,        // large batches: the orientation as a launch of its own
     PH_ACTIVE,        // representative refresh, and the doubling marks and reversal of long paths
     PH_MARK,          // Euler-tour marks
-    PH_REVERSE        // path walks (Euler: reversal scatter + attach)
+    PH_REVERSE        // large batches: path walks; Euler: reversal scatter + attach
 };
 static const char *kPhaseNames[DRSF_NUM_PHASES] = {
     "begin", "ins_claim", "ins_place", "del_claim", "affected", "jump", "scan", "hook", "orient", "active",
@@ -625,7 +625,6 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.grid = (unsigned)nsm * 8u;
     h->dev.coop_jump = coop_blocks_jump(nsm);
     h->dev.coop_hook = coop_blocks_hook(nsm);
-    h->dev.coop_hook_small = coop_blocks_hook_small(nsm);
     h->dev.coop_orient = coop_blocks_orient(nsm);
     h->dev.coop_finish = coop_blocks_finish(nsm);
     h->dev.coop_bfs = coop_blocks_bfs(nsm);
@@ -691,8 +690,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         prof_begin(h, PH_INS_PLACE, s);
         CK(launch_ins_place(h->dev, h->nkey, h->nslot, ctl, g, h->ix, h->ovf, h->ovf_cap, h->rep, sg, h->pt,
                             h->ck[0], h->ca[0], h->cb[0], h->cand_cap, hook_slots(h), s));
-        if (sg) CK(launch_pairs_compact(h->dev, ctl, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap, s));
-        prof_end(h, PH_INS_PLACE, sg ? 2 : 1, s);
+        prof_end(h, PH_INS_PLACE, 1, s);
     } else {
         // Algorithm 1, delete: remove B, cut tree edges, re-label the cut trees
         prof_begin(h, PH_DEL_CLAIM, s);
@@ -722,16 +720,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         CK(launch_scan_rows(h->dev, rows(h), ctl, g, h->rep, sg, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap,
                             s));
         CK(launch_scan_ovf(h->dev, h->ovf, ctl, h->rep, sg, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap, s));
-        if (sg) CK(launch_pairs_compact(h->dev, ctl, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap, s));
-        prof_end(h, PH_SCAN, sg ? 3 : 2, s);
+        prof_end(h, PH_SCAN, 2, s);
     }
-    prof_begin(h, PH_HOOK, s);
-    // an HS insert's candidates all come from k_ins_place, which set up
-    // their hook-forest slots; otherwise the hooking sets them up itself
-    // (inside the scan of a large delete that costs more than it saves)
-    CK(launch_boruvka(h->dev, ctl, h->ck[0], h->ca[0], h->cb[0], h->ck[1], h->ca[1], h->cb[1], hook_slots(h), h->er,
-                      h->n, (op == DRSF_INSERT && !sg) ? 0 : 1, glen > (1 << 18), s));
-    prof_end(h, PH_HOOK, 1, s);
     OrientArgs oa{};
     oa.er = h->er;
     oa.rep = h->rep;
@@ -764,18 +754,46 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     oa.cel = h->nx1;   // (the grid ranking's second buffer: unused on the one-block path)
     oa.parent = h->parent;
     oa.aff_ep = h->aff_ep;
+    oa.long_ep = h->long_ep;
     oa.n = h->n;
-    prof_begin(h, PH_ORIENT, s);
-    CK(launch_orient(h->dev, ctl, oa, s));
-    prof_end(h, PH_ORIENT, 1, s);
-    // Path reversal: by default short paths are reversed by walking and only
-    // the pieces with long paths go through the marks; the Euler-tour
-    // variant (Algorithm 3) takes every re-rooted piece.
+    // Path reversal: by default short paths are reversed by walking, as each
+    // replacement edge is oriented, and only the pieces with long paths go
+    // through the marks; the Euler-tour variant (Algorithm 3) takes every
+    // re-rooted piece.
     const bool euler = (h->flags & DRSF_EULER_REVERSAL) != 0;
-    if (!euler) {
-        prof_begin(h, PH_REVERSE, s);
-        CK(launch_walk(h->dev, ctl, h->chx, h->chy, h->rep, h->parent, h->long_ep, s));
-        prof_end(h, PH_REVERSE, 1, s);
+    const bool large = glen > LARGE_BATCH;
+    oa.walk = euler || large ? 0 : 1;
+    HookArgs ha{};
+    for (int b = 0; b < 2; ++b) {
+        ha.ck[b] = h->ck[b];
+        ha.ca[b] = h->ca[b];
+        ha.cb[b] = h->cb[b];
+    }
+    ha.cand_cap = h->cand_cap;
+    ha.hs = hook_slots(h);
+    ha.er = h->er;
+    ha.er_cap = h->n;
+    // an HS insert's candidates all come from k_ins_place, which set up
+    // their hook-forest slots; otherwise the hooking sets them up itself
+    // (inside the scan of a large delete that costs more than it saves)
+    ha.init = (op == DRSF_INSERT && !sg && !large) ? 0 : 1;
+    ha.pairs = sg ? 1 : 0;
+    ha.pt = h->pt;
+    prof_begin(h, PH_HOOK, s);
+    if (large) {
+        CK(launch_hook_large(h->dev, ctl, ha, s));
+        prof_end(h, PH_HOOK, sg ? 2 : 1, s);
+        prof_begin(h, PH_ORIENT, s);
+        CK(launch_orient(h->dev, ctl, oa, s));
+        prof_end(h, PH_ORIENT, 1, s);
+        if (!euler) {
+            prof_begin(h, PH_REVERSE, s);
+            CK(launch_walk(h->dev, ctl, oa, s));
+            prof_end(h, PH_REVERSE, 1, s);
+        }
+    } else {
+        CK(launch_replace(h->dev, ctl, ha, oa, s));
+        prof_end(h, PH_HOOK, 1, s);
     }
     FinishArgs fa{};
     fa.A = h->A;

@@ -302,7 +302,6 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
                 } else {
                     atomicOr(&ctl->err, ERR_CAPACITY);
                 }
-                atomicAdd((u64 *)&ctl->overflow_total, 1ull);
             }
             const int ra = GL(S.rep[a]), rb = GL(S.rep[b]);
             if (ra != rb) pool_put(G, S, k, ra, rb);

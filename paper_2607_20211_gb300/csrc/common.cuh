@@ -79,7 +79,6 @@ struct Ctl {
     long long jump_visits;
     long long reversed;
     long long batch_len;
-    long long overflow_total;
     const int *batch;       // the current batch (device), set by k_begin
     int td;                 // delete: the detached vertices were found top-down (else: pointer jumping)
     int need_root;          // delete: a cut tree's root piece is re-rooted (read after a top-down delete)

@@ -21,12 +21,8 @@
 #define ORIENT_SMEM_ARCS 12288
 #define ORIENT_SMEM_BYTES (4 * ORIENT_SMEM_ARCS * (int)sizeof(int))
 #define ORIENT_THREADS 1024
-// hooking: threads per block (one block per SM) and the live candidates at
-// the start of a round (after round 0) up to which block 0 finishes alone
-// (the kernel comes in two block sizes: 1024 threads, one block per SM, so
-// that block 0 has the threads for the tail, and 256 threads, four per SM,
-// for batches whose candidates stay in the millions past round 0, where
-// the grid rounds measured faster with smaller blocks)
+// hooking: the live candidates at the start of a round (after round 0) up to
+// which block 0 finishes alone
 #define HOOK_TAIL 8192
 // a core of at most this many edges is oriented by one block (measured on
 // R-MAT-22: faster than the grid phases for small batches' cores of tens of
@@ -846,6 +842,55 @@ __global__ void __launch_bounds__(BLK, 6)
     }
 }
 
+// Move the pair table into the candidate list (one candidate per piece
+// pair, its minimum key) and free the slots for the next batch.
+__device__ __forceinline__ void compact_pairs(Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap) {
+    // four slots per thread and iteration, one counter reservation per
+    // block (the table has far more slots than warps have lanes, and most
+    // warps hold an occupied slot: a per-warp append would queue on the
+    // counter)
+    const long long T = (long long)pt.mask + 1;
+    const long long S = (long long)gridDim.x * blockDim.x;
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < T; base += 4 * S) {
+        u64 pair[4], k[4];
+        bool on[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            long long i = base + q * S + threadIdx.x;
+            pair[q] = i < T ? pt.pk[i] : EMPTY_KEY;
+            on[q] = pair[q] != EMPTY_KEY;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            k[q] = 0;
+            if (on[q]) {
+                long long i = base + q * S + threadIdx.x;
+                k[q] = pt.mk[i];
+                pt.pk[i] = EMPTY_KEY;
+                pt.mk[i] = EMPTY_KEY;
+            }
+        }
+        long long p[4];
+        block_reserve4(&ctl->ncand, on, p);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (!on[q]) continue;
+            if ((u64)p[q] < cand_cap) {
+                ck[p[q]] = k[q];
+                ca[p[q]] = (int)(pair[q] >> 32);
+                cb[p[q]] = (int)(pair[q] & 0xFFFFFFFFu);
+            } else {
+                atomicOr(&ctl->err, ERR_CAPACITY);
+            }
+        }
+    }
+}
+__global__ void __launch_bounds__(BLK) k_pairs_compact(Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb,
+                                                       u64 cand_cap) {
+    if (*(volatile int *)&ctl->skip) return;
+    compact_pairs(ctl, pt, ck, ca, cb, cand_cap);
+}
+
 // Per-block table of hot indices for 64-bit minimum updates: lanes of a
 // warp with the same index combine first; an index held by two or more
 // lanes of a warp (one piece, such as the giant one, can be an endpoint of
@@ -1017,35 +1062,72 @@ __device__ __forceinline__ int hook_rounds(Ctl *ctl, HotMin &hm, int r, long lon
     return 0;
 }
 
-template <int HT>
-__global__ void __launch_bounds__(HT, 1024 / HT) k_boruvka(Ctl *ctl, u64 *ck0, int *ca0, int *cb0, u64 *ck1,
-                                                          int *ca1, int *cb1, HookSlots hs, u64 *er,
-                                                          long long er_cap, int init) {
+// Set up each candidate endpoint once (the first lane to stamp it).
+__device__ __forceinline__ void hook_init(const HookArgs &h, long long c0, unsigned ep) {
+    for (long long i = gtid(); i < c0; i += gstride()) {
+        hook_slot_init(h.hs, LD(h.ca[0][i]), ep);
+        hook_slot_init(h.hs, LD(h.cb[0][i]), ep);
+    }
+}
+
+// Hooking as a launch of its own, for batches above LARGE_BATCH edges, whose
+// candidates stay in the millions past round 0: 256-thread blocks, four per
+// SM (R-MAT scale 20, 1M deletes: 5.0 against 5.4 ms with 1024).
+__global__ void __launch_bounds__(256, 4) k_hook_large(Ctl *ctl, HookArgs h) {
     if (*(volatile int *)&ctl->skip) return;
     __shared__ HotMin hm;
-    const unsigned ep = ctl->epoch;
     const long long c0 = (long long)ctl->ncand;
     if (gtid() == 0) {
         ctl->cnt[1] = ctl->cnt[2] = 0;
         ctl->flag[0] = ctl->flag[1] = ctl->flag[2] = 0;
     }
     hm_init(hm);
-    if (init) {
-        // set up each candidate endpoint once (the first lane to stamp it);
-        // with init == 0 the kernel that wrote the candidates did it and
-        // round 0 starts at once
-        for (long long i = gtid(); i < c0; i += gstride()) {
-            hook_slot_init(hs, ca0[i], ep);
-            hook_slot_init(hs, cb0[i], ep);
-        }
-        if (!grid_barrier(ctl, &ctl->bar[1])) return;
-    } else {
-        __syncthreads();
-    }
-    const int r = hook_rounds<false>(ctl, hm, 0, c0, ck0, ca0, cb0, ck1, ca1, cb1, hs.comp, hs.best0, hs.best1, er,
-                                     er_cap);
+    hook_init(h, c0, ctl->epoch);
+    if (!grid_barrier(ctl, &ctl->bar[1])) return;
+    const int r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
+                                     h.hs.best0, h.hs.best1, h.er, h.er_cap);
     if (r > 0 && blockIdx.x == 0)
-        hook_rounds<true>(ctl, hm, r, c0, ck0, ca0, cb0, ck1, ca1, cb1, hs.comp, hs.best0, hs.best1, er, er_cap);
+        hook_rounds<true>(ctl, hm, r, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp, h.hs.best0,
+                          h.hs.best1, h.er, h.er_cap);
+}
+
+// Path reversal by walking (ReversePaths, Algorithm 1): the path x = v0, v1 =
+// parent[v0], ..., vL (the piece root) is read first and then reversed
+// (parent[v_j] <- v_{j-1}, parent[v0] <- y).  Each child piece has exactly
+// one oriented edge and pieces are disjoint, so the walks never touch the
+// same vertex, and a walk needs nothing but its own edge: whoever orients an
+// edge can walk it at once.  A path of more than WALK_MAX edges stays as it
+// is: its piece is stamped in long_ep and reversed by the pointer-doubling
+// marks.  Returns the vertices reversed.
+// Reversing while walking, each load behind a store into sectors that other
+// walks read and write, took five times as long: 283 -> 51 us per delete
+// batch on the 4096 x 4096 grid (100K edges), 118 -> 27 us on the 256-graph
+// union (1.6M edges).
+__device__ __forceinline__ int walk_path(Ctl *ctl, int *parent, int x, int y, unsigned *long_ep, int piece,
+                                         unsigned ep) {
+    int path[WALK_MAX];   // path[j] = parent[v_j]
+    int len = 0, cur = x;
+    for (; len < WALK_MAX; ++len) {
+        const int nxt = LD(parent[cur]);
+        if (nxt == cur) break;
+        path[len] = nxt;
+        cur = nxt;
+    }
+    if (len == WALK_MAX) {
+        long_ep[piece] = ep;
+        ctl->nlong = 1;
+        return 0;
+    }
+    int prev = y;
+    cur = x;
+    for (int j = 0; j < len; ++j) {
+        const int nxt = path[j];
+        parent[cur] = prev;
+        prev = cur;
+        cur = nxt;
+    }
+    parent[cur] = prev;
+    return len;
 }
 
 // Orientation of replacement edge i: down = its lower-id endpoint's piece
@@ -1056,8 +1138,8 @@ __global__ void __launch_bounds__(HT, 1024 / HT) k_boruvka(Ctl *ctl, u64 *ck0, i
 // representative).  A child that is the root piece of a cut tree (its root
 // was stamped by the cut) is noted: after a top-down delete the affected list
 // holds the detached vertices only, and the refresh then has to pass over
-// all vertices.
-__device__ __forceinline__ void orient_one(Ctl *ctl, const OrientArgs &a, long long i, bool down, unsigned ep) {
+// all vertices.  Returns the vertices that its walk reversed.
+__device__ __forceinline__ int orient_one(Ctl *ctl, const OrientArgs &a, long long i, bool down, unsigned ep) {
     const u64 k = a.er[i];
     const int x0 = (int)klo(k), x1 = (int)khi(k);
     const int p0 = LD(a.ep[2 * i]), p1 = LD(a.ep[2 * i + 1]);
@@ -1070,6 +1152,7 @@ __device__ __forceinline__ void orient_one(Ctl *ctl, const OrientArgs &a, long l
     a.newrep[child] = LD(a.minp[LD(a.eroot[i])]);
     a.rep_ep[child] = ep;
     if (a.aff_ep[child] == ep) ctl->need_root = 1;
+    return a.walk ? walk_path(ctl, a.parent, x, y, a.long_ep, child, ep) : 0;
 }
 
 // Wyllie list ranking of ncore list cells in shared memory by one block:
@@ -1151,10 +1234,12 @@ __device__ void orient_small_core(Ctl *ctl, const OrientArgs &a, const int *cel,
     __syncthreads();
     int *rank = nullptr;
     const int rounds = rank_block(ctl, svc, svn, snc, snn, ncore, &rank);
+    int rev = 0;
     for (long long t = threadIdx.x; t < nce; t += blockDim.x) {
         const long long i = LD(cel[t]);
-        orient_one(ctl, a, i, rank[a.apos[2 * i]] > rank[a.apos[2 * i + 1]], ep);
+        rev += orient_one(ctl, a, i, rank[a.apos[2 * i]] > rank[a.apos[2 * i + 1]], ep);
     }
+    block_add(&ctl->reversed, rev);
     if (threadIdx.x == 0) {
         ctl->ncore = (u64)ncore;
         ctl->rank_rounds = rounds;
@@ -1172,9 +1257,8 @@ __device__ void orient_small_core(Ctl *ctl, const OrientArgs &a, const int *cel,
 // each edge is oriented by its arc that comes first.  The child piece P of
 // edge {x, y} (x in P) gets the oriented replacement edge x -> y; every piece
 // of the super-tree gets the root as its new representative.
-__global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
-    const long long ner = (long long)ctl->ner;
+__device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
+    const long long ner = (long long)*(volatile u64 *)&ctl->ner;
     const unsigned ep = ctl->epoch;
     u64 *bar = &ctl->bar[2];
     // Arc j of edge j/2 runs from the piece of its (j odd ? larger : smaller)
@@ -1183,9 +1267,9 @@ __global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs 
     // (eroot), so no phase re-walks rep / pidx / the hook forest.
     // phase 1: dense ids for the pieces touched by E_r
     if (gtid() == 0) ctl->ncore = ctl->cnt[0] = ctl->cnt[1] = 0;
-    // the path walks after this kernel follow parent pointers one dependent
-    // load at a time: pull the forest into L2 now, while the phases below
-    // wait at their barriers (one 128-byte line per thread or so)
+    // the path walks follow parent pointers one dependent load at a time:
+    // pull the forest into L2 now, while the phases below wait at their
+    // barriers (one 128-byte line per thread or so)
     if (ner > 0) l2_prefetch(a.parent, 4 * a.n, gtid(), gstride());
     // (block-uniform loop: the dense ids are reserved once per block)
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < 2 * ner; b0 += gstride()) {
@@ -1311,11 +1395,18 @@ __global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs 
             cel = cel2;
         }
         if (nce <= ORIENT_SMALL_EDGES) {
-            for (long long i = gtid(); i < ner; i += gstride()) {
-                const unsigned char lf = LD(a.lf[i]);
-                if (lf) orient_one(ctl, a, i, lf == 2, ep);
-            }
+            // (block 0 leaves the leaf edges to the others: its core and
+            // their walks run side by side)
             if (blockIdx.x == 0) orient_small_core(ctl, a, cel, nce, ep);
+            const bool alone = gridDim.x == 1;
+            if (blockIdx.x == 0 && !alone) return;
+            const long long t0 = alone ? gtid() : gtid() - blockDim.x, st = alone ? gstride() : gstride() - blockDim.x;
+            int rev = 0;
+            for (long long i = t0; i < ner; i += st) {
+                const unsigned char lf = LD(a.lf[i]);
+                if (lf) rev += orient_one(ctl, a, i, lf == 2, ep);
+            }
+            block_add(&ctl->reversed, rev);
             return;
         }
     }
@@ -1420,56 +1511,279 @@ __global__ void __launch_bounds__(ORIENT_THREADS) k_orient(Ctl *ctl, OrientArgs 
         if (gtid() == 0) ctl->rank_rounds = r + 1;
     }
     // phase 7: orient, attach points, new roots
+    int rev = 0;
     for (long long i = gtid(); i < ner; i += gstride()) {
         const unsigned char lf = LD(a.lf[i]);
         const bool down = lf ? lf == 2 : LD(vc[LD(a.apos[2 * i])]) > LD(vc[LD(a.apos[2 * i + 1])]);
-        orient_one(ctl, a, i, down, ep);
+        rev += orient_one(ctl, a, i, down, ep);
+    }
+    block_add(&ctl->reversed, rev);
+}
+__global__ void __launch_bounds__(ORIENT_THREADS, 1) k_orient(Ctl *ctl, OrientArgs a) {
+    if (*(volatile int *)&ctl->skip) return;
+    orient_grid(ctl, a);
+}
+
+// Replacement edges, orientation and walks of a batch with at most SMALL_CAND
+// candidates, by one block, everything but the walks in shared memory: the
+// pieces get dense ids through a hash table, the hook-and-compress rounds and
+// the orientation run on those, and only the results go to global memory.
+// On the grid the same batch is a chain of some twenty phases with a grid
+// barrier, two or three dependent global loads and up to a launch between
+// them, whatever its size.
+struct SmallTail {
+    u64 key[SMALL_CAND], best[2 * SMALL_CAND];
+    int hk[4 * SMALL_CAND];                       // hash table: piece, -1 free
+    int pid[2 * SMALL_CAND], comp[2 * SMALL_CAND], minp[2 * SMALL_CAND];
+    unsigned short hl[4 * SMALL_CAND];            // its dense id
+    unsigned short a[SMALL_CAND], b[SMALL_CAND], er[SMALL_CAND];
+    unsigned char vis[2 * SMALL_CAND];
+    int np, ner;
+};
+static_assert(sizeof(SmallTail) <= ORIENT_SMEM_BYTES, "one block's shared memory");
+
+// slot of piece p in the hash table (entered when absent; at most half full)
+__device__ __forceinline__ int tail_slot(SmallTail &t, int p) {
+    unsigned h = ((unsigned)p * 0x9E3779B1u) % (4 * SMALL_CAND);
+    for (;;) {
+        int k = *(volatile int *)&t.hk[h];
+        if (k == -1) {
+            k = atomicCAS(&t.hk[h], -1, p);
+            if (k == -1) {
+                const int l = atomicAdd(&t.np, 1);
+                t.pid[l] = p;
+                t.hl[h] = (unsigned short)l;
+                t.comp[l] = l;
+                t.best[l] = EMPTY_KEY;
+                t.minp[l] = INT_MAX;
+                t.vis[l] = 0;
+                return (int)h;
+            }
+        }
+        if (k == p) return (int)h;
+        h = (h + 1) % (4 * SMALL_CAND);
+    }
+}
+// root of dense piece x (hooking only ever links roots, so chains are short)
+__device__ __forceinline__ int tail_root(const SmallTail &t, int x) {
+    for (int it = 0; it < 2 * SMALL_CAND; ++it) {
+        const int p = *(volatile const int *)&t.comp[x];
+        if (p == x) break;
+        x = p;
+    }
+    return x;
+}
+// best[x] = min(best[x], k): lanes with one x combine first (one piece, such
+// as the giant one, can be an endpoint of most candidates)
+__device__ __forceinline__ void tail_min(SmallTail &t, int x, u64 k, bool on) {
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (!on) return;
+    const unsigned grp = __match_any_sync(m, x);
+    const u64 kmin = group_min_u64(grp, k);
+    if ((int)(threadIdx.x & 31) == __ffs(grp) - 1 && kmin < *(volatile u64 *)&t.best[x]) atomicMin(&t.best[x], kmin);
+}
+
+__device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa, int c0, unsigned ep) {
+    extern __shared__ __align__(16) int s_rank[];
+    SmallTail &t = *reinterpret_cast<SmallTail *>(s_rank);
+    constexpr int IT = SMALL_CAND / ORIENT_THREADS;   // candidates per thread
+    for (int i = threadIdx.x; i < 4 * SMALL_CAND; i += ORIENT_THREADS) t.hk[i] = -1;
+    if (threadIdx.x == 0) t.np = t.ner = 0;
+    __syncthreads();
+    u64 key[IT];
+    int ra[IT], rb[IT];
+    bool alive[IT];
+#pragma unroll
+    for (int q = 0; q < IT; ++q) {
+        const int i = q * ORIENT_THREADS + threadIdx.x;
+        alive[q] = i < c0;
+        key[q] = alive[q] ? LD(h.ck[0][i]) : 0;
+        ra[q] = alive[q] ? LD(h.ca[0][i]) : 0;
+        rb[q] = alive[q] ? LD(h.cb[0][i]) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < IT; ++q) {
+        if (alive[q]) {
+            ra[q] = tail_slot(t, ra[q]);
+            rb[q] = tail_slot(t, rb[q]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < IT; ++q) {
+        const int i = q * ORIENT_THREADS + threadIdx.x;
+        if (alive[q]) {
+            ra[q] = t.hl[ra[q]];
+            rb[q] = t.hl[rb[q]];
+            t.key[i] = key[q];
+            t.a[i] = (unsigned short)ra[q];
+            t.b[i] = (unsigned short)rb[q];
+        }
+    }
+    // hook and compress (as in hook_rounds)
+    int r = 0;
+    for (; r < MAX_ROUNDS; ++r) {
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            if (alive[q]) {
+                ra[q] = tail_root(t, ra[q]);
+                rb[q] = tail_root(t, rb[q]);
+                alive[q] = ra[q] != rb[q];
+            }
+            any |= alive[q];
+            tail_min(t, ra[q], key[q], alive[q]);
+            tail_min(t, rb[q], key[q], alive[q]);
+        }
+        if (!__syncthreads_or(any)) break;
+        bool used[IT];
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            used[q] = alive[q];
+            if (!alive[q]) continue;
+            const int a = ra[q], b = rb[q];
+            const bool ba = t.best[a] == key[q], bb = t.best[b] == key[q];
+            if (ba && bb) t.comp[t.pid[a] > t.pid[b] ? a : b] = t.pid[a] > t.pid[b] ? b : a;
+            else if (ba) t.comp[a] = b;
+            else if (bb) t.comp[b] = a;
+            if (ba || bb) {
+                alive[q] = false;
+                t.er[atomicAdd(&t.ner, 1)] = (unsigned short)(q * ORIENT_THREADS + threadIdx.x);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < IT; ++q)
+            if (used[q]) t.best[ra[q]] = t.best[rb[q]] = EMPTY_KEY;
+        __syncthreads();
+    }
+    __syncthreads();
+    if (r >= MAX_ROUNDS && threadIdx.x == 0) atomicOr(&ctl->err, ERR_ROUNDS);
+    // super-roots: the smallest piece of every super-tree
+    const int np = t.np, ner = t.ner;
+    for (int l = threadIdx.x; l < np; l += ORIENT_THREADS) {
+        const int root = tail_root(t, l), p = t.pid[l];
+        if (p < *(volatile int *)&t.minp[root]) atomicMin(&t.minp[root], p);
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < np; l += ORIENT_THREADS)
+        if (t.minp[tail_root(t, l)] == t.pid[l]) t.vis[l] = 1;
+    __syncthreads();
+    // orientation: an edge with one visited end makes the other end its
+    // child (every piece is reached over one edge only)
+    int child[IT];
+    bool open[IT];
+#pragma unroll
+    for (int q = 0; q < IT; ++q) {
+        open[q] = q * ORIENT_THREADS + (int)threadIdx.x < ner;
+        child[q] = -1;
+    }
+    for (int lvl = 0; lvl <= ner; ++lvl) {
+        bool more = false;
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            if (!open[q]) continue;
+            const int i = t.er[q * ORIENT_THREADS + threadIdx.x];
+            const int a = t.a[i], b = t.b[i];
+            const bool va = *(volatile unsigned char *)&t.vis[a], vb = *(volatile unsigned char *)&t.vis[b];
+            if (va == vb) {
+                more = true;
+                continue;
+            }
+            open[q] = false;
+            child[q] = va ? b : a;
+            t.vis[child[q]] = 1;
+        }
+        if (!__syncthreads_or(more)) break;
+    }
+    // results: attach points and new roots (as in orient_one), and the walks
+    int rev = 0;
+#pragma unroll
+    for (int q = 0; q < IT; ++q) {
+        if (child[q] < 0) continue;
+        const int e = q * ORIENT_THREADS + threadIdx.x;
+        const u64 k = t.key[t.er[e]];
+        const int p = t.pid[child[q]], x0 = (int)klo(k), x1 = (int)khi(k);
+        const bool low = oa.rep[x0] == p;
+        const int x = low ? x0 : x1, y = low ? x1 : x0;
+        oa.chx[e] = x;
+        oa.chy[e] = y;
+        oa.att_x[p] = x;
+        oa.att_ep[p] = ep;
+        oa.newrep[p] = t.minp[tail_root(t, child[q])];
+        oa.rep_ep[p] = ep;
+        if (oa.aff_ep[p] == ep) ctl->need_root = 1;
+        if (oa.walk) rev += walk_path(ctl, oa.parent, x, y, oa.long_ep, p, ep);
+    }
+    block_add(&ctl->reversed, rev);
+    if (threadIdx.x == 0) {
+        ctl->ner = (u64)ner;
+        ctl->hook_rounds = r;
+        ctl->ncore = 0;
     }
 }
 
-// Path reversal by walking (ReversePaths, Algorithm 1), one thread per
-// oriented replacement edge x -> y: the path x = v0, v1 = parent[v0], ...,
-// vL (the piece root) is reversed in place while it is walked (parent[v_j]
-// <- v_{j-1}, parent[v0] <- y).  Each child piece has exactly one oriented
-// edge and pieces are disjoint, so the walks never touch the same vertex.
-// A walk that has not met its root after WALK_MAX steps restores the part
-// it reversed and stamps its piece in long_ep: such pieces are reversed by
-// the pointer-doubling marks instead.
-__global__ void k_walk(Ctl *ctl, const int *chx, const int *chy, const int *rep, int *parent, unsigned *long_ep) {
+// Replacement edges of a batch in one cooperative launch: the pair table is
+// moved into the candidate list (h.pairs), the candidates are hooked, the
+// replacement edges oriented and their paths walked.  Up to SMALL_CAND
+// candidates go to one block (replace_small); the other blocks then only pull
+// the forest into L2 for its walks (and the representatives for the refresh
+// that follows an insert).  As launches of their own the pair compaction,
+// hooking, orientation and walks of a 100-edge batch took 68 us on R-MAT
+// scale 22.
+__global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArgs h, OrientArgs a) {
+    if (*(volatile int *)&ctl->skip) return;
+    __shared__ HotMin hm;
+    const unsigned ep = ctl->epoch;
+    if (gtid() == 0) {
+        ctl->cnt[1] = ctl->cnt[2] = 0;
+        ctl->flag[0] = ctl->flag[1] = ctl->flag[2] = 0;
+    }
+    if (h.pairs) {
+        compact_pairs(ctl, h.pt, h.ck[0], h.ca[0], h.cb[0], h.cand_cap);
+        if (!grid_barrier(ctl, &ctl->bar[1])) return;
+    }
+    const long long c0 = (long long)*(volatile u64 *)&ctl->ncand;
+    if (c0 <= SMALL_CAND) {
+        if (c0 == 0) return;
+        if (blockIdx.x == 0) {
+            replace_small(ctl, h, a, (int)c0, ep);
+        } else {
+            const long long t = gtid() - blockDim.x, nt = gstride() - blockDim.x;
+            l2_prefetch(a.parent, 4 * a.n, t, nt);
+            if (ctl->op == DRSF_INSERT) l2_prefetch(a.rep, 4 * a.n, t, nt);
+        }
+        return;
+    }
+    hm_init(hm);
+    if (h.init) {
+        hook_init(h, c0, ep);
+        if (!grid_barrier(ctl, &ctl->bar[1])) return;
+    }
+    const int r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
+                                     h.hs.best0, h.hs.best1, h.er, h.er_cap);
+    if (r < 0) return;
+    if (r > 0 && blockIdx.x == 0)
+        hook_rounds<true>(ctl, hm, r, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp, h.hs.best0,
+                          h.hs.best1, h.er, h.er_cap);
+    if (!grid_barrier(ctl, &ctl->bar[1])) return;
+    orient_grid(ctl, a);
+}
+
+// The walks as a launch of their own, for batches above LARGE_BATCH edges: one
+// thread per replacement edge at full occupancy, where the orientation (one
+// block per SM) would take them in several rounds.  For a 100K-edge batch the
+// launch costs 10 us more than it saves (R-MAT scale 22).
+__global__ void k_walk(Ctl *ctl, OrientArgs a) {
     if (*(volatile int *)&ctl->skip) return;
     const unsigned ep = ctl->epoch;
     const long long ner = (long long)ctl->ner;
-    long long rev = 0;
+    int rev = 0;
     GS_LOOP(i, ner) {
-        const int x = chx[i];
-        int prev = chy[i], cur = x, steps = 0;
-        bool done = false;
-        for (; steps < WALK_MAX; ++steps) {
-            int nxt = parent[cur];
-            parent[cur] = prev;
-            if (nxt == cur) {
-                done = true;
-                break;
-            }
-            prev = cur;
-            cur = nxt;
-        }
-        if (done) {
-            rev += steps;   // the path's vertices below the root
-        } else {
-            // v0 .. v_{WALK_MAX-1} reversed, cur = v_WALK_MAX untouched
-            int up = cur, v = prev;
-            for (int t = 0; t < WALK_MAX; ++t) {
-                int nv = parent[v];
-                parent[v] = up;
-                up = v;
-                v = nv;
-            }
-            long_ep[rep[x]] = ep;
-            ctl->nlong = 1;
-        }
+        const int x = a.chx[i];
+        rev += walk_path(ctl, a.parent, x, a.chy[i], a.long_ep, a.rep[x], ep);
     }
-    if (rev) atomicAdd((u64 *)&ctl->reversed, (u64)rev);
+    block_add(&ctl->reversed, rev);
 }
 
 // Path-reversal set-up fused with the representative refresh: every vertex
@@ -1516,7 +1830,7 @@ __device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, cons
             for (unsigned m = chg; m; m &= m - 1) {
                 const int k = __ffs(m) - 1;
                 const int pk = p[k];
-                if (a.sel_ep[pk] == ep && a.att_x[pk] != pk) on |= 1u << k;
+                if (LD(a.sel_ep[pk]) == ep && a.att_x[pk] != pk) on |= 1u << k;
             }
             q = block_reserve(&ctl->nact, __popc(on));
         }
@@ -1526,7 +1840,7 @@ __device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, cons
             const long long i = i0 + (long long)k * blockDim.x;
             const int v = L ? L[i] : (int)i;
             if ((on >> k) & 1u) {
-                const int pv = a.parent[v];
+                const int pv = LD(a.parent[v]);
                 a.act[q] = v;
                 a.pold[q] = pv;
                 a.J0[v] = pv;
@@ -1580,7 +1894,7 @@ __device__ bool mark_paths(Ctl *ctl, const FinishArgs &a, long long na) {
                 if (!ok[k]) continue;
                 if (mk[k]) a.mark[w[k]] = 1;
                 Jn[v[k]] = w2[k];
-                more |= a.parent[w2[k]] != w2[k];
+                more |= LD(a.parent[w2[k]]) != w2[k];
             }
         }
         if (__syncthreads_or(more) && threadIdx.x == 0) atomicOr(&ctl->flag[r % 3], 1);
@@ -1608,7 +1922,7 @@ __device__ __forceinline__ void reverse_marked(Ctl *ctl, const FinishArgs &a, lo
             ++c;
         }
     }
-    if (c) atomicAdd((u64 *)&ctl->reversed, (u64)c);
+    block_add(&ctl->reversed, c);
     GS_LOOP(i, ner) a.parent[a.chx[i]] = a.chy[i];
 }
 
@@ -1686,23 +2000,22 @@ unsigned coop_blocks_jump(int nsm) {
              c = coop_blocks((const void *)k_jump<2>, nsm, 8);
     return a < b ? (a < c ? a : c) : (b < c ? b : c);
 }
-static unsigned coop_blocks_hook_t(const void *fn, int threads, int nsm) {
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, 0) != cudaSuccess || per < 1) per = 1;
-    if (per > 1024 / threads) per = 1024 / threads;
-    return (unsigned)(per * nsm);
-}
-unsigned coop_blocks_hook(int nsm) { return coop_blocks_hook_t((const void *)k_boruvka<1024>, 1024, nsm); }
-unsigned coop_blocks_hook_small(int nsm) { return coop_blocks_hook_t((const void *)k_boruvka<256>, 256, nsm); }
+unsigned coop_blocks_hook(int nsm) { return coop_blocks((const void *)k_hook_large, nsm, 4); }
+// one block per SM (both kernels take the same dynamic shared memory)
 unsigned coop_blocks_orient(int nsm) {
     cudaFuncSetAttribute((const void *)k_orient, cudaFuncAttributeMaxDynamicSharedMemorySize, ORIENT_SMEM_BYTES);
+    cudaFuncSetAttribute((const void *)k_replace, cudaFuncAttributeMaxDynamicSharedMemorySize, ORIENT_SMEM_BYTES);
     int per = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, (const void *)k_orient, ORIENT_THREADS,
                                                       ORIENT_SMEM_BYTES) != cudaSuccess ||
         per < 1)
         per = 1;
-    if (per > 2) per = 2;
-    return (unsigned)(per * nsm);
+    int per2 = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, (const void *)k_replace, ORIENT_THREADS,
+                                                      ORIENT_SMEM_BYTES) != cudaSuccess ||
+        per2 < 1)
+        per2 = 1;
+    return (unsigned)((per < per2 ? per : per2) * nsm);
 }
 
 cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s) {
@@ -1740,22 +2053,25 @@ cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_
                                       : (sync_rounds ? (const void *)k_jump<1> : (const void *)k_jump<0>);
     return cudaLaunchCooperativeKernel(fn, d.coop_jump, BLK, args, 0, s);
 }
-cudaError_t launch_boruvka(const Dev &d, Ctl *ctl, u64 *ck0, int *ca0, int *cb0, u64 *ck1, int *ca1, int *cb1,
-                           HookSlots hs, u64 *er, long long er_cap, int init, bool large, cudaStream_t s) {
-    void *args[] = {(void *)&ctl, (void *)&ck0, (void *)&ca0, (void *)&cb0, (void *)&ck1, (void *)&ca1,
-                    (void *)&cb1, (void *)&hs, (void *)&er, (void *)&er_cap, (void *)&init};
-    if (large)
-        return cudaLaunchCooperativeKernel((const void *)k_boruvka<256>, d.coop_hook_small, 256, args, 0, s);
-    return cudaLaunchCooperativeKernel((const void *)k_boruvka<1024>, d.coop_hook, 1024, args, 0, s);
+cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s) {
+    void *args[] = {(void *)&ctl, (void *)&h, (void *)&a};
+    return cudaLaunchCooperativeKernel((const void *)k_replace, d.coop_orient, ORIENT_THREADS, args,
+                                       ORIENT_SMEM_BYTES, s);
+}
+cudaError_t launch_hook_large(const Dev &d, Ctl *ctl, HookArgs h, cudaStream_t s) {
+    if (h.pairs)
+        k_pairs_compact<<<grid_for(((long long)h.pt.mask + 4) / 4, BLK, (unsigned)d.nsm * 8u), BLK, 0, s>>>(
+            ctl, h.pt, h.ck[0], h.ca[0], h.cb[0], h.cand_cap);
+    void *args[] = {(void *)&ctl, (void *)&h};
+    return cudaLaunchCooperativeKernel((const void *)k_hook_large, d.coop_hook, BLK, args, 0, s);
 }
 cudaError_t launch_orient(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&a};
     return cudaLaunchCooperativeKernel((const void *)k_orient, d.coop_orient, ORIENT_THREADS, args,
                                        ORIENT_SMEM_BYTES, s);
 }
-cudaError_t launch_walk(const Dev &d, Ctl *ctl, const int *chx, const int *chy, const int *rep, int *parent,
-                        unsigned *long_ep, cudaStream_t s) {
-    k_walk<<<d.grid, BLK, 0, s>>>(ctl, chx, chy, rep, parent, long_ep);
+cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
+    k_walk<<<d.grid, BLK, 0, s>>>(ctl, a);
     return cudaGetLastError();
 }
 cudaError_t launch_finish(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s) {

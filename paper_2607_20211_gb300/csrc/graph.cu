@@ -230,12 +230,12 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
     // block-uniform loop: the candidate append is aggregated per block
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nb; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
-        bool cross = false;
+        bool cross = false, over = false;
         int ra = 0, rb = 0;
-        u64 k = 0;
+        u64 k = 0, s = 0;
         if (i < nb) {
             k = nkey[i];
-            u64 s = nslot[i];
+            s = nslot[i];
             uint32_t a = klo(k), b = khi(k);
             const Row ha = row_head(g, (int)a), hb = row_head(g, (int)b);
             const int pa = row_take(g, (int)a, ha, &dead), pb = row_take(g, (int)b, hb, &dead);
@@ -246,21 +246,25 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                 ix.e[s].pos = make_uint2(qa, qb);
                 dead -= 2;
             } else {
-                // (a slot taken in the row that had one stays empty and
-                // unlisted until the next rebuild)
-                u64 o = atomicAdd(&ctl->ovf_count, 1ull);
-                if (o < ovf_cap) {
-                    ovf[o] = k;
-                    ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
-                } else {
-                    atomicOr(&ctl->err, ERR_CAPACITY);
-                }
-                atomicAdd((u64 *)&ctl->overflow_total, 1ull);
+                over = true;   // (a slot taken in the row that had one stays empty
+                               // and unlisted until the next rebuild)
             }
             ra = rep[a];
             rb = rep[b];
             cross = ra != rb;
             if (SG && cross) cross = !pair_min(pt.pk, pt.mk, pt.mask, ra, rb, k);   // no slot: plain candidate
+        }
+        // (one atomic per block: a million-edge batch can overflow 100K rows)
+        if (__syncthreads_or(over)) {
+            const long long o = block_append(&ctl->ovf_count, over);
+            if (over) {
+                if ((u64)o < ovf_cap) {
+                    ovf[o] = k;
+                    ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
+                } else {
+                    atomicOr(&ctl->err, ERR_CAPACITY);
+                }
+            }
         }
         long long p = block_append(&ctl->ncand, cross);
         if (cross) {
@@ -269,8 +273,9 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                 ca[p] = ra;
                 cb[p] = rb;
                 // HS: these are all the candidates, so the hooking needs no
-                // initialisation phase of its own (see HookSlots)
-                if (!SG) {
+                // initialisation phase of its own (see HookSlots); few
+                // candidates are hooked in shared memory
+                if (!SG && nb > SMALL_CAND) {
                     hook_slot_init(hs, ra, ep);
                     hook_slot_init(hs, rb, ep);
                 }
@@ -505,51 +510,6 @@ __global__ void k_scan_ovf(const u64 *ovf, Ctl *ctl, const int *rep, PairTable p
     }
 }
 
-// Move the pair table into the candidate list (one candidate per piece
-// pair, its minimum key) and free the slots for the next batch.
-__global__ void k_pairs_compact(Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap) {
-    if (*(volatile int *)&ctl->skip) return;
-    // four slots per thread and iteration, one counter reservation per
-    // block (the table has far more slots than warps have lanes, and most
-    // warps hold an occupied slot: a per-warp append would queue on the
-    // counter)
-    const long long T = (long long)pt.mask + 1;
-    const long long S = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < T; base += 4 * S) {
-        u64 pair[4], k[4];
-        bool on[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            long long i = base + q * S + threadIdx.x;
-            pair[q] = i < T ? pt.pk[i] : EMPTY_KEY;
-            on[q] = pair[q] != EMPTY_KEY;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            k[q] = 0;
-            if (on[q]) {
-                long long i = base + q * S + threadIdx.x;
-                k[q] = pt.mk[i];
-                pt.pk[i] = EMPTY_KEY;
-                pt.mk[i] = EMPTY_KEY;
-            }
-        }
-        long long p[4];
-        block_reserve4(&ctl->ncand, on, p);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (!on[q]) continue;
-            if ((u64)p[q] < cand_cap) {
-                ck[p[q]] = k[q];
-                ca[p[q]] = (int)(pair[q] >> 32);
-                cb[p[q]] = (int)(pair[q] & 0xFFFFFFFFu);
-            } else {
-                atomicOr(&ctl->err, ERR_CAPACITY);
-            }
-        }
-    }
-}
-
 // Edge-list export (rebuild and drsf_export_edges): warp per row, pairs
 // (u, x) with u < x, then the live overflow edges.
 __global__ void k_extract(int n, Csr g, const u64 *ovf, const Ctl *ctl, int *out, long long cap, u64 *cnt,
@@ -695,12 +655,6 @@ cudaError_t launch_scan_ovf(const Dev &d, const u64 *ovf, Ctl *ctl, const int *r
         k_scan_ovf<true><<<d.nsm * 2, BLK, 0, s>>>(ovf, ctl, rep, pt, ck, ca, cb, cand_cap);
     else
         k_scan_ovf<false><<<d.nsm * 2, BLK, 0, s>>>(ovf, ctl, rep, pt, ck, ca, cb, cand_cap);
-    return cudaGetLastError();
-}
-cudaError_t launch_pairs_compact(const Dev &d, Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap,
-                                 cudaStream_t s) {
-    k_pairs_compact<<<grid_for(((long long)pt.mask + 4) / 4, BLK, (unsigned)d.nsm * 8u), BLK, 0, s>>>(ctl, pt, ck, ca,
-                                                                                                   cb, cand_cap);
     return cudaGetLastError();
 }
 cudaError_t launch_extract(const Dev &d, int n, Csr g, const u64 *ovf, u64 novf_max, Ctl *ctl, int *out,

@@ -6,13 +6,15 @@
 
 // Fixed launch shapes.
 #define BLK 256
+// batches with at most this many candidates are replaced, oriented and walked
+// by one block in shared memory (what fits beside the hash table)
+#define SMALL_CAND 2048
 
 struct Dev {
     int nsm;
     unsigned grid;        // grid-stride kernels: nsm * 8 blocks of BLK
     unsigned coop_jump;   // cooperative kernels: co-resident block counts
-    unsigned coop_hook;        // (1024-thread blocks)
-    unsigned coop_hook_small;  // (256-thread blocks, for large batches)
+    unsigned coop_hook;
     unsigned coop_orient;
     unsigned coop_finish;
     unsigned coop_bfs;
@@ -67,8 +69,6 @@ cudaError_t launch_scan_rows(const Dev &d, RowList rl, Ctl *ctl, Csr g, const in
                              u64 *ck, int *ca, int *cb, u64 cand_cap, cudaStream_t s);
 cudaError_t launch_scan_ovf(const Dev &d, const u64 *ovf, Ctl *ctl, const int *rep, bool sg, PairTable pt, u64 *ck,
                             int *ca, int *cb, u64 cand_cap, cudaStream_t s);
-cudaError_t launch_pairs_compact(const Dev &d, Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap,
-                                 cudaStream_t s);
 cudaError_t launch_extract(const Dev &d, int n, Csr g, const u64 *ovf, u64 novf_max, Ctl *ctl, int *out,
                            long long cap, u64 *cnt, cudaStream_t s);
 cudaError_t launch_check_tree_edges(int n, const int *parent, Index ix, int *bad, cudaStream_t s);
@@ -93,10 +93,17 @@ cudaError_t launch_jump_async(const Dev &d, const int *A, Ctl *ctl, int *J, int 
 cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par,
                         int *J, int *J1, int *rep, RowList rl, int mode, const int *rold, unsigned *w, u64 *heavy,
                         Csr g, int sync_rounds, int *X, int *Y, const int *cuts, cudaStream_t s);
-// init: set up the candidates' endpoints first (0: their writer did, HookSlots);
-// large: a batch whose candidates stay many past round 0 (smaller blocks)
-cudaError_t launch_boruvka(const Dev &d, Ctl *ctl, u64 *ck0, int *ca0, int *cb0, u64 *ck1, int *ca1, int *cb1,
-                           HookSlots hs, u64 *er, long long er_cap, int init, bool large, cudaStream_t s);
+struct HookArgs {
+    u64 *ck[2];          // candidates: key and the two pieces (ping-pong)
+    int *ca[2], *cb[2];
+    u64 cand_cap;
+    HookSlots hs;
+    u64 *er;             // replacement edges
+    long long er_cap;
+    int init;            // set up the candidates' endpoints first (0: their writer did, HookSlots)
+    int pairs;           // move the pair table into the candidate list first
+    PairTable pt;
+};
 struct OrientArgs {
     const u64 *er;
     const int *rep;
@@ -113,13 +120,18 @@ struct OrientArgs {
     int *ep, *eid;       // per arc: source piece, its dense id
     int *eroot;          // per edge: hook-forest root of its super-tree
     int *cel;            // core edges (for the one-block path of small cores)
-    const int *parent;   // the forest: pulled into L2 for the walks that follow
+    int *parent;         // the forest: paths are reversed in place
+    unsigned *long_ep;   // pieces whose path is too long to walk
+    int walk;            // walk each path as its edge is oriented (0: k_walk does, or the Euler tour's marks)
     const unsigned *aff_ep;   // old roots of this batch's cut trees
     long long n;
 };
+cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s);
+// the same in three launches, for batches above LARGE_BATCH edges
+#define LARGE_BATCH (1 << 18)
+cudaError_t launch_hook_large(const Dev &d, Ctl *ctl, HookArgs h, cudaStream_t s);
 cudaError_t launch_orient(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);
-cudaError_t launch_walk(const Dev &d, Ctl *ctl, const int *chx, const int *chy, const int *rep, int *parent,
-                        unsigned *long_ep, cudaStream_t s);
+cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);
 struct FinishArgs {
     const int *A;             // delete: the affected list
     long long n;
@@ -141,7 +153,6 @@ unsigned coop_blocks_jump(int nsm);
 unsigned grid_vertex_pass(int nsm);
 unsigned coop_blocks_finish(int nsm);
 unsigned coop_blocks_hook(int nsm);
-unsigned coop_blocks_hook_small(int nsm);
 unsigned coop_blocks_orient(int nsm);
 cudaError_t launch_barrier_selftest(Ctl *ctl, cudaStream_t s);
 // static.cu ------------------------------------------------------------

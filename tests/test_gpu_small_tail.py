@@ -1,0 +1,77 @@
+"""Batches around the candidate limit of the one-block replacement path
+(2,048), with super-forests of every shape, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_20211_gb300 as drsf
+from tests.gpu_util import _tiny_graph, check_batch, make_forest
+
+pytestmark = pytest.mark.gpu
+LIMIT = 2048
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    drsf.build()
+
+
+def _shape(kind, b, rng):
+    """b edges over at most 2 b vertices: all candidates of an insert into an edgeless graph."""
+    i = np.arange(b)
+    if kind == "star":          # one piece is an end of every candidate
+        return np.stack([np.zeros(b, np.int64) + b, i], 1)
+    if kind == "path":          # the deepest super-forest
+        return np.stack([i, i + 1], 1)
+    if kind == "pairs":         # 2 b pieces, b super-trees
+        return np.stack([2 * i, 2 * i + 1], 1)
+    if kind == "dense":         # many rounds, most candidates inside one component
+        e = rng.integers(0, 80, (8 * b, 2))
+        e = np.unique(np.sort(e[e[:, 0] != e[:, 1]], 1), axis=0)
+        return e[rng.permutation(len(e))[:b]]
+    e = rng.integers(0, b, (3 * b, 2))
+    e = np.unique(np.sort(e[e[:, 0] != e[:, 1]], 1), axis=0)
+    return e[rng.permutation(len(e))[:b]]
+
+
+@pytest.mark.parametrize("b", [1, 2, 33, 1023, 1024, 1025, LIMIT - 1, LIMIT, LIMIT + 1, 3 * LIMIT])
+@pytest.mark.parametrize("kind", ["star", "path", "pairs", "dense", "random"])
+def test_insert_shapes(kind, b):
+    """An insert whose every edge is a candidate, the same edges deleted
+    (one tree edge in three kept) and inserted again, ids permuted."""
+    rng = np.random.default_rng(b)
+    e = _shape(kind, b, rng)
+    n = 2 * b + 100
+    e = rng.permutation(n)[e].astype(np.int32)
+    g = _tiny_graph(n, [], list(range(n)))
+    f = make_forest(g)
+    try:
+        keys, par, _ = check_batch(f, n, g.keys, g.parent, drsf.INSERT, e)
+        keys, par, _ = check_batch(f, n, keys, par, drsf.DELETE, e[np.arange(len(e)) % 3 != 0])
+        check_batch(f, n, keys, par, drsf.INSERT, e)
+    finally:
+        f.close()
+
+
+@pytest.mark.parametrize("flags", [drsf.REPL_SG, drsf.REPL_HS])
+@pytest.mark.parametrize("cuts", [5, 700, 1500])
+def test_delete_candidates(flags, cuts):
+    """Deletes whose detached pieces keep several cross edges each: a path
+    with chords, cut in many places; both replacement variants."""
+    n = 6000
+    rng = np.random.default_rng(cuts)
+    chords = rng.integers(0, n, (2 * cuts, 2))
+    chords = chords[np.abs(chords[:, 0] - chords[:, 1]) > 1]
+    edges = [(i, i + 1) for i in range(n - 1)] + [tuple(c) for c in chords.tolist()]
+    g = _tiny_graph(n, edges, [max(i - 1, 0) for i in range(n)])
+    f = make_forest(g, flags=drsf.DETERMINISTIC | flags)
+    at = np.sort(rng.permutation(n - 1)[:cuts])
+    b = np.stack([at, at + 1], 1).astype(np.int32)
+    try:
+        keys, par, _ = check_batch(f, n, g.keys, g.parent, drsf.DELETE, b)
+        keys, par, _ = check_batch(f, n, keys, par, drsf.INSERT, b)
+        check_batch(f, n, keys, par, drsf.DELETE, b)
+    finally:
+        f.close()
