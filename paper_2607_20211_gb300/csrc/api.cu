@@ -34,7 +34,7 @@ struct drsf_ctx {
     void *alloc_ctx = nullptr;
     std::vector<Buf> bufs;
     bool poisoned = false;
-    int jump_sync = 2;   // root search: 2 asynchronous doubling, 1 synchronous rounds, 0 path halving
+    int jump_sync = 2;   // root search: 2 hops, then asynchronous doubling; 1 synchronous rounds, 0 path halving
     int pending_einval = 0;
     int last_sg = 0;     // the last batch took the supergraph variant
     // captured per-batch launch sequences (CUDA graphs), valid for storage
@@ -132,11 +132,11 @@ enum {
     PH_INS_CLAIM,     // insert: normalisation + index claim
     PH_INS_PLACE,     // insert: CSR append + cross test
     PH_DEL_CLAIM,     // delete: normalisation, removal, tree-edge cut
-    PH_AFF,           // delete: affected-vertex list
-    PH_JUMP,          // delete: pointer jumping (representatives)
+    PH_AFF,           // delete: affected-vertex list (selectable root searches)
+    PH_JUMP,          // delete: top-down search, pointer jumping (representatives)
     PH_SCAN,          // delete: cross-edge scan of detached rows + overflow
     PH_HOOK,          // replacement edges: hook-and-compress, orientation, path walks
-    PH_ORIENT,        // large batches: the orientation as a launch of its own
+    PH_ORIENT,        // (part of the above)
     PH_ACTIVE,        // representative refresh, and the doubling marks and reversal of long paths
     PH_MARK,          // Euler-tour marks
     PH_REVERSE        // large batches: path walks; Euler: reversal scatter + attach
@@ -292,8 +292,9 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
         }
         h->cand_cap = need;
     }
-    // tiles of the scanned rows: at most one per 32 CSR slots, plus one
-    const long long ntile = total / 32 + 2;
+    // tiles of the scanned rows: at most one per 32 CSR slots, plus one; or
+    // the jobs of long rows (k_scan), two words per 32 slots at most
+    const long long ntile = total / 16 + 2;
     if (ntile > h->tile_cap) {
         hfree(h, &h->tile, s);
         CKA(halloc(h, &h->tile, (size_t)ntile, s));
@@ -456,8 +457,10 @@ static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     CKA(halloc(h, &h->att_x, n, s));
     CKA(halloc(h, &h->newrep, n, s));
     CKA(halloc(h, &h->A, n, s));
-    CKA(halloc(h, &h->act, n, s));
-    CKA(halloc(h, &h->pold, n, s));
+    // (the warps' lists of k_relabel: see relabel_room)
+    const size_t nl = (size_t)relabel_room(h->n, h->dev.coop_relabel);
+    CKA(halloc(h, &h->act, nl, s));
+    CKA(halloc(h, &h->pold, nl, s));
     CKA(halloc(h, &h->D, n, s));
     CKA(halloc(h, &h->chx, n, s));
     CKA(halloc(h, &h->chy, n, s));
@@ -477,7 +480,7 @@ static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     CKA(halloc(h, &h->roff, n + 1, s));
     CKA(halloc(h, &h->rbase, n, s));
     CKA(halloc(h, &h->rmeta, n, s));
-    CKA(halloc(h, &h->xlist, n, s));
+    CKA(halloc(h, &h->xlist, nl, s));
     CKA(halloc(h, &h->aidx, n, s));
     CKA(halloc(h, &h->aroot, n, s));
     CKA(halloc(h, &h->oep, 2 * n + 2, s));
@@ -624,8 +627,8 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.nsm = nsm;
     h->dev.grid = (unsigned)nsm * 8u;
     h->dev.coop_jump = coop_blocks_jump(nsm);
-    h->dev.coop_hook = coop_blocks_hook(nsm);
-    h->dev.coop_orient = coop_blocks_orient(nsm);
+    h->dev.coop_replace = coop_blocks_replace(nsm);
+    h->dev.coop_relabel = coop_blocks_relabel(nsm);
     h->dev.coop_finish = coop_blocks_finish(nsm);
     h->dev.coop_bfs = coop_blocks_bfs(nsm);
     h->dev.grid_scan = scan_grid(nsm);
@@ -694,8 +697,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     } else {
         // Algorithm 1, delete: remove B, cut tree edges, re-label the cut trees
         prof_begin(h, PH_DEL_CLAIM, s);
-        CK(launch_del_claim(glen, h->ix, g, h->ovf, h->parent, h->rep, ctl, h->aff_ep, h->cut_ep, h->cutlist,
-                            h->wgt, h->rold, s));
+        const PieceSlots ps{h->aff_ep, h->rold, h->comp, h->best0, h->heavy, h->wgt, (unsigned *)h->pdeg};
+        CK(launch_del_claim(glen, h->ix, g, h->ovf, h->parent, h->rep, ctl, ps, h->cutlist, s));
         prof_end(h, PH_DEL_CLAIM, 1, s);
         if (h->detach_now) {
             // the detached vertices top-down from the cut vertices; over its
@@ -707,20 +710,60 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
                              std::max<long long>(1 << 20, 4 * n), DETACH_LEVELS, h->act, h->xlist, s));
             prof_end(h, PH_JUMP, 1, s);
         }
-        prof_begin(h, PH_AFF, s);
-        CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, h->parent,
-                              h->jump_sync == 2 ? h->J0 : nullptr, s));
-        prof_end(h, PH_AFF, 1, s);
-        prof_begin(h, PH_JUMP, s);
-        if (h->jump_sync == 2) CK(launch_jump_async(h->dev, h->A, ctl, h->J0, h->act, h->xlist, s));
-        CK(launch_jump(h->dev, h->A, 1, 0, ctl, h->parent, h->J0, h->J1, h->rep, rows(h), 1, h->rold, h->wgt,
-                       h->heavy, g, h->jump_sync, h->act, h->xlist, h->cutlist, s));
-        prof_end(h, PH_JUMP, h->jump_sync == 2 ? 2 : 1, s);   // the asynchronous doubling is a launch of its own
+        if (h->jump_sync == 2) {
+            RelabelArgs ra{};
+            ra.n = h->n;
+            ra.rep = h->rep;
+            ra.par = h->parent;
+            ra.aff_ep = h->aff_ep;
+            ra.J = h->J0;
+            ra.X = h->act;
+            ra.Y = h->xlist;
+            ra.L = h->pold;
+            ra.D = h->D;
+            ra.rold = h->rold;
+            ra.w = h->wgt;
+            ra.wsum = (unsigned *)h->pdeg;
+            ra.heavy = h->heavy;
+            ra.left = h->minp;
+            ra.cuts = h->cutlist;
+            prof_begin(h, PH_JUMP, s);
+            CK(launch_relabel(h->dev, ctl, ra, s));
+            prof_end(h, PH_JUMP, 1, s);
+        } else {
+            prof_begin(h, PH_AFF, s);
+            CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, s));
+            prof_end(h, PH_AFF, 1, s);
+            prof_begin(h, PH_JUMP, s);
+            CK(launch_jump(h->dev, h->A, 1, 0, ctl, h->parent, h->J0, h->J1, h->rep, rows(h), 1, h->rold, h->wgt,
+                           h->heavy, g, h->jump_sync, h->act, h->xlist, h->cutlist, s));
+            prof_end(h, PH_JUMP, 1, s);
+        }
+        LightArgs la{};
+        la.n = h->n;
+        la.g = g;
+        la.rep = h->rep;
+        la.aff_ep = h->aff_ep;
+        la.rold = h->rold;
+        la.left = h->minp;
+        la.rows = (unsigned *)h->plist;
+        la.D = h->D;
+        la.job = h->tile;
+        la.comp = h->comp;
+        la.best = h->best0;
+        la.root_ep = h->cut_ep;
+        la.cuts = h->cutlist;
+        la.er = h->er;
+        la.ovf = h->ovf;
+        la.pt = h->pt;
+        la.ck = h->ck[0];
+        la.ca = h->ca[0];
+        la.cb = h->cb[0];
+        la.cand_cap = h->cand_cap;
+        la.listed = h->jump_sync != 2;
         prof_begin(h, PH_SCAN, s);
-        CK(launch_scan_rows(h->dev, rows(h), ctl, g, h->rep, sg, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap,
-                            s));
-        CK(launch_scan_ovf(h->dev, h->ovf, ctl, h->rep, sg, h->pt, h->ck[0], h->ca[0], h->cb[0], h->cand_cap, s));
-        prof_end(h, PH_SCAN, 2, s);
+        CK(launch_scan(h->dev, ctl, rows(h), la, sg, s));
+        prof_end(h, PH_SCAN, 1, s);
     }
     OrientArgs oa{};
     oa.er = h->er;
@@ -776,24 +819,16 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     // an HS insert's candidates all come from k_ins_place, which set up
     // their hook-forest slots; otherwise the hooking sets them up itself
     // (inside the scan of a large delete that costs more than it saves)
-    ha.init = (op == DRSF_INSERT && !sg && !large) ? 0 : 1;
+    ha.init = (op == DRSF_INSERT && !sg) ? 0 : 1;
     ha.pairs = sg ? 1 : 0;
     ha.pt = h->pt;
     prof_begin(h, PH_HOOK, s);
-    if (large) {
-        CK(launch_hook_large(h->dev, ctl, ha, s));
-        prof_end(h, PH_HOOK, sg ? 2 : 1, s);
-        prof_begin(h, PH_ORIENT, s);
-        CK(launch_orient(h->dev, ctl, oa, s));
-        prof_end(h, PH_ORIENT, 1, s);
-        if (!euler) {
-            prof_begin(h, PH_REVERSE, s);
-            CK(launch_walk(h->dev, ctl, oa, s));
-            prof_end(h, PH_REVERSE, 1, s);
-        }
-    } else {
-        CK(launch_replace(h->dev, ctl, ha, oa, s));
-        prof_end(h, PH_HOOK, 1, s);
+    CK(launch_replace(h->dev, ctl, ha, oa, s));
+    prof_end(h, PH_HOOK, 1, s);
+    if (large && !euler) {
+        prof_begin(h, PH_REVERSE, s);
+        CK(launch_walk(h->dev, ctl, oa, s));
+        prof_end(h, PH_REVERSE, 1, s);
     }
     FinishArgs fa{};
     fa.A = h->A;

@@ -45,7 +45,7 @@ struct Ctl {
     int skip;               // current batch rejected (ERR_BATCH_ID seen)
     unsigned epoch;         // batch counter; epoch stamps compare against it
     int op;
-    u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs, Euler marks, detach
+    u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs / scan, Euler marks, detach
                             // (reset at each batch's start and before each static BFS)
     int flag[3];            // per-round "another round needed" flags
     u64 cnt[3];             // per-round list sizes (hook-and-compress)
@@ -82,6 +82,8 @@ struct Ctl {
     const int *batch;       // the current batch (device), set by k_begin
     int td;                 // delete: the detached vertices were found top-down (else: pointer jumping)
     int need_root;          // delete: a cut tree's root piece is re-rooted (read after a top-down delete)
+    int njobs;              // delete: parts of long rows to read
+    int pre;                // delete: the first hooking round was taken from the rows (k_scan)
     int nlong;              // some path was too long to be reversed by its walk
     long long det_levels;   // top-down levels of the batch (0: not taken)
     long long det_entries;  // adjacency entries the top-down search read
@@ -181,7 +183,7 @@ __device__ __forceinline__ void l2_prefetch(const void *p, long long bytes, long
         asm volatile("prefetch.global.L2 [%0];" ::"l"(c + off));
 }
 
-// Hook-forest slots of the candidates' endpoints (read by k_boruvka): the
+// Hook-forest slots of the candidates' endpoints (read by k_replace): the
 // kernel that writes a candidate sets up each of its endpoints once per
 // batch (whoever stamps it first): its own root in comp, both per-round
 // minimum slots empty.
@@ -295,23 +297,12 @@ __device__ __forceinline__ long long pair_slot(u64 *pk, u64 mask, u64 pair) {
     return -1;
 }
 __device__ __forceinline__ bool pair_min(u64 *pk, u64 *mk, u64 mask, int a, int b, u64 key) {
-    u64 pair = a < b ? ((u64)(unsigned)a << 32) | (unsigned)b : ((u64)(unsigned)b << 32) | (unsigned)a;
-    u64 s = hslot(pair, mask);
-    for (int p = 0; p < PAIR_PROBES; ++p) {
-        u64 cur = __ldcg(&pk[s]);
-        if (cur == EMPTY_KEY) {
-            u64 old = atomicCAS(&pk[s], EMPTY_KEY, pair);
-            if (old == EMPTY_KEY || old == pair) {
-                atomicMin(&mk[s], key);
-                return true;
-            }
-        } else if (cur == pair) {
-            atomicMin(&mk[s], key);
-            return true;
-        }
-        s = (s + 1) & mask;
-    }
-    return false;
+    const u64 pair = a < b ? ((u64)(unsigned)a << 32) | (unsigned)b : ((u64)(unsigned)b << 32) | (unsigned)a;
+    const long long s = pair_slot(pk, mask, pair);
+    if (s < 0) return false;
+    // (most edges of a pair that has many are no new minimum)
+    if (key < __ldcg(&mk[s])) atomicMin(&mk[s], key);
+    return true;
 }
 
 // Block-wide sum of per-thread counts added to a counter: one atomic per

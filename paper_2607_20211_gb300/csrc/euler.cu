@@ -1,7 +1,7 @@
 // Path marking by the Euler tour (Algorithm 3, ReversePathsEulerTour), the
 // alternative to pointer-doubling marks (selected with DRSF_EULER_REVERSAL).
 //
-// The re-rooted pieces (active vertices, listed densely by k_active) are
+// The re-rooted pieces (active vertices, listed densely by k_finish) are
 // toured: children lists from the old parent pointers, one down arc
 // (parent -> v) and one up arc (v -> parent) per non-root vertex, successor
 // of down(v) = down(first child of v) or up(v) for a leaf, successor of

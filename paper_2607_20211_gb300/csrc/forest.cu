@@ -39,9 +39,7 @@
 // passes are one dependent gather behind a streaming load)
 #define IPT 4
 #define IPN 16
-// k_aff_collect keeps more per item (old root, list position): 8 items per
-// thread (48 registers) measured faster than 16 (64 registers, fewer
-// resident blocks): 0.036 vs 0.041 ms per pass on R-MAT scale 22
+// k_aff_collect keeps more per item (old root, list position)
 #define IPA 8
 // top-down delete: after a search that gave up at its level limit, the
 // deletes that skip it before it is tried again
@@ -99,7 +97,7 @@ __global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
     ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
     ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
     ctl->jump_visits = 0;
-    ctl->td = ctl->need_root = ctl->nlong = 0;
+    ctl->td = ctl->need_root = ctl->nlong = ctl->njobs = ctl->pre = 0;
     if (ctl->det_skip) {   // the last batch skipped the top-down search
         if (ctl->depth_hint > 0) ctl->depth_hint -= 1;
         ctl->det_skip = 0;
@@ -126,10 +124,10 @@ __global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
 // 32 consecutive vertices), with all IPN loads and gathers in flight before
 // any is used.  A warp's listed vertices take consecutive slots (one block
 // reservation of the warps' totals), in vertex order within the warp.
-// It runs only when the top-down search of the detached vertices did not (the
-// pointer-jumping path).
+// It runs for the selectable root searches (k_jump) only, and only when the
+// top-down search of the detached vertices did not find them.
 __global__ void __launch_bounds__(BLK) k_aff_collect(int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                                                     unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J) {
+                                                     unsigned *w, u64 *heavy, Ctl *ctl) {
     static_assert(IPA <= 32, "item masks are 32 bits");
     if (*(volatile int *)&ctl->skip) return;
     if (*(volatile int *)&ctl->td) return;
@@ -162,7 +160,6 @@ __global__ void __launch_bounds__(BLK) k_aff_collect(int n, const int *rep, cons
                 const int v = (int)(v0 + (long long)k * blockDim.x);
                 A[p + __popc(bk & lt)] = v;
                 rold[v] = r[k];
-                if (J) J[v] = par[v];   // seed of the asynchronous doubling
                 if (r[k] == v) {        // the old root: piece-weight and heaviest-piece slots
                     w[v] = 0;
                     heavy[v] = 0;
@@ -281,81 +278,6 @@ __device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long v
     warp_list_rows(pc, pb, rl, on && len > 0, w, st, len, p, ro);
 }
 
-// Representatives by asynchronous pointer doubling in place (delete batches
-// with DRSF_JUMP=async): no grid barrier between steps.  J holds a copy of
-// the cut forest for the listed vertices; afterwards J[v] is the complemented
-// root of every listed vertex, and k_jump<2> carries on from there.
-__global__ void __launch_bounds__(BLK, 6) k_jump_async(const int *A, Ctl *ctl, int *J, int *X, int *Y) {
-    if (*(volatile int *)&ctl->skip || *(volatile int *)&ctl->td) return;
-    const long long cnt = (long long)ctl->naff;
-    // asynchronous doubling in place (one buffer, no grid barrier
-    // between steps): each warp owns a slice of the list and repeats
-    // J[v] <- J[J[v]] over its open vertices until none is left.  A
-    // pointer only ever moves to an ancestor, whatever mix of old and
-    // new values a step reads, so every step moves an open vertex up
-    // at least one level and the result is the same roots.
-    // (list positions are below 2^31: at most n entries)
-    const int lane = threadIdx.x & 31;
-    const int nwarp = (int)(gstride() >> 5);
-    const int slice = (int)((cnt + nwarp - 1) / nwarp);
-    const int wlo = (int)(gtid() >> 5) * slice;
-    int wlen = wlo < cnt ? (int)(wlo + slice < cnt ? slice : cnt - wlo) : 0;
-    const int *in = A + wlo;
-    int *out = X + wlo, *spare = Y + wlo;
-    int it = 0;
-    long long vis = 0;
-    while (wlen > 0) {
-        if (it >= MAX_ROUNDS * 64) {
-            if (lane == 0) atomicOr(&ctl->err, ERR_ROUNDS);
-            return;
-        }
-        vis += wlen;
-        int nopen = 0;
-        for (int b0 = 0; b0 < wlen; b0 += 32 * JU) {
-            int v[JU], w0[JU], w2[JU];
-            bool ok[JU], open[JU];
-#pragma unroll
-            for (int k = 0; k < JU; ++k) {
-                const int i = b0 + k * 32 + lane;
-                ok[k] = i < wlen;
-                v[k] = ok[k] ? in[i] : 0;
-            }
-#pragma unroll
-            for (int k = 0; k < JU; ++k) w0[k] = ok[k] ? LD(J[v[k]]) : -1;
-#pragma unroll
-            for (int k = 0; k < JU; ++k) w2[k] = (ok[k] && w0[k] >= 0) ? LD(J[w0[k]]) : 0;
-#pragma unroll
-            for (int k = 0; k < JU; ++k) {
-                open[k] = false;
-                if (!ok[k]) continue;
-                int nv;
-                if (w0[k] < 0) nv = w0[k];
-                else if (w2[k] < 0) nv = w2[k];
-                else if (w2[k] == w0[k]) nv = ~w0[k];
-                else {
-                    nv = w2[k];
-                    open[k] = true;
-                }
-                J[v[k]] = nv;
-            }
-#pragma unroll
-            for (int k = 0; k < JU; ++k) {
-                const unsigned m = __ballot_sync(0xffffffffu, open[k]);
-                if (open[k]) out[nopen + __popc(m & ((1u << lane) - 1u))] = v[k];
-                nopen += __popc(m);
-            }
-        }
-        wlen = nopen;
-        in = out;
-        int *t = out; out = spare; spare = t;
-        ++it;
-    }
-    if (lane == 0 && vis) {
-        atomicAdd((u64 *)&ctl->jump_visits, (u64)vis);
-        atomicMax((unsigned long long *)&ctl->jump_rounds, (unsigned long long)it);
-    }
-}
-
 // Warp-aggregated list appends of the top-down search (no block barrier):
 // the calling lanes with `on` take consecutive slots of A, those with a
 // non-empty row (`len` > 0) consecutive rows of the row list and their entry
@@ -371,7 +293,7 @@ __global__ void __launch_bounds__(BLK, 6) k_jump_async(const int *A, Ctl *ctl, i
 // touches every vertex of every cut tree.  Each level's rows are appended to
 // the row list of the cross-edge scan as they are found (rows and entry
 // ranges from one packed counter, 32-entry tiles), so level k reads exactly
-// the rows appended in level k-1 with the tile-window scan of k_scan_lb, and
+// the rows appended in level k-1 with the tile-window scan of scan_rows, and
 // the scan afterwards reuses the list (the piece left out of every tree is
 // its root piece).  Every level appends through counters of its own (a ring
 // of three: level k appends to slot k+1, reads the final count of slot k
@@ -572,6 +494,245 @@ __global__ void __launch_bounds__(BLK, 4)
     }
 }
 
+// heavy[r] = the piece left out of the scan of the cut tree with old root r
+// (weight << 32 | piece; the root piece stays it unless a detached piece
+// outweighs it by HEAVY_SWAP_MIN vertices), over the cut list: a cut tree's
+// pieces are its root piece and one piece per cut vertex.
+__device__ __forceinline__ void heaviest_pieces(const int *cuts, long long nc, const int *rold, const unsigned *w,
+                                                u64 *heavy) {
+    for (long long i = gtid(); i < nc; i += gstride()) {
+        int c = cuts[i];
+        int r = rold[c];
+        u64 kc = ((u64)LD(w[c]) << 32) | (unsigned)c;
+        unsigned act = __activemask();
+        unsigned grp = __match_any_sync(act, r);
+        unsigned hi = (unsigned)(kc >> 32), lo = (unsigned)kc;
+        unsigned hmax = __reduce_max_sync(grp, hi);
+        unsigned lmax = __reduce_max_sync(grp, hi == hmax ? lo : 0u);
+        if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) {
+            atomicMax(&heavy[r], ((u64)hmax << 32) | lmax);
+            atomicMax(&heavy[r], ((u64)(LD(w[r]) + HEAVY_SWAP_MIN) << 32) | (unsigned)r);
+        }
+    }
+}
+
+// Delete: the pieces of the cut trees (Algorithm 1, representatives by pointer
+// jumping) and the detached vertices, in one launch over all vertices:
+//   1. each vertex of a cut tree (its old root was stamped by the cut) follows
+//      its parents for up to RELABEL_HOPS steps in the forest, which nobody
+//      writes here, and leaves the ancestor it reached, or its root
+//      complemented, in J;
+//   2. after a grid barrier each warp's vertices still open (deep trees) go on
+//      by asynchronous pointer doubling in place, J[v] <- J[J[v]]: a pointer
+//      only ever moves to an ancestor, whatever mix of old and new values a
+//      step reads, so every step moves an open vertex up at least one level;
+//   3. the vertices whose root changed (the detached ones; on R-MAT a few
+//      percent) get their new representative and are listed;
+//   4. every cut tree gets the piece that the scan for cross edges leaves out:
+//      every cross edge joins two pieces of one old tree, so scanning the rows
+//      of all pieces but one finds each of them.  That is the root piece,
+//      unless a detached piece has HEAVY_SWAP_MIN more vertices (a cut near
+//      the root that detaches most of a tree): then the heaviest piece.  The
+//      root piece's size is its tree's (counted in 1) less the detached
+//      pieces'.
+// Listing the affected vertices, doubling from distance 1 and a pass over that
+// whole list took 38 + 99 us of a 100K-edge delete batch on R-MAT scale 22
+// (2.5M affected vertices, 100K detached).
+#define RELABEL_HOPS 4
+#define RI 4   // vertices per lane and iteration
+
+// Piece counts of a block: a small open-addressing table in shared memory (one
+// global atomic per piece and block at the end; a large piece spans many
+// blocks), or straight to global memory when the table has no slot.
+struct PieceTable {
+    int k[WT_SLOTS];
+    unsigned c[WT_SLOTS];
+};
+__device__ __forceinline__ void pt_init(PieceTable &t) {
+    for (int i = threadIdx.x; i < WT_SLOTS; i += blockDim.x) {
+        t.k[i] = -1;
+        t.c[i] = 0;
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ void pt_flush(PieceTable &t, unsigned *w) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < WT_SLOTS; i += blockDim.x)
+        if (t.k[i] != -1) atomicAdd(&w[t.k[i]], t.c[i]);
+}
+// the lanes with `on` count 1 for their piece p (all 32 lanes call)
+__device__ __forceinline__ void pt_count(PieceTable &t, unsigned *w, int p, bool on) {
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (!on) return;
+    const unsigned grp = __match_any_sync(m, p);
+    if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) piece_count(t.k, t.c, w, p, (unsigned)__popc(grp));
+}
+
+__global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
+    if (*(volatile int *)&ctl->skip) return;
+    if (*(volatile int *)&ctl->td) return;   // the top-down search found the pieces
+    const unsigned ep = ctl->epoch;
+    const long long nc = (long long)ctl->ncut;
+    if (nc == 0) return;   // no tree was cut
+    u64 *bar = &ctl->bar[0];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    __shared__ PieceTable pt;
+    pt_init(pt);
+    // chunks of consecutive vertices, dealt out to the blocks in turn (graphs
+    // or regions with deep trees spread over all of them); a warp's lists
+    // have room for its part of every chunk of its block
+    constexpr int CH = BLK * RI;
+    const long long nch = ((long long)a.n + CH - 1) / CH, per = (nch + gridDim.x - 1) / gridDim.x;
+    const long long own = ((long long)blockIdx.x * CH + (threadIdx.x & ~31) * RI) * per;
+    int *const X = a.X + own, *const Y = a.Y + own, *const L = a.L + own;
+    int nopen = 0, nd = 0;
+    long long naff = 0, vis = 0;
+    int tr = -1;           // the tree that this warp counts, and its count so far
+    unsigned tc = 0;
+    for (long long c = blockIdx.x; c < nch; c += gridDim.x) {
+        const int v0 = (int)(c * CH) + (int)(threadIdx.x & ~31) * RI + lane;
+        int r[RI], x[RI];
+        unsigned on = 0, done = 0;   // vertices of cut trees; those at their root
+#pragma unroll
+        for (int k = 0; k < RI; ++k) {
+            const bool ok = (long long)v0 + k * 32 < a.n;
+            r[k] = ok ? a.rep[v0 + k * 32] : -1;
+            x[k] = ok ? a.par[v0 + k * 32] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < RI; ++k) {
+            if (r[k] >= 0 && a.aff_ep[r[k]] == ep) on |= 1u << k;
+            if (x[k] == v0 + k * 32) done |= 1u << k;
+        }
+        if (!__any_sync(0xffffffffu, on)) continue;
+#pragma unroll
+        for (int h = 0; h < RELABEL_HOPS; ++h) {
+            int nx[RI];
+#pragma unroll
+            for (int k = 0; k < RI; ++k) nx[k] = (on & ~done) >> k & 1u ? a.par[x[k]] : -1;
+#pragma unroll
+            for (int k = 0; k < RI; ++k) {
+                if (nx[k] < 0) continue;
+                if (nx[k] == x[k]) done |= 1u << k;
+                x[k] = nx[k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < RI; ++k) {
+            const bool in = on >> k & 1u, at = done >> k & 1u;
+            if (in) a.J[v0 + k * 32] = at ? ~x[k] : x[k];
+            const unsigned mi = __ballot_sync(0xffffffffu, in);
+            if (!mi) continue;
+            const unsigned mo = __ballot_sync(0xffffffffu, in && !at), md = __ballot_sync(0xffffffffu, in && at && x[k] != r[k]);
+            if (in && !at) X[nopen + __popc(mo & lt)] = v0 + k * 32;
+            if (in && at && x[k] != r[k]) L[nd + __popc(md & lt)] = v0 + k * 32;
+            nopen += __popc(mo);
+            nd += __popc(md);
+            // tree sizes: one tree for the whole warp is the common case
+            const int r0 = __shfl_sync(0xffffffffu, r[k], __ffs(mi) - 1);
+            if (__all_sync(0xffffffffu, !in || r[k] == r0)) {
+                if (r0 != tr) {
+                    if (lane == 0 && tc) piece_count(pt.k, pt.c, a.w, tr, tc);
+                    tr = r0;
+                    tc = 0;
+                }
+                tc += __popc(mi);
+            } else {
+                pt_count(pt, a.w, r[k], in);
+            }
+        }
+        naff += __popc(on);
+    }
+    if (lane == 0 && tc) piece_count(pt.k, pt.c, a.w, tr, tc);
+    block_add((long long *)&ctl->naff, naff);
+    if (!grid_barrier(ctl, bar)) return;
+    // (each warp reads lists that it wrote itself)
+    int *in = X, *out = Y;
+    int it = 0;
+    __syncwarp();
+    for (; nopen > 0; ++it) {
+        if (it >= MAX_ROUNDS * 64) {
+            if (lane == 0) atomicOr(&ctl->err, ERR_ROUNDS);
+            break;
+        }
+        vis += nopen;
+        int left = 0;
+        for (int b0 = 0; b0 < nopen; b0 += 32 * RI) {
+            int v[RI], w[RI];
+#pragma unroll
+            for (int k = 0; k < RI; ++k) v[k] = b0 + k * 32 + lane < nopen ? in[b0 + k * 32 + lane] : -1;
+#pragma unroll
+            for (int k = 0; k < RI; ++k) w[k] = v[k] >= 0 ? LD(a.J[v[k]]) : -1;
+#pragma unroll
+            for (int k = 0; k < RI; ++k) w[k] = w[k] >= 0 ? LD(a.J[w[k]]) : -1;
+#pragma unroll
+            for (int k = 0; k < RI; ++k) {
+                const bool ok = v[k] >= 0, op = ok && w[k] >= 0;
+                if (ok) a.J[v[k]] = w[k];
+                const bool det = ok && !op && ~w[k] != a.rep[v[k]];
+                const unsigned mo = __ballot_sync(0xffffffffu, op), md = __ballot_sync(0xffffffffu, det);
+                if (op) out[left + __popc(mo & lt)] = v[k];
+                if (det) L[nd + __popc(md & lt)] = v[k];
+                left += __popc(mo);
+                nd += __popc(md);
+            }
+        }
+        __syncwarp();
+        nopen = left;
+        int *t = in; in = out; out = t;
+    }
+    if (lane == 0 && vis) {
+        atomicAdd((u64 *)&ctl->jump_visits, (u64)vis);
+        atomicMax((unsigned long long *)&ctl->jump_rounds, (unsigned long long)it);
+    }
+    // detached vertices: the list of all of them (one reservation per block),
+    // representatives and piece weights (those of the cut vertices were zeroed
+    // at the cut)
+    {
+        const long long q = block_reserve(&ctl->ndet, lane == 0 ? nd : 0);
+        int *const D = a.D + __shfl_sync(0xffffffffu, q, 0);
+        for (int i0 = 0; i0 < nd; i0 += 32 * JF) {
+            int v[JF], p[JF];
+#pragma unroll
+            for (int k = 0; k < JF; ++k) v[k] = i0 + k * 32 + lane < nd ? L[i0 + k * 32 + lane] : -1;
+#pragma unroll
+            for (int k = 0; k < JF; ++k) p[k] = v[k] >= 0 ? ~LD(a.J[v[k]]) : 0;
+#pragma unroll
+            for (int k = 0; k < JF; ++k) {
+                if (v[k] >= 0) {
+                    D[i0 + k * 32 + lane] = v[k];
+                    a.rep[v[k]] = p[k];
+                }
+                pt_count(pt, a.w, p[k], v[k] >= 0);
+            }
+        }
+    }
+    pt_flush(pt, a.w);
+    if (!grid_barrier(ctl, bar)) return;
+    // per cut tree: the detached pieces' vertices and the heaviest of them
+    for (long long i = gtid(); i < nc; i += gstride()) {
+        const int c = a.cuts[i], r = a.rold[c];
+        const unsigned wc = LD(a.w[c]);
+        const unsigned grp = __match_any_sync(__activemask(), r);
+        const unsigned sum = __reduce_add_sync(grp, wc);
+        if (lane == __ffs(grp) - 1) atomicAdd(&a.wsum[r], sum);
+        if (wc >= HEAVY_SWAP_MIN) atomicMax(&a.heavy[r], ((u64)wc << 32) | (unsigned)c);
+    }
+    if (!grid_barrier(ctl, bar)) return;
+    bool swap = false;
+    for (long long i = gtid(); i < nc; i += gstride()) {
+        const int r = a.rold[a.cuts[i]];
+        const u64 hv = LD(a.heavy[r]);
+        const bool sw = (hv >> 32) >= (u64)(LD(a.w[r]) - LD(a.wsum[r])) + HEAVY_SWAP_MIN;
+        const int l = sw ? (int)(unsigned)hv : r;
+        a.left[a.cuts[i]] = l;
+        if (LD(a.left[r]) != l) a.left[r] = l;   // (one store per tree, not one per cut)
+        swap |= sw;
+    }
+    if (__syncthreads_or(swap) && threadIdx.x == 0) atomicOr(&ctl->flag[0], 1);
+}
+
 // Representatives (Algorithm 1, parallel pointer jumping) of the listed
 // vertices: rep[v] = root of v in F^ (J starts as a copy of parent).
 // Delete mode (1) then chooses the rows to scan for cross edges: every cross
@@ -583,7 +744,8 @@ __global__ void __launch_bounds__(BLK, 4)
 // and entry ranges are reserved together from one packed counter), their
 // CSR start, their (piece, piece left out) and the row of every 32-entry
 // tile for the load-balanced scan.
-// (6 blocks of BLK threads per SM: the rounds are latency-bound)
+// (The selectable synchronous and halving searches, and the representatives at
+// creation; 6 blocks of BLK threads per SM: the rounds are latency-bound.)
 template <int sync_rounds>
 __global__ void __launch_bounds__(BLK, 6)
     k_jump(const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par, int *J, int *J1, int *rep,
@@ -606,9 +768,6 @@ __global__ void __launch_bounds__(BLK, 6)
         // (par); its converged vertices still write both buffers.
         int *Jc = J, *Jn = J1;
         int r = 0;
-        if constexpr (sync_rounds == 2) {
-            // the roots were found by k_jump_async (complemented in J)
-        } else {
         if (gtid() == 0) {
             ctl->cnt[0] = (u64)cnt;
             ctl->cnt[1] = 0;
@@ -669,7 +828,6 @@ __global__ void __launch_bounds__(BLK, 6)
             int *t = Jc; Jc = Jn; Jn = t;
         }
         if (gtid() == 0) ctl->jump_rounds = r;
-        }
         if (mode == 0) {
             for (long long i = gtid(); i < cnt; i += gstride()) {
                 int v = use_list ? A[i] : (int)i;
@@ -776,22 +934,7 @@ __global__ void __launch_bounds__(BLK, 6)
     // piece per cut vertex, so the cut list covers them all
     const long long nc = (long long)ctl->ncut;
     if (gtid() == 0) ctl->flag[0] = 0;   // set by the swap check below
-    for (long long i = gtid(); i < nc; i += gstride()) {
-        int c = cuts[i];
-        int r = rold[c];
-        u64 kc = ((u64)LD(w[c]) << 32) | (unsigned)c;
-        unsigned act = __activemask();
-        unsigned grp = __match_any_sync(act, r);
-        unsigned hi = (unsigned)(kc >> 32), lo = (unsigned)kc;
-        unsigned hmax = __reduce_max_sync(grp, hi);
-        unsigned lmax = __reduce_max_sync(grp, hi == hmax ? lo : 0u);
-        if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) {
-            atomicMax(&heavy[r], ((u64)hmax << 32) | lmax);
-            // the root piece stays the piece left out unless a detached
-            // piece outweighs it by HEAVY_SWAP_MIN vertices
-            atomicMax(&heavy[r], ((u64)(LD(w[r]) + HEAVY_SWAP_MIN) << 32) | (unsigned)r);
-        }
-    }
+    heaviest_pieces(cuts, nc, rold, w, heavy);
     if (!grid_barrier(ctl, &ctl->bar[0])) return;
     // the provisional list left out each tree's root piece; where another
     // piece is heavier, rebuild the list with the exact rule (rare)
@@ -885,12 +1028,6 @@ __device__ __forceinline__ void compact_pairs(Ctl *ctl, PairTable pt, u64 *ck, i
         }
     }
 }
-__global__ void __launch_bounds__(BLK) k_pairs_compact(Ctl *ctl, PairTable pt, u64 *ck, int *ca, int *cb,
-                                                       u64 cand_cap) {
-    if (*(volatile int *)&ctl->skip) return;
-    compact_pairs(ctl, pt, ck, ca, cb, cand_cap);
-}
-
 // Per-block table of hot indices for 64-bit minimum updates: lanes of a
 // warp with the same index combine first; an index held by two or more
 // lanes of a warp (one piece, such as the giant one, can be an endpoint of
@@ -1070,25 +1207,18 @@ __device__ __forceinline__ void hook_init(const HookArgs &h, long long c0, unsig
     }
 }
 
-// Hooking as a launch of its own, for batches above LARGE_BATCH edges, whose
-// candidates stay in the millions past round 0: 256-thread blocks, four per
-// SM (R-MAT scale 20, 1M deletes: 5.0 against 5.4 ms with 1024).
-__global__ void __launch_bounds__(256, 4) k_hook_large(Ctl *ctl, HookArgs h) {
-    if (*(volatile int *)&ctl->skip) return;
-    __shared__ HotMin hm;
-    const long long c0 = (long long)ctl->ncand;
-    if (gtid() == 0) {
-        ctl->cnt[1] = ctl->cnt[2] = 0;
-        ctl->flag[0] = ctl->flag[1] = ctl->flag[2] = 0;
-    }
-    hm_init(hm);
-    hook_init(h, c0, ctl->epoch);
-    if (!grid_barrier(ctl, &ctl->bar[1])) return;
-    const int r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
-                                     h.hs.best0, h.hs.best1, h.er, h.er_cap);
-    if (r > 0 && blockIdx.x == 0)
+// All rounds: on the grid while many candidates are live, the rest (or all of
+// a short list) by block 0.  Returns -1 when a grid barrier gave up.
+__device__ __forceinline__ int hook_all(Ctl *ctl, HotMin &hm, const HookArgs &h, long long c0) {
+    int r = 0;
+    const bool few = c0 <= SMALL_CAND;
+    if (!few)
+        r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
+                               h.hs.best0, h.hs.best1, h.er, h.er_cap);
+    if ((few || r > 0) && blockIdx.x == 0)
         hook_rounds<true>(ctl, hm, r, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp, h.hs.best0,
                           h.hs.best1, h.er, h.er_cap);
+    return r;
 }
 
 // Path reversal by walking (ReversePaths, Algorithm 1): the path x = v0, v1 =
@@ -1191,7 +1321,7 @@ __device__ int rank_block(Ctl *ctl, int *svc, int *svn, int *snc, int *snn, int 
 // The core of the super-forest (the edges that are not leaf edges, listed
 // in cel) oriented by one block: adjacency ranges claimed by the first arc
 // of each core piece, arcs placed, Euler successors (as in the grid phases
-// of k_orient) written straight into shared memory, ranked there, and each
+// of orient_grid) written straight into shared memory, ranked there, and each
 // core edge oriented by its arc that comes first.  Block barriers only.
 __device__ void orient_small_core(Ctl *ctl, const OrientArgs &a, const int *cel, long long nce, unsigned ep) {
     __shared__ int s_nc;
@@ -1519,11 +1649,6 @@ __device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
     }
     block_add(&ctl->reversed, rev);
 }
-__global__ void __launch_bounds__(ORIENT_THREADS, 1) k_orient(Ctl *ctl, OrientArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
-    orient_grid(ctl, a);
-}
-
 // Replacement edges, orientation and walks of a batch with at most SMALL_CAND
 // candidates, by one block, everything but the walks in shared memory: the
 // pieces get dense ids through a hash table, the hook-and-compress rounds and
@@ -1531,6 +1656,8 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_orient(Ctl *ctl, OrientAr
 // On the grid the same batch is a chain of some twenty phases with a grid
 // barrier, two or three dependent global loads and up to a launch between
 // them, whatever its size.
+// The `pre` replacement edges that k_scan chose join the candidates again (the
+// minimum spanning forest is the same), all with their own pieces as ends.
 struct SmallTail {
     u64 key[SMALL_CAND], best[2 * SMALL_CAND];
     int hk[4 * SMALL_CAND];                       // hash table: piece, -1 free
@@ -1583,7 +1710,7 @@ __device__ __forceinline__ void tail_min(SmallTail &t, int x, u64 k, bool on) {
     if ((int)(threadIdx.x & 31) == __ffs(grp) - 1 && kmin < *(volatile u64 *)&t.best[x]) atomicMin(&t.best[x], kmin);
 }
 
-__device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa, int c0, unsigned ep) {
+__device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa, int c0, int pre, unsigned ep) {
     extern __shared__ __align__(16) int s_rank[];
     SmallTail &t = *reinterpret_cast<SmallTail *>(s_rank);
     constexpr int IT = SMALL_CAND / ORIENT_THREADS;   // candidates per thread
@@ -1596,10 +1723,18 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
 #pragma unroll
     for (int q = 0; q < IT; ++q) {
         const int i = q * ORIENT_THREADS + threadIdx.x;
-        alive[q] = i < c0;
-        key[q] = alive[q] ? LD(h.ck[0][i]) : 0;
-        ra[q] = alive[q] ? LD(h.ca[0][i]) : 0;
-        rb[q] = alive[q] ? LD(h.cb[0][i]) : 0;
+        alive[q] = i < c0 + pre;
+        key[q] = 0;
+        ra[q] = rb[q] = 0;
+        if (!alive[q]) continue;
+        key[q] = i < pre ? LD(h.er[i]) : LD(h.ck[0][i - pre]);
+        if (pre) {
+            ra[q] = oa.rep[klo(key[q])];
+            rb[q] = oa.rep[khi(key[q])];
+        } else {
+            ra[q] = LD(h.ca[0][i]);
+            rb[q] = LD(h.cb[0][i]);
+        }
     }
 #pragma unroll
     for (int q = 0; q < IT; ++q) {
@@ -1739,15 +1874,16 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
         ctl->cnt[1] = ctl->cnt[2] = 0;
         ctl->flag[0] = ctl->flag[1] = ctl->flag[2] = 0;
     }
-    if (h.pairs) {
+    if (h.pairs) {   // 
         compact_pairs(ctl, h.pt, h.ck[0], h.ca[0], h.cb[0], h.cand_cap);
         if (!grid_barrier(ctl, &ctl->bar[1])) return;
     }
     const long long c0 = (long long)*(volatile u64 *)&ctl->ncand;
-    if (c0 <= SMALL_CAND) {
-        if (c0 == 0) return;
+    const long long pre = ctl->pre ? (long long)*(volatile u64 *)&ctl->ner : 0;
+    if (c0 + pre <= SMALL_CAND) {
+        if (c0 + pre == 0) return;
         if (blockIdx.x == 0) {
-            replace_small(ctl, h, a, (int)c0, ep);
+            replace_small(ctl, h, a, (int)c0, (int)pre, ep);
         } else {
             const long long t = gtid() - blockDim.x, nt = gstride() - blockDim.x;
             l2_prefetch(a.parent, 4 * a.n, t, nt);
@@ -1760,12 +1896,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
         hook_init(h, c0, ep);
         if (!grid_barrier(ctl, &ctl->bar[1])) return;
     }
-    const int r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
-                                     h.hs.best0, h.hs.best1, h.er, h.er_cap);
-    if (r < 0) return;
-    if (r > 0 && blockIdx.x == 0)
-        hook_rounds<true>(ctl, hm, r, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp, h.hs.best0,
-                          h.hs.best1, h.er, h.er_cap);
+    if (hook_all(ctl, hm, h, c0) < 0) return;
     if (!grid_barrier(ctl, &ctl->bar[1])) return;
     orient_grid(ctl, a);
 }
@@ -1930,16 +2061,16 @@ __device__ __forceinline__ void reverse_marked(Ctl *ctl, const FinishArgs &a, lo
 // long (ctl->nlong), the doubling marks and the reversal of those pieces, in
 // one cooperative launch: without long walks (the common case) it is one
 // pass and no grid barrier, where two launches that found nothing to do cost
-// 10 us of every batch.  An insert passes over all vertices, a delete over
-// its affected list; after a top-down delete that list holds the detached
-// vertices only, so the rare one that re-rooted a tree's root piece
-// (need_root) passes over all vertices too.  With a.euler the marks are the
+// 10 us of every batch.  A top-down delete passes over the list of its
+// detached vertices, unless it re-rooted a tree's root piece (need_root);
+// the other batches pass over all vertices.  With a.euler the marks are the
 // Euler tour's (a launch of its own) and k_reverse follows it.
 __global__ void __launch_bounds__(BLK, 5) k_finish(Ctl *ctl, FinishArgs a) {
     if (*(volatile int *)&ctl->skip) return;
     const unsigned ep = ctl->epoch;
+    if (ctl->ner == 0) return;   // no piece was merged
     const bool marks = a.euler || *(volatile int *)&ctl->nlong;
-    if (ctl->op == DRSF_DELETE && !(ctl->td && *(volatile int *)&ctl->need_root))
+    if (ctl->op == DRSF_DELETE && ctl->td && !*(volatile int *)&ctl->need_root)
         refresh_pass<IPT>(ctl, a, a.A, (long long)ctl->naff, ep, marks);
     else if (a.n <= gstride() * IPT)
         refresh_pass<IPT>(ctl, a, nullptr, a.n, ep, marks);
@@ -1993,29 +2124,15 @@ static unsigned coop_blocks(const void *fn, int nsm, int cap_per_sm) {
 // The vertex passes (k_aff_collect, k_finish) loop over their range with
 // the blocks that are resident at once: no partial last wave.
 unsigned grid_vertex_pass(int nsm) { return coop_blocks((const void *)k_aff_collect, nsm, 8); }
+unsigned coop_blocks_relabel(int nsm) { return coop_blocks((const void *)k_relabel, nsm, 8); }
 unsigned coop_blocks_finish(int nsm) { return coop_blocks((const void *)k_finish, nsm, 8); }
 unsigned coop_blocks_jump(int nsm) {
-    // the three root-search variants share one launch bound; take the least
-    unsigned a = coop_blocks((const void *)k_jump<0>, nsm, 8), b = coop_blocks((const void *)k_jump<1>, nsm, 8),
-             c = coop_blocks((const void *)k_jump<2>, nsm, 8);
-    return a < b ? (a < c ? a : c) : (b < c ? b : c);
+    const unsigned a = coop_blocks((const void *)k_jump<0>, nsm, 8), b = coop_blocks((const void *)k_jump<1>, nsm, 8);
+    return a < b ? a : b;
 }
-unsigned coop_blocks_hook(int nsm) { return coop_blocks((const void *)k_hook_large, nsm, 4); }
-// one block per SM (both kernels take the same dynamic shared memory)
-unsigned coop_blocks_orient(int nsm) {
-    cudaFuncSetAttribute((const void *)k_orient, cudaFuncAttributeMaxDynamicSharedMemorySize, ORIENT_SMEM_BYTES);
+unsigned coop_blocks_replace(int nsm) {
     cudaFuncSetAttribute((const void *)k_replace, cudaFuncAttributeMaxDynamicSharedMemorySize, ORIENT_SMEM_BYTES);
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, (const void *)k_orient, ORIENT_THREADS,
-                                                      ORIENT_SMEM_BYTES) != cudaSuccess ||
-        per < 1)
-        per = 1;
-    int per2 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, (const void *)k_replace, ORIENT_THREADS,
-                                                      ORIENT_SMEM_BYTES) != cudaSuccess ||
-        per2 < 1)
-        per2 = 1;
-    return (unsigned)((per < per2 ? per : per2) * nsm);
+    return (unsigned)nsm;   // one block per SM (shared memory)
 }
 
 cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s) {
@@ -2023,8 +2140,8 @@ cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cuda
     return cudaGetLastError();
 }
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, cudaStream_t s) {
-    k_aff_collect<<<d.grid_pass, BLK, 0, s>>>(n, rep, aff_ep, A, rold, w, heavy, ctl, par, J);
+                               unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s) {
+    k_aff_collect<<<d.grid_pass, BLK, 0, s>>>(n, rep, aff_ep, A, rold, w, heavy, ctl);
     return cudaGetLastError();
 }
 cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf,
@@ -2038,9 +2155,9 @@ cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *pa
     return cudaLaunchCooperativeKernel((const void *)k_detach, d.coop_detach, BLK, args, 0, s);
 }
 unsigned coop_blocks_detach(int nsm) { return coop_blocks((const void *)k_detach, nsm, 4); }
-cudaError_t launch_jump_async(const Dev &d, const int *A, Ctl *ctl, int *J, int *X, int *Y, cudaStream_t s) {
-    k_jump_async<<<d.coop_jump, BLK, 0, s>>>(A, ctl, J, X, Y);
-    return cudaGetLastError();
+cudaError_t launch_relabel(const Dev &d, Ctl *ctl, RelabelArgs a, cudaStream_t s) {
+    void *args[] = {(void *)&ctl, (void *)&a};
+    return cudaLaunchCooperativeKernel((const void *)k_relabel, d.coop_relabel, BLK, args, 0, s);
 }
 cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par,
                         int *J, int *J1, int *rep, RowList rl, int mode, const int *rold, unsigned *w, u64 *heavy,
@@ -2049,25 +2166,12 @@ cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_
                     (void *)&J,    (void *)&J1,       (void *)&rep,        (void *)&rl,  (void *)&mode,
                     (void *)&rold, (void *)&w,        (void *)&heavy,      (void *)&g,   (void *)&X,
                     (void *)&Y,    (void *)&cuts};
-    const void *fn = sync_rounds == 2 ? (const void *)k_jump<2>
-                                      : (sync_rounds ? (const void *)k_jump<1> : (const void *)k_jump<0>);
+    const void *fn = sync_rounds ? (const void *)k_jump<1> : (const void *)k_jump<0>;
     return cudaLaunchCooperativeKernel(fn, d.coop_jump, BLK, args, 0, s);
 }
 cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&h, (void *)&a};
-    return cudaLaunchCooperativeKernel((const void *)k_replace, d.coop_orient, ORIENT_THREADS, args,
-                                       ORIENT_SMEM_BYTES, s);
-}
-cudaError_t launch_hook_large(const Dev &d, Ctl *ctl, HookArgs h, cudaStream_t s) {
-    if (h.pairs)
-        k_pairs_compact<<<grid_for(((long long)h.pt.mask + 4) / 4, BLK, (unsigned)d.nsm * 8u), BLK, 0, s>>>(
-            ctl, h.pt, h.ck[0], h.ca[0], h.cb[0], h.cand_cap);
-    void *args[] = {(void *)&ctl, (void *)&h};
-    return cudaLaunchCooperativeKernel((const void *)k_hook_large, d.coop_hook, BLK, args, 0, s);
-}
-cudaError_t launch_orient(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
-    void *args[] = {(void *)&ctl, (void *)&a};
-    return cudaLaunchCooperativeKernel((const void *)k_orient, d.coop_orient, ORIENT_THREADS, args,
+    return cudaLaunchCooperativeKernel((const void *)k_replace, d.coop_replace, ORIENT_THREADS, args,
                                        ORIENT_SMEM_BYTES, s);
 }
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {

@@ -14,8 +14,8 @@ struct Dev {
     int nsm;
     unsigned grid;        // grid-stride kernels: nsm * 8 blocks of BLK
     unsigned coop_jump;   // cooperative kernels: co-resident block counts
-    unsigned coop_hook;
-    unsigned coop_orient;
+    unsigned coop_replace;
+    unsigned coop_relabel;
     unsigned coop_finish;
     unsigned coop_bfs;
     unsigned coop_et;
@@ -38,9 +38,16 @@ cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, const int2 *place, lo
 // (the batch kernels read the batch from the control block; len sizes the grid)
 cudaError_t launch_validate_batch(long long len, int n, Ctl *ctl, cudaStream_t s);
 
+// Per-piece slots that a cut sets up: for the cut vertex and for its tree's
+// old root (k_relabel, k_scan).
+struct PieceSlots {
+    unsigned *aff_ep;   // old roots of this batch's cut trees
+    int *rold, *comp;
+    u64 *best, *heavy;
+    unsigned *w, *wsum;
+};
 cudaError_t launch_del_claim(long long len, Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl,
-                             unsigned *aff_ep, unsigned *cut_ep, int *cutlist, unsigned *w, int *rold,
-                             cudaStream_t s);
+                             PieceSlots ps, int *cutlist, cudaStream_t s);
 // The rows a delete batch scans for cross edges, one entry per listed
 // vertex u: u itself, the exclusive prefix sum of the row lengths (roff[nd]
 // = total), the row's start in the CSR, and (rep[u], piece left out of the
@@ -65,10 +72,28 @@ cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *
 cudaError_t launch_ins_place(const Dev &d, const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix,
                              u64 *ovf, u64 ovf_cap, const int *rep, bool sg, PairTable pt, u64 *ck, int *ca, int *cb,
                              u64 cand_cap, HookSlots hs, cudaStream_t s);
-cudaError_t launch_scan_rows(const Dev &d, RowList rl, Ctl *ctl, Csr g, const int *rep, bool sg, PairTable pt,
-                             u64 *ck, int *ca, int *cb, u64 cand_cap, cudaStream_t s);
-cudaError_t launch_scan_ovf(const Dev &d, const u64 *ovf, Ctl *ctl, const int *rep, bool sg, PairTable pt, u64 *ck,
-                            int *ca, int *cb, u64 cand_cap, cudaStream_t s);
+struct LightArgs {
+    int n;
+    Csr g;
+    const int *rep;
+    const unsigned *aff_ep;   // old roots of the cut trees
+    const int *rold, *left;   // per cut vertex: its tree's old root; per piece: the one left out in its tree
+    unsigned *rows;           // per 32 listed rows: those with a cross edge
+    int *D;                   // the vertices whose rows are read
+    int *job;                 // long rows: vertex, part
+    int *comp;                // hook forest of the pieces
+    u64 *best;                // per piece: its minimum cross edge
+    unsigned *root_ep;        // old roots that hooked
+    const int *cuts;
+    u64 *er;                  // replacement edges
+    const u64 *ovf;
+    PairTable pt;
+    u64 *ck;                  // candidates left
+    int *ca, *cb;
+    u64 cand_cap;
+    int listed;               // the rows come as a RowList (selectable root searches)
+};
+cudaError_t launch_scan(const Dev &d, Ctl *ctl, RowList rl, LightArgs a, bool sg, cudaStream_t s);
 cudaError_t launch_extract(const Dev &d, int n, Csr g, const u64 *ovf, u64 novf_max, Ctl *ctl, int *out,
                            long long cap, u64 *cnt, cudaStream_t s);
 cudaError_t launch_check_tree_edges(int n, const int *parent, Index ix, int *bad, cudaStream_t s);
@@ -77,7 +102,7 @@ cudaError_t launch_check_cross(const int *pairs, long long m, const int *rep, in
 // forest.cu ------------------------------------------------------------
 cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s);
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
-                               unsigned *w, u64 *heavy, Ctl *ctl, const int *par, int *J, cudaStream_t s);
+                               unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s);
 // delete: detached vertices top-down from the cut vertices (falls back to
 // the pointer jumping above when over budget).
 // DETACH_LEVELS: its level limit (measured on R-MAT, where it pays, the
@@ -89,7 +114,29 @@ cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *pa
                           const int *rold, long long budget_v, long long budget_e, int max_levels, int *oc, int *op,
                           cudaStream_t s);
 unsigned coop_blocks_detach(int nsm);
-cudaError_t launch_jump_async(const Dev &d, const int *A, Ctl *ctl, int *J, int *X, int *Y, cudaStream_t s);
+struct RelabelArgs {
+    int n;
+    int *rep;
+    const int *par;
+    const unsigned *aff_ep;   // old roots of the cut trees
+    int *J;                   // ancestor, or ~root
+    int *X, *Y, *L;           // per-warp lists: open vertices (ping-pong), detached vertices
+    int *D;                   // all detached vertices
+    const int *rold;          // per cut vertex: the old root of its tree
+    unsigned *w;              // vertices per detached piece; per old root: of its tree
+    unsigned *wsum;           // per old root: vertices of the detached pieces
+    u64 *heavy;               // per old root: the heaviest large detached piece
+    int *left;                // per piece: the one that the scan leaves out in its tree
+    const int *cuts;
+};
+// entries of each list array: blocks take chunks of BLK * 4 vertices in turn,
+// every block has room for as many as the first one
+static inline long long relabel_room(long long n, unsigned blocks) {
+    const long long ch = BLK * 4, nch = (n + ch - 1) / ch, per = (nch + blocks - 1) / blocks;
+    return (nch < (long long)blocks ? nch : (long long)blocks) * per * ch;
+}
+cudaError_t launch_relabel(const Dev &d, Ctl *ctl, RelabelArgs a, cudaStream_t s);
+unsigned coop_blocks_relabel(int nsm);
 cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par,
                         int *J, int *J1, int *rep, RowList rl, int mode, const int *rold, unsigned *w, u64 *heavy,
                         Csr g, int sync_rounds, int *X, int *Y, const int *cuts, cudaStream_t s);
@@ -127,10 +174,8 @@ struct OrientArgs {
     long long n;
 };
 cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s);
-// the same in three launches, for batches above LARGE_BATCH edges
+// batches above this many edges walk their paths in a launch of its own
 #define LARGE_BATCH (1 << 18)
-cudaError_t launch_hook_large(const Dev &d, Ctl *ctl, HookArgs h, cudaStream_t s);
-cudaError_t launch_orient(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);
 struct FinishArgs {
     const int *A;             // delete: the affected list
@@ -152,8 +197,7 @@ cudaError_t launch_labels(int n, const int *rep, int *tmp, int *out, cudaStream_
 unsigned coop_blocks_jump(int nsm);
 unsigned grid_vertex_pass(int nsm);
 unsigned coop_blocks_finish(int nsm);
-unsigned coop_blocks_hook(int nsm);
-unsigned coop_blocks_orient(int nsm);
+unsigned coop_blocks_replace(int nsm);
 cudaError_t launch_barrier_selftest(Ctl *ctl, cudaStream_t s);
 // static.cu ------------------------------------------------------------
 cudaError_t launch_static_forest(const Dev &d, int n, Csr g, const u64 *ovf, Ctl *ctl, int *lab, int *comp,

@@ -1,0 +1,79 @@
+"""The pieces of cut trees found over all vertices (no top-down search):
+depths around the hops of the first step, slices with and without affected
+vertices, and pieces around the weight at which the root piece is scanned
+instead, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_20211_gb300 as drsf
+import workloads
+from tests.gpu_util import _tiny_graph, check_batch, make_forest, run_trajectory
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    drsf.build()
+
+
+@pytest.mark.parametrize("depth", [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 33])
+def test_chains_of_every_depth(depth, monkeypatch):
+    """Many chains of one depth under a common root, some cut at each level,
+    half of them with a second way back to the root."""
+    monkeypatch.setenv("DRSF_DETACH", "0")
+    chains = 700
+    n = 1 + chains * depth
+    edges, parent = [], [0]
+    for c in range(chains):
+        for k in range(depth):
+            v = 1 + c * depth + k
+            edges.append((v, 0 if k == 0 else v - 1))
+            parent.append(0 if k == 0 else v - 1)
+        if c % 2 and depth > 1:
+            edges.append((0, 1 + c * depth + depth - 1))
+    g = _tiny_graph(n, edges, parent)
+    f = make_forest(g)
+    cut = np.array([(1 + c * depth + c % depth, parent[1 + c * depth + c % depth]) for c in range(0, chains, 3)],
+                   np.int32)
+    try:
+        keys, par, _ = check_batch(f, n, g.keys, g.parent, drsf.DELETE, cut)
+        keys, par, _ = check_batch(f, n, keys, par, drsf.INSERT, cut)
+        check_batch(f, n, keys, par, drsf.DELETE, cut[::2])
+    finally:
+        f.close()
+
+
+@pytest.mark.parametrize("below", [4095, 4096, 4097, 9000, 30_000])
+def test_piece_weights_around_the_swap(below, monkeypatch):
+    """A cut below the root detaches `below` vertices of 34,000 (and a second
+    tree is cut in small pieces): the piece left out of the scan changes."""
+    monkeypatch.setenv("DRSF_DETACH", "0")
+    n, m = 34_000, 2000
+    rng = np.random.default_rng(below)
+    # vertex 0 - children 1 .. n - below - 1; vertex n - below heads a piece of `below` vertices
+    h = n - below
+    parent = [0] + [0] * (h - 1) + [0] + [h] * (below - 1)
+    edges = [(v, parent[v]) for v in range(1, n)]
+    edges += [tuple(e) for e in np.stack([rng.integers(1, h, 500), rng.integers(h, n, 500)], 1).tolist()]
+    parent += [n] + [n + i // 2 for i in range(m - 1)]      # second tree, binary
+    edges += [(n + 1 + i, n + i // 2) for i in range(m - 1)]
+    g = _tiny_graph(n + m, edges, parent)
+    f = make_forest(g)
+    cut = np.array([(h, 0)] + [(n + i, parent[n + i]) for i in range(5, m, 7)], np.int32)
+    try:
+        keys, par, _ = check_batch(f, n + m, g.keys, g.parent, drsf.DELETE, cut)
+        check_batch(f, n + m, keys, par, drsf.INSERT, cut)
+    finally:
+        f.close()
+
+
+def test_trajectories_without_the_top_down_search(monkeypatch):
+    monkeypatch.setenv("DRSF_DETACH", "0")
+    I, D = drsf.INSERT, drsf.DELETE
+    run_trajectory(workloads.rmat_graph(16, 16, seed=2), [(I, 1000), (D, 1000), (I, 10_000), (D, 50_000)] * 2, seed=3)
+    run_trajectory(workloads.grid_graph(512, 512, seed=3), [(D, 5000), (I, 5000)] * 2, seed=4, tree_frac=0.9, local=64)
+    run_trajectory(workloads.er_graph(20_001, 25_000, seed=1), [(I, 2000), (D, 2000)] * 2, seed=5)
