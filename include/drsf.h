@@ -98,11 +98,11 @@ enum {
      * per pair of trees (its minimum-key cross edge, through a hash table
      * keyed by the pair of roots), and the hooking then runs on the
      * supergraph.  DRSF_REPL_HS, hooking and shortcutting (Section III-B):
-     * the hooking runs on every cross edge.  Neither flag (or both): chosen
-     * per batch by comparing the number of key edges |M| with n, as the
-     * paper's comparison of the two does (Section V, influencing factors):
-     * SG when |M| > n / 16, where |M| is the batch length for an insert and
-     * the non-tree edges of G (live edges - n) for a delete.  The result is
+     * the hooking runs on every cross edge.  Neither flag (or both): HS for
+     * an insert; for a delete chosen by comparing the number of key edges |M|
+     * with n, as the paper's comparison of the two does (Section V,
+     * influencing factors): SG when |M| > n / 16, where |M| is the non-tree
+     * edges of G (live edges - n).  The result is
      * the same either way (the minimum-key forest does not depend on how
      * parallel super-edges are reduced). */
     DRSF_REPL_SG = 8u,

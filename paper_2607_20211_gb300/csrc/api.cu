@@ -662,17 +662,18 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
 
 // Replacement-edge variant of a batch (Section III): the supergraph (SG)
 // reduction of parallel cross edges, or hooking on every cross edge (HS).
-// A flag forces one; otherwise the key-edge count |M| is compared with n
-// (Section V: HS suits |M| >> n in the paper's implementations, SG the
-// opposite; here the hooking's cost follows the candidate count, so the
-// supergraph's reduction pays off when the key edges outnumber the
-// vertices).  |M| is the batch for an insert and the non-tree edges of G
-// for a delete, from the host-side bound on live edges (no device read).
-static bool use_supergraph(const drsf_ctx *h, int op, long long len) {
+// A flag forces one; otherwise an insert hooks on its cross edges (few of a
+// batch's edges join two trees: reducing them first took 142 us more for the
+// 256-graph union's 1.6M-edge batches, most of it for emptying the pair
+// table), and for a delete the key edges |M| = the non-tree edges of G, from
+// the host-side bound on live edges (no device read), are compared with n:
+// the hooking's cost follows the candidate count, so the reduction pays off
+// when the key edges outnumber the vertices.
+static bool use_supergraph(const drsf_ctx *h, int op) {
     const bool sg = (h->flags & DRSF_REPL_SG) != 0, hs = (h->flags & DRSF_REPL_HS) != 0;
     if (sg != hs) return sg;
-    long long keys = op == DRSF_INSERT ? len : std::max<long long>(0, h->occ_bound - (long long)h->n);
-    return keys > (long long)h->n / 16;
+    if (op == DRSF_INSERT) return false;
+    return std::max<long long>(0, h->occ_bound - (long long)h->n) > (long long)h->n / 16;
 }
 
 // The launch sequence of one batch after k_begin (Algorithm 1).  Its
@@ -892,7 +893,7 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     if (st) return st;
     st = storage_check(h, op, len, s);
     if (st) return st;
-    const bool sg = use_supergraph(h, op, len);
+    const bool sg = use_supergraph(h, op);
     h->last_sg = sg ? 1 : 0;
     // the top-down delete for small batches: its cost follows the detached
     // vertices' rows and its levels, the pointer jumping's the cut trees
