@@ -262,6 +262,18 @@ DRSF_API drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t
                                         int32_t num_classes, drsf_stream stream);
 
 /*
+ * drsf_apply_grouped -- the same batched update (drsf_apply_batched's graphs,
+ * slices, checks and result) through drsf_apply's grid-wide launch sequence:
+ * the graphs' updates are one batch of their union, whose slices are checked
+ * on the device first.  It needs no schedule, and measured faster at every
+ * size tried (2 graphs of 1K vertices to 128 of up to 64K: 1.3 to 9 times).
+ * Errors: as drsf_apply_batched.
+ */
+DRSF_API drsf_status drsf_apply_grouped(drsf_handle h, drsf_op op, const int32_t *batch, int64_t len,
+                                        int32_t num_graphs, const int64_t *vertex_offsets,
+                                        const int64_t *batch_offsets, drsf_stream stream);
+
+/*
  * drsf_reserve -- size the handle's per-batch buffers (device work lists,
  * pair table, the pinned host staging of drsf_apply_host) for batches of up
  * to max_batch edges now, so that later drsf_apply / drsf_apply_host calls

@@ -35,7 +35,7 @@ struct drsf_ctx {
     std::vector<Buf> bufs;
     bool poisoned = false;
     int jump_sync = 2;   // root search: 2 hops, then asynchronous doubling; 1 synchronous rounds, 0 path halving
-    int pending_einval = 0;
+    unsigned epoch = 0;  // batches so far (the stamps of the per-batch arrays)
     int last_sg = 0;     // the last batch took the supergraph variant
     // captured per-batch launch sequences (CUDA graphs), valid for storage
     // generation u_gen; gen moves whenever a storage or batch buffer moves
@@ -99,7 +99,7 @@ struct drsf_ctx {
     bool b_ready = false;
     BState *b_state = nullptr;    // device copies of the per-call state and descriptor
     BDesc *b_desc = nullptr;
-    long long b_gcap = 0;         // graphs the per-graph arrays hold
+    long long b_gcap = 0, b_gcnt_cap = 0;   // graphs that b_meta and the per-graph counters hold
     char *b_meta = nullptr;       // device: voff (G+1) | boff (G+1) | order (G)
     char *b_meta_host = nullptr;  // pinned staging of the same
     cudaEvent_t b_meta_done = nullptr;
@@ -684,8 +684,6 @@ static bool use_supergraph(const drsf_ctx *h, int op) {
 static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cudaStream_t s) {
     Ctl *ctl = h->ctl;
     Csr g{h->row, h->col, h->fpos};
-    CK(launch_validate_batch(glen, h->n, ctl, s));
-    prof_end(h, PH_BEGIN, 2, s);
     if (op == DRSF_INSERT) {
         // Algorithm 1, insert: F^ = F, M = B; rep of the previous batch is current
         prof_begin(h, PH_INS_CLAIM, s);
@@ -888,7 +886,8 @@ static void drop_graphs(drsf_ctx *h) {
     h->u_graphs.clear();
 }
 
-static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t len, cudaStream_t s) {
+static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t len, cudaStream_t s,
+                              int groups = 0, const long long *voff = nullptr, const long long *boff = nullptr) {
     drsf_status st = ensure_batch(h, len, s);
     if (st) return st;
     st = storage_check(h, op, len, s);
@@ -904,7 +903,8 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
         h->prof_nb[op]++;
     }
     prof_begin(h, PH_BEGIN, s);
-    CK(launch_begin(h->ctl, op, len, batch, s));
+    CK(launch_begin(h->ctl, BeginArgs{op, h->n, len, batch, ++h->epoch, groups, voff, boff}, s));
+    prof_end(h, PH_BEGIN, 1, s);
     // per-phase profiling brackets the phases with events: launch directly
     if (h->prof_on || !h->graphs_ok) return launch_rest(h, op, sg, len, s);
     // otherwise replay the captured sequence for this (storage, op, variant,
@@ -978,7 +978,6 @@ static drsf_status batched_scratch(drsf_ctx *h, cudaStream_t s) {
     CKA(halloc(h, &h->b_desc, 1, s));
     CK(cudaStreamCreateWithFlags(&h->b_cap, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&h->b_fork, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&h->b_meta_done, cudaEventDisableTiming));
     for (int c = 0; c < BCLASSES; ++c) {
         CK(cudaStreamCreateWithFlags(&h->b_cls[c], cudaStreamNonBlocking));
         CK(cudaEventCreateWithFlags(&h->b_join[c], cudaEventDisableTiming));
@@ -987,26 +986,75 @@ static drsf_status batched_scratch(drsf_ctx *h, cudaStream_t s) {
     return DRSF_OK;
 }
 
+// The graphs' offsets (and queue order) on the device, copied from pinned
+// staging by each call.
+static drsf_status batched_meta(drsf_ctx *h, long long G, cudaStream_t s) {
+    if (!h->b_meta_done) CK(cudaEventCreateWithFlags(&h->b_meta_done, cudaEventDisableTiming));
+    if (G <= h->b_gcap) return DRSF_OK;
+    CK(cudaStreamSynchronize(s));
+    if (h->b_meta_host) cudaFreeHost(h->b_meta_host);
+    h->b_meta_host = nullptr;
+    hfree(h, &h->b_meta, s);
+    h->b_gcap = 0;
+    const long long cap = std::max<long long>(G, 256);
+    const size_t bytes = (size_t)(2 * (cap + 1)) * sizeof(long long) + (size_t)cap * sizeof(int);
+    CKA(halloc(h, &h->b_meta, bytes, s));
+    CK(cudaMallocHost((void **)&h->b_meta_host, bytes));
+    h->b_gcap = cap;
+    h->b_meta_pending = false;
+    return DRSF_OK;
+}
+
+// The arguments that the two batched calls share; DRSF_OK when they are valid.
+static drsf_status batched_check(drsf_handle h, int op, const int32_t *batch, int64_t len, int32_t num_graphs,
+                                 const int64_t *vertex_offsets, const int64_t *batch_offsets) {
+    if (!h || (op != DRSF_INSERT && op != DRSF_DELETE) || len < 0 || (len > 0 && !batch) || num_graphs < 1 ||
+        !vertex_offsets || !batch_offsets)
+        return DRSF_EINVAL;
+    if (h->poisoned) return DRSF_EPOISONED;
+    if (len > (int64_t)1 << 31) return DRSF_EINVAL;
+    const long long G = num_graphs;
+    if (vertex_offsets[0] < 0 || vertex_offsets[G] > h->n || batch_offsets[0] != 0 || batch_offsets[G] != len)
+        return DRSF_EINVAL;
+    for (long long g = 0; g < G; ++g)
+        if (vertex_offsets[g + 1] < vertex_offsets[g] || batch_offsets[g + 1] < batch_offsets[g]) return DRSF_EINVAL;
+    return DRSF_OK;
+}
+
+drsf_status drsf_apply_grouped(drsf_handle h, drsf_op op, const int32_t *batch, int64_t len, int32_t num_graphs,
+                               const int64_t *vertex_offsets, const int64_t *batch_offsets, drsf_stream stream) {
+    drsf_status st = batched_check(h, (int)op, batch, len, num_graphs, vertex_offsets, batch_offsets);
+    if (st) return st;
+    set_dev(h);
+    cudaStream_t s = (cudaStream_t)stream;
+    const long long G = num_graphs;
+    st = batched_meta(h, G, s);
+    if (st) return st;
+    if (h->b_meta_pending) CK(cudaEventSynchronize(h->b_meta_done));   // the last call's copy out of the staging
+    const size_t bytes = (size_t)(G + 1) * sizeof(long long);
+    memcpy(h->b_meta_host, vertex_offsets, bytes);
+    memcpy(h->b_meta_host + bytes, batch_offsets, bytes);
+    CK(cudaMemcpyAsync(h->b_meta, h->b_meta_host, 2 * bytes, cudaMemcpyHostToDevice, s));
+    CK(cudaEventRecord(h->b_meta_done, s));
+    h->b_meta_pending = true;
+    const long long *off = (const long long *)h->b_meta;
+    return apply_impl(h, (int)op, batch, len, s, (int)G, off, off + (G + 1));
+}
+
 // Per-graph arrays for G graphs and the candidate pool for this call.
 static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cudaStream_t s) {
     BState &b = h->b_st;
-    if (G > h->b_gcap) {
+    drsf_status st = batched_meta(h, G, s);
+    if (st) return st;
+    if (h->b_gcap > h->b_gcnt_cap) {
         CK(cudaStreamSynchronize(s));
-        if (h->b_meta_host) cudaFreeHost(h->b_meta_host);
-        h->b_meta_host = nullptr;
-        hfree(h, &h->b_meta, s);
         hfree(h, &b.gcnt, s);
         hfree(h, &b.gcur, s);
         hfree(h, &b.govf_start, s);
-        long long cap = std::max<long long>(G, 256);
-        size_t bytes = (size_t)(2 * (cap + 1)) * sizeof(long long) + (size_t)cap * sizeof(int);
-        CKA(halloc(h, &h->b_meta, bytes, s));
-        CK(cudaMallocHost((void **)&h->b_meta_host, bytes));
-        CKA(halloc(h, &b.gcnt, (size_t)cap + 1, s));
-        CKA(halloc(h, &b.gcur, (size_t)cap + 1, s));
-        CKA(halloc(h, &b.govf_start, (size_t)cap + 1, s));
-        h->b_gcap = cap;
-        h->b_meta_pending = false;
+        CKA(halloc(h, &b.gcnt, (size_t)h->b_gcap + 1, s));
+        CKA(halloc(h, &b.gcur, (size_t)h->b_gcap + 1, s));
+        CKA(halloc(h, &b.govf_start, (size_t)h->b_gcap + 1, s));
+        h->b_gcnt_cap = h->b_gcap;
     }
     // candidates: at most the batch (insert) or every live edge (delete),
     // plus one partly used chunk per graph
@@ -1042,16 +1090,10 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
 drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, int64_t len, int32_t num_graphs,
                                const int64_t *vertex_offsets, const int64_t *batch_offsets,
                                const drsf_batched_class *classes, int32_t num_classes, drsf_stream stream) {
-    if (!h || (op != DRSF_INSERT && op != DRSF_DELETE) || len < 0 || (len > 0 && !batch) || num_graphs < 1 ||
-        !vertex_offsets || !batch_offsets || !classes || num_classes < 1 || num_classes > BCLASSES)
-        return DRSF_EINVAL;
-    if (h->poisoned) return DRSF_EPOISONED;
-    if (len > (int64_t)1 << 31) return DRSF_EINVAL;
+    if (!classes || num_classes < 1 || num_classes > BCLASSES) return DRSF_EINVAL;
+    drsf_status st = batched_check(h, (int)op, batch, len, num_graphs, vertex_offsets, batch_offsets);
+    if (st) return st;
     const long long G = num_graphs;
-    if (vertex_offsets[0] < 0 || vertex_offsets[G] > h->n || batch_offsets[0] != 0 || batch_offsets[G] != len)
-        return DRSF_EINVAL;
-    for (long long g = 0; g < G; ++g)
-        if (vertex_offsets[g + 1] < vertex_offsets[g] || batch_offsets[g + 1] < batch_offsets[g]) return DRSF_EINVAL;
     for (int c = 0; c < num_classes; ++c) {
         const int t = classes[c].block_threads, cb = classes[c].cluster_blocks;
         if ((t != 128 && t != 256 && t != 512 && t != 1024) || classes[c].blocks_per_sm < 0) return DRSF_EINVAL;
@@ -1060,7 +1102,7 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     }
     set_dev(h);
     cudaStream_t s = (cudaStream_t)stream;
-    drsf_status st = ensure_batch(h, len, s);
+    st = ensure_batch(h, len, s);
     if (st) return st;
     st = storage_check(h, op, len, s);
     if (st) return st;
@@ -1125,6 +1167,7 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     d.order = order_d;
     d.G = (int)G;
     d.op = (int)op;
+    d.epoch = ++h->epoch;
     CK(launch_bset(h->b_state, b, h->b_desc, d, s));
     // one captured launch sequence per (op, class queues, launch shapes)
     std::string key = std::to_string((int)op);

@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(BT) k_bpersist(const BState *Sp, int cls, int 
     G.me = &L_own;
     // every block of the group reads the same skip flag, so they all leave
     // together
-    if (*(volatile int *)&S.ctl->skip) return;
+    if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     const unsigned ep = S.ctl->epoch;
     for (;;) {
@@ -860,8 +860,7 @@ __global__ void k_bbegin(const BState *Sp) {
     const BDesc d = *S.desc;
     Ctl *ctl = S.ctl;
     if (threadIdx.x == 0) {
-        ctl->epoch += 1;
-        ctl->skip = 0;
+        ctl->epoch = d.epoch;
         ctl->op = d.op;
         ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
         ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
@@ -908,7 +907,7 @@ __global__ void k_bvalidate(const BState *Sp) {
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) {
             atomicOr(&S.ctl->err, ERR_BATCH_ID);
-            S.ctl->skip = 1;
+            S.ctl->skip = d.epoch + 1;
         }
     }
 }
@@ -916,7 +915,7 @@ __global__ void k_bvalidate(const BState *Sp) {
 // Overflow edges bucketed per graph (delete calls): count, offsets, fill.
 __global__ void k_bovf_count(const BState *Sp) {
     const BState &S = *Sp;
-    if (*(volatile int *)&S.ctl->skip) return;
+    if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     if (d.op != DRSF_DELETE) return;
     const long long no = (long long)min(S.ctl->ovf_count, S.ovf_cap);
@@ -946,7 +945,7 @@ __global__ void k_bovf_scan(const BState *Sp) {
 }
 __global__ void k_bovf_fill(const BState *Sp) {
     const BState &S = *Sp;
-    if (*(volatile int *)&S.ctl->skip) return;
+    if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     if (d.op != DRSF_DELETE) return;
     const long long no = (long long)min(S.ctl->ovf_count, S.ovf_cap);

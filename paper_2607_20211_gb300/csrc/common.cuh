@@ -42,8 +42,8 @@ typedef unsigned long long u64;
 // per-batch counts.  Statistic fields mirror drsf_batch_stats.
 struct Ctl {
     int err;
-    int skip;               // current batch rejected (ERR_BATCH_ID seen)
-    unsigned epoch;         // batch counter; epoch stamps compare against it
+    unsigned skip;          // epoch + 1 of the last rejected batch (ERR_BATCH_ID seen)
+    unsigned epoch;         // batch counter (the host's); epoch stamps compare against it
     int op;
     u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs / scan, Euler marks, detach
                             // (reset at each batch's start and before each static BFS)
@@ -88,6 +88,11 @@ struct Ctl {
     long long det_levels;   // top-down levels of the batch (0: not taken)
     long long det_entries;  // adjacency entries the top-down search read
 };
+
+// The current batch was rejected: no kernel after k_begin touches anything.
+__device__ __forceinline__ bool batch_skipped(const Ctl *ctl) {
+    return *(const volatile unsigned *)&ctl->skip == ctl->epoch + 1;
+}
 
 // The edge index.  An entry is one 16-byte record: with keys and positions in
 // arrays of their own a deleted edge touched three sectors of a table far

@@ -20,7 +20,7 @@ __device__ __forceinline__ long long etid() { return (long long)blockIdx.x * blo
 __device__ __forceinline__ long long etstride() { return (long long)gridDim.x * blockDim.x; }
 
 __global__ void k_et_marks(Ctl *ctl, EtArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     u64 *bar = &ctl->bar[5];
     const long long na = (long long)ctl->nact;
     // phase 0: clear child counters

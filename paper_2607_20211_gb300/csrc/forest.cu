@@ -84,14 +84,44 @@ __device__ __forceinline__ void load_ipt(const int *a, long long i0, long long c
 __device__ __forceinline__ long long gtid() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ long long gstride() { return (long long)gridDim.x * blockDim.x; }
 
-// Reset the per-batch counters, advance the epoch and record the batch (the
-// kernels after this one read the batch and its length from the control
-// block, so their launches do not depend on them).
-__global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
-    if (threadIdx.x != 0) return;
-    ctl->batch = batch;
-    ctl->epoch += 1;
-    ctl->skip = 0;
+// The graph that owns position i of an offsets array (the last one that starts
+// at or before it).
+__device__ __forceinline__ int owner_of(const long long *off, int G, long long i) {
+    int lo = 0, hi = G - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= i) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Start of a batch: every id is checked (an out-of-range id, or with `groups`
+// an edge that leaves its graph's vertices, rejects the whole batch), and one
+// thread resets the per-batch counters, sets the epoch and records the batch
+// (the kernels after this one read the batch and its length from the control
+// block, so their launches do not depend on them).  The rejection carries the
+// batch's epoch, so it needs no reset that the checks would race with, and no
+// launch of its own.
+__global__ void k_begin(Ctl *ctl, BeginArgs a) {
+    GS_LOOP(i, a.len) {
+        const int u = a.batch[2 * i], v = a.batch[2 * i + 1];
+        bool bad = u < 0 || u >= a.n || v < 0 || v >= a.n;
+        if (a.groups) {
+            const int g = owner_of(a.boff, a.groups, i);
+            const long long lo = a.voff[g], hi = a.voff[g + 1];
+            bad |= u < lo || u >= hi || v < lo || v >= hi;
+        }
+        if (bad) {
+            atomicOr(&ctl->err, ERR_BATCH_ID);
+            ctl->skip = a.epoch + 1;
+        }
+    }
+    if (gtid() != 0) return;
+    const int op = a.op;
+    const long long len = a.len;
+    ctl->batch = a.batch;
+    ctl->epoch = a.epoch;
     ctl->op = op;
     ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
     ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
@@ -129,7 +159,7 @@ __global__ void k_begin(Ctl *ctl, int op, long long len, const int *batch) {
 __global__ void __launch_bounds__(BLK) k_aff_collect(int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
                                                      unsigned *w, u64 *heavy, Ctl *ctl) {
     static_assert(IPA <= 32, "item masks are 32 bits");
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     if (*(volatile int *)&ctl->td) return;
     unsigned ep = ctl->epoch;
     const int lane = threadIdx.x & 31;
@@ -306,7 +336,7 @@ __global__ void __launch_bounds__(BLK, 4)
     k_detach(Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf, u64 ovf_cap, RowList rl,
              int *A, int *J1, unsigned *det_ep, unsigned *det_claim, const int *rold, long long budget_v,
              long long budget_e, int max_levels, int *oc, int *op) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     // Deep trees below the cuts make the search a long chain of levels
     // (one grid barrier each) where pointer doubling needs a logarithmic
     // number of steps: after a search that gave up at the level limit the
@@ -569,7 +599,7 @@ __device__ __forceinline__ void pt_count(PieceTable &t, unsigned *w, int p, bool
 }
 
 __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     if (*(volatile int *)&ctl->td) return;   // the top-down search found the pieces
     const unsigned ep = ctl->epoch;
     const long long nc = (long long)ctl->ncut;
@@ -752,7 +782,7 @@ __global__ void __launch_bounds__(BLK, 6)
            RowList rl, int mode, const int *rold, unsigned *w, u64 *heavy, Csr g, int *X, int *Y, const int *cuts) {
     int *const D = rl.D;
     unsigned *const roff = rl.roff;
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     if (mode == 1 && *(volatile int *)&ctl->td) return;   // the top-down search found the pieces
     long long cnt = use_list ? (long long)ctl->naff : cnt_static;
     if constexpr (sync_rounds != 0) {
@@ -1867,7 +1897,7 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
 // hooking, orientation and walks of a 100-edge batch took 68 us on R-MAT
 // scale 22.
 __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArgs h, OrientArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     __shared__ HotMin hm;
     const unsigned ep = ctl->epoch;
     if (gtid() == 0) {
@@ -1906,7 +1936,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
 // block per SM) would take them in several rounds.  For a 100K-edge batch the
 // launch costs 10 us more than it saves (R-MAT scale 22).
 __global__ void k_walk(Ctl *ctl, OrientArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     const unsigned ep = ctl->epoch;
     const long long ner = (long long)ctl->ner;
     int rev = 0;
@@ -2066,7 +2096,7 @@ __device__ __forceinline__ void reverse_marked(Ctl *ctl, const FinishArgs &a, lo
 // the other batches pass over all vertices.  With a.euler the marks are the
 // Euler tour's (a launch of its own) and k_reverse follows it.
 __global__ void __launch_bounds__(BLK, 5) k_finish(Ctl *ctl, FinishArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     const unsigned ep = ctl->epoch;
     if (ctl->ner == 0) return;   // no piece was merged
     const bool marks = a.euler || *(volatile int *)&ctl->nlong;
@@ -2084,7 +2114,7 @@ __global__ void __launch_bounds__(BLK, 5) k_finish(Ctl *ctl, FinishArgs a) {
     reverse_marked(ctl, a, na);
 }
 __global__ void k_reverse(Ctl *ctl, FinishArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     reverse_marked(ctl, a, (long long)ctl->nact);
 }
 
@@ -2135,8 +2165,8 @@ unsigned coop_blocks_replace(int nsm) {
     return (unsigned)nsm;   // one block per SM (shared memory)
 }
 
-cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s) {
-    k_begin<<<1, 32, 0, s>>>(ctl, op, len, batch);
+cudaError_t launch_begin(Ctl *ctl, BeginArgs a, cudaStream_t s) {
+    k_begin<<<gsz(a.len), BLK, 0, s>>>(ctl, a);
     return cudaGetLastError();
 }
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,

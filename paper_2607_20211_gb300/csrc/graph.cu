@@ -160,23 +160,10 @@ __global__ void k_fill(const u64 *dkey, const u64 *dslot, const int2 *place, lon
 
 // ------------------------------------------------------------ per batch
 
-// Id validation of the batch: an out-of-range id skips the whole batch.
-__global__ void k_validate_batch(int n, Ctl *ctl) {
-    const int *batch = ctl->batch;
-    const long long len = ctl->batch_len;
-    GS_LOOP(i, 2 * len) {
-        int x = batch[i];
-        if (x < 0 || x >= n) {
-            atomicOr(&ctl->err, ERR_BATCH_ID);
-            ctl->skip = 1;
-        }
-    }
-}
-
 // Insert, step 1 (batch normalisation): drop self-loops, repeated pairs and
 // edges already in G; claim an index slot for each new edge.
 __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     const int *batch = ctl->batch;
     const long long len = ctl->batch_len;
     // block-uniform loop: counters and the list append are aggregated per
@@ -223,7 +210,7 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
 template <bool SG>
 __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix, u64 *ovf, u64 ovf_cap,
                             const int *rep, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap, HookSlots hs) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     const unsigned ep = ctl->epoch;
     long long nb = (long long)ctl->nb;
     long long dead = 0;   // change of the slots that scans read and hold no entry
@@ -295,7 +282,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
 // vertex becomes a piece root.
 __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl, PieceSlots ps,
                             int *cutlist) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     const int *batch = ctl->batch;
     const long long len = ctl->batch_len;
     unsigned ep = ctl->epoch;
@@ -767,7 +754,7 @@ __device__ __forceinline__ bool light_hook(const LightArgs &a, int q, u64 *key) 
 
 template <bool SG>
 __global__ void __launch_bounds__(BLK, 4) k_scan(Ctl *ctl, RowList rl, LightArgs a) {
-    if (*(volatile int *)&ctl->skip) return;
+    if (batch_skipped(ctl)) return;
     if (a.listed || *(volatile int *)&ctl->td) {   // the row list is there
         scan_rows<SG>(rl, ctl, a.g, a.rep, a.pt, a.ck, a.ca, a.cb, a.cand_cap);
         scan_ovf<SG>(a.ovf, ctl, a.rep, a.pt, a.ck, a.ca, a.cb, a.cand_cap);
@@ -938,10 +925,6 @@ cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, const int2 *place, lo
 }
 // The batch kernels read the batch and its length from the control block;
 // `len` only sizes their grid (a captured launch sequence is keyed by it).
-cudaError_t launch_validate_batch(long long len, int n, Ctl *ctl, cudaStream_t s) {
-    k_validate_batch<<<gsz(2 * len), BLK, 0, s>>>(n, ctl);
-    return cudaGetLastError();
-}
 cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *nslot, cudaStream_t s) {
     k_ins_claim<<<gsz(len), BLK, 0, s>>>(ix, ctl, nkey, nslot);
     return cudaGetLastError();

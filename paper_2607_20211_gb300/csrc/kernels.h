@@ -36,7 +36,6 @@ cudaError_t launch_rows_init(const long long *off, const int *deg, int n, Row *r
 cudaError_t launch_fill(const u64 *dkey, const u64 *dslot, const int2 *place, long long m, Csr g, Index ix,
                         cudaStream_t s);
 // (the batch kernels read the batch from the control block; len sizes the grid)
-cudaError_t launch_validate_batch(long long len, int n, Ctl *ctl, cudaStream_t s);
 
 // Per-piece slots that a cut sets up: for the cut vertex and for its tree's
 // old root (k_relabel, k_scan).
@@ -100,7 +99,15 @@ cudaError_t launch_check_tree_edges(int n, const int *parent, Index ix, int *bad
 cudaError_t launch_check_cross(const int *pairs, long long m, const int *rep, int *bad, cudaStream_t s);
 
 // forest.cu ------------------------------------------------------------
-cudaError_t launch_begin(Ctl *ctl, int op, long long len, const int *batch, cudaStream_t s);
+struct BeginArgs {
+    int op, n;
+    long long len;
+    const int *batch;
+    unsigned epoch;
+    int groups;                    // graphs with a slice of the batch and a vertex range each; 0: none
+    const long long *voff, *boff;  // their offsets (groups + 1)
+};
+cudaError_t launch_begin(Ctl *ctl, BeginArgs a, cudaStream_t s);
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
                                unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s);
 // delete: detached vertices top-down from the cut vertices (falls back to
@@ -224,6 +231,7 @@ struct BDesc {               // per call
     const int *order;        // graphs in queue order, class by class
     int G;
     int op;
+    unsigned epoch;
 };
 struct BState {              // device pointers of one handle (per call)
     Ctl *ctl;

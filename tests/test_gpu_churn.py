@@ -41,7 +41,8 @@ def test_same_edges_leave_and_come_back(n, m, b, cycles):
         f.close()
 
 
-@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("batched", [None, drsf.DEFAULT_CLASSES, ((2 ** 31 - 1, 512, 0, 2),)],
+                         ids=["plain", "grouped", "persistent"])
 def test_window_neither_overflows_nor_rebuilds(batched):
     """A window of returning edges reuses the rows' freed slots: with
     append-only rows 24 cycles of a sixth of the edges would overflow every
@@ -60,7 +61,7 @@ def test_window_neither_overflows_nor_rebuilds(batched):
         for c in range(24):
             for op in (drsf.DELETE, drsf.INSERT):
                 if batched:
-                    f.apply_batched(op, dev, vo, bo)
+                    f.apply_batched(op, dev, vo, bo, batched)
                 else:
                     f.apply(op, dev)
         st = f.stats()
