@@ -181,11 +181,11 @@ DRSF_API drsf_status drsf_set_allocator(drsf_alloc_fn alloc, drsf_free_fn free_f
  * once (to size the CSR).  Without DRSF_VALIDATE, an F that is not a rooted
  * spanning forest of G gives undefined (but memory-safe) results.
  * The environment variable DRSF_JUMP, read here, selects the root search of
- * the handle's delete batches: unset, asynchronous pointer doubling (per-warp
- * slices stepping in place, no grid barrier between steps); "sync",
+ * the handle's delete batches: unset, a few parent hops and then asynchronous
+ * pointer doubling (in place, no grid barrier between steps); "sync",
  * synchronous doubling rounds; "halving", path-halving walks.  All three give
- * the same representatives.  Before it, a delete batch first looks for its
- * detached vertices top-down from the cut vertices over tree children
+ * the same representatives.  Before the default one, a delete batch first looks
+ * for its detached vertices top-down from the cut vertices over tree children
  * (touching only the detached vertices' rows) and falls back to the root
  * search only when that search exceeds its budget; DRSF_DETACH=0 skips the
  * top-down search, DRSF_DETACH_MAX (default 32768) is the longest delete

@@ -133,8 +133,8 @@ enum {
     PH_INS_PLACE,     // insert: CSR append + cross test
     PH_DEL_CLAIM,     // delete: normalisation, removal, tree-edge cut
     PH_AFF,           // delete: affected-vertex list (selectable root searches)
-    PH_JUMP,          // delete: top-down search, pointer jumping (representatives)
-    PH_SCAN,          // delete: cross-edge scan of detached rows + overflow
+    PH_JUMP,          // large delete: pieces (representatives)
+    PH_SCAN,          // delete: cross-edge scan (small deletes: and the top-down search)
     PH_HOOK,          // replacement edges: hook-and-compress, orientation, path walks
     PH_ORIENT,        // (part of the above)
     PH_ACTIVE,        // representative refresh, and the doubling marks and reversal of long paths
@@ -634,7 +634,7 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.grid_scan = scan_grid(nsm);
     h->dev.grid_pass = grid_vertex_pass(nsm);
     h->dev.coop_et = coop_blocks_et(nsm);
-    h->dev.coop_detach = coop_blocks_detach(nsm);
+    h->dev.coop_cross = coop_blocks_cross(nsm);
     // root search of a delete batch: barrier-free doubling over per-warp
     // slices by default; DRSF_JUMP=sync selects synchronous doubling rounds,
     // DRSF_JUMP=halving the in-place path-halving walks
@@ -699,45 +699,22 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         const PieceSlots ps{h->aff_ep, h->rold, h->comp, h->best0, h->heavy, h->wgt, (unsigned *)h->pdeg};
         CK(launch_del_claim(glen, h->ix, g, h->ovf, h->parent, h->rep, ctl, ps, h->cutlist, s));
         prof_end(h, PH_DEL_CLAIM, 1, s);
-        if (h->detach_now) {
-            // the detached vertices top-down from the cut vertices; over its
-            // budget it hands over to the pointer jumping below
-            prof_begin(h, PH_JUMP, s);
-            const long long n = h->n;
-            CK(launch_detach(h->dev, ctl, h->cutlist, h->parent, h->rep, g, h->ovf, h->ovf_cap, rows(h), h->A, h->J1,
-                             h->det_ep, h->det_claim, h->rold, std::max<long long>(1 << 16, n / 8),
-                             std::max<long long>(1 << 20, 4 * n), DETACH_LEVELS, h->act, h->xlist, s));
-            prof_end(h, PH_JUMP, 1, s);
-        }
-        if (h->jump_sync == 2) {
-            RelabelArgs ra{};
-            ra.n = h->n;
-            ra.rep = h->rep;
-            ra.par = h->parent;
-            ra.aff_ep = h->aff_ep;
-            ra.J = h->J0;
-            ra.X = h->act;
-            ra.Y = h->xlist;
-            ra.L = h->pold;
-            ra.D = h->D;
-            ra.rold = h->rold;
-            ra.w = h->wgt;
-            ra.wsum = (unsigned *)h->pdeg;
-            ra.heavy = h->heavy;
-            ra.left = h->minp;
-            ra.cuts = h->cutlist;
-            prof_begin(h, PH_JUMP, s);
-            CK(launch_relabel(h->dev, ctl, ra, s));
-            prof_end(h, PH_JUMP, 1, s);
-        } else {
-            prof_begin(h, PH_AFF, s);
-            CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, s));
-            prof_end(h, PH_AFF, 1, s);
-            prof_begin(h, PH_JUMP, s);
-            CK(launch_jump(h->dev, h->A, 1, 0, ctl, h->parent, h->J0, h->J1, h->rep, rows(h), 1, h->rold, h->wgt,
-                           h->heavy, g, h->jump_sync, h->act, h->xlist, h->cutlist, s));
-            prof_end(h, PH_JUMP, 1, s);
-        }
+        RelabelArgs ra{};
+        ra.n = h->n;
+        ra.rep = h->rep;
+        ra.par = h->parent;
+        ra.aff_ep = h->aff_ep;
+        ra.J = h->J0;
+        ra.X = h->act;
+        ra.Y = h->xlist;
+        ra.L = h->pold;
+        ra.D = h->D;
+        ra.rold = h->rold;
+        ra.w = h->wgt;
+        ra.wsum = (unsigned *)h->pdeg;
+        ra.heavy = h->heavy;
+        ra.left = h->minp;
+        ra.cuts = h->cutlist;
         LightArgs la{};
         la.n = h->n;
         la.g = g;
@@ -760,12 +737,51 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         la.cb = h->cb[0];
         la.cand_cap = h->cand_cap;
         la.listed = h->jump_sync != 2;
-        prof_begin(h, PH_SCAN, s);
-        CK(launch_scan(h->dev, ctl, rows(h), la, sg, s));
-        prof_end(h, PH_SCAN, 1, s);
+        if (h->detach_now) {
+            // the detached vertices top-down from the cut vertices; over its
+            // budget the search hands over to what large deletes do
+            const long long n = h->n;
+            DetachArgs da{};
+            da.cuts = h->cutlist;
+            da.par = h->parent;
+            da.rold = h->rold;
+            da.rep = h->rep;
+            da.g = g;
+            da.ovf = h->ovf;
+            da.ovf_cap = h->ovf_cap;
+            da.A = h->A;
+            da.J1 = h->J1;
+            da.det_ep = h->det_ep;
+            da.det_claim = h->det_claim;
+            da.budget_v = std::max<long long>(1 << 16, n / 8);
+            da.budget_e = std::max<long long>(1 << 20, 4 * n);
+            da.max_levels = DETACH_LEVELS;
+            da.oc = h->act;
+            da.op = h->xlist;
+            prof_begin(h, PH_SCAN, s);
+            CK(launch_cross(h->dev, ctl, da, ra, rows(h), la, sg, s));
+            prof_end(h, PH_SCAN, 1, s);
+        } else {
+            if (h->jump_sync == 2) {
+                prof_begin(h, PH_JUMP, s);
+                CK(launch_relabel(h->dev, ctl, ra, s));
+                prof_end(h, PH_JUMP, 1, s);
+            } else {
+                prof_begin(h, PH_AFF, s);
+                CK(launch_aff_collect(h->dev, h->n, h->rep, h->aff_ep, h->A, h->rold, h->wgt, h->heavy, ctl, s));
+                prof_end(h, PH_AFF, 1, s);
+                prof_begin(h, PH_JUMP, s);
+                CK(launch_jump(h->dev, h->A, 1, 0, ctl, h->parent, h->J0, h->J1, h->rep, rows(h), 1, h->rold, h->wgt,
+                               h->heavy, g, h->jump_sync, h->act, h->xlist, h->cutlist, s));
+                prof_end(h, PH_JUMP, 1, s);
+            }
+            prof_begin(h, PH_SCAN, s);
+            CK(launch_scan(h->dev, ctl, rows(h), la, sg, s));
+            prof_end(h, PH_SCAN, 1, s);
+        }
     }
     OrientArgs oa{};
-    oa.er = h->er;
+    oa.er = oa.er_out = h->er;
     oa.rep = h->rep;
     oa.comp = h->comp;
     oa.minp = h->minp;
@@ -896,7 +912,7 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     h->last_sg = sg ? 1 : 0;
     // the top-down delete for small batches: its cost follows the detached
     // vertices' rows and its levels, the pointer jumping's the cut trees
-    h->detach_now = op == DRSF_DELETE && h->detach && len <= h->detach_max;
+    h->detach_now = op == DRSF_DELETE && h->detach && len <= h->detach_max && h->jump_sync == 2;
     if (h->prof_on) {
         h->prof_batches++;
         h->prof_op = op;

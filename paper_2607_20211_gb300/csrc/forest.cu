@@ -81,6 +81,8 @@ __device__ __forceinline__ void load_ipt(const int *a, long long i0, long long c
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (long long)(n); \
          i += (long long)gridDim.x * blockDim.x)
 
+#include "scan.cuh"
+
 __device__ __forceinline__ long long gtid() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ long long gstride() { return (long long)gridDim.x * blockDim.x; }
 
@@ -332,11 +334,15 @@ __device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long v
 // go to J1 and are committed only when the search ends within its budget
 // (vertices, entries, levels); otherwise nothing is published and the
 // pointer-jumping path runs.
-__global__ void __launch_bounds__(BLK, 4)
-    k_detach(Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf, u64 ovf_cap, RowList rl,
-             int *A, int *J1, unsigned *det_ep, unsigned *det_claim, const int *rold, long long budget_v,
-             long long budget_e, int max_levels, int *oc, int *op) {
-    if (batch_skipped(ctl)) return;
+// Returns 1 when the pieces were found, 0 when they were not, -1 when a grid
+// barrier gave up.
+__device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl) {
+    const int *const cuts = a.cuts, *const par = a.par, *const rold = a.rold;
+    int *const rep = a.rep, *const A = a.A, *const J1 = a.J1, *const oc = a.oc, *const op = a.op;
+    unsigned *const det_ep = a.det_ep, *const det_claim = a.det_claim;
+    const Csr &g = a.g;
+    const u64 *const ovf = a.ovf;
+    const int max_levels = a.max_levels;
     // Deep trees below the cuts make the search a long chain of levels
     // (one grid barrier each) where pointer doubling needs a logarithmic
     // number of steps: after a search that gave up at the level limit the
@@ -346,7 +352,7 @@ __global__ void __launch_bounds__(BLK, 4)
     // all blocks take the same branch.
     if (*(volatile unsigned *)&ctl->depth_hint > (unsigned)max_levels) {
         if (gtid() == 0) ctl->det_skip = 1;
-        return;
+        return 0;
     }
     const unsigned ep = ctl->epoch;
     const long long nc = (long long)ctl->ncut;
@@ -374,7 +380,7 @@ __global__ void __launch_bounds__(BLK, 4)
     // parent): listed once, read by every level (few: edges land there
     // only when a row is full)
     {
-        const long long no = (long long)min((u64)ctl->ovf_count, ovf_cap);
+        const long long no = (long long)min((u64)ctl->ovf_count, a.ovf_cap);
         for (long long b0 = gtid() & ~31ll; b0 < no; b0 += gstride()) {
             const long long i = b0 + lane;
             int cw = -1, pv = -1;
@@ -404,7 +410,7 @@ __global__ void __launch_bounds__(BLK, 4)
     int lvl = 0;
     bool ok = true;
     for (;; ++lvl) {
-        if (!grid_barrier(ctl, bar)) return;
+        if (!grid_barrier(ctl, bar)) return -1;
         // the level found in the last round (slot lvl % 3) is final
         const int sl = lvl % 3, sn = (lvl + 1) % 3;
         const long long dv = (long long)*(volatile u64 *)&ctl->dv[sl];
@@ -415,7 +421,7 @@ __global__ void __launch_bounds__(BLK, 4)
         const u64 pn = pb + dp;
         const unsigned e_hi = (unsigned)pn, r_hi = (unsigned)(pn >> 32);
         if (dv == 0) break;   // the last level found nothing
-        if (lvl >= max_levels || vn > budget_v || (long long)e_hi > budget_e) {
+        if (lvl >= max_levels || vn > a.budget_v || (long long)e_hi > a.budget_e) {
             ok = false;
             break;
         }
@@ -483,7 +489,7 @@ __global__ void __launch_bounds__(BLK, 4)
                     child = true;
                     w = cw;
                     p = LD(J1[pv]);
-                    ro = rep[w];   // rep still holds the old roots
+                    ro = LD(rep[w]);   // rep still holds the old roots (read again, new, by the scan)
                 }
             }
             if (child) {
@@ -506,7 +512,7 @@ __global__ void __launch_bounds__(BLK, 4)
             ctl->det_levels = -lvl;
             if (lvl >= max_levels) ctl->depth_hint = (unsigned)max_levels + DETACH_BACKOFF;
         }
-        return;
+        return 0;
     }
     // commit the representatives of the detached vertices
     for (long long i = gtid(); i < vb; i += gstride()) {
@@ -522,6 +528,7 @@ __global__ void __launch_bounds__(BLK, 4)
         ctl->depth_hint = (unsigned)lvl;
         ctl->td = 1;
     }
+    return 1;
 }
 
 // heavy[r] = the piece left out of the scan of the cut tree with old root r
@@ -598,12 +605,10 @@ __device__ __forceinline__ void pt_count(PieceTable &t, unsigned *w, int p, bool
     if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) piece_count(t.k, t.c, w, p, (unsigned)__popc(grp));
 }
 
-__global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
-    if (batch_skipped(ctl)) return;
-    if (*(volatile int *)&ctl->td) return;   // the top-down search found the pieces
+__device__ bool relabel(Ctl *ctl, const RelabelArgs &a) {
     const unsigned ep = ctl->epoch;
     const long long nc = (long long)ctl->ncut;
-    if (nc == 0) return;   // no tree was cut
+    if (nc == 0) return true;   // no tree was cut
     u64 *bar = &ctl->bar[0];
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -676,7 +681,7 @@ __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
     }
     if (lane == 0 && tc) piece_count(pt.k, pt.c, a.w, tr, tc);
     block_add((long long *)&ctl->naff, naff);
-    if (!grid_barrier(ctl, bar)) return;
+    if (!grid_barrier(ctl, bar)) return false;
     // (each warp reads lists that it wrote itself)
     int *in = X, *out = Y;
     int it = 0;
@@ -739,7 +744,7 @@ __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
         }
     }
     pt_flush(pt, a.w);
-    if (!grid_barrier(ctl, bar)) return;
+    if (!grid_barrier(ctl, bar)) return false;
     // per cut tree: the detached pieces' vertices and the heaviest of them
     for (long long i = gtid(); i < nc; i += gstride()) {
         const int c = a.cuts[i], r = a.rold[c];
@@ -749,7 +754,7 @@ __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
         if (lane == __ffs(grp) - 1) atomicAdd(&a.wsum[r], sum);
         if (wc >= HEAVY_SWAP_MIN) atomicMax(&a.heavy[r], ((u64)wc << 32) | (unsigned)c);
     }
-    if (!grid_barrier(ctl, bar)) return;
+    if (!grid_barrier(ctl, bar)) return false;
     bool swap = false;
     for (long long i = gtid(); i < nc; i += gstride()) {
         const int r = a.rold[a.cuts[i]];
@@ -761,6 +766,34 @@ __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
         swap |= sw;
     }
     if (__syncthreads_or(swap) && threadIdx.x == 0) atomicOr(&ctl->flag[0], 1);
+    return true;
+}
+
+// Large deletes: pieces and scan as launches of their own (the first fits five
+// blocks on an SM, the second four).
+__global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
+    if (batch_skipped(ctl)) return;
+    relabel(ctl, a);
+}
+template <bool SG>
+__global__ void __launch_bounds__(BLK, 4) k_scan(Ctl *ctl, RowList rl, LightArgs a) {
+    if (batch_skipped(ctl)) return;
+    if (a.listed) scan_listed<SG>(ctl, rl, a);
+    else scan_light<SG>(ctl, a);
+}
+// Small deletes: the top-down search and the scan of the rows it listed, or,
+// where it gives up, what large deletes do, in one launch (as four, the ones
+// that found nothing to do took 8 us of every batch).
+template <bool SG>
+__global__ void __launch_bounds__(BLK, 4)
+    k_cross(Ctl *ctl, DetachArgs d, RelabelArgs r, RowList rl, LightArgs a) {
+    if (batch_skipped(ctl)) return;
+    const int found = detach_top_down(ctl, d, rl);
+    if (found < 0) return;
+    if (!found && !relabel(ctl, r)) return;
+    if (!grid_barrier(ctl, &ctl->bar[6])) return;
+    if (found) scan_listed<SG>(ctl, rl, a);
+    else scan_light<SG>(ctl, a);
 }
 
 // Representatives (Algorithm 1, parallel pointer jumping) of the listed
@@ -1090,15 +1123,38 @@ __device__ __forceinline__ int hm_slot(HotMin &t, int idx, bool ins) {
     }
     return -1;
 }
+// The lanes of the first two indices seen in the warp combine their keys (one
+// piece, such as the giant one, can be an end of most candidates); the other
+// lanes go to global memory one by one, unless their key is no new minimum.
+// (A reduction over each group of equal lanes runs the groups one after
+// another: up to 32 times two reductions where most indices differ.)
 __device__ __forceinline__ void hm_min(HotMin &t, u64 *arr, int idx, u64 k, bool pred) {
     unsigned m = __ballot_sync(__activemask(), pred);
     if (!pred) return;
-    unsigned grp = __match_any_sync(m, idx);
-    u64 kmin = group_min_u64(grp, k);
-    if ((int)(threadIdx.x & 31) != __ffs(grp) - 1) return;
-    int sl = __popc(grp) > 1 ? hm_slot(t, idx, true) : -1;
-    if (sl >= 0) atomicMin(&t.v[sl], kmin);
-    else atomicMin(&arr[idx], kmin);
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int round = 0; round < 2; ++round) {
+        const int l0 = __ffs(m) - 1, i0 = __shfl_sync(m, idx, l0);
+        const unsigned g = __ballot_sync(m, idx == i0);
+        if (__popc(g) > 1) {
+            if (idx == i0) {
+                const u64 kmin = group_min_u64(g, k);
+                if (lane == l0) {
+                    const int sl = hm_slot(t, idx, true);
+                    if (sl >= 0) atomicMin(&t.v[sl], kmin);
+                    else atomicMin(&arr[idx], kmin);
+                }
+                return;
+            }
+            m &= ~g;
+            if (!m) return;
+        } else if (round == 0) {
+            if (lane == l0) break;
+            m &= ~g;
+            if (!m) return;
+        }
+    }
+    if (k < __ldcg(&arr[idx])) atomicMin(&arr[idx], k);
 }
 // bestn[idx] = EMPTY_KEY, once per block for the table's indices
 __device__ __forceinline__ void hm_reset(HotMin &t, u64 *arr, int idx, bool pred) {
@@ -1679,73 +1735,91 @@ __device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
     }
     block_add(&ctl->reversed, rev);
 }
-// Replacement edges, orientation and walks of a batch with at most SMALL_CAND
-// candidates, by one block, everything but the walks in shared memory: the
-// pieces get dense ids through a hash table, the hook-and-compress rounds and
-// the orientation run on those, and only the results go to global memory.
-// On the grid the same batch is a chain of some twenty phases with a grid
-// barrier, two or three dependent global loads and up to a launch between
-// them, whatever its size.
+// Replacement edges and their orientation for a batch with at most SMALL_CAND
+// candidates, by one block in shared memory: the pieces get dense ids through
+// a hash table, the hook-and-compress rounds and the orientation run on
+// those.  On the grid the same batch is a chain of some twenty phases with a
+// grid barrier, two or three dependent global loads and up to a launch between
+// them, whatever its size.  The results (attach points, new roots, walks) are
+// scattered stores and pointer chains: up to SMALL_OUT edges the same block
+// writes them, more go to the whole grid after one barrier (35 of 90 us for
+// 3,300 edges on one SM).
 // The `pre` replacement edges that k_scan chose join the candidates again (the
 // minimum spanning forest is the same), all with their own pieces as ends.
+// Pieces: at most two per candidate.  A piece's minimum key is taken in two
+// halves, which shared memory has native atomics for; what is needed one after
+// the other shares memory.
+#define TAIL_P (2 * SMALL_CAND)
+#define TAIL_H (3 * SMALL_CAND)   // hash slots (two thirds full at most)
+#define SMALL_OUT 256
 struct SmallTail {
-    u64 key[SMALL_CAND], best[2 * SMALL_CAND];
-    int hk[4 * SMALL_CAND];                       // hash table: piece, -1 free
-    int pid[2 * SMALL_CAND], comp[2 * SMALL_CAND], minp[2 * SMALL_CAND];
-    unsigned short hl[4 * SMALL_CAND];            // its dense id
+    u64 key[SMALL_CAND];
+    union {
+        unsigned short hl[TAIL_H];   // a hash slot's dense id
+        struct {
+            unsigned bhi[TAIL_P], blo[TAIL_P];   // a piece's minimum key
+        };
+        struct {
+            int minp[TAIL_P];
+            unsigned char vis[TAIL_P];
+        };
+    };
+    int hk[TAIL_H];                       // hash table: piece, -1 free
+    int pid[TAIL_P];
+    unsigned short comp[TAIL_P];
     unsigned short a[SMALL_CAND], b[SMALL_CAND], er[SMALL_CAND];
-    unsigned char vis[2 * SMALL_CAND];
-    int np, ner;
+    int ner;
 };
-static_assert(sizeof(SmallTail) <= ORIENT_SMEM_BYTES, "one block's shared memory");
+#define REPLACE_SMEM_BYTES ((int)(sizeof(SmallTail) > ORIENT_SMEM_BYTES ? sizeof(SmallTail) : ORIENT_SMEM_BYTES))
+static_assert(sizeof(SmallTail) <= 225 * 1024, "one block's shared memory");
+static_assert(TAIL_H % ORIENT_THREADS == 0, "hash slots per thread");
 
-// slot of piece p in the hash table (entered when absent; at most half full)
+// slot of piece p in the hash table (entered when absent)
 __device__ __forceinline__ int tail_slot(SmallTail &t, int p) {
-    unsigned h = ((unsigned)p * 0x9E3779B1u) % (4 * SMALL_CAND);
+    unsigned h = ((unsigned)p * 0x9E3779B1u) % TAIL_H;
     for (;;) {
         int k = *(volatile int *)&t.hk[h];
-        if (k == -1) {
-            k = atomicCAS(&t.hk[h], -1, p);
-            if (k == -1) {
-                const int l = atomicAdd(&t.np, 1);
-                t.pid[l] = p;
-                t.hl[h] = (unsigned short)l;
-                t.comp[l] = l;
-                t.best[l] = EMPTY_KEY;
-                t.minp[l] = INT_MAX;
-                t.vis[l] = 0;
-                return (int)h;
-            }
-        }
-        if (k == p) return (int)h;
-        h = (h + 1) % (4 * SMALL_CAND);
+        if (k == -1) k = atomicCAS(&t.hk[h], -1, p);
+        if (k == -1 || k == p) return (int)h;
+        h = h + 1 == TAIL_H ? 0 : h + 1;
     }
 }
 // root of dense piece x (hooking only ever links roots, so chains are short)
 __device__ __forceinline__ int tail_root(const SmallTail &t, int x) {
-    for (int it = 0; it < 2 * SMALL_CAND; ++it) {
-        const int p = *(volatile const int *)&t.comp[x];
+    for (int it = 0; it < TAIL_P; ++it) {
+        const int p = *(volatile const unsigned short *)&t.comp[x];
         if (p == x) break;
         x = p;
     }
     return x;
 }
-// best[x] = min(best[x], k): lanes with one x combine first (one piece, such
-// as the giant one, can be an endpoint of most candidates)
-__device__ __forceinline__ void tail_min(SmallTail &t, int x, u64 k, bool on) {
-    const unsigned m = __ballot_sync(0xffffffffu, on);
-    if (!on) return;
-    const unsigned grp = __match_any_sync(m, x);
-    const u64 kmin = group_min_u64(grp, k);
-    if ((int)(threadIdx.x & 31) == __ffs(grp) - 1 && kmin < *(volatile u64 *)&t.best[x]) atomicMin(&t.best[x], kmin);
+
+// Results of one oriented edge: child piece p of edge k takes its attach point
+// and new root (as in orient_one) and its path is reversed.  Returns the
+// vertices reversed.
+__device__ __forceinline__ int tail_out(Ctl *ctl, const OrientArgs &oa, long long e, u64 k, int p, int root,
+                                        unsigned ep) {
+    const int x0 = (int)klo(k), x1 = (int)khi(k);
+    const bool low = oa.rep[x0] == p;
+    const int x = low ? x0 : x1, y = low ? x1 : x0;
+    oa.chx[e] = x;
+    oa.chy[e] = y;
+    oa.att_x[p] = x;
+    oa.att_ep[p] = ep;
+    oa.newrep[p] = root;
+    oa.rep_ep[p] = ep;
+    if (oa.aff_ep[p] == ep) ctl->need_root = 1;
+    return oa.walk ? walk_path(ctl, oa.parent, x, y, oa.long_ep, p, ep) : 0;
 }
 
 __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa, int c0, int pre, unsigned ep) {
     extern __shared__ __align__(16) int s_rank[];
     SmallTail &t = *reinterpret_cast<SmallTail *>(s_rank);
     constexpr int IT = SMALL_CAND / ORIENT_THREADS;   // candidates per thread
-    for (int i = threadIdx.x; i < 4 * SMALL_CAND; i += ORIENT_THREADS) t.hk[i] = -1;
-    if (threadIdx.x == 0) t.np = t.ner = 0;
+    const int lane = threadIdx.x & 31;
+    const int all = c0 + pre;
+    for (int i = threadIdx.x; i < TAIL_H; i += ORIENT_THREADS) t.hk[i] = -1;
+    if (threadIdx.x == 0) t.ner = 0;
     __syncthreads();
     u64 key[IT];
     int ra[IT], rb[IT];
@@ -1753,7 +1827,7 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
 #pragma unroll
     for (int q = 0; q < IT; ++q) {
         const int i = q * ORIENT_THREADS + threadIdx.x;
-        alive[q] = i < c0 + pre;
+        alive[q] = i < all;
         key[q] = 0;
         ra[q] = rb[q] = 0;
         if (!alive[q]) continue;
@@ -1774,6 +1848,27 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
         }
     }
     __syncthreads();
+    // dense ids in slot order
+    int np;
+    {
+        constexpr int HT = TAIL_H / ORIENT_THREADS;
+        const int s0 = threadIdx.x * HT;
+        int cnt = 0;
+#pragma unroll
+        for (int q = 0; q < HT; ++q) cnt += t.hk[s0 + q] != -1;
+        long long tot;
+        int l = (int)block_excl_scan_ll(cnt, &tot);
+        np = (int)tot;
+#pragma unroll
+        for (int q = 0; q < HT; ++q) {
+            if (t.hk[s0 + q] == -1) continue;
+            t.hl[s0 + q] = (unsigned short)l;
+            t.pid[l] = t.hk[s0 + q];
+            t.comp[l] = (unsigned short)l;
+            ++l;
+        }
+    }
+    __syncthreads();
 #pragma unroll
     for (int q = 0; q < IT; ++q) {
         const int i = q * ORIENT_THREADS + threadIdx.x;
@@ -1785,47 +1880,71 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
             t.b[i] = (unsigned short)rb[q];
         }
     }
+    __syncthreads();
+    for (int l = threadIdx.x; l < np; l += ORIENT_THREADS) t.bhi[l] = t.blo[l] = 0xFFFFFFFFu;
+    __syncthreads();
     // hook and compress (as in hook_rounds)
     int r = 0;
     for (; r < MAX_ROUNDS; ++r) {
         bool any = false;
 #pragma unroll
         for (int q = 0; q < IT; ++q) {
-            if (alive[q]) {
-                ra[q] = tail_root(t, ra[q]);
-                rb[q] = tail_root(t, rb[q]);
-                alive[q] = ra[q] != rb[q];
-            }
-            any |= alive[q];
-            tail_min(t, ra[q], key[q], alive[q]);
-            tail_min(t, rb[q], key[q], alive[q]);
+            if (!alive[q]) continue;
+            ra[q] = tail_root(t, ra[q]);
+            rb[q] = tail_root(t, rb[q]);
+            alive[q] = ra[q] != rb[q];
+            if (!alive[q]) continue;
+            any = true;
+            const unsigned hi = (unsigned)(key[q] >> 32);
+            if (hi < *(volatile unsigned *)&t.bhi[ra[q]]) atomicMin(&t.bhi[ra[q]], hi);
+            if (hi < *(volatile unsigned *)&t.bhi[rb[q]]) atomicMin(&t.bhi[rb[q]], hi);
         }
         if (!__syncthreads_or(any)) break;
-        bool used[IT];
 #pragma unroll
         for (int q = 0; q < IT; ++q) {
-            used[q] = alive[q];
             if (!alive[q]) continue;
-            const int a = ra[q], b = rb[q];
-            const bool ba = t.best[a] == key[q], bb = t.best[b] == key[q];
-            if (ba && bb) t.comp[t.pid[a] > t.pid[b] ? a : b] = t.pid[a] > t.pid[b] ? b : a;
-            else if (ba) t.comp[a] = b;
-            else if (bb) t.comp[b] = a;
-            if (ba || bb) {
-                alive[q] = false;
-                t.er[atomicAdd(&t.ner, 1)] = (unsigned short)(q * ORIENT_THREADS + threadIdx.x);
+            const unsigned hi = (unsigned)(key[q] >> 32), lo = (unsigned)key[q];
+            if (t.bhi[ra[q]] == hi) atomicMin(&t.blo[ra[q]], lo);
+            if (t.bhi[rb[q]] == hi) atomicMin(&t.blo[rb[q]], lo);
+        }
+        __syncthreads();
+        unsigned used = 0;
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            bool hook = false;
+            if (alive[q]) {
+                used |= 1u << q;
+                const int a = ra[q], b = rb[q];
+                const unsigned hi = (unsigned)(key[q] >> 32), lo = (unsigned)key[q];
+                const bool ba = t.bhi[a] == hi && t.blo[a] == lo, bb = t.bhi[b] == hi && t.blo[b] == lo;
+                if (ba && bb) t.comp[a > b ? a : b] = (unsigned short)(a > b ? b : a);
+                else if (ba) t.comp[a] = (unsigned short)b;
+                else if (bb) t.comp[b] = (unsigned short)a;
+                hook = ba || bb;
+                alive[q] = !hook;
             }
+            const unsigned m = __ballot_sync(0xffffffffu, hook);
+            if (!m) continue;
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&t.ner, __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (hook) t.er[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(q * ORIENT_THREADS + threadIdx.x);
         }
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < IT; ++q)
-            if (used[q]) t.best[ra[q]] = t.best[rb[q]] = EMPTY_KEY;
+            if (used >> q & 1u) t.bhi[ra[q]] = t.bhi[rb[q]] = t.blo[ra[q]] = t.blo[rb[q]] = 0xFFFFFFFFu;
         __syncthreads();
     }
     __syncthreads();
     if (r >= MAX_ROUNDS && threadIdx.x == 0) atomicOr(&ctl->err, ERR_ROUNDS);
     // super-roots: the smallest piece of every super-tree
-    const int np = t.np, ner = t.ner;
+    const int ner = t.ner;
+    for (int l = threadIdx.x; l < np; l += ORIENT_THREADS) {
+        t.minp[l] = INT_MAX;
+        t.vis[l] = 0;
+    }
+    __syncthreads();
     for (int l = threadIdx.x; l < np; l += ORIENT_THREADS) {
         const int root = tail_root(t, l), p = t.pid[l];
         if (p < *(volatile int *)&t.minp[root]) atomicMin(&t.minp[root], p);
@@ -1861,24 +1980,20 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
         }
         if (!__syncthreads_or(more)) break;
     }
-    // results: attach points and new roots (as in orient_one), and the walks
     int rev = 0;
 #pragma unroll
     for (int q = 0; q < IT; ++q) {
         if (child[q] < 0) continue;
         const int e = q * ORIENT_THREADS + threadIdx.x;
         const u64 k = t.key[t.er[e]];
-        const int p = t.pid[child[q]], x0 = (int)klo(k), x1 = (int)khi(k);
-        const bool low = oa.rep[x0] == p;
-        const int x = low ? x0 : x1, y = low ? x1 : x0;
-        oa.chx[e] = x;
-        oa.chy[e] = y;
-        oa.att_x[p] = x;
-        oa.att_ep[p] = ep;
-        oa.newrep[p] = t.minp[tail_root(t, child[q])];
-        oa.rep_ep[p] = ep;
-        if (oa.aff_ep[p] == ep) ctl->need_root = 1;
-        if (oa.walk) rev += walk_path(ctl, oa.parent, x, y, oa.long_ep, p, ep);
+        const int p = t.pid[child[q]], root = t.minp[tail_root(t, child[q])];
+        if (all <= SMALL_OUT) {
+            rev += tail_out(ctl, oa, e, k, p, root, ep);
+        } else {
+            oa.er_out[e] = k;
+            oa.ep[e] = p;
+            oa.eid[e] = root;
+        }
     }
     block_add(&ctl->reversed, rev);
     if (threadIdx.x == 0) {
@@ -1893,7 +2008,8 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
 // replacement edges oriented and their paths walked.  Up to SMALL_CAND
 // candidates go to one block (replace_small); the other blocks then only pull
 // the forest into L2 for its walks (and the representatives for the refresh
-// that follows an insert).  As launches of their own the pair compaction,
+// that follows an insert) and take part in the results.  As launches of their
+// own the pair compaction,
 // hooking, orientation and walks of a 100-edge batch took 68 us on R-MAT
 // scale 22.
 __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArgs h, OrientArgs a) {
@@ -1919,6 +2035,17 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
             l2_prefetch(a.parent, 4 * a.n, t, nt);
             if (ctl->op == DRSF_INSERT) l2_prefetch(a.rep, 4 * a.n, t, nt);
         }
+        if (c0 + pre <= SMALL_OUT) return;
+        if (!grid_barrier(ctl, &ctl->bar[1])) return;
+        const long long ner = (long long)*(volatile u64 *)&ctl->ner;
+        int rev = 0;
+        // (one warp of every block after another: few edges reach many SMs)
+        for (long long w = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w * 32 < ner;
+             w += (long long)gridDim.x * (blockDim.x >> 5)) {
+            const long long e = w * 32 + (threadIdx.x & 31);
+            if (e < ner) rev += tail_out(ctl, a, e, LD(a.er_out[e]), LD(a.ep[e]), LD(a.eid[e]), ep);
+        }
+        block_add(&ctl->reversed, rev);
         return;
     }
     hm_init(hm);
@@ -2161,7 +2288,7 @@ unsigned coop_blocks_jump(int nsm) {
     return a < b ? a : b;
 }
 unsigned coop_blocks_replace(int nsm) {
-    cudaFuncSetAttribute((const void *)k_replace, cudaFuncAttributeMaxDynamicSharedMemorySize, ORIENT_SMEM_BYTES);
+    cudaFuncSetAttribute((const void *)k_replace, cudaFuncAttributeMaxDynamicSharedMemorySize, REPLACE_SMEM_BYTES);
     return (unsigned)nsm;   // one block per SM (shared memory)
 }
 
@@ -2174,17 +2301,32 @@ cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsign
     k_aff_collect<<<d.grid_pass, BLK, 0, s>>>(n, rep, aff_ep, A, rold, w, heavy, ctl);
     return cudaGetLastError();
 }
-cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf,
-                          u64 ovf_cap, RowList rl, int *A, int *J1, unsigned *det_ep, unsigned *det_claim,
-                          const int *rold, long long budget_v, long long budget_e, int max_levels, int *oc, int *op,
-                          cudaStream_t s) {
-    void *args[] = {(void *)&ctl,     (void *)&cuts,     (void *)&par,      (void *)&rep,        (void *)&g,
-                    (void *)&ovf,     (void *)&ovf_cap,  (void *)&rl,       (void *)&A,          (void *)&J1,
-                    (void *)&det_ep,  (void *)&det_claim, (void *)&rold,    (void *)&budget_v,   (void *)&budget_e,
-                    (void *)&max_levels, (void *)&oc,    (void *)&op};
-    return cudaLaunchCooperativeKernel((const void *)k_detach, d.coop_detach, BLK, args, 0, s);
+cudaError_t launch_cross(const Dev &d, Ctl *ctl, DetachArgs da, RelabelArgs ra, RowList rl, LightArgs la, bool sg,
+                         cudaStream_t s) {
+    void *args[] = {(void *)&ctl, (void *)&da, (void *)&ra, (void *)&rl, (void *)&la};
+    return cudaLaunchCooperativeKernel(sg ? (const void *)k_cross<true> : (const void *)k_cross<false>, d.coop_cross,
+                                       BLK, args, 0, s);
 }
-unsigned coop_blocks_detach(int nsm) { return coop_blocks((const void *)k_detach, nsm, 4); }
+unsigned coop_blocks_cross(int nsm) {
+    const unsigned a = coop_blocks((const void *)k_cross<true>, nsm, 4), b = coop_blocks((const void *)k_cross<false>, nsm, 4);
+    return a < b ? a : b;
+}
+cudaError_t launch_scan(const Dev &d, Ctl *ctl, RowList rl, LightArgs a, bool sg, cudaStream_t s) {
+    void *args[] = {(void *)&ctl, (void *)&rl, (void *)&a};
+    return cudaLaunchCooperativeKernel(sg ? (const void *)k_scan<true> : (const void *)k_scan<false>, d.grid_scan, BLK,
+                                       args, 0, s);
+}
+// The blocks that are resident at once (grid barriers; the row list's tiles
+// are dealt out in equal shares).
+unsigned scan_grid(int nsm) {
+    int per = 8;
+    for (const void *fn : {(const void *)k_scan<true>, (const void *)k_scan<false>}) {
+        int o = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, BLK, 0) != cudaSuccess || o < 1) o = 1;
+        if (o < per) per = o;
+    }
+    return (unsigned)(per * nsm);
+}
 cudaError_t launch_relabel(const Dev &d, Ctl *ctl, RelabelArgs a, cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&a};
     return cudaLaunchCooperativeKernel((const void *)k_relabel, d.coop_relabel, BLK, args, 0, s);
@@ -2202,7 +2344,7 @@ cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_
 cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&h, (void *)&a};
     return cudaLaunchCooperativeKernel((const void *)k_replace, d.coop_replace, ORIENT_THREADS, args,
-                                       ORIENT_SMEM_BYTES, s);
+                                       REPLACE_SMEM_BYTES, s);
 }
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
     k_walk<<<d.grid, BLK, 0, s>>>(ctl, a);

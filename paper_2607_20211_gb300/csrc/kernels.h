@@ -8,7 +8,7 @@
 #define BLK 256
 // batches with at most this many candidates are replaced, oriented and walked
 // by one block in shared memory (what fits beside the hash table)
-#define SMALL_CAND 2048
+#define SMALL_CAND 4096
 
 struct Dev {
     int nsm;
@@ -19,7 +19,7 @@ struct Dev {
     unsigned coop_finish;
     unsigned coop_bfs;
     unsigned coop_et;
-    unsigned coop_detach;
+    unsigned coop_cross;
     unsigned grid_scan;   // row scan: the co-resident block count
     unsigned grid_pass;   // affected list: co-resident blocks
 };
@@ -116,11 +116,18 @@ cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsign
 // search takes 2-7 levels; on deep trees each level costs about as much as
 // a whole pointer-jumping round)
 #define DETACH_LEVELS 16
-cudaError_t launch_detach(const Dev &d, Ctl *ctl, const int *cuts, const int *par, int *rep, Csr g, const u64 *ovf,
-                          u64 ovf_cap, RowList rl, int *A, int *J1, unsigned *det_ep, unsigned *det_claim,
-                          const int *rold, long long budget_v, long long budget_e, int max_levels, int *oc, int *op,
-                          cudaStream_t s);
-unsigned coop_blocks_detach(int nsm);
+struct DetachArgs {
+    const int *cuts, *par, *rold;
+    int *rep;
+    Csr g;
+    const u64 *ovf;
+    u64 ovf_cap;
+    int *A, *J1;                    // detached vertices; their new representatives until the search ends
+    unsigned *det_ep, *det_claim;
+    long long budget_v, budget_e;
+    int max_levels;
+    int *oc, *op;                   // tree edges held outside the rows
+};
 struct RelabelArgs {
     int n;
     int *rep;
@@ -143,6 +150,9 @@ static inline long long relabel_room(long long n, unsigned blocks) {
     return (nch < (long long)blocks ? nch : (long long)blocks) * per * ch;
 }
 cudaError_t launch_relabel(const Dev &d, Ctl *ctl, RelabelArgs a, cudaStream_t s);
+cudaError_t launch_cross(const Dev &d, Ctl *ctl, DetachArgs da, RelabelArgs ra, RowList rl, LightArgs la, bool sg,
+                         cudaStream_t s);
+unsigned coop_blocks_cross(int nsm);
 unsigned coop_blocks_relabel(int nsm);
 cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_static, Ctl *ctl, const int *par,
                         int *J, int *J1, int *rep, RowList rl, int mode, const int *rold, unsigned *w, u64 *heavy,
@@ -160,6 +170,7 @@ struct HookArgs {
 };
 struct OrientArgs {
     const u64 *er;
+    u64 *er_out;         // (the same array: replace_small's edges for the grid)
     const int *rep;
     int *comp, *minp, *pidx, *plist;
     unsigned *pstamp;

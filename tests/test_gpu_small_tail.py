@@ -1,5 +1,5 @@
 """Batches around the candidate limit of the one-block replacement path
-(2,048), with super-forests of every shape, against the oracle."""
+(4,096), with super-forests of every shape, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -8,7 +8,7 @@ import paper_2607_20211_gb300 as drsf
 from tests.gpu_util import _tiny_graph, check_batch, make_forest
 
 pytestmark = pytest.mark.gpu
-LIMIT = 2048
+LIMIT = 4096
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -36,7 +36,7 @@ def _shape(kind, b, rng):
     return e[rng.permutation(len(e))[:b]]
 
 
-@pytest.mark.parametrize("b", [1, 2, 33, 1023, 1024, 1025, LIMIT - 1, LIMIT, LIMIT + 1, 3 * LIMIT])
+@pytest.mark.parametrize("b", [1, 2, 33, 1023, 1024, 1025, 2049, LIMIT - 1, LIMIT, LIMIT + 1, 3 * LIMIT])
 @pytest.mark.parametrize("kind", ["star", "path", "pairs", "dense", "random"])
 def test_insert_shapes(kind, b):
     """An insert whose every edge is a candidate, the same edges deleted
@@ -56,11 +56,11 @@ def test_insert_shapes(kind, b):
 
 
 @pytest.mark.parametrize("flags", [drsf.REPL_SG, drsf.REPL_HS])
-@pytest.mark.parametrize("cuts", [5, 700, 1500])
+@pytest.mark.parametrize("cuts", [5, 700, 1500, 2800])
 def test_delete_candidates(flags, cuts):
     """Deletes whose detached pieces keep several cross edges each: a path
     with chords, cut in many places; both replacement variants."""
-    n = 6000
+    n = 9000
     rng = np.random.default_rng(cuts)
     chords = rng.integers(0, n, (2 * cuts, 2))
     chords = chords[np.abs(chords[:, 0] - chords[:, 1]) > 1]
