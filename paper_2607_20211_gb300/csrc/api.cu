@@ -684,6 +684,7 @@ static bool use_supergraph(const drsf_ctx *h, int op) {
 static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cudaStream_t s) {
     Ctl *ctl = h->ctl;
     Csr g{h->row, h->col, h->fpos};
+    const bool wide = glen > (1 << 16);   // the replacement kernel's form
     if (op == DRSF_INSERT) {
         // Algorithm 1, insert: F^ = F, M = B; rep of the previous batch is current
         prof_begin(h, PH_INS_CLAIM, s);
@@ -691,7 +692,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         prof_end(h, PH_INS_CLAIM, 1, s);
         prof_begin(h, PH_INS_PLACE, s);
         CK(launch_ins_place(h->dev, h->nkey, h->nslot, ctl, g, h->ix, h->ovf, h->ovf_cap, h->rep, sg, h->pt,
-                            h->ck[0], h->ca[0], h->cb[0], h->cand_cap, hook_slots(h), s));
+                            h->ck[0], h->ca[0], h->cb[0], h->cand_cap, hook_slots(h), wide ? SMALL_CAND_LARGE : SMALL_CAND,
+                            s));
         prof_end(h, PH_INS_PLACE, 1, s);
     } else {
         // Algorithm 1, delete: remove B, cut tree edges, re-label the cut trees
@@ -838,7 +840,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     ha.pairs = sg ? 1 : 0;
     ha.pt = h->pt;
     prof_begin(h, PH_HOOK, s);
-    CK(launch_replace(h->dev, ctl, ha, oa, s));
+    CK(launch_replace(h->dev, ctl, ha, oa, wide, s));
     prof_end(h, PH_HOOK, 1, s);
     if (large && !euler) {
         prof_begin(h, PH_REVERSE, s);

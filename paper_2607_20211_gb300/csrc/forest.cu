@@ -17,13 +17,21 @@
 
 #include "kernels.h"
 
-// cores of up to this many arcs are list-ranked in one block's shared memory
-#define ORIENT_SMEM_ARCS 12288
-#define ORIENT_SMEM_BYTES (4 * ORIENT_SMEM_ARCS * (int)sizeof(int))
+// cores of up to this many arcs are list-ranked in one block's shared memory:
+// for batches of up to 64K edges, and for larger ones, whose grid phases want
+// the rest of the SM's memory as L1 (with 216 instead of 128 KB of shared
+// memory the hooking and orientation of a 100K-edge batch took 98 + 66 instead
+// of 77 + 54 us on R-MAT scale 22, the 256-graph union's 241 + 440 instead of
+// 182 + 337)
+#define RANK_ARCS 12288
+#define RANK_ARCS_LARGE 8192
 #define ORIENT_THREADS 1024
 // hooking: the live candidates at the start of a round (after round 0) up to
-// which block 0 finishes alone
+// which block 0 finishes alone, and the candidates that it takes on from the
+// start (what k_scan's first round left: usually none or a few; 3,300 took 90
+// us by one block against 60 by the grid)
 #define HOOK_TAIL 8192
+#define HOOK_FEW 1024
 // a core of at most this many edges is oriented by one block (measured on
 // R-MAT-22: faster than the grid phases for small batches' cores of tens of
 // edges, slower for the 100K batches' cores of about 900 edges)
@@ -1297,7 +1305,7 @@ __device__ __forceinline__ void hook_init(const HookArgs &h, long long c0, unsig
 // a short list) by block 0.  Returns -1 when a grid barrier gave up.
 __device__ __forceinline__ int hook_all(Ctl *ctl, HotMin &hm, const HookArgs &h, long long c0) {
     int r = 0;
-    const bool few = c0 <= SMALL_CAND;
+    const bool few = c0 <= HOOK_FEW;
     if (!few)
         r = hook_rounds<false>(ctl, hm, 0, c0, h.ck[0], h.ca[0], h.cb[0], h.ck[1], h.ca[1], h.cb[1], h.hs.comp,
                                h.hs.best0, h.hs.best1, h.er, h.er_cap);
@@ -1429,7 +1437,7 @@ __device__ void orient_small_core(Ctl *ctl, const OrientArgs &a, const int *cel,
     }
     __syncthreads();
     extern __shared__ int s_rank[];
-    int *svc = s_rank, *svn = svc + ORIENT_SMEM_ARCS, *snc = svn + ORIENT_SMEM_ARCS, *snn = snc + ORIENT_SMEM_ARCS;
+    int *svc = s_rank, *svn = svc + a.rank_arcs, *snc = svn + a.rank_arcs, *snn = snc + a.rank_arcs;
     for (long long t = threadIdx.x; t < 2 * nce; t += blockDim.x) {
         const long long j = 2 * (long long)LD(cel[t >> 1]) + (t & 1);
         const long long tw = j ^ 1;
@@ -1676,16 +1684,15 @@ __device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
     }
     if (!grid_barrier(ctl, bar)) return;
     // phase 6: list ranking (Wyllie): val = arcs from here to the tour end.
-    // A core of at most ORIENT_SMEM_ARCS arcs is ranked by block 0 alone in
+    // A core of at most rank_arcs arcs is ranked by block 0 alone in
     // shared memory (block barriers instead of grid barriers per round).
     const long long ncore = (long long)*(volatile u64 *)&ctl->ncore;
     int *vc = a.val0, *vn = a.val1, *nc = a.nx0, *nn = a.nx1;
     int r = 0;
-    if (ncore <= ORIENT_SMEM_ARCS) {
+    if (ncore <= a.rank_arcs) {
         if (blockIdx.x == 0) {
             extern __shared__ int s_rank[];
-            int *svc = s_rank, *svn = svc + ORIENT_SMEM_ARCS, *snc = svn + ORIENT_SMEM_ARCS,
-                *snn = snc + ORIENT_SMEM_ARCS;
+            int *svc = s_rank, *svn = svc + a.rank_arcs, *snc = svn + a.rank_arcs, *snn = snc + a.rank_arcs;
             for (long long i = threadIdx.x; i < ncore; i += blockDim.x) {
                 svc[i] = LD(a.val0[i]);
                 snc[i] = LD(a.nx0[i]);
@@ -1735,7 +1742,7 @@ __device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
     }
     block_add(&ctl->reversed, rev);
 }
-// Replacement edges and their orientation for a batch with at most SMALL_CAND
+// Replacement edges and their orientation for a batch with at most C
 // candidates, by one block in shared memory: the pieces get dense ids through
 // a hash table, the hook-and-compress rounds and the orientation run on
 // those.  On the grid the same batch is a chain of some twenty phases with a
@@ -1749,44 +1756,44 @@ __device__ void orient_grid(Ctl *ctl, const OrientArgs &a) {
 // Pieces: at most two per candidate.  A piece's minimum key is taken in two
 // halves, which shared memory has native atomics for; what is needed one after
 // the other shares memory.
-#define TAIL_P (2 * SMALL_CAND)
-#define TAIL_H (3 * SMALL_CAND)   // hash slots (two thirds full at most)
 #define SMALL_OUT 256
+template <int C>
 struct SmallTail {
-    u64 key[SMALL_CAND];
+    static constexpr int cand = C, pieces = 2 * C, slots = 3 * C;   // hash slots: two thirds full at most
+    u64 key[C];
     union {
-        unsigned short hl[TAIL_H];   // a hash slot's dense id
+        unsigned short hl[slots];   // a hash slot's dense id
         struct {
-            unsigned bhi[TAIL_P], blo[TAIL_P];   // a piece's minimum key
+            unsigned bhi[pieces], blo[pieces];   // a piece's minimum key
         };
         struct {
-            int minp[TAIL_P];
-            unsigned char vis[TAIL_P];
+            int minp[pieces];
+            unsigned char vis[pieces];
         };
     };
-    int hk[TAIL_H];                       // hash table: piece, -1 free
-    int pid[TAIL_P];
-    unsigned short comp[TAIL_P];
-    unsigned short a[SMALL_CAND], b[SMALL_CAND], er[SMALL_CAND];
+    int hk[slots];                  // hash table: piece, -1 free
+    int pid[pieces];
+    unsigned short comp[pieces];
+    unsigned short a[C], b[C], er[C];
     int ner;
+    static_assert(slots % ORIENT_THREADS == 0, "hash slots per thread");
 };
-#define REPLACE_SMEM_BYTES ((int)(sizeof(SmallTail) > ORIENT_SMEM_BYTES ? sizeof(SmallTail) : ORIENT_SMEM_BYTES))
-static_assert(sizeof(SmallTail) <= 225 * 1024, "one block's shared memory");
-static_assert(TAIL_H % ORIENT_THREADS == 0, "hash slots per thread");
 
 // slot of piece p in the hash table (entered when absent)
-__device__ __forceinline__ int tail_slot(SmallTail &t, int p) {
-    unsigned h = ((unsigned)p * 0x9E3779B1u) % TAIL_H;
+template <class T>
+__device__ __forceinline__ int tail_slot(T &t, int p) {
+    unsigned h = ((unsigned)p * 0x9E3779B1u) % T::slots;
     for (;;) {
         int k = *(volatile int *)&t.hk[h];
         if (k == -1) k = atomicCAS(&t.hk[h], -1, p);
         if (k == -1 || k == p) return (int)h;
-        h = h + 1 == TAIL_H ? 0 : h + 1;
+        h = h + 1 == T::slots ? 0 : h + 1;
     }
 }
 // root of dense piece x (hooking only ever links roots, so chains are short)
-__device__ __forceinline__ int tail_root(const SmallTail &t, int x) {
-    for (int it = 0; it < TAIL_P; ++it) {
+template <class T>
+__device__ __forceinline__ int tail_root(const T &t, int x) {
+    for (int it = 0; it < T::pieces; ++it) {
         const int p = *(volatile const unsigned short *)&t.comp[x];
         if (p == x) break;
         x = p;
@@ -1812,13 +1819,14 @@ __device__ __forceinline__ int tail_out(Ctl *ctl, const OrientArgs &oa, long lon
     return oa.walk ? walk_path(ctl, oa.parent, x, y, oa.long_ep, p, ep) : 0;
 }
 
+template <class T>
 __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa, int c0, int pre, unsigned ep) {
     extern __shared__ __align__(16) int s_rank[];
-    SmallTail &t = *reinterpret_cast<SmallTail *>(s_rank);
-    constexpr int IT = SMALL_CAND / ORIENT_THREADS;   // candidates per thread
+    T &t = *reinterpret_cast<T *>(s_rank);
+    constexpr int IT = T::cand / ORIENT_THREADS;   // candidates per thread
     const int lane = threadIdx.x & 31;
     const int all = c0 + pre;
-    for (int i = threadIdx.x; i < TAIL_H; i += ORIENT_THREADS) t.hk[i] = -1;
+    for (int i = threadIdx.x; i < T::slots; i += ORIENT_THREADS) t.hk[i] = -1;
     if (threadIdx.x == 0) t.ner = 0;
     __syncthreads();
     u64 key[IT];
@@ -1851,7 +1859,7 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
     // dense ids in slot order
     int np;
     {
-        constexpr int HT = TAIL_H / ORIENT_THREADS;
+        constexpr int HT = T::slots / ORIENT_THREADS;
         const int s0 = threadIdx.x * HT;
         int cnt = 0;
 #pragma unroll
@@ -2005,13 +2013,13 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
 
 // Replacement edges of a batch in one cooperative launch: the pair table is
 // moved into the candidate list (h.pairs), the candidates are hooked, the
-// replacement edges oriented and their paths walked.  Up to SMALL_CAND
-// candidates go to one block (replace_small); the other blocks then only pull
+// replacement edges oriented and their paths walked.  Up to C candidates go to
+// one block (replace_small); the other blocks then only pull
 // the forest into L2 for its walks (and the representatives for the refresh
 // that follows an insert) and take part in the results.  As launches of their
-// own the pair compaction,
-// hooking, orientation and walks of a 100-edge batch took 68 us on R-MAT
-// scale 22.
+// own the pair compaction, hooking, orientation and walks of a 100-edge batch
+// took 68 us on R-MAT scale 22.
+template <int C>
 __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArgs h, OrientArgs a) {
     if (batch_skipped(ctl)) return;
     __shared__ HotMin hm;
@@ -2026,10 +2034,10 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
     }
     const long long c0 = (long long)*(volatile u64 *)&ctl->ncand;
     const long long pre = ctl->pre ? (long long)*(volatile u64 *)&ctl->ner : 0;
-    if (c0 + pre <= SMALL_CAND) {
+    if (c0 + pre <= C) {
         if (c0 + pre == 0) return;
         if (blockIdx.x == 0) {
-            replace_small(ctl, h, a, (int)c0, (int)pre, ep);
+            replace_small<SmallTail<C>>(ctl, h, a, (int)c0, (int)pre, ep);
         } else {
             const long long t = gtid() - blockDim.x, nt = gstride() - blockDim.x;
             l2_prefetch(a.parent, 4 * a.n, t, nt);
@@ -2287,9 +2295,16 @@ unsigned coop_blocks_jump(int nsm) {
     const unsigned a = coop_blocks((const void *)k_jump<0>, nsm, 8), b = coop_blocks((const void *)k_jump<1>, nsm, 8);
     return a < b ? a : b;
 }
+template <int C>
+static constexpr int replace_smem(int arcs) {
+    return (int)sizeof(SmallTail<C>) > 16 * arcs ? (int)sizeof(SmallTail<C>) : 16 * arcs;
+}
 unsigned coop_blocks_replace(int nsm) {
-    cudaFuncSetAttribute((const void *)k_replace, cudaFuncAttributeMaxDynamicSharedMemorySize, REPLACE_SMEM_BYTES);
-    return (unsigned)nsm;   // one block per SM (shared memory)
+    cudaFuncSetAttribute((const void *)k_replace<SMALL_CAND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         replace_smem<SMALL_CAND>(RANK_ARCS));
+    cudaFuncSetAttribute((const void *)k_replace<SMALL_CAND_LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         replace_smem<SMALL_CAND_LARGE>(RANK_ARCS_LARGE));
+    return (unsigned)nsm;   // one block per SM (threads and registers)
 }
 
 cudaError_t launch_begin(Ctl *ctl, BeginArgs a, cudaStream_t s) {
@@ -2341,10 +2356,14 @@ cudaError_t launch_jump(const Dev &d, const int *A, int use_list, long long cnt_
     const void *fn = sync_rounds ? (const void *)k_jump<1> : (const void *)k_jump<0>;
     return cudaLaunchCooperativeKernel(fn, d.coop_jump, BLK, args, 0, s);
 }
-cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s) {
+cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, bool large, cudaStream_t s) {
+    static_assert(replace_smem<SMALL_CAND>(RANK_ARCS) <= 225 * 1024, "one block's shared memory");
+    a.rank_arcs = large ? RANK_ARCS_LARGE : RANK_ARCS;
     void *args[] = {(void *)&ctl, (void *)&h, (void *)&a};
-    return cudaLaunchCooperativeKernel((const void *)k_replace, d.coop_replace, ORIENT_THREADS, args,
-                                       REPLACE_SMEM_BYTES, s);
+    return large ? cudaLaunchCooperativeKernel((const void *)k_replace<SMALL_CAND_LARGE>, d.coop_replace,
+                                               ORIENT_THREADS, args, replace_smem<SMALL_CAND_LARGE>(RANK_ARCS_LARGE), s)
+                 : cudaLaunchCooperativeKernel((const void *)k_replace<SMALL_CAND>, d.coop_replace, ORIENT_THREADS, args,
+                                               replace_smem<SMALL_CAND>(RANK_ARCS), s);
 }
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
     k_walk<<<d.grid, BLK, 0, s>>>(ctl, a);

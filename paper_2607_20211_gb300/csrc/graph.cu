@@ -209,7 +209,8 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
 // Section III-B) every cross edge is a candidate of the hooking.
 template <bool SG>
 __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix, u64 *ovf, u64 ovf_cap,
-                            const int *rep, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap, HookSlots hs) {
+                            const int *rep, PairTable pt, u64 *ck, int *ca, int *cb, u64 cand_cap, HookSlots hs,
+                            int small) {
     if (batch_skipped(ctl)) return;
     const unsigned ep = ctl->epoch;
     long long nb = (long long)ctl->nb;
@@ -262,7 +263,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
                 // HS: these are all the candidates, so the hooking needs no
                 // initialisation phase of its own (see HookSlots); few
                 // candidates are hooked in shared memory
-                if (!SG && nb > SMALL_CAND) {
+                if (!SG && nb > small) {
                     hook_slot_init(hs, ra, ep);
                     hook_slot_init(hs, rb, ep);
                 }
@@ -464,13 +465,13 @@ cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *
 }
 cudaError_t launch_ins_place(const Dev &d, const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix,
                              u64 *ovf, u64 ovf_cap, const int *rep, bool sg, PairTable pt, u64 *ck, int *ca, int *cb,
-                             u64 cand_cap, HookSlots hs, cudaStream_t s) {
+                             u64 cand_cap, HookSlots hs, int small, cudaStream_t s) {
     if (sg)
         k_ins_place<true><<<d.grid, BLK, 0, s>>>(nkey, nslot, ctl, g, ix, ovf, ovf_cap, rep, pt, ck, ca, cb, cand_cap,
-                                                 hs);
+                                                 hs, small);
     else
         k_ins_place<false><<<d.grid, BLK, 0, s>>>(nkey, nslot, ctl, g, ix, ovf, ovf_cap, rep, pt, ck, ca, cb,
-                                                  cand_cap, hs);
+                                                  cand_cap, hs, small);
     return cudaGetLastError();
 }
 cudaError_t launch_del_claim(long long len, Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl,

@@ -6,9 +6,11 @@
 
 // Fixed launch shapes.
 #define BLK 256
-// batches with at most this many candidates are replaced, oriented and walked
-// by one block in shared memory (what fits beside the hash table)
+// batches with at most this many candidates are replaced and oriented by one
+// block in shared memory: batches of up to 64K edges, and larger ones (which
+// leave more of the SM's memory to L1)
 #define SMALL_CAND 4096
+#define SMALL_CAND_LARGE 2048
 
 struct Dev {
     int nsm;
@@ -67,10 +69,11 @@ struct PairTable {
 // sg: supergraph variant (pair-table dedupe to one minimum-key edge per
 // pair of trees), else every cross edge is a candidate (hooking variant)
 cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *nslot, cudaStream_t s);
-// (HS: the candidates' hook-forest slots are set up here, see HookSlots)
+// (HS: the hook-forest slots of more than `small` candidates are set up here,
+// see HookSlots)
 cudaError_t launch_ins_place(const Dev &d, const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix,
                              u64 *ovf, u64 ovf_cap, const int *rep, bool sg, PairTable pt, u64 *ck, int *ca, int *cb,
-                             u64 cand_cap, HookSlots hs, cudaStream_t s);
+                             u64 cand_cap, HookSlots hs, int small, cudaStream_t s);
 struct LightArgs {
     int n;
     Csr g;
@@ -170,6 +173,7 @@ struct HookArgs {
 };
 struct OrientArgs {
     const u64 *er;
+    int rank_arcs;       // core arcs that one block ranks in shared memory
     u64 *er_out;         // (the same array: replace_small's edges for the grid)
     const int *rep;
     int *comp, *minp, *pidx, *plist;
@@ -191,7 +195,7 @@ struct OrientArgs {
     const unsigned *aff_ep;   // old roots of this batch's cut trees
     long long n;
 };
-cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, cudaStream_t s);
+cudaError_t launch_replace(const Dev &d, Ctl *ctl, HookArgs h, OrientArgs a, bool large, cudaStream_t s);
 // batches above this many edges walk their paths in a launch of its own
 #define LARGE_BATCH (1 << 18)
 cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s);

@@ -75,3 +75,26 @@ def test_delete_candidates(flags, cuts):
         check_batch(f, n, keys, par, drsf.DELETE, b)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("cross", [0, 1, 200, 300, 2047, 2048, 2049, 3000, 4096, 4097, 9000])
+def test_large_batches_with_few_candidates(cross):
+    """Batches above 64K edges (the replacement kernel's form with less shared
+    memory) most of whose edges lie inside one tree: candidate counts around
+    both forms' limits, inserted and deleted again."""
+    core, b = 30_000, 70_000
+    n = core + 10_000
+    rng = np.random.default_rng(cross)
+    inner = rng.integers(0, core, (2 * b, 2))
+    inner = inner[np.abs(inner[:, 0] - inner[:, 1]) > 1][:b]
+    outer = np.stack([rng.integers(0, core, cross), core + rng.permutation(n - core)[:cross]], 1)
+    g = _tiny_graph(n, [(i, i + 1) for i in range(core - 1)], [max(i - 1, 0) for i in range(core)] + list(range(core, n)))
+    f = make_forest(g)
+    e = rng.permutation(np.concatenate([inner, outer])).astype(np.int32)
+    try:
+        keys, par, st = check_batch(f, n, g.keys, g.parent, drsf.INSERT, e)
+        assert st["replacement"] == cross
+        keys, par, _ = check_batch(f, n, keys, par, drsf.DELETE, e)
+        check_batch(f, n, keys, par, drsf.INSERT, e)
+    finally:
+        f.close()
