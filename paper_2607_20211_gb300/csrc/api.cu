@@ -635,6 +635,7 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.grid_pass = grid_vertex_pass(nsm);
     h->dev.coop_et = coop_blocks_et(nsm);
     h->dev.coop_cross = coop_blocks_cross(nsm);
+    h->dev.few = n <= FEW_VERTICES;
     // root search of a delete batch: barrier-free doubling over per-warp
     // slices by default; DRSF_JUMP=sync selects synchronous doubling rounds,
     // DRSF_JUMP=halving the in-place path-halving walks

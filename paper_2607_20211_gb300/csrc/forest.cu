@@ -2319,8 +2319,8 @@ cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsign
 cudaError_t launch_cross(const Dev &d, Ctl *ctl, DetachArgs da, RelabelArgs ra, RowList rl, LightArgs la, bool sg,
                          cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&da, (void *)&ra, (void *)&rl, (void *)&la};
-    return cudaLaunchCooperativeKernel(sg ? (const void *)k_cross<true> : (const void *)k_cross<false>, d.coop_cross,
-                                       BLK, args, 0, s);
+    return cudaLaunchCooperativeKernel(sg ? (const void *)k_cross<true> : (const void *)k_cross<false>,
+                                       d.few ? (unsigned)d.nsm : d.coop_cross, BLK, args, 0, s);
 }
 unsigned coop_blocks_cross(int nsm) {
     const unsigned a = coop_blocks((const void *)k_cross<true>, nsm, 4), b = coop_blocks((const void *)k_cross<false>, nsm, 4);
@@ -2371,7 +2371,7 @@ cudaError_t launch_walk(const Dev &d, Ctl *ctl, OrientArgs a, cudaStream_t s) {
 }
 cudaError_t launch_finish(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s) {
     void *args[] = {(void *)&ctl, (void *)&a};
-    return cudaLaunchCooperativeKernel((const void *)k_finish, d.coop_finish, BLK, args, 0, s);
+    return cudaLaunchCooperativeKernel((const void *)k_finish, d.few ? (unsigned)d.nsm : d.coop_finish, BLK, args, 0, s);
 }
 cudaError_t launch_reverse(const Dev &d, Ctl *ctl, FinishArgs a, cudaStream_t s) {
     k_reverse<<<d.grid, BLK, 0, s>>>(ctl, a);

@@ -290,6 +290,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
     // block-uniform loop: counters and the cut list append are aggregated
     // per block (one atomic per block instead of one per warp)
     long long loops = 0, drops = 0, wins = 0, dead = 0;
+    const bool early = len <= 1 << 16;
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < len; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
         int c = -1, rc = -1;
@@ -300,7 +301,10 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                 // loaded up front, beside the index probe: parent[u] changes in
                 // this kernel only by the cut of the edge {u, parent[u]}, which
                 // only the thread deleting that edge makes
-                const int par_u = parent[u], par_v = parent[v], rep_u = rep[u], rep_v = rep[v];
+                const int par_u = parent[u], par_v = parent[v];
+                // (the old root is needed for cuts only: large batches, bound
+                // by the sectors they touch, load it then)
+                const int rep_u = early ? rep[u] : 0, rep_v = early ? rep[v] : 0;
                 const unsigned st_u = g.row[u].start, st_v = g.row[v].start;
                 u64 key = ekey((uint32_t)u, (uint32_t)v);
                 uint2 pos;
@@ -316,10 +320,10 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                     }
                     if (par_u == v) {
                         c = u;
-                        rc = rep_u;
+                        rc = early ? rep_u : rep[u];
                     } else if (par_v == u) {
                         c = v;
-                        rc = rep_v;
+                        rc = early ? rep_v : rep[v];
                     }
                     if (c >= 0) {   // c roots a new piece
                         parent[c] = c;

@@ -12,6 +12,10 @@
 #define SMALL_CAND 4096
 #define SMALL_CAND_LARGE 2048
 
+// graphs of at most this many vertices: a grid barrier of one block per SM
+// takes 1.3 us, of four 2.5, and the passes are short
+#define FEW_VERTICES (1 << 18)
+
 struct Dev {
     int nsm;
     unsigned grid;        // grid-stride kernels: nsm * 8 blocks of BLK
@@ -22,6 +26,7 @@ struct Dev {
     unsigned coop_bfs;
     unsigned coop_et;
     unsigned coop_cross;
+    bool few;             // few vertices: one block per SM where blocks wait for each other
     unsigned grid_scan;   // row scan: the co-resident block count
     unsigned grid_pass;   // affected list: co-resident blocks
 };
