@@ -457,8 +457,11 @@ static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     CKA(halloc(h, &h->att_x, n, s));
     CKA(halloc(h, &h->newrep, n, s));
     CKA(halloc(h, &h->A, n, s));
-    // (the warps' lists of k_relabel: see relabel_room)
-    const size_t nl = (size_t)relabel_room(h->n, h->dev.coop_relabel);
+    // the warps' lists of the pieces' pass (relabel_room), which runs with
+    // each of these grids
+    size_t nl = 0;
+    for (unsigned g : {h->dev.coop_relabel, h->dev.coop_cross, (unsigned)h->dev.nsm})
+        nl = std::max(nl, (size_t)relabel_room(h->n, g));
     CKA(halloc(h, &h->act, nl, s));
     CKA(halloc(h, &h->pold, nl, s));
     CKA(halloc(h, &h->D, n, s));

@@ -77,3 +77,23 @@ def test_trajectories_without_the_top_down_search(monkeypatch):
     run_trajectory(workloads.rmat_graph(16, 16, seed=2), [(I, 1000), (D, 1000), (I, 10_000), (D, 50_000)] * 2, seed=3)
     run_trajectory(workloads.grid_graph(512, 512, seed=3), [(D, 5000), (I, 5000)] * 2, seed=4, tree_frac=0.9, local=64)
     run_trajectory(workloads.er_graph(20_001, 25_000, seed=1), [(I, 2000), (D, 2000)] * 2, seed=5)
+
+
+@pytest.mark.parametrize("n", [155_000, 156_673, 200_000, 262_144, 262_145, 622_593, 700_001, 778_241, 1_300_000])
+def test_list_room_for_every_grid(n):
+    """Chains of 40 over all vertices, each cut once, with a batch that tries
+    the top-down search first (it gives up: 40 levels) and with one that does
+    not: every block lists vertices, whatever the grid and the vertices per
+    block (the lists' room is bounded on the host)."""
+    parent = np.arange(n) - (np.arange(n) % 40 != 0)
+    edges = np.stack([np.arange(n), parent], 1)[parent != np.arange(n)]
+    extra = np.stack([np.arange(0, n - 40, 80) + 5, np.arange(0, n - 40, 80) + 37], 1)   # a second way round
+    g = _tiny_graph(n, np.concatenate([edges, extra]).tolist(), parent)
+    f = make_forest(g)
+    cut = edges[edges[:, 0] % 40 == 9].astype(np.int32)
+    more = np.concatenate([cut, edges[edges[:, 0] % 40 == 30], edges[edges[:, 0] % 2 == 1]]).astype(np.int32)
+    try:
+        keys, par, _ = check_batch(f, n, g.keys, g.parent, drsf.DELETE, cut[:32_000])
+        check_batch(f, n, keys, par, drsf.DELETE, more)
+    finally:
+        f.close()
