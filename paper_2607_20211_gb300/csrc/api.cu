@@ -189,6 +189,35 @@ static bool halloc(drsf_ctx *h, T **out, size_t count, cudaStream_t s) {
     return true;
 }
 
+// Several arrays out of one allocation (each 256-byte aligned): a handle's work
+// arrays and a build's temporaries are some seventy arrays, and every call of
+// the allocator costs host time (a framework's allocator behind the hooks:
+// 5 to 10 us).
+struct Slab {
+    struct Part {
+        void **out;
+        size_t bytes;
+    };
+    std::vector<Part> parts;
+    size_t total = 0;
+    template <class T>
+    void add(T **out, size_t count) {
+        const size_t bytes = (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~(size_t)255;
+        parts.push_back({(void **)out, bytes});
+        total += bytes;
+    }
+    // false: out of memory (nothing set); base: the allocation, for hfree
+    bool take(drsf_ctx *h, char **base, cudaStream_t s) {
+        if (!halloc(h, base, total, s)) return false;
+        char *p = *base;
+        for (auto &x : parts) {
+            *x.out = p;
+            p += x.bytes;
+        }
+        return true;
+    }
+};
+
 template <class T>
 static void hfree(drsf_ctx *h, T **ptr, cudaStream_t s) {
     if (!*ptr) return;
@@ -237,17 +266,21 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     CK(cudaMemsetAsync(ix.e, 0xFF, H * sizeof(Entry), s));
 
     u64 *dkey = nullptr, *dslot = nullptr, *cnt = nullptr;
-    long long *tmp64 = nullptr, *bs = nullptr;
+    long long *tmp64 = nullptr, *bs = nullptr, *off = nullptr;
     int *deg = nullptr;
     int2 *place = nullptr;
-    CKA(halloc(h, &dkey, (size_t)std::max<long long>(m, 1), s));
-    CKA(halloc(h, &dslot, (size_t)std::max<long long>(m, 1), s));
-    CKA(halloc(h, &place, (size_t)std::max<long long>(m, 1), s));
-    CKA(halloc(h, &cnt, 4, s));
-    CKA(halloc(h, &deg, (size_t)n, s));
-    CKA(halloc(h, &tmp64, (size_t)n + 1, s));
-    long long tiles = ((long long)n + 4095) / 4096 + 1;
-    CKA(halloc(h, &bs, (size_t)tiles, s));
+    char *tmp = nullptr;
+    const long long tiles = ((long long)n + 4095) / 4096 + 1;
+    Slab t;
+    t.add(&dkey, (size_t)m);
+    t.add(&dslot, (size_t)m);
+    t.add(&place, (size_t)m);
+    t.add(&cnt, 4);
+    t.add(&deg, (size_t)n);
+    t.add(&tmp64, (size_t)n + 1);
+    t.add(&off, (size_t)n + 1);
+    t.add(&bs, (size_t)tiles);
+    CKA(t.take(h, &tmp, s));
     CK(cudaMemsetAsync(cnt, 0, 4 * sizeof(u64), s));
     CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(int), s));
     if (m > 0) CK(launch_create_claim(edges, m, ix, dkey, dslot, cnt, (long long *)(cnt + 1), s));
@@ -257,8 +290,6 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     long long m2 = (long long)hc[0];
     CK(launch_degree(dkey, m2, deg, place, s));
     CK(launch_caps(deg, n, tmp64, s));
-    long long *off = nullptr;
-    CKA(halloc(h, &off, (size_t)n + 1, s));
     CK(launch_scan_i64(tmp64, off, n, bs, s));
     long long total = 0;
     CK(cudaMemcpyAsync(&total, off + n, sizeof(long long), cudaMemcpyDeviceToHost, s));
@@ -315,14 +346,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     h->col_cap = total;
     h->ovf = ovf;
     h->ovf_cap = ovf_cap;
-    hfree(h, &dkey, s);
-    hfree(h, &dslot, s);
-    hfree(h, &place, s);
-    hfree(h, &cnt, s);
-    hfree(h, &deg, s);
-    hfree(h, &off, s);
-    hfree(h, &tmp64, s);
-    hfree(h, &bs, s);
+    hfree(h, &tmp, s);
     h->occ_bound = m2;
     h->ovf_bound = 0;
     h->ctomb_bound = 0;
@@ -358,6 +382,7 @@ static drsf_status ensure_batch(drsf_ctx *h, long long len, cudaStream_t s) {
 }
 
 static drsf_status read_ctl(drsf_ctx *h, cudaStream_t s) {
+    if (!h->ctl_host) CK(cudaMallocHost((void **)&h->ctl_host, sizeof(Ctl)));   // (on first use)
     CK(cudaMemcpyAsync(h->ctl_host, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return DRSF_OK;
@@ -446,69 +471,65 @@ static void set_dev(drsf_ctx *h) {
 
 static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     size_t n = (size_t)h->n;
-    CKA(halloc(h, &h->parent, n, s));
-    CKA(halloc(h, &h->rep, n, s));
-    CKA(halloc(h, &h->J0, n, s));
-    CKA(halloc(h, &h->J1, n, s));
-    CKA(halloc(h, &h->comp, n, s));
-    CKA(halloc(h, &h->minp, n, s));
-    CKA(halloc(h, &h->pidx, n, s));
-    CKA(halloc(h, &h->plist, n + 1, s));
-    CKA(halloc(h, &h->att_x, n, s));
-    CKA(halloc(h, &h->newrep, n, s));
-    CKA(halloc(h, &h->A, n, s));
+    Slab w;
+    char *base = nullptr;
+    w.add(&h->parent, n);
+    w.add(&h->rep, n);
+    w.add(&h->J0, n);
+    w.add(&h->J1, n);
+    w.add(&h->comp, n);
+    w.add(&h->minp, n);
+    w.add(&h->pidx, n);
+    w.add(&h->plist, n + 1);
+    w.add(&h->att_x, n);
+    w.add(&h->newrep, n);
+    w.add(&h->A, n);
     // the warps' lists of the pieces' pass (relabel_room), which runs with
     // each of these grids
     size_t nl = 0;
     for (unsigned g : {h->dev.coop_relabel, h->dev.coop_cross, (unsigned)h->dev.nsm})
         nl = std::max(nl, (size_t)relabel_room(h->n, g));
-    CKA(halloc(h, &h->act, nl, s));
-    CKA(halloc(h, &h->pold, nl, s));
-    CKA(halloc(h, &h->D, n, s));
-    CKA(halloc(h, &h->chx, n, s));
-    CKA(halloc(h, &h->chy, n, s));
-    CKA(halloc(h, &h->aff_ep, n, s));
-    CKA(halloc(h, &h->cut_ep, n, s));
-    CKA(halloc(h, &h->pstamp, n, s));
-    CKA(halloc(h, &h->att_ep, n, s));
-    CKA(halloc(h, &h->long_ep, n, s));
-    CKA(halloc(h, &h->hstamp, n, s));
-    CKA(halloc(h, &h->rep_ep, n, s));
-    CKA(halloc(h, &h->det_ep, n, s));
-    CKA(halloc(h, &h->det_claim, n, s));
-    CKA(halloc(h, &h->best0, n, s));
-    CKA(halloc(h, &h->best1, n, s));
-    CKA(halloc(h, &h->heavy, n, s));
-    CKA(halloc(h, &h->rold, n, s));
-    CKA(halloc(h, &h->roff, n + 1, s));
-    CKA(halloc(h, &h->rbase, n, s));
-    CKA(halloc(h, &h->rmeta, n, s));
-    CKA(halloc(h, &h->xlist, nl, s));
-    CKA(halloc(h, &h->aidx, n, s));
-    CKA(halloc(h, &h->aroot, n, s));
-    CKA(halloc(h, &h->oep, 2 * n + 2, s));
-    CKA(halloc(h, &h->oeid, 2 * n + 2, s));
-    CKA(halloc(h, &h->oeroot, n + 1, s));
-    CKA(halloc(h, &h->cdeg, n + 1, s));
-    CKA(halloc(h, &h->lf, n + 1, s));
-    CKA(halloc(h, &h->wgt, n, s));
-    CKA(halloc(h, &h->er, n, s));
-    CKA(halloc(h, &h->mark, n, s));
-    CKA(halloc(h, &h->pdeg, n + 1, s));
-    CKA(halloc(h, &h->pcur, n + 1, s));
-    CKA(halloc(h, &h->poff, n + 1, s));
-    CKA(halloc(h, &h->adj, 2 * n + 2, s));
-    CKA(halloc(h, &h->apos, 2 * n + 2, s));
-    CKA(halloc(h, &h->val0, 2 * n + 2, s));
-    CKA(halloc(h, &h->val1, 2 * n + 2, s));
-    CKA(halloc(h, &h->nx0, 2 * n + 2, s));
-    CKA(halloc(h, &h->nx1, 2 * n + 2, s));
-    CKA(halloc(h, &h->bsum, 8192, s));
-    CKA(halloc(h, &h->ctl, 1, s));
-    unsigned *eps[] = {h->aff_ep, h->cut_ep, h->pstamp, h->att_ep, h->rep_ep, h->long_ep, h->hstamp, h->det_ep,
-                       h->det_claim};
-    for (unsigned *e : eps) CK(cudaMemsetAsync(e, 0, n * sizeof(unsigned), s));
-    CK(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), s));
+    w.add(&h->act, nl);
+    w.add(&h->pold, nl);
+    w.add(&h->D, n);
+    w.add(&h->chx, n);
+    w.add(&h->chy, n);
+    w.add(&h->best0, n);
+    w.add(&h->best1, n);
+    w.add(&h->heavy, n);
+    w.add(&h->rold, n);
+    w.add(&h->roff, n + 1);
+    w.add(&h->rbase, n);
+    w.add(&h->rmeta, n);
+    w.add(&h->xlist, nl);
+    w.add(&h->aidx, n);
+    w.add(&h->aroot, n);
+    w.add(&h->oep, 2 * n + 2);
+    w.add(&h->oeid, 2 * n + 2);
+    w.add(&h->oeroot, n + 1);
+    w.add(&h->cdeg, n + 1);
+    w.add(&h->lf, n + 1);
+    w.add(&h->wgt, n);
+    w.add(&h->er, n);
+    w.add(&h->mark, n);
+    w.add(&h->pdeg, n + 1);
+    w.add(&h->pcur, n + 1);
+    w.add(&h->poff, n + 1);
+    w.add(&h->adj, 2 * n + 2);
+    w.add(&h->apos, 2 * n + 2);
+    w.add(&h->val0, 2 * n + 2);
+    w.add(&h->val1, 2 * n + 2);
+    w.add(&h->nx0, 2 * n + 2);
+    w.add(&h->nx1, 2 * n + 2);
+    w.add(&h->bsum, 8192);
+    // (the epoch stamps and the control block, which start at zero, last)
+    const size_t clear = w.total;
+    unsigned **eps[] = {&h->aff_ep, &h->cut_ep, &h->pstamp, &h->att_ep, &h->rep_ep, &h->long_ep, &h->hstamp,
+                        &h->det_ep, &h->det_claim};
+    for (unsigned **e : eps) w.add(e, n);
+    w.add(&h->ctl, 1);
+    CKA(w.take(h, &base, s));
+    CK(cudaMemsetAsync(base + clear, 0, w.total - clear, s));
     return DRSF_OK;
 }
 
@@ -553,7 +574,6 @@ static drsf_status create_impl(drsf_ctx *h, const int32_t *edges, int64_t m, con
     if (st) return st;
     st = ensure_batch(h, 1, s);
     if (st) return st;
-    CK(cudaMallocHost((void **)&h->ctl_host, sizeof(Ctl)));
     int *bad = nullptr;
     CKA(halloc(h, &bad, 4, s));
     CK(cudaMemsetAsync(bad, 0, 4 * sizeof(int), s));
@@ -762,6 +782,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
             da.budget_v = std::max<long long>(1 << 16, n / 8);
             da.budget_e = std::max<long long>(1 << 20, 4 * n);
             da.max_levels = DETACH_LEVELS;
+            da.nsm = (unsigned)h->dev.nsm;
             da.oc = h->act;
             da.op = h->xlist;
             prof_begin(h, PH_SCAN, s);

@@ -45,7 +45,7 @@ struct Ctl {
     unsigned skip;          // epoch + 1 of the last rejected batch (ERR_BATCH_ID seen)
     unsigned epoch;         // batch counter (the host's); epoch stamps compare against it
     int op;
-    u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs / scan, Euler marks, detach
+    u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs / scan, Euler marks, detach, cross
                             // (reset at each batch's start and before each static BFS)
     int flag[3];            // per-round "another round needed" flags
     u64 cnt[3];             // per-round list sizes (hook-and-compress)
@@ -472,16 +472,16 @@ __device__ __forceinline__ u64 ld_acquire_u64(const u64 *p) {
 // Grid-wide barrier for cooperative launches (all blocks co-resident).
 // Ticket barrier on a monotonic counter owned by one kernel (always launched
 // with the same block count, so the counter is a multiple of gridDim.x
-// between barriers): each block takes a ticket t and waits until the counter
-// reaches the end of t's group.  The wait is bounded: after
+// between barriers; or by the first nb blocks only, always the same nb): each
+// block takes a ticket t and waits until the counter reaches the end of t's
+// group.  The wait is bounded: after
 // BARRIER_TIMEOUT_NS it latches ERR_TIMEOUT and returns false, and a block
 // that sees another block's timeout returns false too, so the kernel unwinds
 // instead of hanging.
-__device__ __forceinline__ bool grid_barrier(Ctl *ctl, u64 *bar) {
+__device__ __forceinline__ bool grid_barrier(Ctl *ctl, u64 *bar, u64 nb = gridDim.x) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const u64 nb = gridDim.x;
         __threadfence();
         u64 t = atomicAdd(bar, 1ull);
         u64 target = (t / nb + 1) * nb;

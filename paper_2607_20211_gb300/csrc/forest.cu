@@ -49,6 +49,8 @@
 #define IPN 16
 // k_aff_collect keeps more per item (old root, list position)
 #define IPA 8
+// top-down delete: the longest batch searched by one block per SM
+#define SEARCH_FEW 4096
 // top-down delete: after a search that gave up at its level limit, the
 // deletes that skip it before it is tried again
 #define DETACH_BACKOFF 8
@@ -344,7 +346,8 @@ __device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long v
 // pointer-jumping path runs.
 // Returns 1 when the pieces were found, 0 when they were not, -1 when a grid
 // barrier gave up.
-__device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl) {
+__device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl, unsigned nb) {
+    const long long S = (long long)nb * blockDim.x;   // the threads that search
     const int *const cuts = a.cuts, *const par = a.par, *const rold = a.rold;
     int *const rep = a.rep, *const A = a.A, *const J1 = a.J1, *const oc = a.oc, *const op = a.op;
     unsigned *const det_ep = a.det_ep, *const det_claim = a.det_claim;
@@ -367,7 +370,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
     u64 *bar = &ctl->bar[6];
     const int lane = threadIdx.x & 31;
     // level 0: the cut vertices (pieces of their own), slot 0
-    for (long long b0 = gtid() & ~31ll; b0 < nc; b0 += gstride()) {
+    for (long long b0 = gtid() & ~31ll; b0 < nc; b0 += S) {
         const long long i = b0 + lane;
         const bool on = i < nc;
         int c = 0, len = 0, ro = 0;
@@ -389,7 +392,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
     // only when a row is full)
     {
         const long long no = (long long)min((u64)ctl->ovf_count, a.ovf_cap);
-        for (long long b0 = gtid() & ~31ll; b0 < no; b0 += gstride()) {
+        for (long long b0 = gtid() & ~31ll; b0 < no; b0 += S) {
             const long long i = b0 + lane;
             int cw = -1, pv = -1;
             if (i < no) {
@@ -418,7 +421,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
     int lvl = 0;
     bool ok = true;
     for (;; ++lvl) {
-        if (!grid_barrier(ctl, bar)) return -1;
+        if (!grid_barrier(ctl, bar, nb)) return -1;
         // the level found in the last round (slot lvl % 3) is final
         const int sl = lvl % 3, sn = (lvl + 1) % 3;
         const long long dv = (long long)*(volatile u64 *)&ctl->dv[sl];
@@ -438,7 +441,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
         // a contiguous range of tiles per warp
         const unsigned T0 = e_lo >> 5, T1 = (e_hi + 31) >> 5;
         const unsigned NT = T1 - T0;
-        const unsigned nw = (unsigned)(gstride() >> 5), wid = (unsigned)(gtid() >> 5);
+        const unsigned nw = (unsigned)(S >> 5), wid = (unsigned)(gtid() >> 5);
         const unsigned per = (NT + nw - 1) / nw;
         for (unsigned it = 0; it < per; ++it) {
             const unsigned T = T0 + wid * per + it;
@@ -484,7 +487,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
         // children joined by a tree edge outside the rows: a vertex whose
         // parent is detached (published: its J1 before its stamp)
         const long long nt = (long long)*(volatile u64 *)&ctl->dovf;
-        for (long long b0 = gtid() & ~31ll; b0 < nt; b0 += gstride()) {
+        for (long long b0 = gtid() & ~31ll; b0 < nt; b0 += S) {
             const long long i = b0 + lane;
             bool child = false;
             int w = -1, p = 0, ro = 0, len = 0;
@@ -523,7 +526,7 @@ __device__ int detach_top_down(Ctl *ctl, const DetachArgs &a, const RowList &rl)
         return 0;
     }
     // commit the representatives of the detached vertices
-    for (long long i = gtid(); i < vb; i += gstride()) {
+    for (long long i = gtid(); i < vb; i += S) {
         const int v = A[i];
         rep[v] = LD(J1[v]);
     }
@@ -796,10 +799,20 @@ template <bool SG>
 __global__ void __launch_bounds__(BLK, 4)
     k_cross(Ctl *ctl, DetachArgs d, RelabelArgs r, RowList rl, LightArgs a) {
     if (batch_skipped(ctl)) return;
-    const int found = detach_top_down(ctl, d, rl);
-    if (found < 0) return;
+    // a batch of up to SEARCH_FEW edges is searched by one block per SM (a
+    // level of its search is a barrier and little work), the others wait
+    const unsigned nb = ctl->batch_len <= SEARCH_FEW && gridDim.x > d.nsm ? d.nsm : gridDim.x;
+    int found = 0;
+    if (blockIdx.x < nb) {
+        found = detach_top_down(ctl, d, rl, nb);
+        if (found < 0) return;
+    }
+    if (nb < gridDim.x) {
+        if (!grid_barrier(ctl, &ctl->bar[7])) return;
+        found = *(volatile int *)&ctl->td;
+    }
     if (!found && !relabel(ctl, r)) return;
-    if (!grid_barrier(ctl, &ctl->bar[6])) return;
+    if ((!found || nb == gridDim.x) && !grid_barrier(ctl, &ctl->bar[7])) return;
     if (found) scan_listed<SG>(ctl, rl, a);
     else scan_light<SG>(ctl, a);
 }

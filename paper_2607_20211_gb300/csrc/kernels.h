@@ -134,6 +134,7 @@ struct DetachArgs {
     unsigned *det_ep, *det_claim;
     long long budget_v, budget_e;
     int max_levels;
+    unsigned nsm;
     int *oc, *op;                   // tree edges held outside the rows
 };
 struct RelabelArgs {
