@@ -35,11 +35,16 @@ struct drsf_ctx {
     std::vector<Buf> bufs;
     bool poisoned = false;
     int jump_sync = 2;   // root search: 2 hops, then asynchronous doubling; 1 synchronous rounds, 0 path halving
-    unsigned epoch = 0;  // batches so far (the stamps of the per-batch arrays)
     int last_sg = 0;     // the last batch took the supergraph variant
     // captured per-batch launch sequences (CUDA graphs), valid for storage
     // generation u_gen; gen moves whenever a storage or batch buffer moves
-    std::vector<std::pair<std::string, cudaGraphExec_t>> u_graphs;
+    struct Captured {
+        std::string key;
+        cudaGraphExec_t exec;
+        cudaGraph_t graph;       // kept: it names the node below
+        cudaGraphNode_t begin;   // k_begin, whose arguments change with the batch
+    };
+    std::vector<Captured> u_graphs;
     std::map<std::string, int> u_seen;   // uses of each shape (capture on the second)
     long long gen = 0, u_gen = 0;
     bool graphs_ok = true;
@@ -533,6 +538,15 @@ static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     return DRSF_OK;
 }
 
+// Forget the captured launch sequences (the storage they point into moved).
+static void drop_graphs(drsf_ctx *h) {
+    for (auto &c : h->u_graphs) {
+        cudaGraphExecDestroy(c.exec);
+        cudaGraphDestroy(c.graph);
+    }
+    h->u_graphs.clear();
+}
+
 static void destroy_all(drsf_ctx *h) {
     if (!h) return;
     set_dev(h);
@@ -544,7 +558,7 @@ static void destroy_all(drsf_ctx *h) {
     if (h->stage_done) cudaEventDestroy(h->stage_done);
     for (cudaEvent_t e : h->prof_ev) cudaEventDestroy(e);
     for (auto &ge : h->b_graphs) cudaGraphExecDestroy(ge.second);
-    for (auto &ge : h->u_graphs) cudaGraphExecDestroy(ge.second);
+    drop_graphs(h);
     if (h->u_cap) cudaStreamDestroy(h->u_cap);
     if (h->b_meta_host) cudaFreeHost(h->b_meta_host);
     if (h->b_meta_done) cudaEventDestroy(h->b_meta_done);
@@ -923,12 +937,6 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     return DRSF_OK;
 }
 
-// Forget the captured launch sequences (the storage they point into moved).
-static void drop_graphs(drsf_ctx *h) {
-    for (auto &ge : h->u_graphs) cudaGraphExecDestroy(ge.second);
-    h->u_graphs.clear();
-}
-
 static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t len, cudaStream_t s,
                               int groups = 0, const long long *voff = nullptr, const long long *boff = nullptr) {
     drsf_status st = ensure_batch(h, len, s);
@@ -945,13 +953,18 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
         h->prof_op = op;
         h->prof_nb[op]++;
     }
-    prof_begin(h, PH_BEGIN, s);
-    CK(launch_begin(h->ctl, BeginArgs{op, h->n, len, batch, ++h->epoch, groups, voff, boff}, s));
-    prof_end(h, PH_BEGIN, 1, s);
+    const BeginArgs ba{op, h->n, len, batch, groups, voff, boff};
+    auto direct = [&]() -> drsf_status {
+        prof_begin(h, PH_BEGIN, s);
+        CK(launch_begin(h->ctl, ba, len, s));
+        prof_end(h, PH_BEGIN, 1, s);
+        return launch_rest(h, op, sg, len, s);
+    };
     // per-phase profiling brackets the phases with events: launch directly
-    if (h->prof_on || !h->graphs_ok) return launch_rest(h, op, sg, len, s);
+    if (h->prof_on || !h->graphs_ok) return direct();
     // otherwise replay the captured sequence for this (storage, op, variant,
-    // grid size class of the batch kernels); capture it on first use
+    // grid size class of the batch kernels), with its first kernel's
+    // arguments set to this batch
     long long glen = 4096;
     while (glen < len) glen <<= 2;
     if (h->u_gen != h->gen) {
@@ -961,39 +974,44 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     }
     const std::string key = std::to_string(op) + ":" + std::to_string(sg ? 1 : 0) + ":" + std::to_string(glen) +
                             ":" + std::to_string(h->detach_now ? 1 : 0);
-    cudaGraphExec_t exec = nullptr;
-    for (auto &ge : h->u_graphs)
-        if (ge.first == key) exec = ge.second;
-    if (!exec) {
-        // a shape is captured on its second use: recording and instantiating
-        // costs more host time than one direct launch sequence, and a
-        // handle that sees a shape once (a tenant with few batches) never
-        // pays it
-        int &seen = h->u_seen[key];
-        if (++seen < 2) return launch_rest(h, op, sg, len, s);
-        // recorded on a stream of the library's own (the caller's stream may
-        // be the legacy default stream, which cannot be captured); nothing
-        // runs while recording, the replay below is ordered on s
-        if (!h->u_cap) CK(cudaStreamCreateWithFlags(&h->u_cap, cudaStreamNonBlocking));
-        CK(cudaStreamBeginCapture(h->u_cap, cudaStreamCaptureModeThreadLocal));
-        drsf_status rs = launch_rest(h, op, sg, glen, h->u_cap);
-        cudaGraph_t graph = nullptr;
-        cudaError_t e = cudaStreamEndCapture(h->u_cap, &graph);
-        if (rs == DRSF_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        if (rs != DRSF_OK || e != cudaSuccess || !exec) {
-            // capture not possible here: launch directly from now on
-            cudaGetLastError();
-            h->graphs_ok = false;
-            return launch_rest(h, op, sg, len, s);
+    for (auto &c : h->u_graphs)
+        if (c.key == key) {
+            CK(set_begin(c.exec, c.begin, h->ctl, ba, glen));
+            CK(cudaGraphLaunch(c.exec, s));
+            return DRSF_OK;
         }
-        if (h->u_graphs.size() >= 16) {
-            cudaGraphExecDestroy(h->u_graphs.front().second);
-            h->u_graphs.erase(h->u_graphs.begin());
-        }
-        h->u_graphs.emplace_back(key, exec);
+    // a shape is captured on its second use: recording and instantiating
+    // costs more host time than one direct launch sequence, and a handle that
+    // sees a shape once (a tenant with few batches) never pays it
+    int &seen = h->u_seen[key];
+    if (++seen < 2) return direct();
+    // recorded on a stream of the library's own (the caller's stream may be
+    // the legacy default stream, which cannot be captured); nothing runs
+    // while recording, the replay below is ordered on s
+    if (!h->u_cap) CK(cudaStreamCreateWithFlags(&h->u_cap, cudaStreamNonBlocking));
+    CK(cudaStreamBeginCapture(h->u_cap, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = launch_begin(h->ctl, ba, glen, h->u_cap);
+    const drsf_status rs = e == cudaSuccess ? launch_rest(h, op, sg, glen, h->u_cap) : DRSF_ECUDA;
+    drsf_ctx::Captured c{key, nullptr, nullptr, nullptr};
+    cudaError_t e2 = cudaStreamEndCapture(h->u_cap, &c.graph);
+    if (e == cudaSuccess) e = e2;
+    size_t roots = 1;
+    if (rs == DRSF_OK && e == cudaSuccess) e = cudaGraphGetRootNodes(c.graph, &c.begin, &roots);
+    if (rs == DRSF_OK && e == cudaSuccess && roots == 1) e = cudaGraphInstantiate(&c.exec, c.graph, 0);
+    if (rs != DRSF_OK || e != cudaSuccess || !c.exec) {
+        // capture not possible here: launch directly from now on
+        cudaGetLastError();
+        if (c.graph) cudaGraphDestroy(c.graph);
+        h->graphs_ok = false;
+        return direct();
     }
-    CK(cudaGraphLaunch(exec, s));
+    if (h->u_graphs.size() >= 16) {
+        cudaGraphExecDestroy(h->u_graphs.front().exec);
+        cudaGraphDestroy(h->u_graphs.front().graph);
+        h->u_graphs.erase(h->u_graphs.begin());
+    }
+    h->u_graphs.push_back(c);
+    CK(cudaGraphLaunch(c.exec, s));   // (recorded with this batch's arguments)
     return DRSF_OK;
 }
 
@@ -1210,7 +1228,6 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     d.order = order_d;
     d.G = (int)G;
     d.op = (int)op;
-    d.epoch = ++h->epoch;
     CK(launch_bset(h->b_state, b, h->b_desc, d, s));
     // one captured launch sequence per (op, class queues, launch shapes)
     std::string key = std::to_string((int)op);

@@ -860,7 +860,8 @@ __global__ void k_bbegin(const BState *Sp) {
     const BDesc d = *S.desc;
     Ctl *ctl = S.ctl;
     if (threadIdx.x == 0) {
-        ctl->epoch = d.epoch;
+        ctl->base += 1;
+        ctl->epoch = ctl->base;
         ctl->op = d.op;
         ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
         ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
@@ -907,7 +908,7 @@ __global__ void k_bvalidate(const BState *Sp) {
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) {
             atomicOr(&S.ctl->err, ERR_BATCH_ID);
-            S.ctl->skip = d.epoch + 1;
+            S.ctl->skip = S.ctl->epoch + 1;
         }
     }
 }

@@ -43,7 +43,9 @@ typedef unsigned long long u64;
 struct Ctl {
     int err;
     unsigned skip;          // epoch + 1 of the last rejected batch (ERR_BATCH_ID seen)
-    unsigned epoch;         // batch counter (the host's); epoch stamps compare against it
+    unsigned epoch;         // batch counter; epoch stamps compare against it
+    unsigned base;          // the batches before this one (k_begin's blocks all read it; the claim
+                            // kernels move it on)
     int op;
     u64 bar[8];             // grid-barrier counters: jump, hook, orient, mark, bfs / scan, Euler marks, detach, cross
                             // (reset at each batch's start and before each static BFS)

@@ -49,6 +49,10 @@
 #define IPN 16
 // k_aff_collect keeps more per item (old root, list position)
 #define IPA 8
+// the refresh after a large delete, most of whose vertices may change (the
+// 4096 x 4096 grid: three quarters): their new representatives are loaded
+// together
+#define IPD 8
 // top-down delete: the longest batch searched by one block per SM
 #define SEARCH_FEW 4096
 // top-down delete: after a search that gave up at its level limit, the
@@ -116,6 +120,7 @@ __device__ __forceinline__ int owner_of(const long long *off, int G, long long i
 // batch's epoch, so it needs no reset that the checks would race with, and no
 // launch of its own.
 __global__ void k_begin(Ctl *ctl, BeginArgs a) {
+    const unsigned epoch = ctl->base + 1;
     GS_LOOP(i, a.len) {
         const int u = a.batch[2 * i], v = a.batch[2 * i + 1];
         bool bad = u < 0 || u >= a.n || v < 0 || v >= a.n;
@@ -126,14 +131,14 @@ __global__ void k_begin(Ctl *ctl, BeginArgs a) {
         }
         if (bad) {
             atomicOr(&ctl->err, ERR_BATCH_ID);
-            ctl->skip = a.epoch + 1;
+            ctl->skip = epoch + 1;
         }
     }
     if (gtid() != 0) return;
     const int op = a.op;
     const long long len = a.len;
     ctl->batch = a.batch;
-    ctl->epoch = a.epoch;
+    ctl->epoch = epoch;
     ctl->op = op;
     ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
     ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
@@ -2103,8 +2108,9 @@ __global__ void k_walk(Ctl *ctl, OrientArgs a) {
 // IP items per thread and iteration (IPT over a list or few vertices, IPN
 // over many), k-major as in k_aff_collect, one slot reservation per block.
 // Only the pieces stay in registers; the few items whose piece changed are
-// handled from bit masks (the common item costs one stamp gather).
-template <int IP>
+// handled from bit masks (the common item costs one stamp gather).  With DENSE
+// many change, and their new representatives are loaded side by side.
+template <int IP, bool DENSE>
 __device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, const int *L, long long cnt, unsigned ep,
                                              bool marks) {
     static_assert(IP <= 32, "item masks are 32 bits");
@@ -2135,15 +2141,37 @@ __device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, cons
             if (i0 + (long long)k * blockDim.x < cnt && a.rep_ep[p[k]] == ep) chg |= 1u << k;
         unsigned on = 0;
         long long q = 0;
+        int nr[DENSE ? IP : 1];
+        if (DENSE) {
+#pragma unroll
+            for (int k = 0; k < IP; ++k) nr[k] = chg >> k & 1u ? a.newrep[p[k]] : 0;
+        }
         if (marks) {   // (the same value in every thread)
-            for (unsigned m = chg; m; m &= m - 1) {
-                const int k = __ffs(m) - 1;
-                const int pk = p[k];
-                if (LD(a.sel_ep[pk]) == ep && a.att_x[pk] != pk) on |= 1u << k;
+            if (DENSE) {
+#pragma unroll
+                for (int k = 0; k < IP; ++k)
+                    if ((chg >> k & 1u) && LD(a.sel_ep[p[k]]) == ep) on |= 1u << k;
+                for (unsigned m = on; m; m &= m - 1) {
+                    const int k = __ffs(m) - 1;
+                    if (a.att_x[p[k]] == p[k]) on &= ~(1u << k);
+                }
+            } else {
+                for (unsigned m = chg; m; m &= m - 1) {
+                    const int k = __ffs(m) - 1;
+                    const int pk = p[k];
+                    if (LD(a.sel_ep[pk]) == ep && a.att_x[pk] != pk) on |= 1u << k;
+                }
             }
             q = block_reserve(&ctl->nact, __popc(on));
         }
-        for (unsigned m = chg; m; m &= m - 1) {
+        if (DENSE) {
+#pragma unroll
+            for (int k = 0; k < IP; ++k) {
+                const long long i = i0 + (long long)k * blockDim.x;
+                if (chg >> k & 1u) a.rep[L ? L[i] : (int)i] = nr[k];
+            }
+        }
+        for (unsigned m = DENSE ? on : chg; m; m &= m - 1) {
             const int k = __ffs(m) - 1;
             const int pk = p[k];
             const long long i = i0 + (long long)k * blockDim.x;
@@ -2158,7 +2186,7 @@ __device__ __forceinline__ void refresh_pass(Ctl *ctl, const FinishArgs &a, cons
                 a.aroot[q] = pk;      // the piece root
                 ++q;
             }
-            a.rep[v] = a.newrep[pk];
+            if (!DENSE) a.rep[v] = a.newrep[pk];
         }
     }
 }
@@ -2249,11 +2277,13 @@ __global__ void __launch_bounds__(BLK, 5) k_finish(Ctl *ctl, FinishArgs a) {
     if (ctl->ner == 0) return;   // no piece was merged
     const bool marks = a.euler || *(volatile int *)&ctl->nlong;
     if (ctl->op == DRSF_DELETE && ctl->td && !*(volatile int *)&ctl->need_root)
-        refresh_pass<IPT>(ctl, a, a.A, (long long)ctl->naff, ep, marks);
+        refresh_pass<IPT, true>(ctl, a, a.A, (long long)ctl->naff, ep, marks);
     else if (a.n <= gstride() * IPT)
-        refresh_pass<IPT>(ctl, a, nullptr, a.n, ep, marks);
+        refresh_pass<IPT, false>(ctl, a, nullptr, a.n, ep, marks);
+    else if (ctl->op == DRSF_DELETE)
+        refresh_pass<IPD, true>(ctl, a, nullptr, a.n, ep, marks);
     else
-        refresh_pass<IPN>(ctl, a, nullptr, a.n, ep, marks);
+        refresh_pass<IPN, false>(ctl, a, nullptr, a.n, ep, marks);
     if (a.euler || !marks) return;
     if (!grid_barrier(ctl, &ctl->bar[3])) return;
     const long long na = (long long)*(volatile u64 *)&ctl->nact;
@@ -2320,9 +2350,18 @@ unsigned coop_blocks_replace(int nsm) {
     return (unsigned)nsm;   // one block per SM (threads and registers)
 }
 
-cudaError_t launch_begin(Ctl *ctl, BeginArgs a, cudaStream_t s) {
-    k_begin<<<gsz(a.len), BLK, 0, s>>>(ctl, a);
+cudaError_t launch_begin(Ctl *ctl, BeginArgs a, long long grid_len, cudaStream_t s) {
+    k_begin<<<gsz(grid_len), BLK, 0, s>>>(ctl, a);
     return cudaGetLastError();
+}
+cudaError_t set_begin(cudaGraphExec_t exec, cudaGraphNode_t node, Ctl *ctl, BeginArgs a, long long grid_len) {
+    void *args[] = {(void *)&ctl, (void *)&a};
+    cudaKernelNodeParams p = {};
+    p.func = (void *)k_begin;
+    p.gridDim = dim3(gsz(grid_len));
+    p.blockDim = dim3(BLK);
+    p.kernelParams = args;
+    return cudaGraphExecKernelNodeSetParams(exec, node, &p);
 }
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
                                unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s) {

@@ -163,6 +163,7 @@ __global__ void k_fill(const u64 *dkey, const u64 *dslot, const int2 *place, lon
 // Insert, step 1 (batch normalisation): drop self-loops, repeated pairs and
 // edges already in G; claim an index slot for each new edge.
 __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->base = ctl->epoch;
     if (batch_skipped(ctl)) return;
     const int *batch = ctl->batch;
     const long long len = ctl->batch_len;
@@ -283,6 +284,7 @@ __global__ void k_ins_place(const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, 
 // vertex becomes a piece root.
 __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl, PieceSlots ps,
                             int *cutlist) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->base = ctl->epoch;
     if (batch_skipped(ctl)) return;
     const int *batch = ctl->batch;
     const long long len = ctl->batch_len;

@@ -111,11 +111,13 @@ struct BeginArgs {
     int op, n;
     long long len;
     const int *batch;
-    unsigned epoch;
     int groups;                    // graphs with a slice of the batch and a vertex range each; 0: none
     const long long *voff, *boff;  // their offsets (groups + 1)
 };
-cudaError_t launch_begin(Ctl *ctl, BeginArgs a, cudaStream_t s);
+// (grid_len sizes the grid)
+cudaError_t launch_begin(Ctl *ctl, BeginArgs a, long long grid_len, cudaStream_t s);
+// the same launch's node in an instantiated graph, for another batch
+cudaError_t set_begin(cudaGraphExec_t exec, cudaGraphNode_t node, Ctl *ctl, BeginArgs a, long long grid_len);
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
                                unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s);
 // delete: detached vertices top-down from the cut vertices (falls back to
@@ -252,7 +254,6 @@ struct BDesc {               // per call
     const int *order;        // graphs in queue order, class by class
     int G;
     int op;
-    unsigned epoch;
 };
 struct BState {              // device pointers of one handle (per call)
     Ctl *ctl;
