@@ -135,7 +135,7 @@ struct drsf_ctx {
 enum {
     PH_BEGIN = 0,     // k_begin + id validation
     PH_INS_CLAIM,     // insert: normalisation + index claim
-    PH_INS_PLACE,     // insert: CSR append + cross test
+    PH_INS_PLACE,     // insert: CSR append + cross test (small batches: and the claim)
     PH_DEL_CLAIM,     // delete: normalisation, removal, tree-edge cut
     PH_AFF,           // delete: affected-vertex list (selectable root searches)
     PH_JUMP,          // large delete: pieces (representatives)
@@ -725,13 +725,17 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     const bool wide = glen > (1 << 16);   // the replacement kernel's form
     if (op == DRSF_INSERT) {
         // Algorithm 1, insert: F^ = F, M = B; rep of the previous batch is current
-        prof_begin(h, PH_INS_CLAIM, s);
-        CK(launch_ins_claim(glen, h->ix, ctl, h->nkey, h->nslot, s));
-        prof_end(h, PH_INS_CLAIM, 1, s);
+        const PlaceArgs pa{g,          h->ix,    h->ovf,      h->ovf_cap,    h->rep,
+                           h->pt,      h->ck[0], h->ca[0],    h->cb[0],      h->cand_cap,
+                           hook_slots(h), wide ? SMALL_CAND_LARGE : SMALL_CAND};
+        if (glen > SMALL_INSERT) {
+            prof_begin(h, PH_INS_CLAIM, s);
+            CK(launch_ins_claim(glen, h->ix, ctl, h->nkey, h->nslot, s));
+            prof_end(h, PH_INS_CLAIM, 1, s);
+        }
         prof_begin(h, PH_INS_PLACE, s);
-        CK(launch_ins_place(h->dev, h->nkey, h->nslot, ctl, g, h->ix, h->ovf, h->ovf_cap, h->rep, sg, h->pt,
-                            h->ck[0], h->ca[0], h->cb[0], h->cand_cap, hook_slots(h), wide ? SMALL_CAND_LARGE : SMALL_CAND,
-                            s));
+        if (glen > SMALL_INSERT) CK(launch_ins_place(h->dev, h->nkey, h->nslot, ctl, pa, sg, s));
+        else CK(launch_ins_small(glen, ctl, pa, sg, s));
         prof_end(h, PH_INS_PLACE, 1, s);
     } else {
         // Algorithm 1, delete: remove B, cut tree edges, re-label the cut trees

@@ -74,11 +74,24 @@ struct PairTable {
 // sg: supergraph variant (pair-table dedupe to one minimum-key edge per
 // pair of trees), else every cross edge is a candidate (hooking variant)
 cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *nslot, cudaStream_t s);
-// (HS: the hook-forest slots of more than `small` candidates are set up here,
-// see HookSlots)
-cudaError_t launch_ins_place(const Dev &d, const u64 *nkey, const u64 *nslot, Ctl *ctl, Csr g, Index ix,
-                             u64 *ovf, u64 ovf_cap, const int *rep, bool sg, PairTable pt, u64 *ck, int *ca, int *cb,
-                             u64 cand_cap, HookSlots hs, int small, cudaStream_t s);
+struct PlaceArgs {
+    Csr g;
+    Index ix;
+    u64 *ovf;
+    u64 ovf_cap;
+    const int *rep;
+    PairTable pt;
+    u64 *ck;             // candidates
+    int *ca, *cb;
+    u64 cand_cap;
+    HookSlots hs;
+    int small;           // HS: the slots of more than this many candidates are set up (HookSlots)
+};
+cudaError_t launch_ins_place(const Dev &d, const u64 *nkey, const u64 *nslot, Ctl *ctl, PlaceArgs p, bool sg,
+                             cudaStream_t s);
+// claim and placement in one launch
+#define SMALL_INSERT (1 << 18)
+cudaError_t launch_ins_small(long long len, Ctl *ctl, PlaceArgs p, bool sg, cudaStream_t s);
 struct LightArgs {
     int n;
     Csr g;

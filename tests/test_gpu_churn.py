@@ -72,3 +72,29 @@ def test_window_neither_overflows_nor_rebuilds(batched):
         keys, par, _ = check_batch(f, g.n, keys, par, drsf.INSERT, back)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("flags", [0, drsf.REPL_HS, drsf.REPL_SG], ids=["default", "hs", "sg"])
+@pytest.mark.parametrize("b", [1, 513, 2 ** 18 - 1, 2 ** 18, 2 ** 18 + 1])
+def test_claim_and_place_around_the_one_launch_limit(b, flags):
+    """Inserts around the 2^18 edges up to which one launch claims and places
+    them: repeats in both directions, self-loops, edges that exist, rows that
+    overflow; the edges go in a second time (all dropped) and out again."""
+    n = 60_000
+    g = workloads.er_graph(n, n // 2, seed=23)
+    rng = np.random.default_rng(b)
+    e = rng.integers(0, n, (b, 2)).astype(np.int32)
+    e[: b // 4, 0] %= 97                                  # full rows: the overflow list
+    q = b // 8
+    e[b - q:] = e[:q, ::-1]                               # repeats, turned round
+    e[q: q + b // 16, 1] = e[q: q + b // 16, 0]           # self-loops
+    e[2 * q: 2 * q + b // 16] = g.edges()[rng.integers(0, g.m, b // 16)]
+    e = rng.permutation(e)
+    f = make_forest(g, flags=drsf.DETERMINISTIC | flags)
+    keys, par = g.keys, g.parent
+    try:
+        for op in (drsf.INSERT, drsf.INSERT, drsf.DELETE):
+            keys, par, _ = check_batch(f, n, keys, par, op, e)
+        assert np.array_equal(workloads.edges_to_keys(f.export_edges().cpu().numpy()), keys)
+    finally:
+        f.close()
