@@ -67,7 +67,7 @@ struct drsf_ctx {
     int *J0 = nullptr, *J1 = nullptr, *comp = nullptr, *minp = nullptr, *pidx = nullptr, *plist = nullptr;
     int *att_x = nullptr, *newrep = nullptr, *A = nullptr, *act = nullptr, *pold = nullptr, *D = nullptr;
     int *chx = nullptr, *chy = nullptr;
-    unsigned *aff_ep = nullptr, *cut_ep = nullptr, *pstamp = nullptr, *att_ep = nullptr, *rep_ep = nullptr;
+    unsigned *aff_ep = nullptr, *pstamp = nullptr, *att_ep = nullptr, *rep_ep = nullptr;
     unsigned *long_ep = nullptr, *hstamp = nullptr;
     unsigned *det_ep = nullptr, *det_claim = nullptr;   // top-down delete stamps
     bool detach = true;                                 // DRSF_DETACH=0 turns the top-down delete off
@@ -529,7 +529,7 @@ static drsf_status alloc_work(drsf_ctx *h, cudaStream_t s) {
     w.add(&h->bsum, 8192);
     // (the epoch stamps and the control block, which start at zero, last)
     const size_t clear = w.total;
-    unsigned **eps[] = {&h->aff_ep, &h->cut_ep, &h->pstamp, &h->att_ep, &h->rep_ep, &h->long_ep, &h->hstamp,
+    unsigned **eps[] = {&h->aff_ep, &h->pstamp, &h->att_ep, &h->rep_ep, &h->long_ep, &h->hstamp,
                         &h->det_ep, &h->det_claim};
     for (unsigned **e : eps) w.add(e, n);
     w.add(&h->ctl, 1);
@@ -770,8 +770,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         la.D = h->D;
         la.job = h->tile;
         la.comp = h->comp;
+        la.root = h->J0;
         la.best = h->best0;
-        la.root_ep = h->cut_ep;
         la.cuts = h->cutlist;
         la.er = h->er;
         la.ovf = h->ovf;

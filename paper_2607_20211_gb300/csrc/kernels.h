@@ -102,8 +102,8 @@ struct LightArgs {
     int *D;                   // the vertices whose rows are read
     int *job;                 // long rows: vertex, part
     int *comp;                // hook forest of the pieces
+    int *root;                // per cut vertex, while the hook forest is flattened: its root
     u64 *best;                // per piece: its minimum cross edge
-    unsigned *root_ep;        // old roots that hooked
     const int *cuts;
     u64 *er;                  // replacement edges
     const u64 *ovf;

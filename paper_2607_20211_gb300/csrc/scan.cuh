@@ -174,6 +174,7 @@ __device__ __forceinline__ void scan_ovf(const u64 *ovf, Ctl *ctl, const int *re
 #define LONG_ROW 32
 #define JOB_LEN 128
 #define LU 8
+#define FLAT_WALK 16
 __device__ __forceinline__ void piece_min(u64 *best, int p, u64 k) {
     if (k < __ldcg(&best[p])) atomicMin(&best[p], k);
 }
@@ -435,8 +436,11 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
     const long long nd = (long long)*(volatile u64 *)&ctl->ndet;
     if (!light_pass<true, SG>(ctl, a, nd, bar)) return;
     if (!grid_barrier(ctl, bar)) return;
-    // every scanned piece: the cut vertices' pieces and, once per tree, the
-    // root piece (block-uniform loop: the edges are appended per block)
+    // every scanned piece: the cut vertices' pieces and, where a detached piece
+    // is left out in its place, the root piece, by the thread that meets the
+    // one left out (a cut vertex like the others; when every cut asked its old
+    // root's stamp, all warps went to one sector).  Block-uniform loop: the
+    // edges are appended per block.
     for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nc; b0 += (long long)gridDim.x * blockDim.x) {
         const long long i = b0 + threadIdx.x;
         bool h1 = false, h2 = false;
@@ -444,7 +448,7 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
         if (i < nc) {
             const int c = a.cuts[i], r = a.rold[c], l = a.left[r];
             if (c != l) h1 = light_hook(a, c, &k1);
-            if (l != r && __ldcg(&a.root_ep[r]) != ep && atomicExch(&a.root_ep[r], ep) != ep) h2 = light_hook(a, r, &k2);
+            else h2 = light_hook(a, r, &k2);
         }
         const long long q1 = block_append(&ctl->ner, h1);
         if (h1) a.er[q1] = k1;
@@ -454,20 +458,27 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
         }
     }
     if (!grid_barrier(ctl, bar)) return;
-    // flatten: first the paths are shortened (walks that halve them), then
-    // every piece gets its root by a read-only walk (a walk that halved paths
-    // could put an older ancestor back where the piece's own thread wrote the
-    // root)
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x)
-        find_root(a.comp, a.cuts[i], ctl);
+    // flatten: every piece's root is found by a walk that writes nothing (a
+    // path of more than FLAT_WALK steps is halved as it is walked) and kept
+    // aside; after a barrier it is stored.  (Walks that halved every path, and
+    // stores of roots beside walks that were still reading, made each other's
+    // loads miss: R-MAT scale 20, 1M deletes, 500K pieces, paths of at most 6
+    // steps: the whole scan 694 us so, 545 in this way.)
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
+        int x = __ldcg(&a.comp[a.cuts[i]]);
+        bool at = false;
+        for (int h = 0; h < FLAT_WALK && !at; ++h) {
+            const int p = __ldcg(&a.comp[x]);
+            at = p == x;
+            x = p;
+        }
+        a.root[i] = at ? x : find_root(a.comp, x, ctl);
+    }
     if (!grid_barrier(ctl, bar)) return;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
         const int c = a.cuts[i], r = a.rold[c];
-        a.comp[c] = find_root_ro(a.comp, c, ctl);
-        if (a.left[r] != r) {   // (one store: every cut of the tree comes here)
-            const int up = __ldcg(&a.comp[r]), root = find_root_ro(a.comp, up, ctl);
-            if (root != up) a.comp[r] = root;
-        }
+        a.comp[c] = a.root[i];
+        if (c == a.left[r]) a.comp[r] = find_root_ro(a.comp, r, ctl);
     }
     if (!grid_barrier(ctl, bar)) return;
     light_pass<false, SG>(ctl, a, nd, bar);

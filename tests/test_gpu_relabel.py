@@ -97,3 +97,24 @@ def test_list_room_for_every_grid(n):
         check_batch(f, n, keys, par, drsf.DELETE, more)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("depth", [1, 2, 15, 16, 17, 18, 19, 33, 1000, 39_999])
+def test_hook_paths_around_the_read_only_walk(depth, monkeypatch):
+    """Every vertex of a star is cut off at once and hooks to the vertex before
+    it: paths of `depth` hooks, around the 16 steps that a walk takes before it
+    halves its path, and one of all pieces."""
+    monkeypatch.setenv("DRSF_DETACH", "0")
+    n = 40_001
+    v = np.arange(1, n)
+    star = np.stack([np.zeros(n - 1, np.int64), v], 1)
+    path = np.stack([v[:-1], v[1:]], 1)
+    path = path[(v[:-1] % (depth + 1)) != 0]
+    g = _tiny_graph(n, np.concatenate([star, path]).tolist(), [0] * n)
+    f = make_forest(g)
+    try:
+        keys, par, st = check_batch(f, n, g.keys, g.parent, drsf.DELETE, star)
+        assert st["tree_cut"] == n - 1
+        check_batch(f, n, keys, par, drsf.INSERT, star)
+    finally:
+        f.close()
