@@ -576,9 +576,13 @@ __device__ __forceinline__ void heaviest_pieces(const int *cuts, long long nc, c
 //      writes here, and leaves the ancestor it reached, or its root
 //      complemented, in J;
 //   2. after a grid barrier each warp's vertices still open (deep trees) go on
-//      by asynchronous pointer doubling in place, J[v] <- J[J[v]]: a pointer
-//      only ever moves to an ancestor, whatever mix of old and new values a
-//      step reads, so every step moves an open vertex up at least one level;
+//      by asynchronous pointer jumping in place, RELABEL_STEPS pointers at
+//      once: a pointer only ever moves to an ancestor, whatever mix of old and
+//      new values a step reads, so every step moves an open vertex up at least
+//      one level (one pointer a step, J[v] <- J[J[v]], is as many loads in all
+//      but more passes over the lists and stores that others' loads miss on:
+//      the 4096 x 4096 grid's 16M vertices 550 us, three 456, five 462, seven
+//      475);
 //   3. the vertices whose root changed (the detached ones; on R-MAT a few
 //      percent) get their new representative and are listed;
 //   4. every cut tree gets the piece that the scan for cross edges leaves out:
@@ -592,6 +596,7 @@ __device__ __forceinline__ void heaviest_pieces(const int *cuts, long long nc, c
 // whole list took 38 + 99 us of a 100K-edge delete batch on R-MAT scale 22
 // (2.5M affected vertices, 100K detached).
 #define RELABEL_HOPS 4
+#define RELABEL_STEPS 3
 #define RI 4   // vertices per lane and iteration
 
 // Piece counts of a block: a small open-addressing table in shared memory (one
@@ -716,7 +721,10 @@ __device__ bool relabel(Ctl *ctl, const RelabelArgs &a) {
 #pragma unroll
             for (int k = 0; k < RI; ++k) w[k] = v[k] >= 0 ? LD(a.J[v[k]]) : -1;
 #pragma unroll
-            for (int k = 0; k < RI; ++k) w[k] = w[k] >= 0 ? LD(a.J[w[k]]) : -1;
+            for (int h = 0; h < RELABEL_STEPS; ++h) {
+#pragma unroll
+                for (int k = 0; k < RI; ++k) w[k] = w[k] >= 0 ? LD(a.J[w[k]]) : w[k];
+            }
 #pragma unroll
             for (int k = 0; k < RI; ++k) {
                 const bool ok = v[k] >= 0, op = ok && w[k] >= 0;
