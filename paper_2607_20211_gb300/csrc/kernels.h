@@ -102,7 +102,8 @@ struct LightArgs {
     int *D;                   // the vertices whose rows are read
     int *job;                 // long rows: vertex, part
     int *comp;                // hook forest of the pieces
-    int *root;                // per cut vertex, while the hook forest is flattened: its root
+    int *root;                // per cut vertex, while the hook forest is flattened: its root; then the rows
+                              // read again
     u64 *best;                // per piece: its minimum cross edge
     const int *cuts;
     u64 *er;                  // replacement edges

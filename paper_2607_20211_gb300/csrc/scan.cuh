@@ -256,10 +256,11 @@ __device__ __forceinline__ u64 light_entries(Ctl *ctl, const LightArgs &a, const
 
 // One pass over the listed rows and the overflow edges (step 1 or 3).  Step 1
 // keeps which rows have a cross edge, one bit each, and step 3 reads only
-// those again (in the 4096 x 4096 grid's pieces a third).  Vertex, piece and
-// row head, and what the piece says are loaded up to three rows ahead.
+// those again (in the 4096 x 4096 grid's pieces a third; with `again`, the
+// list of those that are in no component of a piece left out).  Vertex, piece
+// and row head, and what the piece says are loaded up to three rows ahead.
 template <bool FIND, bool SG>
-__device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long long nd, u64 *bar) {
+__device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long long nd, u64 *bar, bool again = false) {
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -267,8 +268,9 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
     const long long nb = (nd + 31) >> 5;
     auto vertex = [&](long long b) {
         if (b >= nb || b * 32 + lane >= nd) return -1;
-        if (!FIND && !(__ldcg(&a.rows[b]) >> lane & 1u)) return -1;
-        return __ldcg(&a.D[b * 32 + lane]);
+        if (FIND) return __ldcg(&a.D[b * 32 + lane]);
+        if (again) return __ldcg(&a.root[b * 32 + lane]);
+        return __ldcg(&a.rows[b]) >> lane & 1u ? __ldcg(&a.D[b * 32 + lane]) : -1;
     };
     LightRow r0, r1;
     light_head(a, r0, vertex(warp));
@@ -397,6 +399,41 @@ __device__ __forceinline__ bool light_hook(const LightArgs &a, int q, u64 *key) 
     return true;
 }
 
+// Lists the rows that step 3 reads: those with a cross edge whose component
+// does not hold the piece left out.  From AGAIN_MIN rows on: few rows of many
+// are left (one in ten of those with a cross edge in the 4096 x 4096 grid), and
+// a warp that met one of them among its 32 read it alone.  Scan, us: the grid
+// 404 -> 348, the 256-graph union 635 -> 521, R-MAT scale 20 (1M deletes)
+// 554 -> 524; a list of 100K rows (R-MAT scale 22) keeps too few blocks busy:
+// 72 us without it, 92 with.
+#define AGAIN_MIN (1 << 19)
+__device__ __forceinline__ void list_again(Ctl *ctl, const LightArgs &a, long long nd) {
+    const long long step = (long long)blockDim.x * LU;
+    for (long long b0 = blockIdx.x * step; b0 < nd; b0 += gridDim.x * step) {
+        int v[LU], p[LU], l[LU], cp[LU];
+        unsigned in = 0;
+#pragma unroll
+        for (int u = 0; u < LU; ++u) {
+            const long long i = b0 + u * blockDim.x + threadIdx.x;
+            v[u] = i < nd && (__ldcg(&a.rows[i >> 5]) >> (i & 31) & 1u) ? __ldcg(&a.D[i]) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < LU; ++u) p[u] = v[u] >= 0 ? __ldcg(&a.rep[v[u]]) : -1;
+#pragma unroll
+        for (int u = 0; u < LU; ++u) {
+            l[u] = p[u] >= 0 ? a.left[p[u]] : -1;
+            cp[u] = p[u] >= 0 ? __ldcg(&a.comp[p[u]]) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < LU; ++u)
+            if (p[u] >= 0 && __ldcg(&a.comp[l[u]]) != cp[u]) in |= 1u << u;
+        long long q = block_reserve(&ctl->nagain, __popc(in));
+#pragma unroll
+        for (int u = 0; u < LU; ++u)
+            if (in >> u & 1u) a.root[q++] = v[u];
+    }
+}
+
 // The scan of a row list (top-down deletes, selectable root searches).
 template <bool SG>
 __device__ __forceinline__ void scan_listed(Ctl *ctl, const RowList &rl, const LightArgs &a) {
@@ -481,6 +518,12 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
         if (c == a.left[r]) a.comp[r] = find_root_ro(a.comp, r, ctl);
     }
     if (!grid_barrier(ctl, bar)) return;
-    light_pass<false, SG>(ctl, a, nd, bar);
+    if (nd < AGAIN_MIN) {
+        light_pass<false, SG>(ctl, a, nd, bar);
+    } else {
+        list_again(ctl, a, nd);
+        if (!grid_barrier(ctl, bar)) return;
+        light_pass<false, SG>(ctl, a, (long long)*(volatile u64 *)&ctl->nagain, bar, true);
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->pre = 1;
 }

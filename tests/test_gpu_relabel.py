@@ -118,3 +118,25 @@ def test_hook_paths_around_the_read_only_walk(depth, monkeypatch):
         check_batch(f, n, keys, par, drsf.INSERT, star)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("detached", [2 ** 19 - 1, 2 ** 19, 2 ** 19 + 2049])
+def test_second_reading_around_its_list(detached):
+    """2^19 listed rows and more are listed anew before they are read again:
+    a star cut at every edge, whose vertices keep random edges among them
+    (hubs with rows in parts too)."""
+    n = detached + 1
+    rng = np.random.default_rng(detached)
+    v = np.arange(1, n)
+    star = np.stack([np.zeros(n - 1, np.int64), v], 1)
+    e = rng.integers(1, n, (n, 2))
+    e[: n // 8, 0] = 1 + e[: n // 8, 0] % 50
+    e = e[e[:, 0] != e[:, 1]]
+    keys = np.unique(workloads.edges_to_keys(np.concatenate([star, np.sort(e, 1)])))
+    g = _tiny_graph(n, workloads.keys_to_edges(keys).tolist(), [0] * n)
+    f = make_forest(g)
+    try:
+        _, _, st = check_batch(f, n, g.keys, g.parent, drsf.DELETE, star)
+        assert st["tree_cut"] == detached
+    finally:
+        f.close()
