@@ -966,6 +966,12 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     };
     // per-phase profiling brackets the phases with events: launch directly
     if (h->prof_on || !h->graphs_ok) return direct();
+    // a stream that the caller is capturing records plain launches: its graph
+    // keeps the batch's arguments, which the handle's graphs get before each
+    // replay
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) return direct();
     // otherwise replay the captured sequence for this (storage, op, variant,
     // grid size class of the batch kernels), with its first kernel's
     // arguments set to this batch

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2607_20211_gb300 as drsf
 import workloads
 from tests.gpu_util import check_batch, make_forest
@@ -96,5 +97,41 @@ def test_claim_and_place_around_the_one_launch_limit(b, flags):
         for op in (drsf.INSERT, drsf.INSERT, drsf.DELETE):
             keys, par, _ = check_batch(f, n, keys, par, op, e)
         assert np.array_equal(workloads.edges_to_keys(f.export_edges().cpu().numpy()), keys)
+    finally:
+        f.close()
+
+
+@pytest.mark.parametrize("b,detach", [(100, "1"), (5000, "1"), (5000, "0")])
+def test_batches_captured_by_the_caller(b, detach, monkeypatch):
+    """The caller captures an insert and a delete after the handle has captured
+    both shapes itself, runs other batches, and replays its graph on new
+    contents of the captured buffer."""
+    monkeypatch.setenv("DRSF_DETACH", detach)
+    n = 50_000
+    g = workloads.er_graph(n, 100_000, seed=31)
+    f = make_forest(g)
+    keys, par = g.keys, g.parent
+    buf = torch.empty((b, 2), dtype=torch.int32, device="cuda")
+    rng = np.random.default_rng(b)
+    try:
+        for c in range(3):
+            batch = workloads.insert_batch(n, keys, b, 50 + c)
+            for op in (drsf.INSERT, drsf.DELETE):
+                keys, par, _ = check_batch(f, n, keys, par, op, batch, labels=False)
+        graphs = {}
+        for op in (drsf.INSERT, drsf.DELETE):
+            graphs[op] = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graphs[op]):
+                f.apply(op, buf)
+        for c in range(3):
+            for op in (drsf.INSERT, drsf.DELETE):
+                batch = (workloads.insert_batch(n, keys, b, 70 + c) if op == drsf.INSERT
+                         else workloads.keys_to_edges(rng.permutation(keys)[:b]))
+                buf.copy_(torch.from_numpy(np.ascontiguousarray(batch, np.int32)))
+                graphs[op].replay()
+                ref = oracle.apply(n, keys, par, op, batch, want_keys=True)
+                assert np.array_equal(f.parent().cpu().numpy(), ref.parent)
+                keys, par = ref.keys, ref.parent
+                keys, par, _ = check_batch(f, n, keys, par, op, batch[:50], labels=False)
     finally:
         f.close()
