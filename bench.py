@@ -359,9 +359,14 @@ def run_ours(args, rank, ws, local):
     # algorithmic byte model over the same K steps
     pbytes = {}
     opbytes = {"insert": {}, "delete": {}}
+    # a phase without launches of its own is part of another's kernel
+    within = {"ins_claim": "ins_place", "affected": "jump", "jump": "scan", "orient": "hook", "reverse": "hook",
+              "mark": "active"}
     for k in range(K):
         for op, oname in ((0, "insert"), (1, "delete")):
             for ph, by in phase_bytes(steps[W + k][op][1], g.n, op).items():
+                while ph in within and prof[oname].get(ph, (0.0, 0))[1] == 0:
+                    ph = within[ph]
                 pbytes[ph] = pbytes.get(ph, 0) + by
                 opbytes[oname][ph] = opbytes[oname].get(ph, 0) + by
     phases = {}

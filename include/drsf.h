@@ -128,10 +128,13 @@ typedef struct {
     int64_t detached;      /* rows scanned for cross edges: vertices of cut trees
                               outside the piece left out of the scan, the root
                               piece unless a detached piece has 4096 more
-                              vertices, then the heaviest piece (delete) */
+                              vertices, then the heaviest piece, whose
+                              vertices are counted too (delete) */
     int64_t scanned;       /* adjacency entries scanned for cross edges */
-    int64_t candidates;    /* cross edges found */
-    int64_t hook_rounds;   /* hook-and-compress rounds */
+    int64_t candidates;    /* cross edges found; deletes without the top-down
+                              search: those left when every scanned piece has
+                              hooked along its smallest one */
+    int64_t hook_rounds;   /* hook-and-compress rounds over the candidates */
     int64_t replacement;   /* replacement edges |E_r| */
     int64_t rank_rounds;   /* list-ranking rounds of the Euler tour */
     int64_t active;        /* vertices of the re-rooted trees whose path goes
