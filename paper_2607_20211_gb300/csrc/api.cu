@@ -141,7 +141,7 @@ enum {
     PH_JUMP,          // large delete: pieces (representatives)
     PH_SCAN,          // delete: cross-edge scan (small deletes: and the top-down search)
     PH_HOOK,          // replacement edges: hook-and-compress, orientation, path walks
-    PH_ORIENT,        // (part of the above)
+    PH_ORIENT,        // (part of PH_HOOK)
     PH_ACTIVE,        // representative refresh, and the doubling marks and reversal of long paths
     PH_MARK,          // Euler-tour marks
     PH_REVERSE        // large batches: path walks; Euler: reversal scatter + attach

@@ -61,27 +61,6 @@
 // longest path reversed by one walking thread (longer ones: doubling marks)
 #define WALK_MAX 64
 
-// x[k] = a[i0 + k] for k < IP (IP a multiple of 4, i0 a multiple of IP, a
-// 16-byte aligned): vector loads when all IP items are in range.
-template <int IP>
-__device__ __forceinline__ void load_vec(const int *a, long long i0, long long cnt, int (&x)[IP]) {
-    if (i0 + IP <= cnt) {
-#pragma unroll
-        for (int j = 0; j < IP / 4; ++j) {
-            const int4 q = *reinterpret_cast<const int4 *>(a + i0 + 4 * j);
-            x[4 * j] = q.x;
-            x[4 * j + 1] = q.y;
-            x[4 * j + 2] = q.z;
-            x[4 * j + 3] = q.w;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < IP; ++k) x[k] = i0 + k < cnt ? a[i0 + k] : 0;
-    }
-}
-__device__ __forceinline__ void load_ipt(const int *a, long long i0, long long cnt, int (&x)[IPT]) {
-    load_vec<IPT>(a, i0, cnt, x);
-}
 // a detached piece is left out of the cross-edge scan instead of its tree's
 // root piece only if it has this many more vertices (the swap costs a full
 // pass over the affected list)
@@ -595,7 +574,8 @@ __device__ __forceinline__ void heaviest_pieces(const int *cuts, long long nc, c
 //      pieces'.
 // Listing the affected vertices, doubling from distance 1 and a pass over that
 // whole list took 38 + 99 us of a 100K-edge delete batch on R-MAT scale 22
-// (2.5M affected vertices, 100K detached).
+// (2.5M affected vertices, 100K detached); this 65.  Bound by the gathers of
+// the hops, from L2, and by its barriers.
 #define RELABEL_HOPS 4
 #define RELABEL_STEPS 3
 #define RI 4   // vertices per lane and iteration

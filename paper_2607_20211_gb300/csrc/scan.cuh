@@ -163,8 +163,8 @@ __device__ __forceinline__ void scan_ovf(const u64 *ovf, Ctl *ctl, const int *re
 //      one (HS).
 // A batch that detaches much of a graph has more pairs of pieces than the pair
 // table (or a hash table of any size that fits L2) can take: R-MAT scale 20,
-// 1M deletes, 4.1M pairs; scan and hooking 1,410 + 1,120 us.  Few of them are
-// left after the first round.
+// 1M deletes, 4.1M pairs; scan and hooking 1,410 + 1,120 us, 437 + 330 in this
+// way.  Few of them are left after the first round.
 //
 // A lane reads a row of up to LONG_ROW entries by itself, LU entries in flight
 // (flattening the rows of a warp by a prefix sum and reading 32 entries per
