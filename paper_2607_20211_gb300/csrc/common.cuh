@@ -85,7 +85,7 @@ struct Ctl {
     int td;                 // delete: the detached vertices were found top-down (else: pointer jumping)
     int need_root;          // delete: a cut tree's root piece is re-rooted (read after a top-down delete)
     int njobs;              // delete: parts of long rows to read
-    u64 nagain;             // large delete: rows read again
+    u64 nagain[2];          // large delete: rows read again, after the first and a second round
     int pre;                // delete: the first hooking round was taken from the rows (k_scan)
     int nlong;              // some path was too long to be reversed by its walk
     long long det_levels;   // top-down levels of the batch (0: not taken)

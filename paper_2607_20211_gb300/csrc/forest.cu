@@ -123,7 +123,7 @@ __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
     ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
     ctl->jump_visits = 0;
-    ctl->nagain = 0;
+    ctl->nagain[0] = ctl->nagain[1] = 0;
     ctl->td = ctl->need_root = ctl->nlong = ctl->njobs = ctl->pre = 0;
     if (ctl->det_skip) {   // the last batch skipped the top-down search
         if (ctl->depth_hint > 0) ctl->depth_hint -= 1;

@@ -157,7 +157,8 @@ __device__ __forceinline__ void scan_ovf(const u64 *ovf, Ctl *ctl, const int *re
 //      out, whose rows are not read, need not choose.
 //   3. The hook forest of the pieces is flattened and the rows of every
 //      component without the piece left out are read once more (on R-MAT most
-//      pieces hang under that one by now): the cross edges that still join two
+//      pieces hang under that one by now; where most do not, after a second
+//      round from the rows): the cross edges that still join two
 //      components are the candidates of the rounds that follow (k_replace),
 //      reduced per pair of components through the pair table (SG) or one by
 //      one (HS).
@@ -175,6 +176,9 @@ __device__ __forceinline__ void scan_ovf(const u64 *ovf, Ctl *ctl, const int *re
 #define JOB_LEN 128
 #define LU 8
 #define FLAT_WALK 16
+// what a pass over the rows does: step 1's minima per piece, a further round's
+// minima per component, or the candidates left
+enum { FIND = 0, AGAIN = 1, EMIT = 2 };
 __device__ __forceinline__ void piece_min(u64 *best, int p, u64 k) {
     if (k < __ldcg(&best[p])) atomicMin(&best[p], k);
 }
@@ -195,19 +199,18 @@ __device__ __forceinline__ void light_head(const LightArgs &a, LightRow &r, int 
 }
 // Step 1 skips the piece left out, step 3 its whole component: another
 // component's cross edges are all in its own rows.
-template <bool FIND>
+template <int MODE>
 __device__ __forceinline__ void light_piece(const LightArgs &a, LightRow &r) {
     r.lp = r.cp = 0;
     r.best = EMPTY_KEY;
     if (r.v < 0) return;
     r.lp = a.left[r.p];
     r.cp = r.p;
-    if (FIND) {
-        r.best = __ldcg(&a.best[r.p]);
-    } else {
+    if (MODE != FIND) {
         r.cp = __ldcg(&a.comp[r.p]);
         r.lp = __ldcg(&a.comp[r.lp]);
     }
+    if (MODE != EMIT) r.best = __ldcg(&a.best[r.cp]);
     if (r.cp == r.lp) r.used = 0;
 }
 // A cross edge of step 3, seen from component cv: appended to the candidates
@@ -226,9 +229,9 @@ __device__ __forceinline__ void light_emit(Ctl *ctl, const LightArgs &a, bool ra
         atomicOr(&ctl->err, ERR_CAPACITY);
     }
 }
-// Entries at, at + step, ... (LU of them, below `used`) of row r: FIND, the
-// minimum of their cross edges; else they are emitted.
-template <bool FIND, bool SG>
+// Entries at, at + step, ... (LU of them, below `used`) of row r: the minimum of
+// their cross edges, or (EMIT) they are emitted.
+template <int MODE, bool SG>
 __device__ __forceinline__ u64 light_entries(Ctl *ctl, const LightArgs &a, const LightRow &r, int at, int step) {
     int x[LU], rx[LU];
     u64 k = EMPTY_KEY;
@@ -236,11 +239,19 @@ __device__ __forceinline__ u64 light_entries(Ctl *ctl, const LightArgs &a, const
     for (int u = 0; u < LU; ++u) x[u] = at + u * step < r.used ? a.g.col[(size_t)r.st + at + u * step] : -1;
 #pragma unroll
     for (int u = 0; u < LU; ++u) rx[u] = x[u] >= 0 ? a.rep[x[u]] : r.p;
-    if (FIND) {
+    if (MODE == FIND) {
 #pragma unroll
         for (int u = 0; u < LU; ++u) {
             const u64 key = ekey((uint32_t)r.v, (uint32_t)x[u]);
             if (rx[u] != r.p && key < k) k = key;
+        }
+    } else if (MODE == AGAIN) {
+#pragma unroll
+        for (int u = 0; u < LU; ++u) rx[u] = rx[u] != r.p ? __ldcg(&a.comp[rx[u]]) : r.cp;
+#pragma unroll
+        for (int u = 0; u < LU; ++u) {
+            const u64 key = ekey((uint32_t)r.v, (uint32_t)x[u]);
+            if (rx[u] != r.cp && key < k) k = key;
         }
     } else {
 #pragma unroll
@@ -259,8 +270,8 @@ __device__ __forceinline__ u64 light_entries(Ctl *ctl, const LightArgs &a, const
 // those again (in the 4096 x 4096 grid's pieces a third; with `again`, the
 // list of those that are in no component of a piece left out).  Vertex, piece
 // and row head, and what the piece says are loaded up to three rows ahead.
-template <bool FIND, bool SG>
-__device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long long nd, u64 *bar, bool again = false) {
+template <int MODE, bool SG>
+__device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long long nd, u64 *bar, bool again) {
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -268,22 +279,22 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
     const long long nb = (nd + 31) >> 5;
     auto vertex = [&](long long b) {
         if (b >= nb || b * 32 + lane >= nd) return -1;
-        if (FIND) return __ldcg(&a.D[b * 32 + lane]);
+        if (MODE == FIND) return __ldcg(&a.D[b * 32 + lane]);
         if (again) return __ldcg(&a.root[b * 32 + lane]);
         return __ldcg(&a.rows[b]) >> lane & 1u ? __ldcg(&a.D[b * 32 + lane]) : -1;
     };
     LightRow r0, r1;
     light_head(a, r0, vertex(warp));
-    light_piece<FIND>(a, r0);
+    light_piece<MODE>(a, r0);
     light_head(a, r1, vertex(warp + nw));
     int v2 = vertex(warp + 2 * nw);
     for (long long b = warp; b < nb; b += nw) {
         const int v3 = vertex(b + 3 * nw);
         LightRow r2;
         light_head(a, r2, v2);
-        light_piece<FIND>(a, r1);
+        light_piece<MODE>(a, r1);
         const bool big = r0.used > LONG_ROW;
-        if (FIND) {
+        if (MODE == FIND) {
             read += r0.used;
             unsigned bm = __ballot_sync(0xffffffffu, big);
             if (bm) {
@@ -313,21 +324,21 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
         const int most = __reduce_max_sync(0xffffffffu, r0.used);
         u64 k = EMPTY_KEY;
         for (int at = 0; at < most; at += LU) {
-            const u64 e = light_entries<FIND, SG>(ctl, a, r0, at, 1);
+            const u64 e = light_entries<MODE, SG>(ctl, a, r0, at, 1);
             k = e < k ? e : k;
         }
-        if (FIND) {
+        if (MODE != EMIT) {
             const bool hit = k != EMPTY_KEY;
             const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (lane == 0) a.rows[b] = m;
+            if (MODE == FIND && lane == 0) a.rows[b] = m;
             if (m) {
                 // rows of one piece combine first (a large piece's rows fill warps)
-                const int p0 = __shfl_sync(0xffffffffu, r0.p, __ffs(m) - 1);
-                if (__all_sync(0xffffffffu, !hit || r0.p == p0)) {
+                const int p0 = __shfl_sync(0xffffffffu, r0.cp, __ffs(m) - 1);
+                if (__all_sync(0xffffffffu, !hit || r0.cp == p0)) {
                     k = group_min_u64(0xffffffffu, k);
                     if (lane == __ffs(m) - 1 && k < r0.best) atomicMin(&a.best[p0], k);
                 } else if (hit && k < r0.best) {
-                    atomicMin(&a.best[r0.p], k);
+                    atomicMin(&a.best[r0.cp], k);
                 }
             }
         }
@@ -335,7 +346,7 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
         r1 = r2;
         v2 = v3;
     }
-    if (FIND && !grid_barrier(ctl, bar)) return false;   // the jobs are all listed
+    if (MODE == FIND && !grid_barrier(ctl, bar)) return false;   // the jobs are all listed
     const long long nj = *(volatile int *)&ctl->njobs;
     auto job = [&](long long t) {
         return t < nj ? __ldcg(reinterpret_cast<const int2 *>(&a.job[2 * t])) : make_int2(-1, 0);
@@ -344,24 +355,24 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
     light_head(a, r0, j0.x);
     for (long long t = warp; t < nj; t += nw) {
         const int2 j2 = job(t + 2 * nw);
-        light_piece<FIND>(a, r0);
+        light_piece<MODE>(a, r0);
         light_head(a, r1, j1.x);
         const int at = j0.y * JOB_LEN;
         r0.used = min(r0.used, at + JOB_LEN);
         u64 k = EMPTY_KEY;
         for (int i = at; i < r0.used; i += 32 * LU) {
-            const u64 e = light_entries<FIND, SG>(ctl, a, r0, i + lane, 32);
+            const u64 e = light_entries<MODE, SG>(ctl, a, r0, i + lane, 32);
             k = e < k ? e : k;
         }
-        if (FIND) {
+        if (MODE != EMIT) {
             k = group_min_u64(0xffffffffu, k);
-            if (lane == 0 && k < r0.best) atomicMin(&a.best[r0.p], k);
+            if (lane == 0 && k < r0.best) atomicMin(&a.best[r0.cp], k);
         }
         r0 = r1;
         j0 = j1;
         j1 = j2;
     }
-    if (FIND) block_add(&ctl->scanned, read);
+    if (MODE == FIND) block_add(&ctl->scanned, read);
     // edges held outside the rows
     const long long no = (long long)ctl->ovf_count;
     const long long S = (long long)gridDim.x * blockDim.x;
@@ -372,7 +383,7 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
             ra = __ldcg(&a.rep[klo(k)]);
             rb = __ldcg(&a.rep[khi(k)]);
         }
-        if (FIND) {
+        if (MODE == FIND) {
             if (ra == rb) continue;
             // (the piece left out does not choose: its minimum stays empty)
             const int l = a.left[ra];
@@ -380,7 +391,13 @@ __device__ __forceinline__ bool light_pass(Ctl *ctl, const LightArgs &a, long lo
             if (rb != l) piece_min(a.best, rb, k);
         } else {
             const int ca = ra != rb ? __ldcg(&a.comp[ra]) : 0, cb = ra != rb ? __ldcg(&a.comp[rb]) : 0;
-            light_emit<SG>(ctl, a, ca != cb, k, ca, cb);
+            if (MODE == EMIT) {
+                light_emit<SG>(ctl, a, ca != cb, k, ca, cb);
+            } else if (ca != cb) {
+                const int l = __ldcg(&a.comp[a.left[ra]]);
+                if (ca != l) piece_min(a.best, ca, k);
+                if (cb != l) piece_min(a.best, cb, k);
+            }
         }
     }
     return true;
@@ -407,7 +424,16 @@ __device__ __forceinline__ bool light_hook(const LightArgs &a, int q, u64 *key) 
 // 554 -> 524; a list of 100K rows (R-MAT scale 22) keeps too few blocks busy:
 // 72 us without it, 92 with.
 #define AGAIN_MIN (1 << 19)
-__device__ __forceinline__ void list_again(Ctl *ctl, const LightArgs &a, long long nd) {
+// From so many listed rows on, a quarter of all or more, a second round is taken from them, not only the
+// first: most of the graph is in components without the piece left out, and
+// their pairs would fill the pair table (R-MAT scale 20, 1M deletes of a graph
+// that has lost half its tree edges ten times over: 2.5M candidates; scan and
+// hooking 1,400 + 1,320 us, 1,002 + 359 with the round).  With fewer rows the
+// reading costs more than the candidates it saves: at 2^17 the 256-graph
+// union's scan and hooking took 584 + 310 us instead of 521 + 337, the grid's
+// (one row in twenty left) 503 + 185 instead of 347 + 223.
+#define ROUND_MIN (1 << 19)
+__device__ __forceinline__ void list_again(Ctl *ctl, const LightArgs &a, long long nd, u64 *count) {
     const long long step = (long long)blockDim.x * LU;
     for (long long b0 = blockIdx.x * step; b0 < nd; b0 += gridDim.x * step) {
         int v[LU], p[LU], l[LU], cp[LU];
@@ -427,11 +453,86 @@ __device__ __forceinline__ void list_again(Ctl *ctl, const LightArgs &a, long lo
 #pragma unroll
         for (int u = 0; u < LU; ++u)
             if (p[u] >= 0 && __ldcg(&a.comp[l[u]]) != cp[u]) in |= 1u << u;
-        long long q = block_reserve(&ctl->nagain, __popc(in));
+        long long q = block_reserve(count, __popc(in));
 #pragma unroll
         for (int u = 0; u < LU; ++u)
             if (in >> u & 1u) a.root[q++] = v[u];
     }
+}
+
+// The same in a further round, for component q: comp keeps the hooked ones
+// complemented until a barrier (the others go on asking which component a
+// piece is in: a complemented piece is the root of its own).
+__device__ __forceinline__ int light_component(const LightArgs &a, int p) {
+    const int c = __ldcg(&a.comp[p]);
+    return c < 0 ? p : c;
+}
+__device__ __forceinline__ bool light_hook_again(const LightArgs &a, int q, u64 *key) {
+    const u64 k = __ldcg(&a.best[q]);
+    if (k == EMPTY_KEY || __ldcg(&a.comp[q]) != q) return false;
+    const int pa = light_component(a, __ldcg(&a.rep[klo(k)])), pb = light_component(a, __ldcg(&a.rep[khi(k)]));
+    const int o = pa == q ? pb : pa;
+    if (__ldcg(&a.best[o]) == k && q < o) return false;
+    a.comp[q] = ~o;
+    *key = k;
+    return true;
+}
+
+// Hooks every scanned piece (or, AGAIN, every component of them) along its
+// minimum edge: the cut vertices' pieces and, where a detached piece is left
+// out in its place, the root piece, by the thread that meets the one left out
+// (a cut vertex like the others; when every cut asked its old root's stamp, all
+// warps went to one sector).  Block-uniform loop: the edges are appended per
+// block.
+template <int MODE>
+__device__ __forceinline__ void hook_pieces(Ctl *ctl, const LightArgs &a, long long nc) {
+    for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nc; b0 += (long long)gridDim.x * blockDim.x) {
+        const long long i = b0 + threadIdx.x;
+        bool h1 = false, h2 = false;
+        u64 k1 = 0, k2 = 0;
+        if (i < nc) {
+            const int c = a.cuts[i], r = a.rold[c], l = a.left[r];
+            if (MODE == FIND) {
+                if (c != l) h1 = light_hook(a, c, &k1);
+                else h2 = light_hook(a, r, &k2);
+            } else {
+                h1 = light_hook_again(a, c, &k1);
+                if (c == l) h2 = light_hook_again(a, r, &k2);
+            }
+        }
+        const long long q1 = block_append(&ctl->ner, h1);
+        if (h1) a.er[q1] = k1;
+        if (__syncthreads_or(h2)) {
+            const long long q2 = block_append(&ctl->ner, h2);
+            if (h2) a.er[q2] = k2;
+        }
+    }
+}
+
+// Flattens the hook forest: every piece's root is found by a walk that writes
+// nothing (a path of more than FLAT_WALK steps is halved as it is walked) and
+// kept aside; after a barrier it is stored.  (Walks that halved every path, and
+// stores of roots beside walks that were still reading, made each other's
+// loads miss: R-MAT scale 20, 1M deletes, 500K pieces, paths of at most 6
+// steps: the whole scan 694 us so, 545 in this way.)
+__device__ __forceinline__ bool flatten_pieces(Ctl *ctl, const LightArgs &a, long long nc, u64 *bar) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
+        int x = __ldcg(&a.comp[a.cuts[i]]);
+        bool at = false;
+        for (int h = 0; h < FLAT_WALK && !at; ++h) {
+            const int p = __ldcg(&a.comp[x]);
+            at = p == x;
+            x = p;
+        }
+        a.root[i] = at ? x : find_root(a.comp, x, ctl);
+    }
+    if (!grid_barrier(ctl, bar)) return false;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
+        const int c = a.cuts[i], r = a.rold[c];
+        a.comp[c] = a.root[i];
+        if (c == a.left[r]) a.comp[r] = find_root_ro(a.comp, r, ctl);
+    }
+    return grid_barrier(ctl, bar);
 }
 
 // The scan of a row list (top-down deletes, selectable root searches).
@@ -471,59 +572,42 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
         if (!grid_barrier(ctl, bar)) return;
     }
     const long long nd = (long long)*(volatile u64 *)&ctl->ndet;
-    if (!light_pass<true, SG>(ctl, a, nd, bar)) return;
+    if (!light_pass<FIND, SG>(ctl, a, nd, bar, false)) return;
     if (!grid_barrier(ctl, bar)) return;
-    // every scanned piece: the cut vertices' pieces and, where a detached piece
-    // is left out in its place, the root piece, by the thread that meets the
-    // one left out (a cut vertex like the others; when every cut asked its old
-    // root's stamp, all warps went to one sector).  Block-uniform loop: the
-    // edges are appended per block.
-    for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < nc; b0 += (long long)gridDim.x * blockDim.x) {
-        const long long i = b0 + threadIdx.x;
-        bool h1 = false, h2 = false;
-        u64 k1 = 0, k2 = 0;
-        if (i < nc) {
-            const int c = a.cuts[i], r = a.rold[c], l = a.left[r];
-            if (c != l) h1 = light_hook(a, c, &k1);
-            else h2 = light_hook(a, r, &k2);
-        }
-        const long long q1 = block_append(&ctl->ner, h1);
-        if (h1) a.er[q1] = k1;
-        if (__syncthreads_or(h2)) {
-            const long long q2 = block_append(&ctl->ner, h2);
-            if (h2) a.er[q2] = k2;
-        }
-    }
-    if (!grid_barrier(ctl, bar)) return;
-    // flatten: every piece's root is found by a walk that writes nothing (a
-    // path of more than FLAT_WALK steps is halved as it is walked) and kept
-    // aside; after a barrier it is stored.  (Walks that halved every path, and
-    // stores of roots beside walks that were still reading, made each other's
-    // loads miss: R-MAT scale 20, 1M deletes, 500K pieces, paths of at most 6
-    // steps: the whole scan 694 us so, 545 in this way.)
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
-        int x = __ldcg(&a.comp[a.cuts[i]]);
-        bool at = false;
-        for (int h = 0; h < FLAT_WALK && !at; ++h) {
-            const int p = __ldcg(&a.comp[x]);
-            at = p == x;
-            x = p;
-        }
-        a.root[i] = at ? x : find_root(a.comp, x, ctl);
-    }
-    if (!grid_barrier(ctl, bar)) return;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
-        const int c = a.cuts[i], r = a.rold[c];
-        a.comp[c] = a.root[i];
-        if (c == a.left[r]) a.comp[r] = find_root_ro(a.comp, r, ctl);
-    }
+    hook_pieces<FIND>(ctl, a, nc);
     if (!grid_barrier(ctl, bar)) return;
     if (nd < AGAIN_MIN) {
-        light_pass<false, SG>(ctl, a, nd, bar);
+        if (!flatten_pieces(ctl, a, nc, bar)) return;
+        light_pass<EMIT, SG>(ctl, a, nd, bar, false);
     } else {
-        list_again(ctl, a, nd);
+        if (!flatten_pieces(ctl, a, nc, bar)) return;
+        list_again(ctl, a, nd, &ctl->nagain[0]);
         if (!grid_barrier(ctl, bar)) return;
-        light_pass<false, SG>(ctl, a, (long long)*(volatile u64 *)&ctl->nagain, bar, true);
+        long long na = (long long)*(volatile u64 *)&ctl->nagain[0];
+        if (na >= ROUND_MIN && na >= nd / 4) {
+            // another round from the rows: minima per component, which hook
+            for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+                 i += (long long)gridDim.x * blockDim.x) {
+                const int c = a.cuts[i], r = a.rold[c];
+                a.best[c] = EMPTY_KEY;
+                if (c == a.left[r]) a.best[r] = EMPTY_KEY;
+            }
+            if (!grid_barrier(ctl, bar)) return;
+            if (!light_pass<AGAIN, SG>(ctl, a, na, bar, true) || !grid_barrier(ctl, bar)) return;
+            hook_pieces<AGAIN>(ctl, a, nc);
+            if (!grid_barrier(ctl, bar)) return;
+            for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+                 i += (long long)gridDim.x * blockDim.x) {
+                const int c = a.cuts[i], r = a.rold[c], x = __ldcg(&a.comp[c]);
+                if (x < 0) a.comp[c] = ~x;
+                if (c == a.left[r] && __ldcg(&a.comp[r]) < 0) a.comp[r] = ~__ldcg(&a.comp[r]);
+            }
+            if (!grid_barrier(ctl, bar) || !flatten_pieces(ctl, a, nc, bar)) return;
+            list_again(ctl, a, nd, &ctl->nagain[1]);
+            if (!grid_barrier(ctl, bar)) return;
+            na = (long long)*(volatile u64 *)&ctl->nagain[1];
+        }
+        light_pass<EMIT, SG>(ctl, a, na, bar, true);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->pre = 1;
 }

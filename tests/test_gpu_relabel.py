@@ -120,23 +120,28 @@ def test_hook_paths_around_the_read_only_walk(depth, monkeypatch):
         f.close()
 
 
-@pytest.mark.parametrize("detached", [2 ** 19 - 1, 2 ** 19, 2 ** 19 + 2049])
-def test_second_reading_around_its_list(detached):
-    """2^19 listed rows and more are listed anew before they are read again:
-    a star cut at every edge, whose vertices keep random edges among them
-    (hubs with rows in parts too)."""
+@pytest.mark.parametrize("detached,flags", [(2 ** 19 - 1, 0), (2 ** 19, 0), (2 ** 19 + 2049, 0), (2 ** 20 + 1, 0),
+                                            (2 ** 20 + 1, drsf.REPL_HS)])
+def test_second_reading_around_its_list(detached, flags):
+    """2^19 listed rows and more are listed anew before they are read again,
+    and a second round is taken from as many that are left (the last two): a
+    star cut at every edge, whose vertices keep random edges among them (hubs
+    with rows in parts, and edges outside the rows)."""
     n = detached + 1
     rng = np.random.default_rng(detached)
     v = np.arange(1, n)
     star = np.stack([np.zeros(n - 1, np.int64), v], 1)
     e = rng.integers(1, n, (n, 2))
     e[: n // 8, 0] = 1 + e[: n // 8, 0] % 50
-    e = e[e[:, 0] != e[:, 1]]
-    keys = np.unique(workloads.edges_to_keys(np.concatenate([star, np.sort(e, 1)])))
+    e = np.sort(e[e[:, 0] != e[:, 1]], 1)
+    h = len(e) * 7 // 8
+    late = rng.permutation(e)[h:]
+    keys = np.unique(workloads.edges_to_keys(np.concatenate([star, e[:h]])))
     g = _tiny_graph(n, workloads.keys_to_edges(keys).tolist(), [0] * n)
-    f = make_forest(g)
+    f = make_forest(g, flags=drsf.DETERMINISTIC | flags)
     try:
-        _, _, st = check_batch(f, n, g.keys, g.parent, drsf.DELETE, star)
+        keys, par, _ = check_batch(f, n, g.keys, g.parent, drsf.INSERT, late.astype(np.int32), labels=False)
+        _, _, st = check_batch(f, n, keys, par, drsf.DELETE, star)
         assert st["tree_cut"] == detached
     finally:
         f.close()
