@@ -63,6 +63,8 @@ struct Ctl {
     u64 ndet;               // detached list
     u64 ncand;              // candidates
     u64 ner;                // replacement edges
+    u64 npre;               // delete: those of them that the scan chose (k_replace's blocks branch on this
+                            // and on ncand: nothing in that launch writes it, where block 0 counts ner on)
     u64 npc;                // distinct pieces touched by E_r
     u64 nact;               // active vertices (path reversal)
     u64 ncore;              // core arcs of the super-forest Euler tour
@@ -86,7 +88,6 @@ struct Ctl {
     int need_root;          // delete: a cut tree's root piece is re-rooted (read after a top-down delete)
     int njobs;              // delete: parts of long rows to read
     u64 nagain[2];          // large delete: rows read again, after the first and a second round
-    int pre;                // delete: the first hooking round was taken from the rows (k_scan)
     int nlong;              // some path was too long to be reversed by its walk
     long long det_levels;   // top-down levels of the batch (0: not taken)
     long long det_entries;  // adjacency entries the top-down search read

@@ -124,7 +124,8 @@ __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
     ctl->jump_visits = 0;
     ctl->nagain[0] = ctl->nagain[1] = 0;
-    ctl->td = ctl->need_root = ctl->nlong = ctl->njobs = ctl->pre = 0;
+    ctl->td = ctl->need_root = ctl->nlong = ctl->njobs = 0;
+    ctl->npre = 0;
     if (ctl->det_skip) {   // the last batch skipped the top-down search
         if (ctl->depth_hint > 0) ctl->depth_hint -= 1;
         ctl->det_skip = 0;
@@ -2040,7 +2041,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
         if (!grid_barrier(ctl, &ctl->bar[1])) return;
     }
     const long long c0 = (long long)*(volatile u64 *)&ctl->ncand;
-    const long long pre = ctl->pre ? (long long)*(volatile u64 *)&ctl->ner : 0;
+    const long long pre = (long long)ctl->npre;
     if (c0 + pre <= C) {
         if (c0 + pre == 0) return;
         if (blockIdx.x == 0) {

@@ -609,5 +609,6 @@ __device__ void scan_light(Ctl *ctl, const LightArgs &a) {
         }
         light_pass<EMIT, SG>(ctl, a, na, bar, true);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->pre = 1;
+    // (every hooking round ended at a barrier: the count is final)
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->npre = *(volatile u64 *)&ctl->ner;
 }
