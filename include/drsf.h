@@ -212,6 +212,19 @@ DRSF_API drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, con
  * Errors (immediate): DRSF_EINVAL (bad op, negative len, NULL batch with
  * len > 0), DRSF_ENOMEM, DRSF_ECUDA, DRSF_EPOISONED.  An out-of-range id is
  * reported later as DRSF_EINVAL and the batch is skipped.
+ * Recording: on a stream that the caller is capturing, the batch is recorded
+ * (this call and the three after it; host arguments are copied) and each replay
+ * of the caller's graph applies what the device batch then holds, in the order
+ * of the streams and not after drsf_destroy.  A recording allocates and waits
+ * for nothing of the handle's: a batch longer than any before it and than
+ * drsf_reserve's, or an insert that the conservative bounds leave no room for,
+ * is refused with DRSF_ECUDA, the capture going on without it (a plain call
+ * makes room).  A replayed insert that would overfill the storage is skipped
+ * and reported later as DRSF_ENOMEM; a replay after a plain call moved the
+ * storage (a rebuild, or longer buffers) is skipped and reported later as
+ * DRSF_EINVAL: record it again.  Once a batch has been recorded, plain inserts
+ * read the real counts first (one synchronisation), as replays are not in the
+ * host's bounds.
  */
 DRSF_API drsf_status drsf_apply(drsf_handle h, drsf_op op, const int32_t *batch, int64_t len, drsf_stream stream);
 

@@ -36,8 +36,14 @@ struct drsf_ctx {
     bool poisoned = false;
     int jump_sync = 2;   // root search: 2 hops, then asynchronous doubling; 1 synchronous rounds, 0 path halving
     int last_sg = 0;     // the last batch took the supergraph variant
+    // batches that the caller recorded into graphs of its own: the host's
+    // bounds below miss their replays, and their host arguments are kept on
+    // the device until the handle is destroyed
+    bool recorded = false;
+    std::vector<void *> kept;
     // captured per-batch launch sequences (CUDA graphs), valid for storage
     // generation u_gen; gen moves whenever a storage or batch buffer moves
+    // (storage_moved; the control block has it too)
     struct Captured {
         std::string key;
         cudaGraphExec_t exec;
@@ -248,6 +254,41 @@ static void hfree(drsf_ctx *h, T **ptr, cudaStream_t s) {
         if (!(x)) return DRSF_ENOMEM;             \
     } while (0)
 
+// Storage or batch buffers moved: captured launch sequences point into the old
+// ones.  The handle drops its own; a graph of the caller's finds out by the
+// control block (StorageLimits).
+static cudaError_t storage_moved(drsf_ctx *h, cudaStream_t s) {
+    h->gen++;
+    return cudaMemcpyAsync(&h->ctl->storage, &h->gen, sizeof h->gen, cudaMemcpyHostToDevice, s);
+}
+
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+// A device copy of host arguments for a batch that is being recorded: made at
+// once, on a stream of the library's own, and kept until the handle is
+// destroyed (the recording refers to it; a copy recorded from the staging
+// buffers would read whatever a later call left there).
+static drsf_status keep_copy(drsf_ctx *h, const void *src, size_t bytes, void **out) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    void *p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes ? bytes : 16);
+    const bool full = e != cudaSuccess;
+    if (e == cudaSuccess) h->kept.push_back(p);
+    if (e == cudaSuccess && !h->u_cap) e = cudaStreamCreateWithFlags(&h->u_cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, h->u_cap);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->u_cap);
+    if (e != cudaSuccess) cudaGetLastError();
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    if (e != cudaSuccess) return full ? DRSF_ENOMEM : DRSF_ECUDA;
+    *out = p;
+    return DRSF_OK;
+}
+
 static u64 pow2_at_least(u64 x) {
     u64 p = 1024;
     while (p < x) p <<= 1;
@@ -355,7 +396,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     h->occ_bound = m2;
     h->ovf_bound = 0;
     h->ctomb_bound = 0;
-    h->gen++;   // captured launch sequences point into the old storage
+    CK(storage_moved(h, s));
     *m_out = m2;
     if (self_loops_out) *self_loops_out = (long long)hc[1];
     return DRSF_OK;
@@ -382,7 +423,7 @@ static drsf_status ensure_batch(drsf_ctx *h, long long len, cudaStream_t s) {
     CK(cudaMemsetAsync(h->pt.mk, 0xFF, T * sizeof(u64), s));
     h->pt.mask = T - 1;
     h->batch_cap = cap;
-    h->gen++;
+    CK(storage_moved(h, s));
     return DRSF_OK;
 }
 
@@ -420,6 +461,7 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     if (st) return st;
     // reset the storage counters of the control block
     Ctl c = *h->ctl_host;
+    c.storage = h->gen;
     c.ovf_count = 0;
     c.edges = m2;
     c.htomb = 0;
@@ -430,21 +472,29 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     return DRSF_OK;
 }
 
+static StorageLimits limits(const drsf_ctx *h) {
+    return StorageLimits{h->gen, (long long)(0.7 * (double)h->H), h->ovf_cap};
+}
+
+// By the host-side bounds an insert of `len` edges has room.
+static bool insert_fits(const drsf_ctx *h, long long len) {
+    const StorageLimits l = limits(h);
+    return h->occ_bound + len <= l.index_max && h->ovf_bound + len <= (long long)l.ovf_cap;
+}
+
 // Decide from host-side bounds whether the storage could run out during a
 // batch of `len`; only then read the real counts (one synchronisation) and
-// rebuild if needed.
+// rebuild if needed.  (Replays of recorded inserts are not in the bounds.)
 static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_t s) {
     if (op == DRSF_INSERT) {
-        bool maybe = h->occ_bound + len > (long long)(0.7 * (double)h->H) ||
-                     h->ovf_bound + len > (long long)h->ovf_cap;
-        if (maybe) {
+        if (h->recorded || !insert_fits(h, len)) {
             drsf_status st = read_ctl(h, s);
             if (st) return st;
             long long occ = h->ctl_host->edges + h->ctl_host->htomb;
             long long ovfc = (long long)h->ctl_host->ovf_count;
             h->occ_bound = occ;
             h->ovf_bound = ovfc;
-            if (occ + len > (long long)(0.7 * (double)h->H) || ovfc + len > (long long)h->ovf_cap) {
+            if (!insert_fits(h, len)) {
                 st = rebuild(h, s, len);
                 if (st) return st;
             }
@@ -465,6 +515,20 @@ static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_
         }
     }
     return DRSF_OK;
+}
+
+// What a batch needs of the handle before it is enqueued.  While the caller
+// captures `s` nothing can be read, freed or allocated: a batch that has no
+// room by the bounds is refused, before anything is recorded.
+static drsf_status prepare_batch(drsf_ctx *h, int op, long long len, cudaStream_t s, bool rec) {
+    if (rec) {
+        if (len > h->batch_cap || (op == DRSF_INSERT && !insert_fits(h, len))) return DRSF_ECUDA;
+        h->recorded = true;
+        return DRSF_OK;
+    }
+    drsf_status st = ensure_batch(h, len, s);
+    if (st) return st;
+    return storage_check(h, op, len, s);
 }
 
 static void set_dev(drsf_ctx *h) {
@@ -559,6 +623,7 @@ static void destroy_all(drsf_ctx *h) {
     for (cudaEvent_t e : h->prof_ev) cudaEventDestroy(e);
     for (auto &ge : h->b_graphs) cudaGraphExecDestroy(ge.second);
     drop_graphs(h);
+    for (void *p : h->kept) cudaFree(p);
     if (h->u_cap) cudaStreamDestroy(h->u_cap);
     if (h->b_meta_host) cudaFreeHost(h->b_meta_host);
     if (h->b_meta_done) cudaEventDestroy(h->b_meta_done);
@@ -943,9 +1008,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
 
 static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t len, cudaStream_t s,
                               int groups = 0, const long long *voff = nullptr, const long long *boff = nullptr) {
-    drsf_status st = ensure_batch(h, len, s);
-    if (st) return st;
-    st = storage_check(h, op, len, s);
+    const bool rec = capturing(s);
+    drsf_status st = prepare_batch(h, op, len, s, rec);
     if (st) return st;
     const bool sg = use_supergraph(h, op);
     h->last_sg = sg ? 1 : 0;
@@ -957,7 +1021,7 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
         h->prof_op = op;
         h->prof_nb[op]++;
     }
-    const BeginArgs ba{op, h->n, len, batch, groups, voff, boff};
+    const BeginArgs ba{op, h->n, len, batch, limits(h), groups, voff, boff};
     auto direct = [&]() -> drsf_status {
         prof_begin(h, PH_BEGIN, s);
         CK(launch_begin(h->ctl, ba, len, s));
@@ -969,9 +1033,7 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     // a stream that the caller is capturing records plain launches: its graph
     // keeps the batch's arguments, which the handle's graphs get before each
     // replay
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-    if (cap != cudaStreamCaptureStatusNone) return direct();
+    if (rec) return direct();
     // otherwise replay the captured sequence for this (storage, op, variant,
     // grid size class of the batch kernels), with its first kernel's
     // arguments set to this batch
@@ -1099,10 +1161,21 @@ drsf_status drsf_apply_grouped(drsf_handle h, drsf_op op, const int32_t *batch, 
     set_dev(h);
     cudaStream_t s = (cudaStream_t)stream;
     const long long G = num_graphs;
+    const size_t bytes = (size_t)(G + 1) * sizeof(long long);
+    if (capturing(s)) {
+        std::vector<char> both(2 * bytes);
+        memcpy(both.data(), vertex_offsets, bytes);
+        memcpy(both.data() + bytes, batch_offsets, bytes);
+        st = prepare_batch(h, (int)op, len, s, true);
+        if (st) return st;
+        void *kept = nullptr;
+        st = keep_copy(h, both.data(), 2 * bytes, &kept);
+        if (st) return st;
+        return apply_impl(h, (int)op, batch, len, s, (int)G, (const long long *)kept, (const long long *)kept + (G + 1));
+    }
     st = batched_meta(h, G, s);
     if (st) return st;
     if (h->b_meta_pending) CK(cudaEventSynchronize(h->b_meta_done));   // the last call's copy out of the staging
-    const size_t bytes = (size_t)(G + 1) * sizeof(long long);
     memcpy(h->b_meta_host, vertex_offsets, bytes);
     memcpy(h->b_meta_host + bytes, batch_offsets, bytes);
     CK(cudaMemcpyAsync(h->b_meta, h->b_meta_host, 2 * bytes, cudaMemcpyHostToDevice, s));
@@ -1112,9 +1185,25 @@ drsf_status drsf_apply_grouped(drsf_handle h, drsf_op op, const int32_t *batch, 
     return apply_impl(h, (int)op, batch, len, s, (int)G, off, off + (G + 1));
 }
 
+// Candidates of the persistent kernels: at most the batch (insert) or every
+// live edge (delete), plus one partly used chunk per graph.
+static u64 batched_pool(const drsf_ctx *h, long long G, long long len) {
+    return (u64)std::max<long long>(len, h->col_cap / 2 + (long long)h->ovf_cap) + (u64)(G + 1) * 2048u;
+}
+// Tiles of the scanned rows: graph g's start at row[first vertex].start / 32 + g.
+static long long batched_tiles(const drsf_ctx *h, long long G) { return h->col_cap / 32 + G + 2; }
+
+// The persistent kernels' buffers hold this call as they are.
+static bool batched_fits(const drsf_ctx *h, long long G, long long len) {
+    const BState &b = h->b_st;
+    return h->b_ready && G <= h->b_gcnt_cap && batched_pool(h, G, len) <= b.pool_cap &&
+           batched_tiles(h, G) <= h->b_tile_cap && b.govf && h->b_govf_cap >= h->ovf_cap;
+}
+
 // Per-graph arrays for G graphs and the candidate pool for this call.
 static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cudaStream_t s) {
     BState &b = h->b_st;
+    bool moved = false;
     drsf_status st = batched_meta(h, G, s);
     if (st) return st;
     if (h->b_gcap > h->b_gcnt_cap) {
@@ -1126,10 +1215,9 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
         CKA(halloc(h, &b.gcur, (size_t)h->b_gcap + 1, s));
         CKA(halloc(h, &b.govf_start, (size_t)h->b_gcap + 1, s));
         h->b_gcnt_cap = h->b_gcap;
+        moved = true;
     }
-    // candidates: at most the batch (insert) or every live edge (delete),
-    // plus one partly used chunk per graph
-    const u64 need = (u64)std::max<long long>(len, h->col_cap / 2 + (long long)h->ovf_cap) + (u64)(G + 1) * 2048u;
+    const u64 need = batched_pool(h, G, len);
     if (need > b.pool_cap) {
         CK(cudaStreamSynchronize(s));
         hfree(h, &b.pk, s);
@@ -1139,14 +1227,15 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
         CKA(halloc(h, &b.pa, need, s));
         CKA(halloc(h, &b.pb, need, s));
         b.pool_cap = need;
+        moved = true;
     }
-    // tiles of the scanned rows: graph g's start at row[first vertex].start / 32 + g
-    const long long ntile = h->col_cap / 32 + G + 2;
+    const long long ntile = batched_tiles(h, G);
     if (ntile > h->b_tile_cap) {
         CK(cudaStreamSynchronize(s));
         hfree(h, &b.tile, s);
         CKA(halloc(h, &b.tile, (size_t)ntile, s));
         h->b_tile_cap = ntile;
+        moved = true;
     }
     // overflow buckets: as large as the overflow list (which a rebuild resizes)
     if (!b.govf || h->b_govf_cap < h->ovf_cap) {
@@ -1154,7 +1243,9 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
         hfree(h, &b.govf, s);
         CKA(halloc(h, &b.govf, (size_t)h->ovf_cap, s));
         h->b_govf_cap = h->ovf_cap;
+        moved = true;
     }
+    if (moved) CK(storage_moved(h, s));
     return DRSF_OK;
 }
 
@@ -1173,14 +1264,16 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     }
     set_dev(h);
     cudaStream_t s = (cudaStream_t)stream;
-    st = ensure_batch(h, len, s);
+    const bool rec = capturing(s);
+    if (rec && !batched_fits(h, G, len)) return DRSF_ECUDA;
+    st = prepare_batch(h, (int)op, len, s, rec);
     if (st) return st;
-    st = storage_check(h, op, len, s);
-    if (st) return st;
-    st = batched_scratch(h, s);
-    if (st) return st;
-    st = batched_capacity(h, G, len, s);
-    if (st) return st;
+    if (!rec) {
+        st = batched_scratch(h, s);
+        if (st) return st;
+        st = batched_capacity(h, G, len, s);
+        if (st) return st;
+    }
     BState &b = h->b_st;
     // queue order: size class by vertex count, then the largest work first
     // (batch edges + vertices) so the long graphs start early
@@ -1191,8 +1284,10 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
         while (c < num_classes - 1 && nv > classes[c].max_vertices) ++c;
         per[c].push_back((int)g);
     }
-    char *mh = h->b_meta_host;
-    if (h->b_meta_pending) CK(cudaEventSynchronize(h->b_meta_done));
+    const size_t mbytes = (size_t)(2 * (G + 1)) * sizeof(long long) + (size_t)G * sizeof(int);
+    std::vector<char> rec_meta(rec ? mbytes : 0);
+    char *mh = rec ? rec_meta.data() : h->b_meta_host;
+    if (!rec && h->b_meta_pending) CK(cudaEventSynchronize(h->b_meta_done));
     long long *voff_h = (long long *)mh, *boff_h = voff_h + (G + 1);
     int *order_h = (int *)(boff_h + (G + 1));
     memcpy(voff_h, vertex_offsets, (size_t)(G + 1) * sizeof(long long));
@@ -1210,12 +1305,17 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
         for (int g : v) order_h[pos++] = g;
     }
     q[num_classes] = (int)pos;
-    const size_t mbytes = (size_t)(2 * (G + 1)) * sizeof(long long) + (size_t)G * sizeof(int);
-    long long *voff_d = (long long *)h->b_meta, *boff_d = voff_d + (G + 1);
+    void *meta = h->b_meta;
+    if (rec) {
+        st = keep_copy(h, mh, mbytes, &meta);
+        if (st) return st;
+    } else {
+        CK(cudaMemcpyAsync(meta, mh, mbytes, cudaMemcpyHostToDevice, s));
+        CK(cudaEventRecord(h->b_meta_done, s));
+        h->b_meta_pending = true;
+    }
+    long long *voff_d = (long long *)meta, *boff_d = voff_d + (G + 1);
     int *order_d = (int *)(boff_d + (G + 1));
-    CK(cudaMemcpyAsync(h->b_meta, mh, mbytes, cudaMemcpyHostToDevice, s));
-    CK(cudaEventRecord(h->b_meta_done, s));
-    h->b_meta_pending = true;
     // the per-call state: current storage pointers + scratch
     b.ctl = h->ctl;
     b.parent = h->parent;
@@ -1238,6 +1338,7 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     d.order = order_d;
     d.G = (int)G;
     d.op = (int)op;
+    d.lim = limits(h);
     CK(launch_bset(h->b_state, b, h->b_desc, d, s));
     // one captured launch sequence per (op, class queues, launch shapes)
     std::string key = std::to_string((int)op);
@@ -1262,13 +1363,10 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
                std::to_string(classes[c].block_threads) + ":" + std::to_string(grid[c]) + ":" +
                std::to_string(classes[c].cluster_blocks);
     }
-    cudaGraphExec_t exec = nullptr;
-    for (auto &ge : h->b_graphs)
-        if (ge.first == key) exec = ge.second;
-    if (!exec) {
-        CK(cudaStreamBeginCapture(h->b_cap, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = launch_bprologue(h->dev, h->b_state, h->b_cap);
-        if (e == cudaSuccess) e = cudaEventRecord(h->b_fork, h->b_cap);
+    // the sequence, on a stream that is being captured
+    auto sequence = [&](cudaStream_t cs) -> cudaError_t {
+        cudaError_t e = launch_bprologue(h->dev, h->b_state, cs);
+        if (e == cudaSuccess) e = cudaEventRecord(h->b_fork, cs);
         for (int c = 0; c < num_classes && e == cudaSuccess; ++c) {
             if (q[c + 1] == q[c]) continue;
             e = cudaStreamWaitEvent(h->b_cls[c], h->b_fork, 0);
@@ -1276,8 +1374,21 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
                 e = launch_bpersist(h->b_state, c, q[c], q[c + 1], classes[c].block_threads, grid[c],
                                     classes[c].cluster_blocks, h->b_cls[c]);
             if (e == cudaSuccess) e = cudaEventRecord(h->b_join[c], h->b_cls[c]);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(h->b_cap, h->b_join[c], 0);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, h->b_join[c], 0);
         }
+        return e;
+    };
+    if (rec) {
+        CK(sequence(s));
+        h->last_sg = 0;
+        return DRSF_OK;
+    }
+    cudaGraphExec_t exec = nullptr;
+    for (auto &ge : h->b_graphs)
+        if (ge.first == key) exec = ge.second;
+    if (!exec) {
+        CK(cudaStreamBeginCapture(h->b_cap, cudaStreamCaptureModeThreadLocal));
+        cudaError_t e = sequence(h->b_cap);
         cudaGraph_t graph = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(h->b_cap, &graph);
         if (e == cudaSuccess) e = e2;
@@ -1342,6 +1453,12 @@ drsf_status drsf_apply_host(drsf_handle h, drsf_op op, const int32_t *batch, int
     if (len > (int64_t)1 << 31) return DRSF_EINVAL;
     set_dev(h);
     cudaStream_t s = (cudaStream_t)stream;
+    if (capturing(s)) {
+        drsf_status st = prepare_batch(h, (int)op, len, s, true);
+        void *kept = nullptr;
+        if (!st) st = keep_copy(h, batch, (size_t)len * 2 * sizeof(int), &kept);
+        return st ? st : apply_impl(h, (int)op, (const int32_t *)kept, len, s);
+    }
     drsf_status st = ensure_stage(h, len, s);
     if (st) return st;
     if (h->stage_pending) CK(cudaEventSynchronize(h->stage_done));   // previous copy out of the staging buffer
@@ -1360,11 +1477,12 @@ static drsf_status latched(drsf_ctx *h) {
         h->poisoned = true;
         return (e & ERR_TIMEOUT) ? DRSF_ETIMEOUT : DRSF_EPOISONED;
     }
-    if (e & ERR_BATCH_ID) {
-        // report once, then clear the bit
-        int z = e & ~ERR_BATCH_ID;
+    const int skipped = ERR_BATCH_ID | ERR_MOVED | ERR_FULL;
+    if (e & skipped) {
+        // report once, then clear the bits
+        int z = e & ~skipped;
         cudaMemcpy(&h->ctl->err, &z, sizeof(int), cudaMemcpyHostToDevice);
-        return DRSF_EINVAL;
+        return (e & (ERR_BATCH_ID | ERR_MOVED)) ? DRSF_EINVAL : DRSF_ENOMEM;
     }
     return DRSF_OK;
 }
@@ -1506,7 +1624,7 @@ drsf_status drsf_static_forest(drsf_handle h, int32_t *parent_out, int32_t *labe
     u64 *levels = (u64 *)h->bsum;   // scratch word
     Csr g{h->row, h->col, h->fpos};
     CK(launch_static_forest(h->dev, h->n, g, h->ovf, h->ctl, h->J1, comp, parent_out, h->act, h->xlist, levels,
-                            s));
+                            h->gen, s));
     if (levels_out) {
         long long lv = 0;
         CK(cudaMemcpyAsync(&lv, levels, sizeof lv, cudaMemcpyDeviceToHost, s));

@@ -859,9 +859,11 @@ __global__ void k_bbegin(const BState *Sp) {
     const BState &S = *Sp;
     const BDesc d = *S.desc;
     Ctl *ctl = S.ctl;
+    const bool moved = ctl->storage != d.lim.gen;   // a recorded call: its buffers may be gone
     if (threadIdx.x == 0) {
         ctl->base += 1;
         ctl->epoch = ctl->base;
+        storage_ok(ctl, d.lim, d.op, d.len, ctl->epoch);
         ctl->op = d.op;
         ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
         ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
@@ -873,6 +875,7 @@ __global__ void k_bbegin(const BState *Sp) {
         for (int i = 0; i < 8; ++i) ctl->bar[i] = 0;
         *S.pool_ctr = 0;
     }
+    if (moved) return;
     if (threadIdx.x < BCLASSES) S.qctr[threadIdx.x] = 0;
     for (int i = threadIdx.x; i <= d.G; i += blockDim.x) {
         S.gcnt[i] = 0;
@@ -895,6 +898,7 @@ __device__ __forceinline__ int graph_of(const long long *voff, int G, long long 
 // DRSF_EINVAL latched.  One warp per graph.
 __global__ void k_bvalidate(const BState *Sp) {
     const BState &S = *Sp;
+    if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -929,6 +933,7 @@ __global__ void k_bovf_count(const BState *Sp) {
 __global__ void k_bovf_scan(const BState *Sp) {
     // one block: exclusive scan of the per-graph counts into govf_start
     const BState &S = *Sp;
+    if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     __shared__ long long s_run;
     if (threadIdx.x == 0) s_run = 0;

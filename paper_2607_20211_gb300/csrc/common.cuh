@@ -33,6 +33,8 @@ typedef unsigned long long u64;
 #define ERR_TIMEOUT 2    // a bounded grid barrier gave up
 #define ERR_CAPACITY 4   // an internal buffer would overflow (never expected)
 #define ERR_ROUNDS 8     // an iteration exceeded its round bound (cyclic parent)
+#define ERR_MOVED 16     // a recorded batch was replayed after the storage moved: batch skipped
+#define ERR_FULL 32      // a recorded insert was replayed without room for it: batch skipped
 
 // grid-barrier wait limit in nanoseconds (globaltimer)
 #define BARRIER_TIMEOUT_NS 2000000000ull
@@ -42,7 +44,7 @@ typedef unsigned long long u64;
 // per-batch counts.  Statistic fields mirror drsf_batch_stats.
 struct Ctl {
     int err;
-    unsigned skip;          // epoch + 1 of the last rejected batch (ERR_BATCH_ID seen)
+    unsigned skip;          // epoch + 1 of the last rejected batch (ERR_BATCH_ID, ERR_MOVED, ERR_FULL)
     unsigned epoch;         // batch counter; epoch stamps compare against it
     unsigned base;          // the batches before this one (k_begin's blocks all read it; the claim
                             // kernels move it on)
@@ -69,6 +71,7 @@ struct Ctl {
     u64 nact;               // active vertices (path reversal)
     u64 ncore;              // core arcs of the super-forest Euler tour
     u64 ovf_count;          // overflow list length (grows until rebuild)
+    long long storage;      // generation of the storage and batch buffers (drsf_ctx::gen)
     long long edges;        // live undirected edges of G
     long long htomb;        // index tombstones
     long long ctomb;        // dead CSR entries (deleted ones, and slots lost to overflow edges)
@@ -96,6 +99,27 @@ struct Ctl {
 // The current batch was rejected: no kernel after k_begin touches anything.
 __device__ __forceinline__ bool batch_skipped(const Ctl *ctl) {
     return *(const volatile unsigned *)&ctl->skip == ctl->epoch + 1;
+}
+
+// What a batch may assume of the handle's storage.  A batch that the caller
+// recorded into a graph of its own carries pointers into the storage as it was
+// then, and its room was checked then; k_begin and k_bbegin check again.
+struct StorageLimits {
+    long long gen;          // ctl->storage as the launches' pointers were taken
+    long long index_max;    // index slots in use (live and deleted) after an insert
+    u64 ovf_cap;            // overflow entries after an insert
+};
+// One thread of the batch's first kernel: false (and the batch rejected) when
+// the launches that follow have no business with the storage.
+__device__ __forceinline__ bool storage_ok(Ctl *ctl, const StorageLimits &l, int op, long long len, unsigned epoch) {
+    int e = 0;
+    if (ctl->storage != l.gen) e = ERR_MOVED;
+    else if (op == DRSF_INSERT && (ctl->edges + ctl->htomb + len > l.index_max || ctl->ovf_count + (u64)len > l.ovf_cap))
+        e = ERR_FULL;
+    if (!e) return true;
+    atomicOr(&ctl->err, e);
+    ctl->skip = epoch + 1;
+    return false;
 }
 
 // The edge index.  An entry is one 16-byte record: with keys and positions in

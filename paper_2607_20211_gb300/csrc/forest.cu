@@ -100,7 +100,8 @@ __device__ __forceinline__ int owner_of(const long long *off, int G, long long i
 // launch of its own.
 __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     const unsigned epoch = ctl->base + 1;
-    GS_LOOP(i, a.len) {
+    if (gtid() == 0) storage_ok(ctl, a.lim, a.op, a.len, epoch);
+    if (ctl->storage == a.lim.gen) GS_LOOP(i, a.len) {
         const int u = a.batch[2 * i], v = a.batch[2 * i + 1];
         bool bad = u < 0 || u >= a.n || v < 0 || v >= a.n;
         if (a.groups) {

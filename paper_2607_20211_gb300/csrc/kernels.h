@@ -125,6 +125,7 @@ struct BeginArgs {
     int op, n;
     long long len;
     const int *batch;
+    StorageLimits lim;
     int groups;                    // graphs with a slice of the batch and a vertex range each; 0: none
     const long long *voff, *boff;  // their offsets (groups + 1)
 };
@@ -245,7 +246,7 @@ unsigned coop_blocks_replace(int nsm);
 cudaError_t launch_barrier_selftest(Ctl *ctl, cudaStream_t s);
 // static.cu ------------------------------------------------------------
 cudaError_t launch_static_forest(const Dev &d, int n, Csr g, const u64 *ovf, Ctl *ctl, int *lab, int *comp,
-                                 int *parent, int *f0, int *f1, u64 *levels, cudaStream_t s);
+                                 int *parent, int *f0, int *f1, u64 *levels, long long gen, cudaStream_t s);
 unsigned coop_blocks_bfs(int nsm);
 // euler.cu -------------------------------------------------------------
 struct EtArgs {
@@ -268,6 +269,7 @@ struct BDesc {               // per call
     const int *order;        // graphs in queue order, class by class
     int G;
     int op;
+    StorageLimits lim;
 };
 struct BState {              // device pointers of one handle (per call)
     Ctl *ctl;

@@ -43,7 +43,11 @@ __device__ __forceinline__ void cc_union(int *lab, int a, int b) {
     }
 }
 
-__global__ void k_cc_hook(int n, Csr g, const u64 *ovf, const Ctl *ctl, int *lab) {
+__global__ void k_cc_hook(int n, Csr g, const u64 *ovf, Ctl *ctl, long long gen, int *lab) {
+    if (ctl->storage != gen) {   // a recorded call: the storage is gone
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->err, ERR_MOVED);
+        return;
+    }
     int lane = threadIdx.x & 31;
     long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -89,7 +93,8 @@ __global__ void k_cc_roots(int n, const int *lab, int *comp, int *parent, int *f
 // frontier vertex streams its row; a neighbour claimed by atomicCAS on its
 // parent joins the next frontier.  Frontiers alternate between two lists;
 // counts live in ctl->cnt (3 slots, as in the other round loops).
-__global__ void k_bfs(Ctl *ctl, Csr g, const u64 *ovf, int *parent, int *f0, int *f1, u64 *levels) {
+__global__ void k_bfs(Ctl *ctl, Csr g, const u64 *ovf, int *parent, int *f0, int *f1, u64 *levels, long long gen) {
+    if (ctl->storage != gen) return;
     int lane = threadIdx.x & 31;
     long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -143,18 +148,18 @@ unsigned coop_blocks_bfs(int nsm) {
 }
 
 cudaError_t launch_static_forest(const Dev &d, int n, Csr g, const u64 *ovf, Ctl *ctl, int *lab, int *comp,
-                                 int *parent, int *f0, int *f1, u64 *levels, cudaStream_t s) {
+                                 int *parent, int *f0, int *f1, u64 *levels, long long gen, cudaStream_t s) {
     unsigned gn = grid_for(n, BLK, 152u * 16u);
     cudaError_t e = cudaMemsetAsync(ctl->cnt, 0, sizeof(ctl->cnt), s);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(&ctl->bar[4], 0, sizeof(u64), s);   // BFS barrier counter
     if (e != cudaSuccess) return e;
     k_cc_init<<<gn, BLK, 0, s>>>(n, lab);
-    k_cc_hook<<<d.grid, BLK, 0, s>>>(n, g, ovf, ctl, lab);
+    k_cc_hook<<<d.grid, BLK, 0, s>>>(n, g, ovf, ctl, gen, lab);
     k_cc_roots<<<gn, BLK, 0, s>>>(n, lab, comp, parent, f0, &ctl->cnt[0]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&ctl, (void *)&g, (void *)&ovf, (void *)&parent, (void *)&f0, (void *)&f1,
-                    (void *)&levels};
+                    (void *)&levels, (void *)&gen};
     return cudaLaunchCooperativeKernel((const void *)k_bfs, d.coop_bfs, BLK, args, 0, s);
 }
