@@ -66,7 +66,7 @@ class BatchedClass(ctypes.Structure):
                 ("blocks_per_sm", ctypes.c_int32), ("cluster_blocks", ctypes.c_int32)]
 
 
-# default size classes of the batched form:
+# size classes of the batched form's persistent kernels to start a schedule from:
 # (max vertices, block threads, blocks per SM, blocks per cluster)
 DEFAULT_CLASSES = ((8192, 256, 0, 1), (65536, 512, 0, 2), (2 ** 31 - 1, 1024, 0, 8))
 
@@ -268,23 +268,26 @@ class DynamicForest:
             raise DRSFError(st, "drsf_apply_host")
 
     def apply_batched(self, op: int, batch: torch.Tensor, vertex_offsets, batch_offsets,
-                      classes=DEFAULT_CLASSES) -> None:
+                      classes=None) -> None:
         """Batched form: the handle holds the disjoint union of independent
         graphs (graph g owns vertices vertex_offsets[g] .. vertex_offsets[g+1]
         and batch rows batch_offsets[g] .. batch_offsets[g+1]); every graph's
-        slice is applied.  With the default schedule the slices go through
-        the grid-wide launch sequence as one batch of the union
-        (drsf_apply_grouped: 1.3 to 9 times faster at every size measured);
-        a schedule of the caller's own runs the persistent per-graph kernels
-        with it: `classes` is a sequence of (max_vertices, block_threads,
-        blocks_per_sm[, cluster_blocks]) size classes.  Same result."""
+        slice is applied.  Without `classes` the slices go through the
+        grid-wide launch sequence as one batch of the union
+        (drsf_apply_grouped: 1.3 to 9 times faster at every size measured,
+        2 graphs of 1K vertices to 256 of up to 256K).  With a schedule the
+        persistent per-graph kernels run instead (drsf_apply_batched):
+        `classes` is a sequence of (max_vertices, block_threads,
+        blocks_per_sm[, cluster_blocks]) size classes, for instance
+        DEFAULT_CLASSES.  Same result; choose them only where a measurement of
+        your own graphs says so (the autotuner times schedules)."""
         import numpy as np
         batch = _dev_i32(batch, "batch", 2)
         vo = np.ascontiguousarray(vertex_offsets, np.int64)
         bo = np.ascontiguousarray(batch_offsets, np.int64)
         if vo.shape != bo.shape or vo.ndim != 1 or len(vo) < 2:
             raise ValueError("vertex_offsets and batch_offsets must be 1-D of the same length G + 1")
-        if classes is DEFAULT_CLASSES:
+        if classes is None:
             st = _lib.drsf_apply_grouped(self._h, op, batch.data_ptr() if batch.numel() else None,
                                          int(batch.shape[0]) if batch.numel() else 0, len(vo) - 1, vo.ctypes.data,
                                          bo.ctypes.data, _stream_ptr(self._stream))

@@ -205,7 +205,7 @@ def test_persistent_overflow_and_edge_cases():
         for op, per in ((drsf.INSERT, ins), (drsf.DELETE, dels)):
             ub = dev_tensor(np.concatenate([U.shift(i, b) for i, b in enumerate(per)]).reshape(-1, 2))
             vo, bo = _offsets(U, per)
-            fp.apply_batched(op, ub, vo, bo)
+            fp.apply_batched(op, ub, vo, bo, drsf.DEFAULT_CLASSES)
             got = U.split(fp.parent().cpu().numpy())
             labs = U.split(fp.labels().cpu().numpy())
             for i, g in enumerate(graphs):
@@ -232,7 +232,7 @@ def test_persistent_rejects_an_edge_between_graphs():
         bad = np.concatenate([U.shift(i, b) for i, b in enumerate(per)])
         bad[0, 1] = U.offsets[1] + 2          # graph 0's edge reaches into graph 1
         vo, bo = _offsets(U, per)
-        fp.apply_batched(drsf.INSERT, dev_tensor(bad), vo, bo)
+        fp.apply_batched(drsf.INSERT, dev_tensor(bad), vo, bo, drsf.DEFAULT_CLASSES)
         with pytest.raises(drsf.DRSFError) as e:
             fp.stats()
         assert e.value.status == drsf.EINVAL
@@ -241,7 +241,7 @@ def test_persistent_rejects_an_edge_between_graphs():
         b2 = tr.next_batch(drsf.INSERT, 50)
         per = [np.zeros((0, 2), np.int32), np.zeros((0, 2), np.int32), b2, np.zeros((0, 2), np.int32)]
         vo, bo = _offsets(U, per)
-        fp.apply_batched(drsf.INSERT, dev_tensor(U.shift(2, b2)), vo, bo)
+        fp.apply_batched(drsf.INSERT, dev_tensor(U.shift(2, b2)), vo, bo, drsf.DEFAULT_CLASSES)
         got = U.split(fp.parent().cpu().numpy())[2]
         r = oracle.apply(graphs[2].n, graphs[2].keys, graphs[2].parent, drsf.INSERT, b2)
         assert np.array_equal(got, r.parent)

@@ -42,8 +42,8 @@ def test_same_edges_leave_and_come_back(n, m, b, cycles):
         f.close()
 
 
-@pytest.mark.parametrize("batched", [None, drsf.DEFAULT_CLASSES, ((2 ** 31 - 1, 512, 0, 2),)],
-                         ids=["plain", "grouped", "persistent"])
+@pytest.mark.parametrize("batched", [False, (), (((2 ** 31 - 1, 512, 0, 2),),), (drsf.DEFAULT_CLASSES,)],
+                         ids=["plain", "grouped", "persistent", "persistent-classes"])
 def test_window_neither_overflows_nor_rebuilds(batched):
     """A window of returning edges reuses the rows' freed slots: with
     append-only rows 24 cycles of a sixth of the edges would overflow every
@@ -56,13 +56,13 @@ def test_window_neither_overflows_nor_rebuilds(batched):
     back = workloads.keys_to_edges(rng.permutation(g.keys)[:20_000])
     dev = torch.from_numpy(back).cuda()
     vo = bo = None
-    if batched:
+    if batched is not False:
         vo, bo = np.array([0, g.n], np.int64), np.array([0, len(back)], np.int64)
     try:
         for c in range(24):
             for op in (drsf.DELETE, drsf.INSERT):
-                if batched:
-                    f.apply_batched(op, dev, vo, bo, batched)
+                if batched is not False:
+                    f.apply_batched(op, dev, vo, bo, *batched)
                 else:
                     f.apply(op, dev)
         st = f.stats()
