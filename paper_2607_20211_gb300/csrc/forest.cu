@@ -1778,14 +1778,22 @@ struct SmallTail {
         struct {
             int minp[pieces];
             unsigned char vis[pieces];
+            unsigned short apos[pieces];   // an arc's place among its source's
         };
     };
-    int hk[slots];                  // hash table: piece, -1 free
+    union {
+        int hk[slots];              // hash table: piece, -1 free
+        struct {
+            unsigned short start[pieces];   // a piece's arcs
+            unsigned arc[pieces];           // tour: arcs to the end << 16 | next place
+        };
+    };
     int pid[pieces];
     unsigned short comp[pieces];
     unsigned short a[C], b[C], er[C];
     int ner;
-    static_assert(slots % ORIENT_THREADS == 0, "hash slots per thread");
+    static_assert(slots % ORIENT_THREADS == 0 && pieces % ORIENT_THREADS == 0, "items per thread");
+    static_assert(pieces < 0xFFFF, "places and ranks of the tour are 16 bits");
 };
 
 // slot of piece p in the hash table (entered when absent)
@@ -1799,15 +1807,88 @@ __device__ __forceinline__ int tail_slot(T &t, int p) {
         h = h + 1 == T::slots ? 0 : h + 1;
     }
 }
-// root of dense piece x (hooking only ever links roots, so chains are short)
+// root of dense piece x; the path is halved as it is walked (one round's hooks
+// can make a chain of all pieces: a path whose keys rise), by several threads
+// at once: an entry only ever moves to an ancestor
 template <class T>
-__device__ __forceinline__ int tail_root(const T &t, int x) {
+__device__ __forceinline__ int tail_root(T &t, int x) {
+    volatile unsigned short *const c = t.comp;
     for (int it = 0; it < T::pieces; ++it) {
-        const int p = *(volatile const unsigned short *)&t.comp[x];
+        const int p = c[x];
         if (p == x) break;
-        x = p;
+        const int g = c[p];
+        if (g == p) return p;
+        c[x] = (unsigned short)g;
+        x = g;
     }
     return x;
+}
+
+// Ranks the arcs of the super-forest's Euler tour (as orient_grid does its
+// core's): a piece's arcs side by side, the arc after b->a in b's list follows
+// a->b, the circuit opened at each super-root, Wyllie's ranking with the arcs
+// of a round in registers.  For super-forests deeper than TAIL_LEVELS, which
+// the orientation by levels would take one barrier per level for: an insert
+// that joins 4,000 vertices to a path took 3,852 us by levels and unhalved
+// chains, 124 so (a path of 250: 135 and 61, of 60: 59 and 57; a random tree of
+// 4,000, at most 32 deep: 92 and 89).
+// arc[apos[2 e]] >> 16 and arc[apos[2 e + 1]] >> 16 are then the ranks of edge
+// e's arcs from its first end and from its second.  Returns the rounds.
+#define TAIL_LEVELS 32
+#define TAIL_NIL 0xFFFFu
+template <class T>
+__device__ __noinline__ int tail_rank(int ner, int np) {
+    extern __shared__ __align__(16) int s_rank[];
+    T &t = *reinterpret_cast<T *>(s_rank);
+    const int arcs = 2 * ner;
+    auto source = [&](int j) { return (int)(j & 1 ? t.b[t.er[j >> 1]] : t.a[t.er[j >> 1]]); };
+    for (int l = threadIdx.x; l < np; l += ORIENT_THREADS) t.arc[l] = 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < arcs; j += ORIENT_THREADS) t.apos[j] = (unsigned short)atomicAdd(&t.arc[source(j)], 1u);
+    __syncthreads();
+    {
+        const int per = (np + ORIENT_THREADS - 1) / ORIENT_THREADS, l0 = threadIdx.x * per, l1 = min(np, l0 + per);
+        int deg = 0;
+        for (int l = l0; l < l1; ++l) deg += (int)t.arc[l];
+        long long tot;
+        int at = (int)block_excl_scan_ll(deg, &tot);
+        for (int l = l0; l < l1; ++l) {
+            t.start[l] = (unsigned short)at;
+            at += (int)t.arc[l];
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < arcs; j += ORIENT_THREADS) t.apos[j] = (unsigned short)(t.apos[j] + t.start[source(j)]);
+    __syncthreads();
+    for (int j = threadIdx.x; j < arcs; j += ORIENT_THREADS) {
+        const int head = source(j ^ 1), end = head + 1 < np ? t.start[head + 1] : arcs;
+        unsigned next = t.apos[j ^ 1] + 1u;
+        if ((int)next == end) next = t.minp[tail_root(t, head)] == t.pid[head] ? TAIL_NIL : t.start[head];
+        t.arc[t.apos[j]] = 1u << 16 | next;
+    }
+    __syncthreads();
+    int r = 0;
+    for (;;) {
+        unsigned w[T::pieces / ORIENT_THREADS];
+        bool more = false;
+#pragma unroll
+        for (int q = 0; q < T::pieces / ORIENT_THREADS; ++q) {
+            const int i = q * ORIENT_THREADS + threadIdx.x;
+            w[q] = i < arcs ? t.arc[i] : TAIL_NIL;
+            if ((w[q] & 0xFFFFu) != TAIL_NIL) {
+                const unsigned o = t.arc[w[q] & 0xFFFFu];
+                w[q] = (w[q] & 0xFFFF0000u) + (o & 0xFFFF0000u) | (o & 0xFFFFu);
+                more = true;
+            }
+        }
+        if (!__syncthreads_or(more) || ++r > MAX_ROUNDS) return r;
+#pragma unroll
+        for (int q = 0; q < T::pieces / ORIENT_THREADS; ++q) {
+            const int i = q * ORIENT_THREADS + threadIdx.x;
+            if (i < arcs) t.arc[i] = w[q];
+        }
+        __syncthreads();
+    }
 }
 
 // Results of one oriented edge: child piece p of edge k takes its attach point
@@ -1979,7 +2060,8 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
         open[q] = q * ORIENT_THREADS + (int)threadIdx.x < ner;
         child[q] = -1;
     }
-    for (int lvl = 0; lvl <= ner; ++lvl) {
+    bool deep = ner > 0;
+    for (int lvl = 0; deep && lvl < TAIL_LEVELS; ++lvl) {
         bool more = false;
 #pragma unroll
         for (int q = 0; q < IT; ++q) {
@@ -1995,7 +2077,20 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
             child[q] = va ? b : a;
             t.vis[child[q]] = 1;
         }
-        if (!__syncthreads_or(more)) break;
+        deep = __syncthreads_or(more);
+    }
+    if (deep) {
+        const int rounds = tail_rank<T>(ner, np);
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            if (!open[q]) continue;
+            const int e = q * ORIENT_THREADS + threadIdx.x, i = t.er[e];
+            child[q] = t.arc[t.apos[2 * e]] >> 16 > t.arc[t.apos[2 * e + 1]] >> 16 ? t.b[i] : t.a[i];
+        }
+        if (threadIdx.x == 0) {
+            if (rounds > MAX_ROUNDS) atomicOr(&ctl->err, ERR_ROUNDS);
+            ctl->rank_rounds = rounds;
+        }
     }
     int rev = 0;
 #pragma unroll
@@ -2016,7 +2111,7 @@ __device__ void replace_small(Ctl *ctl, const HookArgs &h, const OrientArgs &oa,
     if (threadIdx.x == 0) {
         ctl->ner = (u64)ner;
         ctl->hook_rounds = r;
-        ctl->ncore = 0;
+        ctl->ncore = deep ? 2 * (u64)ner : 0;
     }
 }
 

@@ -98,3 +98,27 @@ def test_large_batches_with_few_candidates(cross):
         check_batch(f, n, keys, par, drsf.INSERT, e)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("b", [20, 33, 34, 60, 500, 2047, 2048, 2049, LIMIT - 1, LIMIT])
+@pytest.mark.parametrize("shape", ["rising", "falling", "comb"])
+def test_deep_super_forests_take_logarithmic_rounds(shape, b):
+    """Super-forests deeper than the levels that the orientation takes one by
+    one, with hook chains of all pieces (keys that rise along a path): ranked,
+    in as many rounds as the tour's length has binary digits."""
+    n = 2 * b + 100
+    i = np.arange(b)
+    d = b // 3
+    e = np.stack([np.where(i < d, i, i % max(d, 1)), i + 1], 1) if shape == "comb" else np.stack([i, i + 1], 1)
+    e = (n - 1 - e if shape == "falling" else e).astype(np.int32)
+    g = _tiny_graph(n, [], list(range(n)))
+    f = make_forest(g)
+    try:
+        keys, par, st = check_batch(f, n, g.keys, g.parent, drsf.INSERT, e)
+        depth = d if shape == "comb" else b
+        assert (st["rank_rounds"] > 0) == (depth > 32)
+        assert st["rank_rounds"] <= (2 * b).bit_length() and st["hook_rounds"] <= b.bit_length()
+        keys, par, _ = check_batch(f, n, keys, par, drsf.DELETE, e[np.arange(b) % 5 != 0])
+        check_batch(f, n, keys, par, drsf.INSERT, e)
+    finally:
+        f.close()
