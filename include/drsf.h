@@ -292,8 +292,9 @@ DRSF_API drsf_status drsf_apply_grouped(drsf_handle h, drsf_op op, const int32_t
 /*
  * drsf_reserve -- size the handle's per-batch buffers (device work lists,
  * pair table, the pinned host staging of drsf_apply_host) for batches of up
- * to max_batch edges now, so that later drsf_apply / drsf_apply_host calls
- * of at most that size neither allocate nor synchronise for them (storage
+ * to max_batch edges now, and the pinned memory that drsf_sync and drsf_stats
+ * read the counters into, so that later calls of at most that size neither
+ * allocate nor synchronise for them (storage
  * growth of the graph itself can still do so).  Not in the paper: for
  * serving loops, where an allocation or a synchronisation inside one
  * tenant's call stalls every other tenant's work.  Synchronises `stream`.

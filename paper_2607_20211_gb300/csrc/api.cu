@@ -427,8 +427,16 @@ static drsf_status ensure_batch(drsf_ctx *h, long long len, cudaStream_t s) {
     return DRSF_OK;
 }
 
+// The host's copy of the control block: by drsf_reserve, else on first use (a
+// pinned allocation can wait for the device).
+static drsf_status ensure_ctl_host(drsf_ctx *h) {
+    if (!h->ctl_host) CK(cudaMallocHost((void **)&h->ctl_host, sizeof(Ctl)));
+    return DRSF_OK;
+}
+
 static drsf_status read_ctl(drsf_ctx *h, cudaStream_t s) {
-    if (!h->ctl_host) CK(cudaMallocHost((void **)&h->ctl_host, sizeof(Ctl)));   // (on first use)
+    drsf_status st = ensure_ctl_host(h);
+    if (st) return st;
     CK(cudaMemcpyAsync(h->ctl_host, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return DRSF_OK;
@@ -1442,6 +1450,8 @@ drsf_status drsf_reserve(drsf_handle h, int64_t max_batch, drsf_stream stream) {
     drsf_status st = ensure_batch(h, max_batch, s);
     if (st) return st;
     st = ensure_stage(h, max_batch, s);
+    if (st) return st;
+    st = ensure_ctl_host(h);
     if (st) return st;
     CK(cudaStreamSynchronize(s));
     return DRSF_OK;
