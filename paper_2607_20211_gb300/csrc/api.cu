@@ -157,6 +157,10 @@ static const char *kPhaseNames[DRSF_NUM_PHASES] = {
     "mark", "reverse"};
 
 static RowList rows(drsf_ctx *h) { return RowList{h->D, h->roff, h->rbase, h->rmeta, h->tile}; }
+static Ovf overflow(drsf_ctx *h) {
+    unsigned *const pos = (unsigned *)(h->ovf + h->ovf_cap);
+    return Ovf{h->ovf, pos, pos + h->ovf_cap, h->ovf_cap};
+}
 static HookSlots hook_slots(drsf_ctx *h) { return HookSlots{h->hstamp, h->comp, h->best0, h->best1}; }
 
 static void prof_begin(drsf_ctx *h, int phase, cudaStream_t s) {
@@ -353,7 +357,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     CK(launch_fill(dkey, dslot, place, m2, g, ix, s));
     u64 ovf_cap = std::max<u64>(std::max<u64>(1u << 16, (u64)m2 / 16), (u64)(2 * extra));
     u64 *ovf = nullptr;
-    CKA(halloc(h, &ovf, ovf_cap, s));
+    CKA(halloc(h, &ovf, 2 * ovf_cap, s));   // (Ovf's three arrays)
     // candidate buffers: every live undirected edge at most once
     u64 need = (u64)total / 2 + ovf_cap + 1024;
     if (need > h->cand_cap) {
@@ -470,7 +474,7 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     // reset the storage counters of the control block
     Ctl c = *h->ctl_host;
     c.storage = h->gen;
-    c.ovf_count = 0;
+    c.ovf_count = c.ovf_free = 0;
     c.edges = m2;
     c.htomb = 0;
     c.ctomb = 0;
@@ -499,7 +503,7 @@ static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_
             drsf_status st = read_ctl(h, s);
             if (st) return st;
             long long occ = h->ctl_host->edges + h->ctl_host->htomb;
-            long long ovfc = (long long)h->ctl_host->ovf_count;
+            long long ovfc = (long long)(h->ctl_host->ovf_count - h->ctl_host->ovf_free);
             h->occ_bound = occ;
             h->ovf_bound = ovfc;
             if (!insert_fits(h, len)) {
@@ -798,9 +802,9 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
     const bool wide = glen > (1 << 16);   // the replacement kernel's form
     if (op == DRSF_INSERT) {
         // Algorithm 1, insert: F^ = F, M = B; rep of the previous batch is current
-        const PlaceArgs pa{g,          h->ix,    h->ovf,      h->ovf_cap,    h->rep,
-                           h->pt,      h->ck[0], h->ca[0],    h->cb[0],      h->cand_cap,
-                           hook_slots(h), wide ? SMALL_CAND_LARGE : SMALL_CAND};
+        const PlaceArgs pa{g,        h->ix,    overflow(h), h->rep,        h->pt,
+                           h->ck[0], h->ca[0], h->cb[0],    h->cand_cap, hook_slots(h),
+                           wide ? SMALL_CAND_LARGE : SMALL_CAND};
         if (glen > SMALL_INSERT) {
             prof_begin(h, PH_INS_CLAIM, s);
             CK(launch_ins_claim(glen, h->ix, ctl, h->nkey, h->nslot, s));
@@ -814,7 +818,7 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
         // Algorithm 1, delete: remove B, cut tree edges, re-label the cut trees
         prof_begin(h, PH_DEL_CLAIM, s);
         const PieceSlots ps{h->aff_ep, h->rold, h->comp, h->best0, h->heavy, h->wgt, (unsigned *)h->pdeg};
-        CK(launch_del_claim(glen, h->ix, g, h->ovf, h->parent, h->rep, ctl, ps, h->cutlist, s));
+        CK(launch_del_claim(glen, h->ix, g, overflow(h), h->parent, h->rep, ctl, ps, h->cutlist, s));
         prof_end(h, PH_DEL_CLAIM, 1, s);
         RelabelArgs ra{};
         ra.n = h->n;
@@ -1330,8 +1334,7 @@ drsf_status drsf_apply_batched(drsf_handle h, drsf_op op, const int32_t *batch, 
     b.rep = h->rep;
     b.g = Csr{h->row, h->col, h->fpos};
     b.ix = h->ix;
-    b.ovf = h->ovf;
-    b.ovf_cap = h->ovf_cap;
+    b.ovf = overflow(h);
     b.nkey = h->nkey;
     b.nslot = h->nslot;
     b.pt_pk = h->pt.pk;
@@ -1547,7 +1550,7 @@ drsf_status drsf_stats(drsf_handle h, drsf_batch_stats *out, drsf_stream stream)
     out->mark_rounds = c.mark_rounds;
     out->jump_rounds = c.jump_rounds;
     out->edges = c.edges;
-    out->overflow = (int64_t)c.ovf_count;
+    out->overflow = (int64_t)(c.ovf_count - c.ovf_free);
     out->rebuilds = h->rebuilds;
     out->jump_visits = c.jump_visits;
     out->supergraph = h->last_sg;

@@ -295,9 +295,10 @@ __device__ void b_insert(const Grp &G, const BState &S, const BDesc &d, long lon
                 S.ix.e[s].pos = make_uint2(qa, qb);
                 hole -= 2;
             } else {
-                const u64 o = atomicAdd(&ctl->ovf_count, 1ull);
-                if (o < S.ovf_cap) {
-                    S.ovf[o] = k;
+                const u64 o = (u64)ovf_take(ctl, S.ovf);
+                if (o < S.ovf.cap) {
+                    S.ovf.e[o] = k;
+                    S.ovf.pos[o] = pa >= 0 ? ha.start + (unsigned)pa : (pb >= 0 ? hb.start + (unsigned)pb : POS_OVF);
                     S.ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
                 } else {
                     atomicOr(&ctl->err, ERR_CAPACITY);
@@ -350,7 +351,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         }
         ++wins;
         if (pos.x == POS_OVF) {
-            S.ovf[pos.y] = TOMB_KEY;
+            ovf_give(ctl, S.ovf, S.g, pos.y, u, v);
         } else {
             const int lo = (int)klo(key), hi = (int)khi(key);
             row_give(S.g, lo, S.g.row[lo].start, pos.x);
@@ -552,7 +553,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
         if (!pool_ensure(G, S, G.stride)) return;
         const long long q = q0 + G.tid;
         if (q < o1) {
-            const u64 k = GL(S.ovf[S.govf[q]]);
+            const u64 k = GL(S.ovf.e[S.govf[q]]);
             if (k != TOMB_KEY) {
                 const int ra = GL(S.rep[klo(k)]), rb = GL(S.rep[khi(k)]);
                 if (ra != rb) cross_edge(G, S, k, ra, rb);
@@ -923,10 +924,10 @@ __global__ void k_bovf_count(const BState *Sp) {
     if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     if (d.op != DRSF_DELETE) return;
-    const long long no = (long long)min(S.ctl->ovf_count, S.ovf_cap);
+    const long long no = (long long)min(S.ctl->ovf_count, S.ovf.cap);
     const long long vlo = d.voff[0], vhi = d.voff[d.G];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < no; i += (long long)gridDim.x * blockDim.x) {
-        const u64 k = S.ovf[i];
+        const u64 k = S.ovf.e[i];
         if (k != TOMB_KEY && klo(k) >= vlo && klo(k) < vhi) atomicAdd(&S.gcnt[graph_of(d.voff, d.G, klo(k))], 1);
     }
 }
@@ -954,10 +955,10 @@ __global__ void k_bovf_fill(const BState *Sp) {
     if (batch_skipped(S.ctl)) return;
     const BDesc d = *S.desc;
     if (d.op != DRSF_DELETE) return;
-    const long long no = (long long)min(S.ctl->ovf_count, S.ovf_cap);
+    const long long no = (long long)min(S.ctl->ovf_count, S.ovf.cap);
     const long long vlo = d.voff[0], vhi = d.voff[d.G];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < no; i += (long long)gridDim.x * blockDim.x) {
-        const u64 k = S.ovf[i];
+        const u64 k = S.ovf.e[i];
         if (k == TOMB_KEY || klo(k) < vlo || klo(k) >= vhi) continue;
         const int g = graph_of(d.voff, d.G, klo(k));
         S.govf[S.govf_start[g] + atomicAdd(&S.gcur[g], 1)] = (u64)i;   // position, read again after the claim

@@ -10,7 +10,9 @@
 //                                       global col positions of the edge in
 //                                       the rows of min(u,v) and max(u,v),
 //                                       or (POS_OVF, overflow slot)
-//   ovf[ovf_cap]                uint64  edges whose row had no free slot
+//   ovf                         16 B    edges with a full row (key, slot taken
+//                                       in the other row), and a stack of the
+//                                       entries that are free again
 //   per-batch work arrays (epoch-stamped, never cleared per batch)
 #pragma once
 
@@ -70,7 +72,8 @@ struct Ctl {
     u64 npc;                // distinct pieces touched by E_r
     u64 nact;               // active vertices (path reversal)
     u64 ncore;              // core arcs of the super-forest Euler tour
-    u64 ovf_count;          // overflow list length (grows until rebuild)
+    u64 ovf_count;          // overflow list length: entries ever taken since the last rebuild
+    u64 ovf_free;           // entries of it that are free again
     long long storage;      // generation of the storage and batch buffers (drsf_ctx::gen)
     long long edges;        // live undirected edges of G
     long long htomb;        // index tombstones
@@ -107,14 +110,14 @@ __device__ __forceinline__ bool batch_skipped(const Ctl *ctl) {
 struct StorageLimits {
     long long gen;          // ctl->storage as the launches' pointers were taken
     long long index_max;    // index slots in use (live and deleted) after an insert
-    u64 ovf_cap;            // overflow entries after an insert
+    u64 ovf_cap;            // overflow entries in use after an insert
 };
 // One thread of the batch's first kernel: false (and the batch rejected) when
 // the launches that follow have no business with the storage.
 __device__ __forceinline__ bool storage_ok(Ctl *ctl, const StorageLimits &l, int op, long long len, unsigned epoch) {
     int e = 0;
     if (ctl->storage != l.gen) e = ERR_MOVED;
-    else if (op == DRSF_INSERT && (ctl->edges + ctl->htomb + len > l.index_max || ctl->ovf_count + (u64)len > l.ovf_cap))
+    else if (op == DRSF_INSERT && (ctl->edges + ctl->htomb + len > l.index_max || ctl->ovf_count - ctl->ovf_free + (u64)len > l.ovf_cap))
         e = ERR_FULL;
     if (!e) return true;
     atomicOr(&ctl->err, e);
@@ -310,6 +313,38 @@ __device__ __forceinline__ void row_give(const Csr &g, int r, unsigned start, un
     g.fpos[(size_t)start + k] = (int)(pos - start);
 }
 
+// The edges held outside their rows.  An edge of which one row is full took a
+// slot of the other: it stays empty, and is given back with the entry.
+struct Ovf {
+    u64 *e;           // keys; TOMB_KEY where free
+    unsigned *pos;    // that slot's position in col, or POS_OVF
+    unsigned *free;   // stack of ctl->ovf_free free entries
+    u64 cap;
+};
+
+// Entry for an edge outside its rows: from the top of the stack, or the list's
+// end (a draw that found the stack empty is put back, as with the rows'
+// slots).  As with the rows' slots, entries are only taken while a batch is inserted
+// and only given back while one is deleted.
+__device__ __forceinline__ long long ovf_take(Ctl *ctl, const Ovf &o) {
+    const long long have = (long long)atomicAdd(&ctl->ovf_free, ~0ull);   // (minus one)
+    if (have > 0) return o.free[have - 1];
+    atomicAdd(&ctl->ovf_free, 1ull);
+    return (long long)atomicAdd(&ctl->ovf_count, 1ull);
+}
+// Edge {a, b} leaves entry i: the entry is free again, and the slot that the
+// edge held in one of its rows.
+__device__ __forceinline__ void ovf_give(Ctl *ctl, const Ovf &o, const Csr &g, unsigned i, int a, int b) {
+    o.e[i] = TOMB_KEY;
+    const unsigned p = o.pos[i];
+    if (p != POS_OVF) {
+        const Row ha = row_head(g, a);
+        const bool in_a = p - ha.start < (unsigned)ha.cap;
+        row_give(g, in_a ? a : b, in_a ? ha.start : g.row[b].start, p);
+    }
+    o.free[agg_append(&ctl->ovf_free, true)] = i;
+}
+
 // Pair table: piece pair (min, max) -> minimum edge key between the two
 // pieces.  Probing is bounded; a pair that finds no slot returns false and
 // the caller keeps the edge as a plain candidate instead.
@@ -402,6 +437,25 @@ __device__ __forceinline__ long long block_excl_scan_ll(long long v, long long *
     *total = s_ws[nw - 1];
     __syncthreads();
     return pre;
+}
+
+// ovf_take for every thread of a block with `on` (all call): the stack and the
+// list's end are asked once.
+__device__ __forceinline__ long long ovf_take_block(Ctl *ctl, const Ovf &o, bool on) {
+    __shared__ long long s_have, s_end;
+    long long n;
+    const long long k = block_excl_scan_ll(on, &n);
+    if (threadIdx.x == 0) {
+        const long long have = (long long)atomicAdd(&ctl->ovf_free, (u64)-n);
+        const long long got = have < 0 ? 0 : (have < n ? have : n);
+        if (got < n) atomicAdd(&ctl->ovf_free, (u64)(n - got));
+        s_have = have;
+        s_end = got < n ? (long long)atomicAdd(&ctl->ovf_count, (u64)(n - got)) - got : 0;
+    }
+    __syncthreads();
+    const long long i = !on ? -1 : (k < s_have ? (long long)o.free[s_have - 1 - k] : s_end + k);
+    __syncthreads();
+    return i;
 }
 
 // Block-aggregated reservation of `cnt` consecutive slots per thread (one

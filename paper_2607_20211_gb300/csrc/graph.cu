@@ -202,7 +202,7 @@ __global__ void k_ins_claim(Index ix, Ctl *ctl, u64 *nkey, u64 *nslot) {
 
 // Insert, step 2, for the edge of every calling thread with `on` (key k, index
 // slot s; the whole block calls): a free slot of both CSR rows (row_take), or,
-// when one of them is full, whole to the overflow list.  The cross test of the
+// when one of them is full, whole to the overflow list (Ovf).  The cross test of the
 // insert case (M = B, Algorithm 1) is fused here: rep[u] != rep[v] makes a
 // candidate.  With SG (the supergraph variant, Section III-A) a candidate goes
 // into the pair table instead, which keeps the minimum key per pair of trees
@@ -215,6 +215,7 @@ template <bool SG>
 __device__ __forceinline__ void place_edge(bool on, u64 k, u64 s, const PlaceArgs &p, Ctl *ctl, unsigned ep, bool slots,
                                            long long *dead) {
     bool cross = false, over = false;
+    unsigned held = POS_OVF;
     int ra = 0, rb = 0;
     if (on) {
         const uint32_t a = klo(k), b = khi(k);
@@ -227,20 +228,21 @@ __device__ __forceinline__ void place_edge(bool on, u64 k, u64 s, const PlaceArg
             p.ix.e[s].pos = make_uint2(qa, qb);
             *dead -= 2;
         } else {
-            over = true;   // (a slot taken in the row that had one stays empty
-                           // and unlisted until the next rebuild)
+            over = true;
+            held = pa >= 0 ? ha.start + (unsigned)pa : (pb >= 0 ? hb.start + (unsigned)pb : POS_OVF);
         }
         ra = p.rep[a];
         rb = p.rep[b];
         cross = ra != rb;
         if (SG && cross) cross = !pair_min(p.pt.pk, p.pt.mk, p.pt.mask, ra, rb, k);   // no slot: plain candidate
     }
-    // (one atomic per block: a million-edge batch can overflow 100K rows)
+    // (asked for per block: a million-edge batch can overflow 100K rows)
     if (__syncthreads_or(over)) {
-        const long long o = block_append(&ctl->ovf_count, over);
+        const long long o = ovf_take_block(ctl, p.ovf, over);
         if (over) {
-            if ((u64)o < p.ovf_cap) {
-                p.ovf[o] = k;
+            if ((u64)o < p.ovf.cap) {
+                p.ovf.e[o] = k;
+                p.ovf.pos[o] = held;
                 p.ix.e[s].pos = make_uint2(POS_OVF, (uint32_t)o);
             } else {
                 atomicOr(&ctl->err, ERR_CAPACITY);
@@ -330,7 +332,7 @@ __global__ void k_ins_small(Ctl *ctl, PlaceArgs p) {
 // deleted edge {u, v} with parent[u] == v, parent[u] <- u (either
 // orientation).  The old root of a cut tree is stamped "affected"; the cut
 // vertex becomes a piece root.
-__global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl, PieceSlots ps,
+__global__ void k_del_claim(Index ix, Csr g, Ovf ovf, int *parent, const int *rep, Ctl *ctl, PieceSlots ps,
                             int *cutlist) {
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->base = ctl->epoch;
     if (batch_skipped(ctl)) return;
@@ -362,7 +364,7 @@ __global__ void k_del_claim(Index ix, Csr g, u64 *ovf, int *parent, const int *r
                 if (s >= 0) won = atomicCAS(&ix.e[s].key, key, TOMB_KEY) == key;
                 if (won) {
                     if (pos.x == POS_OVF) {
-                        ovf[pos.y] = TOMB_KEY;
+                        ovf_give(ctl, ovf, g, pos.y, u, v);
                     } else {
                         row_give(g, u < v ? u : v, u < v ? st_u : st_v, pos.x);
                         row_give(g, u < v ? v : u, u < v ? st_v : st_u, pos.y);
@@ -528,7 +530,7 @@ cudaError_t launch_ins_small(long long len, Ctl *ctl, PlaceArgs p, bool sg, cuda
     else k_ins_small<false><<<gsz(len), BLK, 0, s>>>(ctl, p);
     return cudaGetLastError();
 }
-cudaError_t launch_del_claim(long long len, Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl,
+cudaError_t launch_del_claim(long long len, Index ix, Csr g, Ovf ovf, int *parent, const int *rep, Ctl *ctl,
                              PieceSlots ps, int *cutlist, cudaStream_t s) {
     k_del_claim<<<gsz(len), BLK, 0, s>>>(ix, g, ovf, parent, rep, ctl, ps, cutlist);
     return cudaGetLastError();

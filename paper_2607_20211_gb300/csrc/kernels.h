@@ -52,7 +52,7 @@ struct PieceSlots {
     u64 *best, *heavy;
     unsigned *w, *wsum;
 };
-cudaError_t launch_del_claim(long long len, Index ix, Csr g, u64 *ovf, int *parent, const int *rep, Ctl *ctl,
+cudaError_t launch_del_claim(long long len, Index ix, Csr g, Ovf ovf, int *parent, const int *rep, Ctl *ctl,
                              PieceSlots ps, int *cutlist, cudaStream_t s);
 // The rows a delete batch scans for cross edges, one entry per listed
 // vertex u: u itself, the exclusive prefix sum of the row lengths (roff[nd]
@@ -77,8 +77,7 @@ cudaError_t launch_ins_claim(long long len, Index ix, Ctl *ctl, u64 *nkey, u64 *
 struct PlaceArgs {
     Csr g;
     Index ix;
-    u64 *ovf;
-    u64 ovf_cap;
+    Ovf ovf;
     const int *rep;
     PairTable pt;
     u64 *ck;             // candidates
@@ -276,8 +275,7 @@ struct BState {              // device pointers of one handle (per call)
     int *parent, *rep;
     Csr g;
     Index ix;
-    u64 *ovf;
-    u64 ovf_cap;
+    Ovf ovf;
     u64 *nkey, *nslot;       // batch-indexed
     // vertex-indexed scratch (graph g uses its own vertex range)
     int *J, *R, *A, *Dv, *roff, *comp, *minp, *pidx, *plist, *pdeg, *poff, *pcur, *newroot, *flist, *chx, *chy;

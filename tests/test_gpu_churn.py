@@ -135,3 +135,48 @@ def test_batches_captured_by_the_caller(b, detach, monkeypatch):
                 keys, par, _ = check_batch(f, n, keys, par, op, batch[:50], labels=False)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("batched", [False, (((2 ** 31 - 1, 256, 0, 1),),)], ids=["plain", "persistent"])
+@pytest.mark.parametrize("b", [300, 5000, 2 ** 18 + 100])
+def test_edges_of_a_full_hub_leave_and_come_back(b, batched):
+    """b edges of hubs whose rows are full go to the overflow list, leave and
+    come back for many cycles: the list does not grow, and the rows of their
+    other ends lose no slots (then, two more edges of each still find one)."""
+    hubs, n = 7, b + 100_000
+    rng = np.random.default_rng(b)
+    ends = np.sort(rng.permutation(np.arange(hubs, n))[:b])
+    e = np.stack([np.arange(b) % hubs, ends], 1).astype(np.int32)
+    g = workloads.Graph.__new__(workloads.Graph)
+    path = np.stack([np.arange(n - 1), np.arange(1, n)], 1)
+    g.name, g.n, g.W, g.keys = "hubs", n, 0, workloads.edges_to_keys(path)
+    g.parent = np.maximum(np.arange(n) - 1, 0).astype(np.int32)
+    f = make_forest(g)
+    dev = torch.from_numpy(e).cuda()
+    vo, bo = np.array([0, n], np.int64), np.array([0, b], np.int64)
+    try:
+        st = {}
+        for c in range(12):
+            for op in (drsf.INSERT, drsf.DELETE):
+                if batched is not False:
+                    f.apply_batched(op, dev, vo, bo, *batched)
+                else:
+                    f.apply(op, dev)
+                st[op] = f.stats()
+            if c == 0:
+                most, rebuilds = (st[drsf.INSERT][k] for k in ("overflow", "rebuilds"))   # (room for a batch so long)
+            assert st[drsf.INSERT]["overflow"] == most and st[drsf.DELETE]["overflow"] == 0
+        assert b - 6 * hubs <= most <= b and f.stats()["rebuilds"] == rebuilds
+        keys, par = g.keys, f.parent().cpu().numpy()
+        keys, par, st = check_batch(f, n, keys, par, drsf.INSERT, e)
+        near = ends[(ends + 5 < n)]
+        more = np.stack([near, near + 2], 1)                   # two more for most ends, three at most
+        keys, par, st = check_batch(f, n, keys, par, drsf.INSERT, more.astype(np.int32), labels=False)
+        assert st["overflow"] == most
+        keys, par, st = check_batch(f, n, keys, par, drsf.DELETE, rng.permutation(e))
+        assert st["overflow"] == 0
+        check_batch(f, n, keys, par, drsf.INSERT, e[::-1], labels=False)
+        assert np.array_equal(workloads.edges_to_keys(f.export_edges().cpu().numpy()),
+                              np.union1d(keys, workloads.edges_to_keys(e)))
+    finally:
+        f.close()
