@@ -864,7 +864,7 @@ __global__ void k_bbegin(const BState *Sp) {
     if (threadIdx.x == 0) {
         ctl->base += 1;
         ctl->epoch = ctl->base;
-        storage_ok(ctl, d.lim, d.op, d.len, ctl->epoch);
+        storage_guard(ctl, storage_counts(ctl), d.lim, d.op, d.len, ctl->epoch);
         ctl->op = d.op;
         ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
         ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;

@@ -112,17 +112,26 @@ struct StorageLimits {
     long long index_max;    // index slots in use (live and deleted) after an insert
     u64 ovf_cap;            // overflow entries in use after an insert
 };
-// One thread of the batch's first kernel: false (and the batch rejected) when
-// the launches that follow have no business with the storage.
-__device__ __forceinline__ bool storage_ok(Ctl *ctl, const StorageLimits &l, int op, long long len, unsigned epoch) {
+// (loaded ahead of the check, beside the first loads of the batch: behind them
+// an insert and a delete of 100 edges took 130 us instead of 126, R-MAT scale 22)
+struct StorageCounts {
+    long long gen, used;
+    u64 ovf;
+};
+__device__ __forceinline__ StorageCounts storage_counts(const Ctl *ctl) {
+    const volatile Ctl *c = ctl;
+    return StorageCounts{c->storage, c->edges + c->htomb, c->ovf_count - c->ovf_free};
+}
+// One thread of the batch's first kernel: rejects the batch when the launches
+// that follow have no business with the storage.
+__device__ __forceinline__ void storage_guard(Ctl *ctl, const StorageCounts &c, const StorageLimits &l, int op,
+                                              long long len, unsigned epoch) {
     int e = 0;
-    if (ctl->storage != l.gen) e = ERR_MOVED;
-    else if (op == DRSF_INSERT && (ctl->edges + ctl->htomb + len > l.index_max || ctl->ovf_count - ctl->ovf_free + (u64)len > l.ovf_cap))
-        e = ERR_FULL;
-    if (!e) return true;
+    if (c.gen != l.gen) e = ERR_MOVED;
+    else if (op == DRSF_INSERT && (c.used + len > l.index_max || c.ovf + (u64)len > l.ovf_cap)) e = ERR_FULL;
+    if (!e) return;
     atomicOr(&ctl->err, e);
     ctl->skip = epoch + 1;
-    return false;
 }
 
 // The edge index.  An entry is one 16-byte record: with keys and positions in

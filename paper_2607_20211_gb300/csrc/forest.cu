@@ -100,8 +100,9 @@ __device__ __forceinline__ int owner_of(const long long *off, int G, long long i
 // launch of its own.
 __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     const unsigned epoch = ctl->base + 1;
-    if (gtid() == 0) storage_ok(ctl, a.lim, a.op, a.len, epoch);
-    if (ctl->storage == a.lim.gen) GS_LOOP(i, a.len) {
+    StorageCounts have{};
+    if (gtid() == 0) have = storage_counts(ctl);
+    GS_LOOP(i, a.len) {
         const int u = a.batch[2 * i], v = a.batch[2 * i + 1];
         bool bad = u < 0 || u >= a.n || v < 0 || v >= a.n;
         if (a.groups) {
@@ -117,6 +118,7 @@ __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     if (gtid() != 0) return;
     const int op = a.op;
     const long long len = a.len;
+    storage_guard(ctl, have, a.lim, op, len, epoch);   // (batch and offsets are the caller's or kept for the recording)
     ctl->batch = a.batch;
     ctl->epoch = epoch;
     ctl->op = op;
