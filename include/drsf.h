@@ -187,7 +187,7 @@ DRSF_API drsf_status drsf_set_allocator(drsf_alloc_fn alloc, drsf_free_fn free_f
  * the handle's delete batches: unset, a few parent hops and then asynchronous
  * pointer doubling (in place, no grid barrier between steps); "sync",
  * synchronous doubling rounds; "halving", path-halving walks.  All three give
- * the same representatives.  Before the default one, a delete batch first looks
+ * the same representatives.  Before it, a delete batch first looks
  * for its detached vertices top-down from the cut vertices over tree children
  * (touching only the detached vertices' rows) and falls back to the root
  * search only when that search exceeds its budget; DRSF_DETACH=0 skips the

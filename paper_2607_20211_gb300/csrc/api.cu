@@ -883,7 +883,8 @@ static drsf_status launch_rest(drsf_ctx *h, int op, bool sg, long long glen, cud
             prof_begin(h, PH_SCAN, s);
             CK(launch_cross(h->dev, ctl, da, ra, rows(h), la, sg, s));
             prof_end(h, PH_SCAN, 1, s);
-        } else {
+        }
+        if (!h->detach_now || la.listed) {
             if (h->jump_sync == 2) {
                 prof_begin(h, PH_JUMP, s);
                 CK(launch_relabel(h->dev, ctl, ra, s));
@@ -1027,7 +1028,7 @@ static drsf_status apply_impl(drsf_ctx *h, int op, const int32_t *batch, int64_t
     h->last_sg = sg ? 1 : 0;
     // the top-down delete for small batches: its cost follows the detached
     // vertices' rows and its levels, the pointer jumping's the cut trees
-    h->detach_now = op == DRSF_DELETE && h->detach && len <= h->detach_max && h->jump_sync == 2;
+    h->detach_now = op == DRSF_DELETE && h->detach && len <= h->detach_max;
     if (h->prof_on) {
         h->prof_batches++;
         h->prof_op = op;

@@ -787,12 +787,14 @@ __global__ void __launch_bounds__(BLK, 5) k_relabel(Ctl *ctl, RelabelArgs a) {
 template <bool SG>
 __global__ void __launch_bounds__(BLK, 4) k_scan(Ctl *ctl, RowList rl, LightArgs a) {
     if (batch_skipped(ctl)) return;
-    if (a.listed) scan_listed<SG>(ctl, rl, a);
-    else scan_light<SG>(ctl, a);
+    if (!a.listed) scan_light<SG>(ctl, a);
+    else if (!ctl->td) scan_listed<SG>(ctl, rl, a);   // (else k_cross has scanned them)
 }
 // Small deletes: the top-down search and the scan of the rows it listed, or,
 // where it gives up, what large deletes do, in one launch (as four, the ones
-// that found nothing to do took 8 us of every batch).
+// that found nothing to do took 8 us of every batch).  With a selectable root
+// search (a.listed) that search and its scan are launches of their own, which
+// find nothing to do when the top-down one found the pieces.
 template <bool SG>
 __global__ void __launch_bounds__(BLK, 4)
     k_cross(Ctl *ctl, DetachArgs d, RelabelArgs r, RowList rl, LightArgs a) {
@@ -809,7 +811,7 @@ __global__ void __launch_bounds__(BLK, 4)
         if (!grid_barrier(ctl, &ctl->bar[7])) return;
         found = *(volatile int *)&ctl->td;
     }
-    if (!found && !relabel(ctl, r)) return;
+    if (!found && (a.listed || !relabel(ctl, r))) return;
     if ((!found || nb == gridDim.x) && !grid_barrier(ctl, &ctl->bar[7])) return;
     if (found) scan_listed<SG>(ctl, rl, a);
     else scan_light<SG>(ctl, a);

@@ -134,8 +134,8 @@ cudaError_t launch_begin(Ctl *ctl, BeginArgs a, long long grid_len, cudaStream_t
 cudaError_t set_begin(cudaGraphExec_t exec, cudaGraphNode_t node, Ctl *ctl, BeginArgs a, long long grid_len);
 cudaError_t launch_aff_collect(const Dev &d, int n, const int *rep, const unsigned *aff_ep, int *A, int *rold,
                                unsigned *w, u64 *heavy, Ctl *ctl, cudaStream_t s);
-// delete: detached vertices top-down from the cut vertices (falls back to
-// the pointer jumping above when over budget).
+// delete: detached vertices top-down from the cut vertices (over budget, the
+// root search takes over).
 // DETACH_LEVELS: its level limit (measured on R-MAT, where it pays, the
 // search takes 2-7 levels; on deep trees each level costs about as much as
 // a whole pointer-jumping round)

@@ -145,3 +145,34 @@ def test_second_reading_around_its_list(detached, flags):
         assert st["tree_cut"] == detached
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("jump", ["sync", "halving", ""])
+@pytest.mark.parametrize("sg", [drsf.REPL_SG, drsf.REPL_HS])
+def test_top_down_search_before_every_root_search(jump, sg, monkeypatch):
+    """Small deletes look top-down first whatever root search the handle has,
+    which takes over where the search gives up (a path is too deep for it)."""
+    if jump:
+        monkeypatch.setenv("DRSF_JUMP", jump)
+    n = 30_000
+    rng = np.random.default_rng(7)
+    flat = np.stack([rng.integers(0, 60, n - 60), np.arange(60, n)], 1)      # 60 hubs with leaves, chords between
+    chords = rng.integers(60, n, (3000, 2))
+    hubs = np.stack([np.zeros(59, np.int64), np.arange(1, 60)], 1)
+    path = np.stack([np.arange(n - 1), np.arange(1, n)], 1)
+    for edges, found in ((np.concatenate([hubs, flat, chords[chords[:, 0] != chords[:, 1]]]), True),
+                         (np.concatenate([path, chords[np.abs(chords[:, 0] - chords[:, 1]) > 1]]), False)):
+        g = _tiny_graph(n, workloads.keys_to_edges(np.unique(workloads.edges_to_keys(edges))).tolist(),
+                        None if found else np.maximum(np.arange(n) - 1, 0))
+        f = make_forest(g, flags=drsf.DETERMINISTIC | sg)
+        keys, par = g.keys, g.parent
+        try:
+            for c in range(3):
+                v = rng.permutation(np.nonzero(par != np.arange(n))[0])[:500]
+                cut = np.stack([v, par[v]], 1).astype(np.int32)
+                keys, par, st = check_batch(f, n, keys, par, drsf.DELETE, cut)
+                if c == 0:
+                    assert (st["detach_levels"] > 0) == found and st["detach_levels"] != 0
+                keys, par, _ = check_batch(f, n, keys, par, drsf.INSERT, cut)
+        finally:
+            f.close()
