@@ -66,7 +66,9 @@ typedef void *drsf_stream;
 typedef enum {
     DRSF_OK = 0,
     DRSF_EINVAL = 1,      /* bad argument or out-of-range vertex id */
-    DRSF_ENOMEM = 2,      /* allocation failed; the handle is unchanged */
+    DRSF_ENOMEM = 2,      /* allocation failed; the handle is unchanged (or, when
+                             not even its old buffers could be had again,
+                             DRSF_EPOISONED from the next call on) */
     DRSF_ECUDA = 3,       /* a CUDA runtime call failed */
     DRSF_ENOT_FOREST = 4, /* DRSF_VALIDATE: parent is not a rooted spanning forest of G */
     DRSF_ETIMEOUT = 5,    /* a bounded device-side wait gave up */

@@ -245,6 +245,23 @@ static void hfree(drsf_ctx *h, T **ptr, cudaStream_t s) {
     *ptr = nullptr;
 }
 
+// Frees what it lists when the function that fills it gives up.
+struct Owned {
+    drsf_ctx *h;
+    cudaStream_t s;
+    std::vector<void *> p;
+    template <class T>
+    bool take(T **out, size_t count) {
+        if (!halloc(h, out, count, s)) return false;
+        p.push_back((void *)*out);
+        return true;
+    }
+    void keep() { p.clear(); }
+    ~Owned() {
+        for (void *x : p) hfree(h, &x, s);
+    }
+};
+
 #define CK(x)                                     \
     do {                                          \
         cudaError_t e_ = (x);                     \
@@ -264,6 +281,50 @@ static void hfree(drsf_ctx *h, T **ptr, cudaStream_t s) {
 static cudaError_t storage_moved(drsf_ctx *h, cudaStream_t s) {
     h->gen++;
     return cudaMemcpyAsync(&h->ctl->storage, &h->gen, sizeof h->gen, cudaMemcpyHostToDevice, s);
+}
+
+// Larger work arrays in place of some (their contents are scratch): allocated
+// beside the old ones, or, without room for both, after giving those up; when
+// that fails too the old sizes are taken again and the handle is as it was.
+// (launches: captured ones refer to them.)
+struct Work {
+    void **p;
+    size_t old_bytes, bytes;
+    bool ones;   // starts filled with ones
+};
+static bool take_work(drsf_ctx *h, const std::vector<Work> &w, bool old, std::vector<char *> *got, cudaStream_t s) {
+    Owned own{h, s, {}};
+    for (const Work &x : w) {
+        const size_t bytes = old ? x.old_bytes : x.bytes;
+        char *p = nullptr;
+        if (bytes && !own.take(&p, bytes)) return false;
+        if (p && x.ones && cudaMemsetAsync(p, 0xFF, bytes, s) != cudaSuccess) return false;
+        got->push_back(p);
+    }
+    own.keep();
+    return true;
+}
+static drsf_status regrow(drsf_ctx *h, const std::vector<Work> &w, cudaStream_t s, bool launches = true) {
+    std::vector<char *> got;
+    bool ok = take_work(h, w, false, &got, s), back = false;
+    for (const Work &x : w) hfree(h, (char **)x.p, s);
+    if (!ok) {
+        got.clear();
+        ok = take_work(h, w, false, &got, s);
+    }
+    if (!ok) {
+        got.clear();
+        back = take_work(h, w, true, &got, s);
+        if (!back) h->poisoned = true;
+    }
+    if (ok || back)
+        for (size_t i = 0; i < w.size(); ++i) *w[i].p = got[i];
+    if (launches) CK(storage_moved(h, s));
+    return ok ? DRSF_OK : DRSF_ENOMEM;
+}
+template <class T>
+static Work work(T **p, size_t old_count, size_t count, bool ones = false) {
+    return Work{(void **)p, *p ? old_count * sizeof(T) : 0, count * sizeof(T), ones};
 }
 
 static bool capturing(cudaStream_t s) {
@@ -311,7 +372,8 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     long long headroom = std::max<long long>(std::max<long long>(m / 2, 1 << 12), 2 * extra);
     u64 H = pow2_at_least((u64)(2 * (m + headroom)));
     Index ix{};
-    CKA(halloc(h, &ix.e, H, s));
+    Owned own{h, s, {}};   // the new storage, until it is swapped in
+    CKA(own.take(&ix.e, H));
     ix.mask = H - 1;
     CK(cudaMemsetAsync(ix.e, 0xFF, H * sizeof(Entry), s));
 
@@ -331,6 +393,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     t.add(&off, (size_t)n + 1);
     t.add(&bs, (size_t)tiles);
     CKA(t.take(h, &tmp, s));
+    Owned temps{h, s, {tmp}};
     CK(cudaMemsetAsync(cnt, 0, 4 * sizeof(u64), s));
     CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(int), s));
     if (m > 0) CK(launch_create_claim(edges, m, ix, dkey, dslot, cnt, (long long *)(cnt + 1), s));
@@ -347,9 +410,9 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     if (total >= (long long)POS_OVF - 1) return DRSF_ENOMEM;   // positions are 32-bit
     int *col = nullptr, *fpos = nullptr;
     Row *row = nullptr;
-    CKA(halloc(h, &col, (size_t)total, s));
-    CKA(halloc(h, &fpos, (size_t)total, s));
-    CKA(halloc(h, &row, (size_t)n + 1, s));
+    CKA(own.take(&col, (size_t)total));
+    CKA(own.take(&fpos, (size_t)total));
+    CKA(own.take(&row, (size_t)n + 1));
     CK(cudaMemsetAsync(col, 0xFF, (size_t)total * sizeof(int), s));
     CK(cudaMemsetAsync(fpos, 0xFF, (size_t)total * sizeof(int), s));
     CK(launch_rows_init(off, deg, n, row, s));
@@ -357,28 +420,26 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     CK(launch_fill(dkey, dslot, place, m2, g, ix, s));
     u64 ovf_cap = std::max<u64>(std::max<u64>(1u << 16, (u64)m2 / 16), (u64)(2 * extra));
     u64 *ovf = nullptr;
-    CKA(halloc(h, &ovf, 2 * ovf_cap, s));   // (Ovf's three arrays)
+    CKA(own.take(&ovf, 2 * ovf_cap));   // (Ovf's three arrays)
     // candidate buffers: every live undirected edge at most once
     u64 need = (u64)total / 2 + ovf_cap + 1024;
     if (need > h->cand_cap) {
+        std::vector<Work> w;
         for (int b = 0; b < 2; ++b) {
-            hfree(h, &h->ck[b], s);
-            hfree(h, &h->ca[b], s);
-            hfree(h, &h->cb[b], s);
+            w.push_back(work(&h->ck[b], h->cand_cap, need));
+            w.push_back(work(&h->ca[b], h->cand_cap, need));
+            w.push_back(work(&h->cb[b], h->cand_cap, need));
         }
-        for (int b = 0; b < 2; ++b) {
-            CKA(halloc(h, &h->ck[b], need, s));
-            CKA(halloc(h, &h->ca[b], need, s));
-            CKA(halloc(h, &h->cb[b], need, s));
-        }
+        const drsf_status st = regrow(h, w, s);
+        if (st) return st;
         h->cand_cap = need;
     }
     // tiles of the scanned rows: at most one per 32 CSR slots, plus one; or
     // the jobs of long rows (k_scan), two words per 32 slots at most
     const long long ntile = total / 16 + 2;
     if (ntile > h->tile_cap) {
-        hfree(h, &h->tile, s);
-        CKA(halloc(h, &h->tile, (size_t)ntile, s));
+        const drsf_status st = regrow(h, {work(&h->tile, (size_t)h->tile_cap, (size_t)ntile)}, s);
+        if (st) return st;
         h->tile_cap = ntile;
     }
     CK(cudaStreamSynchronize(s));
@@ -396,7 +457,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     h->col_cap = total;
     h->ovf = ovf;
     h->ovf_cap = ovf_cap;
-    hfree(h, &tmp, s);
+    own.keep();
     h->occ_bound = m2;
     h->ovf_bound = 0;
     h->ctomb_bound = 0;
@@ -410,24 +471,16 @@ static drsf_status ensure_batch(drsf_ctx *h, long long len, cudaStream_t s) {
     if (len <= h->batch_cap) return DRSF_OK;
     long long cap = std::max<long long>(len, 1 << 12);
     CK(cudaStreamSynchronize(s));
-    hfree(h, &h->nkey, s);
-    hfree(h, &h->nslot, s);
-    hfree(h, &h->cutlist, s);
-    hfree(h, &h->pt.pk, s);
-    hfree(h, &h->pt.mk, s);
-    CKA(halloc(h, &h->nkey, (size_t)cap, s));
-    CKA(halloc(h, &h->nslot, (size_t)cap, s));
-    CKA(halloc(h, &h->cutlist, (size_t)cap, s));
     // pair table: room for ~2 piece pairs per batch edge at load <= 1/2
     // (a pair that finds no slot falls back to a plain candidate)
-    u64 T = pow2_at_least((u64)cap * 4);
-    CKA(halloc(h, &h->pt.pk, T, s));
-    CKA(halloc(h, &h->pt.mk, T, s));
-    CK(cudaMemsetAsync(h->pt.pk, 0xFF, T * sizeof(u64), s));
-    CK(cudaMemsetAsync(h->pt.mk, 0xFF, T * sizeof(u64), s));
+    const u64 T = pow2_at_least((u64)cap * 4);
+    const size_t was = (size_t)h->batch_cap, is = (size_t)cap;
+    const drsf_status st = regrow(h, {work(&h->nkey, was, is), work(&h->nslot, was, is), work(&h->cutlist, was, is),
+                                      work(&h->pt.pk, h->pt.mask + 1, T, true), work(&h->pt.mk, h->pt.mask + 1, T, true)},
+                                  s);
+    if (st) return st;
     h->pt.mask = T - 1;
     h->batch_cap = cap;
-    CK(storage_moved(h, s));
     return DRSF_OK;
 }
 
@@ -454,8 +507,9 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     long long live = h->ctl_host->edges;
     int *tmp = nullptr;
     u64 *cnt = nullptr;
-    CKA(halloc(h, &tmp, (size_t)std::max<long long>(2 * live, 2), s));
-    CKA(halloc(h, &cnt, 2, s));
+    Owned own{h, s, {}};
+    CKA(own.take(&tmp, (size_t)std::max<long long>(2 * live, 2)));
+    CKA(own.take(&cnt, 2));
     CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(u64), s));
     Csr g{h->row, h->col, h->fpos};
     CK(launch_extract(h->dev, h->n, g, h->ovf, h->ovf_cap, h->ctl, tmp, live, cnt, s));
@@ -468,8 +522,6 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     }
     long long m2 = 0;
     st = build_graph(h, tmp, live, s, &m2, nullptr, extra);
-    hfree(h, &tmp, s);
-    hfree(h, &cnt, s);
     if (st) return st;
     // reset the storage counters of the control block
     Ctl c = *h->ctl_host;
@@ -1109,19 +1161,21 @@ static drsf_status batched_scratch(drsf_ctx *h, cudaStream_t s) {
     BState &b = h->b_st;
     int **iv[] = {&b.J, &b.R, &b.A, &b.Dv, &b.roff, &b.comp, &b.minp, &b.pidx, &b.plist, &b.pdeg, &b.poff, &b.pcur,
                   &b.newroot, &b.flist, &b.chx, &b.chy};
-    for (int **p : iv) CKA(halloc(h, p, n + 1, s));
-    CKA(halloc(h, &b.adj, 2 * n + 2, s));
+    Owned own{h, s, {}};
+    for (int **p : iv) CKA(own.take(p, n + 1));
+    CKA(own.take(&b.adj, 2 * n + 2));
     unsigned **st[] = {&b.st_aff, &b.st_cut, &b.st_piece, &b.st_vis, &b.st_rr};
     for (unsigned **p : st) {
-        CKA(halloc(h, p, n + 1, s));
+        CKA(own.take(p, n + 1));
         CK(cudaMemsetAsync(*p, 0, (n + 1) * sizeof(unsigned), s));
     }
-    CKA(halloc(h, &b.best, n + 1, s));
-    CKA(halloc(h, &b.er, n + 1, s));
-    CKA(halloc(h, &b.pool_ctr, 1, s));
-    CKA(halloc(h, &b.qctr, BCLASSES, s));
-    CKA(halloc(h, &h->b_state, 1, s));
-    CKA(halloc(h, &h->b_desc, 1, s));
+    CKA(own.take(&b.best, n + 1));
+    CKA(own.take(&b.er, n + 1));
+    CKA(own.take(&b.pool_ctr, 1));
+    CKA(own.take(&b.qctr, BCLASSES));
+    CKA(own.take(&h->b_state, 1));
+    CKA(own.take(&h->b_desc, 1));
+    own.keep();
     CK(cudaStreamCreateWithFlags(&h->b_cap, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&h->b_fork, cudaEventDisableTiming));
     for (int c = 0; c < BCLASSES; ++c) {
@@ -1216,49 +1270,36 @@ static bool batched_fits(const drsf_ctx *h, long long G, long long len) {
 // Per-graph arrays for G graphs and the candidate pool for this call.
 static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cudaStream_t s) {
     BState &b = h->b_st;
-    bool moved = false;
     drsf_status st = batched_meta(h, G, s);
     if (st) return st;
     if (h->b_gcap > h->b_gcnt_cap) {
         CK(cudaStreamSynchronize(s));
-        hfree(h, &b.gcnt, s);
-        hfree(h, &b.gcur, s);
-        hfree(h, &b.govf_start, s);
-        CKA(halloc(h, &b.gcnt, (size_t)h->b_gcap + 1, s));
-        CKA(halloc(h, &b.gcur, (size_t)h->b_gcap + 1, s));
-        CKA(halloc(h, &b.govf_start, (size_t)h->b_gcap + 1, s));
+        const size_t was = (size_t)h->b_gcnt_cap + 1, is = (size_t)h->b_gcap + 1;
+        st = regrow(h, {work(&b.gcnt, was, is), work(&b.gcur, was, is), work(&b.govf_start, was, is)}, s);
+        if (st) return st;
         h->b_gcnt_cap = h->b_gcap;
-        moved = true;
     }
     const u64 need = batched_pool(h, G, len);
     if (need > b.pool_cap) {
         CK(cudaStreamSynchronize(s));
-        hfree(h, &b.pk, s);
-        hfree(h, &b.pa, s);
-        hfree(h, &b.pb, s);
-        CKA(halloc(h, &b.pk, need, s));
-        CKA(halloc(h, &b.pa, need, s));
-        CKA(halloc(h, &b.pb, need, s));
+        st = regrow(h, {work(&b.pk, b.pool_cap, need), work(&b.pa, b.pool_cap, need), work(&b.pb, b.pool_cap, need)}, s);
+        if (st) return st;
         b.pool_cap = need;
-        moved = true;
     }
     const long long ntile = batched_tiles(h, G);
     if (ntile > h->b_tile_cap) {
         CK(cudaStreamSynchronize(s));
-        hfree(h, &b.tile, s);
-        CKA(halloc(h, &b.tile, (size_t)ntile, s));
+        st = regrow(h, {work(&b.tile, (size_t)h->b_tile_cap, (size_t)ntile)}, s);
+        if (st) return st;
         h->b_tile_cap = ntile;
-        moved = true;
     }
     // overflow buckets: as large as the overflow list (which a rebuild resizes)
     if (!b.govf || h->b_govf_cap < h->ovf_cap) {
         CK(cudaStreamSynchronize(s));
-        hfree(h, &b.govf, s);
-        CKA(halloc(h, &b.govf, (size_t)h->ovf_cap, s));
+        st = regrow(h, {work(&b.govf, (size_t)h->b_govf_cap, (size_t)h->ovf_cap)}, s);
+        if (st) return st;
         h->b_govf_cap = h->ovf_cap;
-        moved = true;
     }
-    if (moved) CK(storage_moved(h, s));
     return DRSF_OK;
 }
 
@@ -1433,14 +1474,16 @@ drsf_status drsf_apply(drsf_handle h, drsf_op op, const int32_t *batch, int64_t 
 static drsf_status ensure_stage(drsf_ctx *h, long long len, cudaStream_t s) {
     if (len > h->stage_cap) {
         CK(cudaStreamSynchronize(s));
-        if (h->stage_host) cudaFreeHost(h->stage_host);
-        h->stage_host = nullptr;
-        hfree(h, &h->stage_dev, s);
-        long long cap = std::max<long long>(len, 1 << 16);
-        CK(cudaMallocHost((void **)&h->stage_host, (size_t)cap * 2 * sizeof(int)));
-        CKA(halloc(h, &h->stage_dev, (size_t)cap * 2, s));
-        h->stage_cap = cap;
         if (!h->stage_done) CK(cudaEventCreateWithFlags(&h->stage_done, cudaEventDisableTiming));
+        const long long cap = std::max<long long>(len, 1 << 16);
+        int *host = nullptr;
+        CK(cudaMallocHost((void **)&host, (size_t)cap * 2 * sizeof(int)));
+        const drsf_status st = regrow(h, {work(&h->stage_dev, 2 * (size_t)h->stage_cap, 2 * (size_t)cap)}, s, false);
+        std::swap(host, h->stage_host);
+        if (st) std::swap(host, h->stage_host);
+        if (host) cudaFreeHost(host);
+        if (st) return st;
+        h->stage_cap = cap;
         h->stage_pending = false;
     }
     return DRSF_OK;

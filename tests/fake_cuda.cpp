@@ -1,35 +1,38 @@
 // A CUDA runtime for the library's host code on a machine without a GPU:
 // device memory is host memory, kernels are counted by name and not run.
-// What the tests set and read: the allocation that fails, the stream that the
-// caller captures, and counts of launches, waits, pinned allocations and of
+// What the tests set and read: the memory there is, the stream that the caller
+// captures, and counts of launches, waits, pinned allocations and of
 // calls that a capture forbids.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
 #include <cstring>
 #include <map>
-#include <set>
 #include <string>
 
 namespace {
 std::map<const void *, std::string> names;
 std::map<std::string, long long> launched;
-std::set<void *> live;
-long long fail_in = -1;        // allocations until one fails (-1: none does)
+std::map<void *, size_t> live;
+bool deny = false;
+size_t held = 0, room = ~(size_t)0 >> 1;   // bytes allocated, and what there is
 cudaStream_t captured = nullptr;
 bool relaxed = false;
 long long waits = 0, pinned = 0, forbidden = 0, recorded_copies = 0;
 
 cudaError_t get(void **p, size_t n) {
     if (captured && !relaxed) ++forbidden;
-    if (fail_in >= 0 && fail_in-- == 0) return cudaErrorMemoryAllocation;
+    if (deny || n + held > room) return cudaErrorMemoryAllocation;
     *p = calloc(n ? n : 1, 1);
-    live.insert(*p);
+    live[*p] = n;
+    held += n;
     return cudaSuccess;
 }
 cudaError_t put(void *p) {
     if (captured && !relaxed) ++forbidden;
-    if (p && live.erase(p) == 0) abort();
+    if (p && !live.count(p)) abort();
+    if (p) held -= live[p];
+    live.erase(p);
     free(p);
     return cudaSuccess;
 }
@@ -55,13 +58,15 @@ cudaStream_t cfg_s;
 
 #pragma GCC visibility push(default)
 extern "C" {
-void fake_fail_alloc(long long k) { fail_in = k; }
+// memory for `more` bytes beside what is held (< 0: no limit)
+void fake_room(long long more) { room = more < 0 ? ~(size_t)0 >> 1 : held + (size_t)more; }
 void fake_capture(void *s) { captured = (cudaStream_t)s; }
 long long fake_waits() { return waits; }
 long long fake_pinned() { return pinned; }
 long long fake_forbidden() { return forbidden; }
 long long fake_recorded_copies() { return recorded_copies; }
-long long fake_live() { return (long long)live.size(); }
+void fake_deny(int on) { deny = on; }   // no memory at all
+long long fake_held() { return (long long)held; }
 // launches since the last call, of kernels whose (mangled) name holds `part`
 long long fake_launches(const char *part) {
     long long n = 0;
@@ -99,10 +104,15 @@ cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3, dim3, void **, size
 cudaError_t cudaMalloc(void **p, size_t n) { return get(p, n); }
 cudaError_t cudaFree(void *p) { return put(p); }
 cudaError_t cudaMallocHost(void **p, size_t n) {
+    if (captured && !relaxed) ++forbidden;
     ++pinned;
-    return get(p, n);
+    *p = calloc(n ? n : 1, 1);
+    return cudaSuccess;
 }
-cudaError_t cudaFreeHost(void *p) { return put(p); }
+cudaError_t cudaFreeHost(void *p) {
+    free(p);
+    return cudaSuccess;
+}
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) {
     memcpy(d, s, n);
     return cudaSuccess;

@@ -35,9 +35,9 @@ def load(tmp):
     lib.drsf_sync.argtypes = [vp, vp]
     lib.drsf_destroy.argtypes = [vp]
     lib.fake_capture.argtypes = [vp]
-    lib.fake_fail_alloc.argtypes = [i64]
+    lib.fake_room.argtypes = [i64]
     lib.fake_launches.argtypes = [ctypes.c_char_p]
-    for name in ("waits", "pinned", "forbidden", "recorded_copies", "live", "launches"):
+    for name in ("waits", "pinned", "forbidden", "recorded_copies", "held", "launches"):
         getattr(lib, "fake_" + name).restype = i64
     _lib = lib
     return lib
@@ -77,5 +77,5 @@ class Handle:
 
     def close(self):
         self.lib.fake_capture(None)
-        self.lib.fake_fail_alloc(-1)
+        self.lib.fake_room(-1)
         self.lib.drsf_destroy(self.h)

@@ -17,11 +17,11 @@ def handle(tmp_path_factory):
 def test_calls_after_reserve_allocate_nothing(handle, size):
     lib = handle.lib
     assert lib.drsf_reserve(handle.h, size, handle.STREAM) == drsf.OK
-    before = lib.fake_pinned(), lib.fake_live()
+    before = lib.fake_pinned(), lib.fake_held()
     assert lib.drsf_sync(handle.h, handle.STREAM) == drsf.OK
     for k in range(3):
         for op in (drsf.INSERT, drsf.DELETE):
             assert handle.apply(op, min(size, 1000), host=True) == drsf.OK
             assert handle.apply(op, min(size, 1000)) == drsf.OK
             assert lib.drsf_sync(handle.h, handle.STREAM) == drsf.OK
-    assert (lib.fake_pinned(), lib.fake_live()) == before
+    assert (lib.fake_pinned(), lib.fake_held()) == before
