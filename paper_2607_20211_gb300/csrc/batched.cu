@@ -354,8 +354,7 @@ __device__ void b_delete(const Grp &G, const BState &S, const BDesc &d, int v0, 
             ovf_give(ctl, S.ovf, S.g, pos.y, u, v);
         } else {
             const int lo = (int)klo(key), hi = (int)khi(key);
-            row_give(S.g, lo, S.g.row[lo].start, pos.x);
-            row_give(S.g, hi, S.g.row[hi].start, pos.y);
+            row_give2(S.g, lo, S.g.row[lo].start, pos.x, hi, S.g.row[hi].start, pos.y);
             dead += 2;
         }
         int c = -1, rc = -1;

@@ -366,8 +366,7 @@ __global__ void k_del_claim(Index ix, Csr g, Ovf ovf, int *parent, const int *re
                     if (pos.x == POS_OVF) {
                         ovf_give(ctl, ovf, g, pos.y, u, v);
                     } else {
-                        row_give(g, u < v ? u : v, u < v ? st_u : st_v, pos.x);
-                        row_give(g, u < v ? v : u, u < v ? st_v : st_u, pos.y);
+                        row_give2(g, u, st_u, u < v ? pos.x : pos.y, v, st_v, u < v ? pos.y : pos.x);
                         dead += 2;
                     }
                     if (par_u == v) {

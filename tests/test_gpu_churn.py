@@ -180,3 +180,34 @@ def test_edges_of_a_full_hub_leave_and_come_back(b, batched):
                               np.union1d(keys, workloads.edges_to_keys(e)))
     finally:
         f.close()
+
+
+def test_removal_at_a_hub_costs_what_it_costs_elsewhere():
+    """Half a million edges of one vertex removed from rows and index in less
+    than twice the time of as many spread over all vertices (an atomic per edge
+    on the hub's row took more than three times as long)."""
+    n, b = 1 << 20, 500_000
+    rng = np.random.default_rng(2)
+    v = np.arange(1, n)
+    star = np.stack([np.zeros(n - 1, np.int64), v], 1)
+    rest = workloads.keys_to_edges(np.unique(workloads.edges_to_keys(np.stack([v, rng.permutation(v)], 1))))
+    rest = rest[rest[:, 0] != rest[:, 1]]
+    g = workloads.Graph.__new__(workloads.Graph)
+    g.name, g.n, g.W, g.keys = "star", n, 0, np.union1d(workloads.edges_to_keys(star), workloads.edges_to_keys(rest))
+    g.parent = np.zeros(n, np.int32)
+    f = make_forest(g)
+    ms = {}
+    try:
+        for name, e in (("spread", rest), ("hub", star)):
+            d = torch.from_numpy(np.ascontiguousarray(rng.permutation(e)[:b], np.int32)).cuda()
+            for _ in range(3):
+                f.delete(d)
+                f.insert(d)
+            f.profile_start(16)
+            for _ in range(8):
+                f.delete(d)
+                f.insert(d)
+            ms[name] = f.profile_stop()["delete"]["del_claim"][0]
+        assert ms["hub"] < 2 * ms["spread"], ms
+    finally:
+        f.close()
