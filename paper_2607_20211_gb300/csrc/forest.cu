@@ -1177,15 +1177,36 @@ __device__ __forceinline__ void hm_min(HotMin &t, u64 *arr, int idx, u64 k, bool
     }
     if (k < __ldcg(&arr[idx])) atomicMin(&arr[idx], k);
 }
-// bestn[idx] = EMPTY_KEY, once per block for the table's indices
+// arr[idx] = EMPTY_KEY, once per block for the table's indices, and for the
+// others by whoever still finds a key there.  (With a match of all lanes'
+// indices and a store for each one an insert of 1M edges between 1,000 trees
+// hooked for 1,195 us instead of 995.)
 __device__ __forceinline__ void hm_reset(HotMin &t, u64 *arr, int idx, bool pred) {
     unsigned m = __ballot_sync(__activemask(), pred);
     if (!pred) return;
-    unsigned grp = __match_any_sync(m, idx);
-    if ((int)(threadIdx.x & 31) != __ffs(grp) - 1) return;
-    int sl = __popc(grp) > 1 ? hm_slot(t, idx, true) : -1;
-    if (sl >= 0) t.rst[sl] = 1;
-    else arr[idx] = EMPTY_KEY;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int round = 0; round < 2; ++round) {
+        const int l0 = __ffs(m) - 1, i0 = __shfl_sync(m, idx, l0);
+        const unsigned g = __ballot_sync(m, idx == i0);
+        if (__popc(g) > 1) {
+            if (idx == i0) {
+                if (lane == l0) {
+                    const int sl = hm_slot(t, idx, true);
+                    if (sl >= 0) t.rst[sl] = 1;
+                    else if (arr[idx] != EMPTY_KEY) arr[idx] = EMPTY_KEY;
+                }
+                return;
+            }
+            m &= ~g;
+            if (!m) return;
+        } else if (round == 0) {
+            if (lane == l0) break;
+            m &= ~g;
+            if (!m) return;
+        }
+    }
+    if (arr[idx] != EMPTY_KEY) arr[idx] = EMPTY_KEY;
 }
 // sends the table's minima to arr (min) and its resets to rst_arr, then
 // clears it; every thread of the block calls it
@@ -1201,6 +1222,20 @@ __device__ __forceinline__ void hm_flush(HotMin &t, u64 *arr, u64 *rst_arr) {
         t.rst[i] = 0;
     }
     __syncthreads();
+}
+
+// Roots of both ends of a candidate, walked side by side.  Nobody hooks
+// meanwhile, and a barrier lies behind those who did: the entries may come from
+// L1 (the roots of few components are read by all candidates).  One after the
+// other and from L2 they took 130 of the 995 us above.
+__device__ __forceinline__ void find_roots(const int *comp, int &a, int &b, Ctl *ctl) {
+    for (int it = 0; it < (1 << 24); ++it) {
+        const int pa = comp[a], pb = comp[b];
+        if (pa == a && pb == b) return;
+        a = pa;
+        b = pb;
+    }
+    atomicOr(&ctl->err, ERR_ROUNDS);
 }
 
 // Replacement edges by hook-and-compress over the trees of F^ (pieces).
@@ -1243,13 +1278,12 @@ __device__ __forceinline__ int hook_rounds(Ctl *ctl, HotMin &hm, int r, long lon
         // phase A: roots of both ends, per-component minimum key
         for (long long i = T; i < c; i += S) {
             int a = LD(ca[i]), b = LD(cb[i]);
+            const u64 k = LD(ck[i]);
             if (r > 0) {   // every endpoint is its own root in round 0
-                a = find_root_ro(comp, a, ctl);
-                b = find_root_ro(comp, b, ctl);
+                find_roots(comp, a, b, ctl);
                 ca[i] = a;
                 cb[i] = b;
             }
-            u64 k = LD(ck[i]);
             hm_min(hm, best, a, k, a != b);
             hm_min(hm, best, b, k, a != b);
         }
@@ -1270,15 +1304,17 @@ __device__ __forceinline__ int hook_rounds(Ctl *ctl, HotMin &hm, int r, long lon
                 k = LD(ck[i]);
             }
             if (alive) {
-                bool ba = __ldcg(&best[a]) == k, bb = __ldcg(&best[b]) == k;
+                const bool ba = best[a] == k, bb = best[b] == k;   // (final since the barrier: from L1)
                 if (ba && bb) comp[a > b ? a : b] = a > b ? b : a;
                 else if (ba) comp[a] = b;
                 else if (bb) comp[b] = a;
                 hook = ba || bb;
                 keep = !hook;
             }
-            hm_reset(hm, bestn, a, alive);
-            hm_reset(hm, bestn, b, alive);
+            if (r > 0) {   // (both arrays start empty)
+                hm_reset(hm, bestn, a, alive);
+                hm_reset(hm, bestn, b, alive);
+            }
             hooked |= hook;
             long long pe = block_append(&ctl->ner, hook);
             if (hook) {

@@ -122,3 +122,25 @@ def test_deep_super_forests_take_logarithmic_rounds(shape, b):
         check_batch(f, n, keys, par, drsf.INSERT, e)
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("flags", [0, drsf.REPL_SG])
+@pytest.mark.parametrize("trees,b", [(2, 30_000), (16, 30_000), (17, 300_000), (100, 100_000), (1000, 400_000)])
+def test_parallel_edges_between_few_trees(trees, b, flags):
+    """Inserts whose every edge joins two of a few trees: minima and resets of
+    few components by all candidates, over several rounds on the grid."""
+    n = 200_000
+    v = np.arange(n)
+    star = np.stack([v % trees, v], 1)[trees:]
+    g = _tiny_graph(n, star.tolist(), v % trees)
+    rng = np.random.default_rng(trees)
+    e = rng.integers(0, n, (b, 2))
+    e = e[(e[:, 0] % trees) != (e[:, 1] % trees)].astype(np.int32)
+    f = make_forest(g, flags=drsf.DETERMINISTIC | flags)
+    try:
+        keys, par, st = check_batch(f, n, g.keys, g.parent, drsf.INSERT, e)
+        assert st["replacement"] == trees - 1
+        keys, par, _ = check_batch(f, n, keys, par, drsf.DELETE, e)
+        check_batch(f, n, keys, par, drsf.INSERT, e[: b // 2])
+    finally:
+        f.close()
