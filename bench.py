@@ -22,7 +22,6 @@ an independent replica (the update of one graph does not shard).
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -232,23 +231,6 @@ def phase_bytes(st: dict, n: int, op: int) -> dict:
     return out
 
 
-def ncu_traffic(kernel_phase: str):
-    """DRAM bytes per launch from a committed ncu summary, if it was taken
-    on the current source of that kernel."""
-    path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
-    if not os.path.exists(path):
-        return None
-    try:
-        d = json.load(open(path)).get(kernel_phase)
-        if not d:
-            return None
-        src = os.path.join(ROOT, d["source"])
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-        return d["bytes_per_launch"] if sha == d["source_sha"] else None
-    except Exception:
-        return None
-
-
 # ------------------------------------------------------------ our arm
 
 def plan(g, cfg, steps, b, seed):
@@ -385,7 +367,7 @@ def run_ours(args, rank, ws, local):
     roofline = {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "phase_timing": "CUDA events around each phase over the same K steps, replayed on a fresh handle "
                                 "with direct launches (the timed run replays captured CUDA graphs)",
-                "frac": round(achieved / peak, 4), "traffic": ncu_traffic(dom),
+                "frac": round(achieved / peak, 4),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic_bytes_per_launch": int(per_launch_bytes),
                 "ms_per_launch": round(per_launch_ms, 5)}
@@ -524,8 +506,8 @@ def replacement_variants(g, edges_d, parent_d, dev_batches, W, K, flush, stream)
         f.close()
         out[name] = {"insert_ms": round(float(np.median(ms[0])), 4), "delete_ms": round(float(np.median(ms[1])), 4),
                      "insert_candidates": int(np.mean(cands[0])), "delete_candidates": int(np.mean(cands[1]))}
-    out["what"] = (f"median batch time over {K} steps after {W} warm-up, each variant forced; the default "
-                   "picks per batch (SG when the key edges exceed n/16)")
+    out["what"] = (f"median batch time over {K} steps after {W} warm-up, each variant forced; the default is HS "
+                   "for inserts and, for deletes, SG when the key edges exceed n/16")
     return out
 
 

@@ -866,7 +866,7 @@ __global__ void k_bbegin(const BState *Sp) {
         storage_guard(ctl, storage_counts(ctl), d.lim, d.op, d.len, ctl->epoch);
         ctl->op = d.op;
         ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
-        ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
+        ctl->scanned = ctl->self_loops = ctl->dropped = 0;
         ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
         ctl->jump_visits = 0;
         ctl->td = ctl->need_root = 0;

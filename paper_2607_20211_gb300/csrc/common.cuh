@@ -81,7 +81,6 @@ struct Ctl {
     long long scanned;      // adjacency entries scanned
     long long self_loops;
     long long dropped;
-    long long tree_cut;
     long long hook_rounds;
     long long rank_rounds;
     long long mark_rounds;

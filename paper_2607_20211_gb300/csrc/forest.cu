@@ -123,7 +123,7 @@ __global__ void k_begin(Ctl *ctl, BeginArgs a) {
     ctl->epoch = epoch;
     ctl->op = op;
     ctl->nb = ctl->ncut = ctl->naff = ctl->ndet = ctl->ncand = ctl->ner = ctl->npc = ctl->nact = 0;
-    ctl->scanned = ctl->self_loops = ctl->dropped = ctl->tree_cut = 0;
+    ctl->scanned = ctl->self_loops = ctl->dropped = 0;
     ctl->hook_rounds = ctl->rank_rounds = ctl->mark_rounds = ctl->jump_rounds = ctl->reversed = 0;
     ctl->jump_visits = 0;
     ctl->nagain[0] = ctl->nagain[1] = 0;
