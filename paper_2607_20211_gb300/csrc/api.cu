@@ -34,7 +34,7 @@ struct drsf_ctx {
     void *alloc_ctx = nullptr;
     std::vector<Buf> bufs;
     bool poisoned = false;
-    int jump_sync = 2;   // root search: 2 hops, then asynchronous doubling; 1 synchronous rounds, 0 path halving
+    int jump_sync = 2;   // root search: 2 a few hops, then asynchronous jumping; 1 synchronous rounds, 0 path halving
     int last_sg = 0;     // the last batch took the supergraph variant
     // batches that the caller recorded into graphs of its own: the host's
     // bounds below miss their replays, and their host arguments are kept on
@@ -43,7 +43,7 @@ struct drsf_ctx {
     std::vector<void *> kept;
     // captured per-batch launch sequences (CUDA graphs), valid for storage
     // generation u_gen; gen moves whenever a storage or batch buffer moves
-    // (storage_moved; the control block has it too)
+    // (publish_storage; the control block has it too)
     struct Captured {
         std::string key;
         cudaGraphExec_t exec;
@@ -57,7 +57,9 @@ struct drsf_ctx {
     cudaStream_t u_cap = nullptr;
 
     Ctl *ctl = nullptr;
-    Ctl *ctl_host = nullptr;   // pinned
+    Ctl *ctl_host = nullptr;   // pinned, once reserved or read by the caller
+    Ctl ctl_page{};            // what batches read the counts into before that
+    const Ctl *seen = nullptr; // the last copy read
 
     // forest
     int *parent = nullptr, *rep = nullptr;
@@ -275,52 +277,49 @@ struct Owned {
         if (!(x)) return DRSF_ENOMEM;             \
     } while (0)
 
-// Storage or batch buffers moved: captured launch sequences point into the old
-// ones.  The handle drops its own; a graph of the caller's finds out by the
-// control block (StorageLimits).
-static cudaError_t storage_moved(drsf_ctx *h, cudaStream_t s) {
-    h->gen++;
+// Storage or batch buffers moved (h->gen went on): captured launch sequences
+// point into the old ones.  The handle drops its own; a graph of the caller's
+// finds out by the control block (StorageLimits), which has to have the new
+// generation before the next batch.
+static cudaError_t publish_storage(drsf_ctx *h, cudaStream_t s) {
     return cudaMemcpyAsync(&h->ctl->storage, &h->gen, sizeof h->gen, cudaMemcpyHostToDevice, s);
 }
 
-// Larger work arrays in place of some (their contents are scratch): allocated
-// beside the old ones, or, without room for both, after giving those up; when
-// that fails too the old sizes are taken again and the handle is as it was.
-// (launches: captured ones refer to them.)
+// Larger work arrays in place of some (their contents are scratch).  The old
+// ones are given up first: an allocator that keeps what it is given back serves
+// the new ones from them (allocated beside them, a rebuild took 0.2 to 0.5 ms
+// more).  Without room for the new sizes the old ones are taken again, and the
+// handle is as it was.  (launches: captured ones refer to the arrays.)
 struct Work {
     void **p;
     size_t old_bytes, bytes;
     bool ones;   // starts filled with ones
 };
-static bool take_work(drsf_ctx *h, const std::vector<Work> &w, bool old, std::vector<char *> *got, cudaStream_t s) {
+static bool take_work(drsf_ctx *h, const std::vector<Work> &w, bool old, cudaStream_t s) {
     Owned own{h, s, {}};
+    std::vector<char *> got;
     for (const Work &x : w) {
         const size_t bytes = old ? x.old_bytes : x.bytes;
         char *p = nullptr;
         if (bytes && !own.take(&p, bytes)) return false;
         if (p && x.ones && cudaMemsetAsync(p, 0xFF, bytes, s) != cudaSuccess) return false;
-        got->push_back(p);
+        got.push_back(p);
     }
     own.keep();
+    for (size_t i = 0; i < w.size(); ++i) *w[i].p = got[i];
     return true;
 }
 static drsf_status regrow(drsf_ctx *h, const std::vector<Work> &w, cudaStream_t s, bool launches = true) {
-    std::vector<char *> got;
-    bool ok = take_work(h, w, false, &got, s), back = false;
     for (const Work &x : w) hfree(h, (char **)x.p, s);
-    if (!ok) {
-        got.clear();
-        ok = take_work(h, w, false, &got, s);
-    }
-    if (!ok) {
-        got.clear();
-        back = take_work(h, w, true, &got, s);
-        if (!back) h->poisoned = true;
-    }
-    if (ok || back)
-        for (size_t i = 0; i < w.size(); ++i) *w[i].p = got[i];
-    if (launches) CK(storage_moved(h, s));
-    return ok ? DRSF_OK : DRSF_ENOMEM;
+    if (launches) h->gen++;
+    if (take_work(h, w, false, s)) return DRSF_OK;
+    if (!take_work(h, w, true, s)) h->poisoned = true;
+    return DRSF_ENOMEM;
+}
+static drsf_status regrow_published(drsf_ctx *h, const std::vector<Work> &w, cudaStream_t s) {
+    const drsf_status st = regrow(h, w, s);
+    CK(publish_storage(h, s));
+    return st;
 }
 template <class T>
 static Work work(T **p, size_t old_count, size_t count, bool ones = false) {
@@ -461,7 +460,7 @@ static drsf_status build_graph(drsf_ctx *h, const int *edges, long long m, cudaS
     h->occ_bound = m2;
     h->ovf_bound = 0;
     h->ctomb_bound = 0;
-    CK(storage_moved(h, s));
+    h->gen++;   // (the caller writes it with the counts)
     *m_out = m2;
     if (self_loops_out) *self_loops_out = (long long)hc[1];
     return DRSF_OK;
@@ -475,27 +474,28 @@ static drsf_status ensure_batch(drsf_ctx *h, long long len, cudaStream_t s) {
     // (a pair that finds no slot falls back to a plain candidate)
     const u64 T = pow2_at_least((u64)cap * 4);
     const size_t was = (size_t)h->batch_cap, is = (size_t)cap;
-    const drsf_status st = regrow(h, {work(&h->nkey, was, is), work(&h->nslot, was, is), work(&h->cutlist, was, is),
-                                      work(&h->pt.pk, h->pt.mask + 1, T, true), work(&h->pt.mk, h->pt.mask + 1, T, true)},
-                                  s);
+    const drsf_status st = regrow_published(
+        h, {work(&h->nkey, was, is), work(&h->nslot, was, is), work(&h->cutlist, was, is),
+            work(&h->pt.pk, h->pt.mask + 1, T, true), work(&h->pt.mk, h->pt.mask + 1, T, true)}, s);
     if (st) return st;
     h->pt.mask = T - 1;
     h->batch_cap = cap;
     return DRSF_OK;
 }
 
-// The host's copy of the control block: by drsf_reserve, else on first use (a
-// pinned allocation can wait for the device).
+// The pinned copy of the control block: by drsf_reserve, else by the first call
+// that reads the counters for the caller (110 to 220 us where no other handle
+// has one; a batch that reads them does without).
 static drsf_status ensure_ctl_host(drsf_ctx *h) {
     if (!h->ctl_host) CK(cudaMallocHost((void **)&h->ctl_host, sizeof(Ctl)));
     return DRSF_OK;
 }
 
 static drsf_status read_ctl(drsf_ctx *h, cudaStream_t s) {
-    drsf_status st = ensure_ctl_host(h);
-    if (st) return st;
-    CK(cudaMemcpyAsync(h->ctl_host, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
+    Ctl *const dst = h->ctl_host ? h->ctl_host : &h->ctl_page;
+    CK(cudaMemcpyAsync(dst, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    h->seen = dst;
     return DRSF_OK;
 }
 
@@ -504,7 +504,7 @@ static drsf_status read_ctl(drsf_ctx *h, cudaStream_t s) {
 static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     drsf_status st = read_ctl(h, s);
     if (st) return st;
-    long long live = h->ctl_host->edges;
+    long long live = h->seen->edges;
     int *tmp = nullptr;
     u64 *cnt = nullptr;
     Owned own{h, s, {}};
@@ -522,9 +522,12 @@ static drsf_status rebuild(drsf_ctx *h, cudaStream_t s, long long extra) {
     }
     long long m2 = 0;
     st = build_graph(h, tmp, live, s, &m2, nullptr, extra);
-    if (st) return st;
+    if (st) {
+        CK(publish_storage(h, s));   // (work buffers may have moved)
+        return st;
+    }
     // reset the storage counters of the control block
-    Ctl c = *h->ctl_host;
+    Ctl c = *h->seen;
     c.storage = h->gen;
     c.ovf_count = c.ovf_free = 0;
     c.edges = m2;
@@ -554,8 +557,8 @@ static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_
         if (h->recorded || !insert_fits(h, len)) {
             drsf_status st = read_ctl(h, s);
             if (st) return st;
-            long long occ = h->ctl_host->edges + h->ctl_host->htomb;
-            long long ovfc = (long long)(h->ctl_host->ovf_count - h->ctl_host->ovf_free);
+            long long occ = h->seen->edges + h->seen->htomb;
+            long long ovfc = (long long)(h->seen->ovf_count - h->seen->ovf_free);
             h->occ_bound = occ;
             h->ovf_bound = ovfc;
             if (!insert_fits(h, len)) {
@@ -570,7 +573,7 @@ static drsf_status storage_check(drsf_ctx *h, int op, long long len, cudaStream_
         if (h->ctomb_bound > h->col_cap / 4) {
             drsf_status st = read_ctl(h, s);
             if (st) return st;
-            long long ct = h->ctl_host->ctomb;
+            long long ct = h->seen->ctomb;
             h->ctomb_bound = ct;
             if (ct > h->col_cap / 4) {
                 st = rebuild(h, s, len);
@@ -758,6 +761,7 @@ static drsf_status create_impl(drsf_ctx *h, const int32_t *edges, int64_t m, con
         if (hb[0]) return DRSF_ENOT_FOREST;
     }
     hfree(h, &bad, s);
+    c.storage = h->gen;
     c.edges = m2;
     c.self_loops = loops;
     CK(cudaMemcpyAsync(h->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
@@ -802,8 +806,8 @@ drsf_status drsf_create(int32_t n, const int32_t *edges, int64_t m, const int32_
     h->dev.coop_et = coop_blocks_et(nsm);
     h->dev.coop_cross = coop_blocks_cross(nsm);
     h->dev.few = n <= FEW_VERTICES;
-    // root search of a delete batch: barrier-free doubling over per-warp
-    // slices by default; DRSF_JUMP=sync selects synchronous doubling rounds,
+    // root search of a delete batch: a few hops and barrier-free jumping over
+    // per-warp lists by default; DRSF_JUMP=sync selects synchronous doubling rounds,
     // DRSF_JUMP=halving the in-place path-halving walks
     const char *jm = getenv("DRSF_JUMP");
     h->jump_sync = jm && strcmp(jm, "halving") == 0 ? 0 : (jm && strcmp(jm, "sync") == 0 ? 1 : 2);
@@ -1275,28 +1279,28 @@ static drsf_status batched_capacity(drsf_ctx *h, long long G, long long len, cud
     if (h->b_gcap > h->b_gcnt_cap) {
         CK(cudaStreamSynchronize(s));
         const size_t was = (size_t)h->b_gcnt_cap + 1, is = (size_t)h->b_gcap + 1;
-        st = regrow(h, {work(&b.gcnt, was, is), work(&b.gcur, was, is), work(&b.govf_start, was, is)}, s);
+        st = regrow_published(h, {work(&b.gcnt, was, is), work(&b.gcur, was, is), work(&b.govf_start, was, is)}, s);
         if (st) return st;
         h->b_gcnt_cap = h->b_gcap;
     }
     const u64 need = batched_pool(h, G, len);
     if (need > b.pool_cap) {
         CK(cudaStreamSynchronize(s));
-        st = regrow(h, {work(&b.pk, b.pool_cap, need), work(&b.pa, b.pool_cap, need), work(&b.pb, b.pool_cap, need)}, s);
+        st = regrow_published(h, {work(&b.pk, b.pool_cap, need), work(&b.pa, b.pool_cap, need), work(&b.pb, b.pool_cap, need)}, s);
         if (st) return st;
         b.pool_cap = need;
     }
     const long long ntile = batched_tiles(h, G);
     if (ntile > h->b_tile_cap) {
         CK(cudaStreamSynchronize(s));
-        st = regrow(h, {work(&b.tile, (size_t)h->b_tile_cap, (size_t)ntile)}, s);
+        st = regrow_published(h, {work(&b.tile, (size_t)h->b_tile_cap, (size_t)ntile)}, s);
         if (st) return st;
         h->b_tile_cap = ntile;
     }
     // overflow buckets: as large as the overflow list (which a rebuild resizes)
     if (!b.govf || h->b_govf_cap < h->ovf_cap) {
         CK(cudaStreamSynchronize(s));
-        st = regrow(h, {work(&b.govf, (size_t)h->b_govf_cap, (size_t)h->ovf_cap)}, s);
+        st = regrow_published(h, {work(&b.govf, (size_t)h->b_govf_cap, (size_t)h->ovf_cap)}, s);
         if (st) return st;
         h->b_govf_cap = h->ovf_cap;
     }
@@ -1529,7 +1533,7 @@ drsf_status drsf_apply_host(drsf_handle h, drsf_op op, const int32_t *batch, int
 }
 
 static drsf_status latched(drsf_ctx *h) {
-    int e = h->ctl_host->err;
+    int e = h->seen->err;
     if (e & (ERR_TIMEOUT | ERR_CAPACITY | ERR_ROUNDS)) {
         h->poisoned = true;
         return (e & ERR_TIMEOUT) ? DRSF_ETIMEOUT : DRSF_EPOISONED;
@@ -1548,7 +1552,8 @@ drsf_status drsf_sync(drsf_handle h, drsf_stream stream) {
     if (!h) return DRSF_EINVAL;
     if (h->poisoned) return DRSF_EPOISONED;
     set_dev(h);
-    drsf_status st = read_ctl(h, (cudaStream_t)stream);
+    drsf_status st = ensure_ctl_host(h);
+    if (!st) st = read_ctl(h, (cudaStream_t)stream);
     if (st) return st;
     return latched(h);
 }
@@ -1574,9 +1579,10 @@ drsf_status drsf_stats(drsf_handle h, drsf_batch_stats *out, drsf_stream stream)
     if (!h || !out) return DRSF_EINVAL;
     if (h->poisoned) return DRSF_EPOISONED;
     set_dev(h);
-    drsf_status st = read_ctl(h, (cudaStream_t)stream);
+    drsf_status st = ensure_ctl_host(h);
+    if (!st) st = read_ctl(h, (cudaStream_t)stream);
     if (st) return st;
-    const Ctl &c = *h->ctl_host;
+    const Ctl &c = *h->seen;
     out->batch_len = c.batch_len;
     out->self_loops = c.self_loops;
     out->dropped = c.dropped;

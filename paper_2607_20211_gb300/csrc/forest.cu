@@ -309,11 +309,6 @@ __device__ __forceinline__ void warp_detach_append(u64 *vc, u64 *pc, long long v
     warp_list_rows(pc, pb, rl, on && len > 0, w, st, len, p, ro);
 }
 
-// Warp-aggregated list appends of the top-down search (no block barrier):
-// the calling lanes with `on` take consecutive slots of A, those with a
-// non-empty row (`len` > 0) consecutive rows of the row list and their entry
-// ranges, from one atomic per warp on each counter (rows in the high and
-// entries in the low 32 bits of the packed row counter).  All 32 lanes call.
 // Delete, top-down alternative to the pointer jumping of Algorithm 1 (same
 // representatives): the detached vertices are the cut vertices and every
 // descendant of one in the cut forest, and a detached vertex's piece is the
@@ -2172,7 +2167,7 @@ __global__ void __launch_bounds__(ORIENT_THREADS, 1) k_replace(Ctl *ctl, HookArg
         ctl->cnt[1] = ctl->cnt[2] = 0;
         ctl->flag[0] = ctl->flag[1] = ctl->flag[2] = 0;
     }
-    if (h.pairs) {   // 
+    if (h.pairs) {
         compact_pairs(ctl, h.pt, h.ck[0], h.ca[0], h.cb[0], h.cand_cap);
         if (!grid_barrier(ctl, &ctl->bar[1])) return;
     }

@@ -25,3 +25,14 @@ def test_calls_after_reserve_allocate_nothing(handle, size):
             assert handle.apply(op, min(size, 1000)) == drsf.OK
             assert lib.drsf_sync(handle.h, handle.STREAM) == drsf.OK
     assert (lib.fake_pinned(), lib.fake_held()) == before
+
+
+def test_batches_allocate_no_host_memory(handle):
+    """Batches that have to read the counters (and rebuild) without drsf_reserve."""
+    lib = handle.lib
+    p, w = lib.fake_pinned(), lib.fake_waits()
+    for k in range(6):
+        for op in (drsf.DELETE, drsf.INSERT):
+            assert handle.apply(op, 4000) == drsf.OK
+    assert lib.fake_waits() > w and lib.fake_pinned() == p
+    assert lib.drsf_sync(handle.h, handle.STREAM) == drsf.OK and lib.fake_pinned() == p + 1
