@@ -163,9 +163,11 @@ __device__ __forceinline__ void scan_ovf(const u64 *ovf, Ctl *ctl, const int *re
 //      reduced per pair of components through the pair table (SG) or one by
 //      one (HS).
 // A batch that detaches much of a graph has more pairs of pieces than the pair
-// table (or a hash table of any size that fits L2) can take: R-MAT scale 20,
-// 1M deletes, 4.1M pairs; scan and hooking 1,410 + 1,120 us, 437 + 330 in this
-// way.  Few of them are left after the first round.
+// table (or a hash table of any size that fits L2) can take.  Few of them are
+// left after the first round: a window of 1M-edge batches over R-MAT scale 20
+// (W below; its deletes cut 480K tree edges, 4.1M pairs) took 1,410 us to scan
+// and 1,120 to hook with every cross edge as a candidate, and takes 435 and 322
+// with all that is said here.
 //
 // A lane reads a row of up to LONG_ROW entries by itself, LU entries in flight
 // (flattening the rows of a warp by a prefix sum and reading 32 entries per
@@ -419,16 +421,18 @@ __device__ __forceinline__ bool light_hook(const LightArgs &a, int q, u64 *key) 
 // Lists the rows that step 3 reads: those with a cross edge whose component
 // does not hold the piece left out.  From AGAIN_MIN rows on: few rows of many
 // are left (one in ten of those with a cross edge in the 4096 x 4096 grid), and
-// a warp that met one of them among its 32 read it alone.  Scan, us: the grid
-// 404 -> 348, the 256-graph union 635 -> 521, R-MAT scale 20 (1M deletes)
-// 554 -> 524; a list of 100K rows (R-MAT scale 22) keeps too few blocks busy:
-// 72 us without it, 92 with.
+// a warp that met one of them among its 32 read it alone.  Scan, us, without and
+// with the list: the grid 404 and 348, the 256-graph union 635 and 521, W 554
+// and 524.  A shorter list keeps too few blocks busy: R-MAT scale 22 with 98K
+// rows 71 and 88, 179K 103 and 119, 378K 172 and 180; scale 20 with 434K 189 and
+// 196; but 64 graphs with 464K rows 141 and 130: the line lies about here.
 #define AGAIN_MIN (1 << 19)
-// From so many listed rows on, a quarter of all or more, a second round is taken from them, not only the
-// first: most of the graph is in components without the piece left out, and
-// their pairs would fill the pair table (R-MAT scale 20, 1M deletes of a graph
-// that has lost half its tree edges ten times over: 2.5M candidates; scan and
-// hooking 1,400 + 1,320 us, 1,002 + 359 with the round).  With fewer rows the
+// From so many listed rows on, a quarter of all or more, a second round is taken
+// from them, not only the first: most of the graph is in components without the
+// piece left out, and their pairs would fill the pair table (R-MAT scale 20
+// after ten batches of 1M deletes, half of them tree edges, which W is not:
+// 2.5M candidates; scan and hooking 1,400 + 1,320 us, 1,002 + 359 with the
+// round).  With fewer rows the
 // reading costs more than the candidates it saves: at 2^17 the 256-graph
 // union's scan and hooking took 584 + 310 us instead of 521 + 337, the grid's
 // (one row in twenty left) 503 + 185 instead of 347 + 223.
@@ -513,8 +517,8 @@ __device__ __forceinline__ void hook_pieces(Ctl *ctl, const LightArgs &a, long l
 // nothing (a path of more than FLAT_WALK steps is halved as it is walked) and
 // kept aside; after a barrier it is stored.  (Walks that halved every path, and
 // stores of roots beside walks that were still reading, made each other's
-// loads miss: R-MAT scale 20, 1M deletes, 500K pieces, paths of at most 6
-// steps: the whole scan 694 us so, 545 in this way.)
+// loads miss: W, 480K pieces, paths of at most 6 steps: the whole scan 694 us
+// so, 545 in this way.)
 __device__ __forceinline__ bool flatten_pieces(Ctl *ctl, const LightArgs &a, long long nc, u64 *bar) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += (long long)gridDim.x * blockDim.x) {
         int x = __ldcg(&a.comp[a.cuts[i]]);
