@@ -251,7 +251,7 @@ DRSF_API drsf_status drsf_apply_host(drsf_handle h, drsf_op op, const int32_t *b
  * graphs, and every edge of a slice must have both ends in its graph's
  * range (else DRSF_EINVAL is latched and the call is skipped, as for an
  * out-of-range id).  drsf_apply_grouped does the same update faster at every
- * size measured (0.31 of the time of this form with a tuned schedule at 256
+ * size measured (0.3 of the time of this form with a tuned schedule at 256
  * graphs); this form is for graphs whose own measurement says otherwise.
  * Instead of the grid-wide launch sequence, persistent
  * kernels keep one group per graph, a thread-block cluster of
