@@ -249,7 +249,10 @@ class DynamicForest:
 
     # -- updates ----------------------------------------------------------
     def apply(self, op: int, batch: torch.Tensor) -> None:
-        """Enqueue one batch (insert or delete) on the handle's stream."""
+        """Enqueue one batch (insert or delete) on the handle's stream.  While
+        the stream is captured the batch is recorded; each replay applies what
+        the tensor then holds (drsf_apply in include/drsf.h says what voids a
+        recording)."""
         batch = _dev_i32(batch, "batch", 2)
         st = _lib.drsf_apply(self._h, op, batch.data_ptr() if batch.numel() else None,
                              int(batch.shape[0]) if batch.numel() else 0, _stream_ptr(self._stream))

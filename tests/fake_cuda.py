@@ -1,7 +1,6 @@
 """The library's host code on the CPU: its objects linked against the runtime
 of fake_cuda.cpp (device memory is host memory, kernels are counted)."""
 import ctypes
-import glob
 import os
 import subprocess
 
@@ -18,12 +17,16 @@ def load(tmp):
     global _lib
     if _lib is not None:
         return _lib
+    bld = drsf._build_mod
     drsf.build()
+    objs = [os.path.join(bld.BUILD, os.path.basename(src)[:-3] + ".o") for src in bld.sources()]
+    if not all(map(os.path.exists, objs)):
+        drsf.build(force=True)
     out = os.path.join(str(tmp), "libdrsf_fake.so")
-    cuda = os.path.dirname(os.path.dirname(drsf._build_mod._nvcc()))
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(bld._nvcc())))
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-O1", "-fvisibility=hidden", "-Wl,-Bsymbolic",
                     "-I", os.path.join(cuda, "include"), os.path.join(HERE, "fake_cuda.cpp"),
-                    *sorted(glob.glob(os.path.join(drsf._build_mod.BUILD, "*.o"))), "-o", out], check=True)
+                    *objs, "-o", out], check=True)
     lib = ctypes.CDLL(out)
     vp, i32, i64, u32 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_uint32
     lib.drsf_create.argtypes = [i32, vp, i64, vp, u32, vp, ctypes.POINTER(ctypes.c_void_p)]
